@@ -1,6 +1,7 @@
-"""ctypes binding of ``libevln.so``: same names as the C entry points, argument marshalling only.
+"""Binding of ``libevln.so``: same names as the C entry points, argument marshalling only.
 
-Every step of the path runs in the library's CUDA kernels.  PyTorch is used for device memory
+The calls a model makes per layer and step (``kHotCalls``) are CPython built-ins compiled from
+``csrc/py_native.cpp``; the others go through ctypes.  Every step of the path runs in the library's CUDA kernels.  PyTorch is used for device memory
 and streams.  There is no fallback: loading fails loudly when the library has not been built
 (``python -c "import __graft_entry__ as g; g.build()"`` or ``build_library()`` below).
 """
@@ -15,6 +16,7 @@ from ctypes import (POINTER, Structure, byref, c_char_p, c_double, c_float, c_in
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
 LIB_PATH = os.path.join(_PKG, "lib", "libevln.so")
+NATIVE_PATH = os.path.join(_PKG, "lib", "_evln_native.so")
 _SOURCES = ["evln_api.cu", "attn_pair.cuh", "attn_simt.cuh", "combine.cuh", "rope_append.cuh",
             "common.cuh", "ptx_sm100.cuh", "gather_rope.cuh", "timeline_debug.cuh"]
 
@@ -80,11 +82,22 @@ class EvlnError(RuntimeError):
 def build_library(force: bool = False, verbose: bool = False) -> str:
     """Compile the CUDA sources into ``lib/libevln.so`` for sm_100a (in-tree)."""
     src_dir = os.path.join(_PKG, "csrc")
-    srcs = [os.path.join(src_dir, s) for s in _SOURCES] + [os.path.join(_ROOT, "include", "evln.h")]
-    if not force and os.path.exists(LIB_PATH) and all(
-            os.path.getmtime(LIB_PATH) >= os.path.getmtime(s) for s in srcs):
-        return LIB_PATH
+    header = os.path.join(_ROOT, "include", "evln.h")
+    srcs = [os.path.join(src_dir, s) for s in _SOURCES] + [header]
     os.makedirs(os.path.dirname(LIB_PATH), exist_ok=True)
+
+    def fresh(path, sources):
+        return not force and os.path.exists(path) and all(os.path.getmtime(path) >= os.path.getmtime(s) for s in sources)
+
+    if not fresh(LIB_PATH, srcs):
+        _build_cuda(src_dir, verbose)
+    native_src = os.path.join(src_dir, "py_native.cpp")
+    if not fresh(NATIVE_PATH, [native_src, header]):
+        _build_native(native_src)
+    return LIB_PATH
+
+
+def _build_cuda(src_dir, verbose):
     tmp = LIB_PATH + f".tmp{os.getpid()}"
     cmd = ["nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
            "-shared", "-Xcompiler", "-fPIC", "-o", tmp, os.path.join(src_dir, "evln_api.cu")]
@@ -92,7 +105,22 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         cmd.insert(1, "-Xptxas=-v")
     subprocess.check_call(cmd)
     os.replace(tmp, LIB_PATH)
-    return LIB_PATH
+
+
+def _build_native(src):
+    """The CPython module of the hot calls (``lib/_evln_native.so``), against torch's C++ headers."""
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension
+    lib_dir, torch_lib = os.path.dirname(LIB_PATH), os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = NATIVE_PATH + f".tmp{os.getpid()}"
+    includes = cpp_extension.include_paths("cuda") + [sysconfig.get_paths()["include"]]
+    subprocess.check_call(
+        ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+        + [a for d in includes for a in ("-isystem", d)] + ["-o", tmp, src, "-L", lib_dir, "-levln", "-L", torch_lib]
+        + ["-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10", "-Wl,-rpath,$ORIGIN", f"-Wl,-rpath,{torch_lib}"])
+    os.replace(tmp, NATIVE_PATH)
 
 
 _lib = None
@@ -244,12 +272,6 @@ def evlnRopeTableBytes(head_dim: int, count: int) -> int:
     return int(lib().evlnRopeTableBytes(int(head_dim), int(count)))
 
 
-def evlnRopeTable(handle, head_dim, rope_theta, first_pos, count, table, stream=None):
-    """(cos, sin) of the positions first_pos .. first_pos+count-1 into ``table`` (device memory)."""
-    _check(lib().evlnRopeTable(handle, int(head_dim), float(rope_theta), int(first_pos), int(count), _ptr(table),
-                               _stream(stream)), "evlnRopeTable")
-
-
 def evlnPagedCheckTable(params, cache_lens, new_offsets, page_table_rows):
     """Host check of a page table given as ``[batch][max_pages_per_seq]`` ints (flattened or nested).
     Returns (status, bad_episode, bad_index)."""
@@ -277,73 +299,11 @@ def evlnStepQRotSize(handle, params) -> int:
     return int(v.value)
 
 
-def evlnRopeAppend(handle, params, q_new, k_new, v_new, q_rot, k_cache, v_cache, stream=None,
-                   strides=None):
-    """q_new/k_new/v_new: [n,H,D] tensors (last two dims contiguous) or raw addresses + strides."""
-    if strides is None:
-        strides = (q_new.stride(0), k_new.stride(0), v_new.stride(0))
-    _check(lib().evlnRopeAppend(handle, byref(params), _ptr(q_new), _ptr(k_new), _ptr(v_new),
-                                int(strides[0]), int(strides[1]), int(strides[2]), _ptr(q_rot),
-                                _ptr(k_cache), _ptr(v_cache), _stream(stream)), "evlnRopeAppend")
-
-
-def evlnStepAttention(handle, params, q_rot, k_cache, v_cache, workspace, workspace_bytes=None,
-                      stream=None):
-    if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    _check(lib().evlnStepAttention(handle, byref(params), _ptr(q_rot), _ptr(k_cache), _ptr(v_cache),
-                                   _ptr(workspace), int(workspace_bytes), _stream(stream)),
-           "evlnStepAttention")
-
-
-def evlnStepCombine(handle, params, workspace, out, lse_out=None, stream=None):
-    _check(lib().evlnStepCombine(handle, byref(params), _ptr(workspace), _ptr(out), _ptr(lse_out),
-                                 _stream(stream)), "evlnStepCombine")
-
-
-def evlnStep(handle, params, q_new, k_new, v_new, q_rot, k_cache, v_cache, workspace, out, lse_out=None,
-             workspace_bytes=None, stream=None, strides=None):
-    """The three calls of a step in one."""
-    if strides is None:
-        strides = (q_new.stride(0), k_new.stride(0), v_new.stride(0))
-    if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    _check(lib().evlnStep(handle, byref(params), _ptr(q_new), _ptr(k_new), _ptr(v_new), int(strides[0]),
-                          int(strides[1]), int(strides[2]), _ptr(q_rot), _ptr(k_cache), _ptr(v_cache),
-                          _ptr(workspace), int(workspace_bytes), _ptr(out), _ptr(lse_out), _stream(stream)),
-           "evlnStep")
-
-
 def evlnPagedWorkspaceSize(handle, params, cache_lens, new_offsets) -> int:
     v = c_size_t(0)
     _check(lib().evlnPagedWorkspaceSize(handle, byref(params), _ints(cache_lens), _ints(new_offsets),
                                         byref(v)), "evlnPagedWorkspaceSize")
     return int(v.value)
-
-
-def evlnPagedRopeAppend(handle, params, q_new, k_new, v_new, cache_lens, new_offsets, page_table,
-                        q_rot, k_pool, v_pool, stream=None):
-    _check(lib().evlnPagedRopeAppend(handle, byref(params), _ptr(q_new), _ptr(k_new), _ptr(v_new),
-                                     _ints(cache_lens), _ints(new_offsets), _ptr(page_table),
-                                     _ptr(q_rot), _ptr(k_pool), _ptr(v_pool), _stream(stream)),
-           "evlnPagedRopeAppend")
-
-
-def evlnPagedStepAttention(handle, params, q_rot, k_pool, v_pool, cache_lens, new_offsets, page_table,
-                           workspace, workspace_bytes=None, stream=None):
-    if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
-    _check(lib().evlnPagedStepAttention(handle, byref(params), _ptr(q_rot), _ptr(k_pool), _ptr(v_pool),
-                                        _ints(cache_lens), _ints(new_offsets), _ptr(page_table),
-                                        _ptr(workspace), int(workspace_bytes), _stream(stream)),
-           "evlnPagedStepAttention")
-
-
-def evlnPagedStepCombine(handle, params, workspace, cache_lens, new_offsets, out, lse_out=None,
-                         stream=None):
-    _check(lib().evlnPagedStepCombine(handle, byref(params), _ptr(workspace), _ints(cache_lens),
-                                      _ints(new_offsets), _ptr(out), _ptr(lse_out), _stream(stream)),
-           "evlnPagedStepCombine")
 
 
 def packed_params(num_q_heads, num_kv_heads, head_dim, instr_len, frame_tokens, action_tokens, num_frames,
@@ -357,23 +317,6 @@ def evlnPackedWorkspaceSize(handle, params) -> int:
     v = c_size_t(0)
     _check(lib().evlnPackedWorkspaceSize(handle, byref(params), byref(v)), "evlnPackedWorkspaceSize")
     return int(v.value)
-
-
-def evlnPackedForward(handle, params, q, k, v, k_cache, v_cache, workspace, out, lse_out=None, stream=None):
-    """A packed sequence I, v_1, a_1, ..., v_N, a_N under the action-isolating mask, in one call."""
-    _check(lib().evlnPackedForward(handle, byref(params), _ptr(q), _ptr(k), _ptr(v), int(q.stride(0)), int(k.stride(0)),
-                                   int(v.stride(0)), _ptr(k_cache), _ptr(v_cache), _ptr(workspace),
-                                   int(workspace.numel() * workspace.element_size()), _ptr(out), _ptr(lse_out),
-                                   _stream(stream)), "evlnPackedForward")
-
-
-def evlnStepAttentionNoAlloc(params, q_rot, k_cache, v_cache, out, lse_out=None, stream=None):
-    """Attention + combine without a handle or a caller workspace: the split partials go to a
-    scratch array built into the library (at most EVLN_NOALLOC_SCRATCH_BYTES).  For callers that
-    must not allocate device memory; calls sharing a device must not overlap."""
-    _check(lib().evlnStepAttentionNoAlloc(byref(params), _ptr(q_rot), _ptr(k_cache), _ptr(v_cache),
-                                          _ptr(out), _ptr(lse_out), _stream(stream)),
-           "evlnStepAttentionNoAlloc")
 
 
 def gather_params(dtype, num_kv_heads, head_dim, store_capacity, work_capacity, rope_theta,
@@ -392,21 +335,6 @@ def evlnSampleFrames(sampler: int, num_frames: int, budget: int, stride: int = 1
     return [int(buf[i]) for i in range(cnt)]
 
 
-def evlnStoreAppend(handle, params, k_new, v_new, store_len, k_store, v_store, stream=None):
-    _check(lib().evlnStoreAppend(handle, byref(params), _ptr(k_new), _ptr(v_new), int(k_new.stride(0)),
-                                 int(v_new.stride(0)), int(store_len), int(k_new.shape[0]), _ptr(k_store),
-                                 _ptr(v_store), _stream(stream)), "evlnStoreAppend")
-
-
-def evlnGatherRope(handle, params, seg_src, seg_len, k_store, v_store, k_work, v_work, stream=None) -> int:
-    """Lays the kept store segments out in the working cache; returns the number of tokens laid out."""
-    total = c_int(0)
-    _check(lib().evlnGatherRope(handle, byref(params), len(seg_src), _ints(seg_src), _ints(seg_len), _ptr(k_store),
-                                _ptr(v_store), _ptr(k_work), _ptr(v_work), byref(total), _stream(stream)),
-           "evlnGatherRope")
-    return int(total.value)
-
-
 def evlnStoreOffload(handle, params, k_store, v_store, src_slot, length, h_k_store, h_v_store, dst_slot, stream=None):
     """Device store slots -> pinned host store ``[Hkv, host_capacity, D]`` (asynchronous DMA)."""
     _check(lib().evlnStoreOffload(handle, byref(params), _ptr(k_store), _ptr(v_store), int(src_slot), int(length),
@@ -419,3 +347,41 @@ def evlnStoreFetch(handle, params, h_k_store, h_v_store, src_slot, length, k_sto
     _check(lib().evlnStoreFetch(handle, byref(params), _ptr(h_k_store), _ptr(h_v_store), int(h_k_store.shape[1]),
                                 int(src_slot), int(length), _ptr(k_store), _ptr(v_store), int(dst_slot),
                                 _stream(stream)), "evlnStoreFetch")
+
+
+# ---- the calls a model makes per layer and step ----------------------------------------------
+
+# Built-ins of lib/_evln_native.so (csrc/py_native.cpp).  Through ctypes an evlnStep cost 16.5 us of
+# host time, twice what its three launches take, and more than the GPU needs for a step of a few tokens.
+kHotCalls = ("evlnRopeTable", "evlnRopeAppend", "evlnStepAttention", "evlnStepCombine", "evlnStep",
+             "evlnPagedRopeAppend", "evlnPagedStepAttention", "evlnPagedStepCombine", "evlnPackedForward",
+             "evlnStepAttentionNoAlloc", "evlnStoreAppend", "evlnGatherRope")
+
+
+def _load_native():
+    """Puts the built-ins in the place of the stand-ins below; raises if the module has not been built."""
+    import importlib.util
+
+    import torch  # noqa: F401  (its libraries carry symbols the module needs)
+    lib()
+    if not os.path.exists(NATIVE_PATH):
+        raise ImportError(f"{NATIVE_PATH} is missing: build it with __graft_entry__.build() (g++); there is no fallback")
+    spec = importlib.util.spec_from_file_location("_evln_native", NATIVE_PATH)
+    native = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(native)
+    native.configure(evlnStepParams, evlnPagedParams, evlnPackedParams, evlnGatherParams, EvlnError, ctypes.ArgumentError)
+    for name in kHotCalls:
+        globals()[name] = getattr(native, name)
+
+
+def _first_call(name):
+    def stand_in(*args, **kwargs):
+        if globals()[name] is stand_in:
+            _load_native()
+        return globals()[name](*args, **kwargs)
+    stand_in.__name__ = name
+    return stand_in
+
+
+for _name in kHotCalls:
+    globals()[_name] = _first_call(_name)
