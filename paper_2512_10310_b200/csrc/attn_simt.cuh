@@ -2,13 +2,25 @@
 //
 // The fp32 configuration asks for 1e-5 agreement with the fp64 oracle, which tf32 tensor-core
 // products cannot give, so this kernel evaluates the same split-KV causal attention with
-// float FMAs.  One warp owns one packed query row (kv head g, row r = i*G + h%G): every lane
-// scores one key of a 32-key chunk, the running maximum and sum of the online softmax are
-// reduced across the warp with shuffles, and each lane accumulates D/32 output channels.
-// It is also the on-device cross-check of the tensor-core kernel for bf16 inputs.
+// float FMAs.  It is also the on-device cross-check of the tensor-core kernel for bf16 inputs, and
+// the path of bf16 with head_dim 64.
+//
+// Bound: the FMA pipes (4 D flop per visible pair; 128 FMA per SM and cycle).  A block of 256 threads
+// owns a tile of 16 * RPT packed query rows of one kv head and walks its split's keys 64 at a time:
+//   thread (ty, tx) = (tid / 16, tid % 16) holds rows ty, ty + 16, ... (RPT of them), scores the keys
+//   tx, tx + 16, tx + 32, tx + 48 of the tile, and accumulates channels 4 tx .. 4 tx + 3 (and + 64).
+//   Everything it multiplies comes out of shared memory as 16-byte vectors and is used RPT (or 4)
+//   times; products go two at a time (packed FMAs over channel pairs).  Rows of Q, K and P are padded
+//   so that neither the 16 keys nor the two rows a warp touches at once meet in a bank.
+//   One K and one V tile are resident: the next K tile is fetched (cp.async) while the products with V
+//   run, the next V tile while the next scores run.
+// RPT = 8 (128 rows): each vector from shared memory feeds 8 rows, the FMA pipes are the limit.
+// RPT = 2 (32 rows): a quarter of the work per block, for calls whose 128-row tiles would leave SMs
+// idle; shared-memory reads bound it at about the same rate per row (K and V vectors feed 2 rows).
 #pragma once
 
 #include "common.cuh"
+#include "ptx_sm100.cuh"
 
 namespace evln {
 
@@ -18,84 +30,211 @@ struct SimtAttnArgs {
     const void* v_cache;
     float* o_part;         // [S, Hkv, R, D]
     float* lse_part;       // [S, Hkv, R]
-    int Hkv, G, D;
+    int Hkv, G;
     int cache_len, num_new, cache_cap;
     int num_splits;
     float scale;
 };
 
-template <typename T, int D>
-__global__ void __launch_bounds__(128)
+constexpr int kSimtThreads = 256;
+constexpr int kSimtKeys = 64;                           // keys per tile
+constexpr int kSimtPStride = kSimtKeys + 16;            // two neighbouring rows 16 banks apart
+template <int D, int RPT> constexpr int simt_smem_bytes()
+{
+    return (16 * RPT * (D + 4) + kSimtKeys * (D + 4) + kSimtKeys * D + 16 * RPT * kSimtPStride) * (int)sizeof(float);
+}
+
+// Row `row` of a tile to shared memory, 4 channels at `d`; rows at or past `rows` read as zeros.
+template <typename T>
+__device__ __forceinline__ void simt_fetch(float* dst, const T* base, int row, int rows, int D, int d)
+{
+    if constexpr (sizeof(T) == 4) {
+        ptx::cp_async16(ptx::smem_u32(dst), base + (row < rows ? (long)row * D + d : 0), row < rows);
+    } else {
+        uint2 raw = make_uint2(0u, 0u);
+        if (row < rows) raw = *reinterpret_cast<const uint2*>(base + (long)row * D + d);
+        *reinterpret_cast<float4*>(dst) = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
+                                                      __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
+    }
+}
+
+template <typename T, int D, int RPT, int NT = 256>
+__global__ void __launch_bounds__(NT)
 attn_simt_kernel(const SimtAttnArgs a)
 {
-    constexpr int C = D / 32;                 // output channels per lane
-    asm volatile("griddepcontrol.wait;" ::: "memory");          // programmatic dependent launch: inputs ready
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __shared__ float s_q[4][D];
+    constexpr int TY = NT / 16, BM = TY * RPT, BN = kSimtKeys, QS = D + 4, PS = kSimtPStride;
+    constexpr int kUnrollQ = RPT >= 8 ? 4 : 8, kUnrollV = RPT >= 8 ? 2 : 4;   // loads in flight ahead of the products
+    constexpr int NV = D / 64;                          // 4-channel groups of O per thread
+    constexpr int kVec = D / 4;                         // 16-byte vectors per row
+    extern __shared__ __align__(16) float simt_smem[];
+    float* s_q = simt_smem;                             // [BM][QS]
+    float* s_k = s_q + BM * QS;                         // [BN][QS]
+    float* s_v = s_k + BN * QS;                         // [BN][D]
+    float* s_p = s_v + BN * D;                          // [BM][PS]
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int R = a.num_new * a.G;
-    const int r = blockIdx.x * 4 + warp;
+    const int row0 = blockIdx.x * BM;
     const int g = blockIdx.y, split = blockIdx.z;
-    const int T_total = a.cache_len + a.num_new;
-    if (r >= R) return;
-
-    const int i = r / a.G;
-    const long t_lo = (long)split * T_total / a.num_splits;
-    long t_hi = (long)(split + 1) * T_total / a.num_splits;
-    const long bound = (long)a.cache_len + i + 1;          // keys 0 .. L+i are visible
-    if (t_hi > bound) t_hi = bound;
-
-    const T* q = (const T*)a.q_rot + ((long)g * R + r) * D;
-    for (int d = lane; d < D; d += 32) s_q[warp][d] = to_float(q[d]);
-    __syncwarp();
-
-    const T* kbase = (const T*)a.k_cache + (long)g * a.cache_cap * D;
-    const T* vbase = (const T*)a.v_cache + (long)g * a.cache_cap * D;
-
-    float m = -INFINITY, l = 0.f;
-    float o[C];
+    const int total = a.cache_len + a.num_new;
+    // splits are whole key tiles
+    const int all_tiles = (total + BN - 1) / BN;
+    const int t_lo = (int)((long)split * all_tiles / a.num_splits) * BN;
+    int t_hi = min(total, (int)((long)(split + 1) * all_tiles / a.num_splits) * BN);
+    // keys past the tile's last token are visible to none of its rows
+    const int last_row = min(row0 + BM, R) - 1;
+    t_hi = min(t_hi, a.cache_len + last_row / a.G + 1);
+    int bound[RPT];                                     // last visible key of the thread's rows
 #pragma unroll
-    for (int c = 0; c < C; ++c) o[c] = 0.f;
+    for (int r = 0; r < RPT; ++r) bound[r] = a.cache_len + (row0 + r * TY + ty) / a.G;
 
-    for (long t0 = t_lo; t0 < t_hi; t0 += 32) {
-        const long t = t0 + lane;
-        float s = -INFINITY;
-        if (t < t_hi) {
-            const T* k = kbase + t * D;
-            float acc = 0.f;
-#pragma unroll 8
-            for (int d = 0; d < D; ++d) acc = fmaf(s_q[warp][d], to_float(k[d]), acc);
-            s = acc * a.scale;
-        }
-        float cmax = s;
+    const T* qb = (const T*)a.q_rot + ((long)g * R + row0) * D;
+    const T* kb = (const T*)a.k_cache + ((long)g * a.cache_cap + t_lo) * D;
+    const T* vb = (const T*)a.v_cache + ((long)g * a.cache_cap + t_lo) * D;
+    const int keys = t_hi - t_lo, ntiles = keys > 0 ? (keys + BN - 1) / BN : 0;
+
+    auto fetch_k = [&](int j) {
+        for (int i = tid; i < BN * kVec; i += NT)
+            simt_fetch(s_k + (i / kVec) * QS + (i % kVec) * 4, kb, j * BN + i / kVec, keys, D, (i % kVec) * 4);
+    };
+    auto fetch_v = [&](int j) {
+        for (int i = tid; i < BN * kVec; i += NT)
+            simt_fetch(s_v + (i / kVec) * D + (i % kVec) * 4, vb, j * BN + i / kVec, keys, D, (i % kVec) * 4);
+    };
+
+    ptx::grid_dependency_wait();                        // programmatic dependent launch: inputs ready
+    ptx::grid_launch_dependents();
+    if (ntiles > 0) {
+        for (int i = tid; i < BM * kVec; i += NT)
+            simt_fetch(s_q + (i / kVec) * QS + (i % kVec) * 4, qb, i / kVec, R - row0, D, (i % kVec) * 4);
+        fetch_k(0);
+    }
+    ptx::cp_async_commit();
+    if (ntiles > 0) fetch_v(0);
+    ptx::cp_async_commit();
+
+    float m[RPT], l[RPT];
+    uint64_t o[RPT][2 * NV];                            // channel pairs
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, off));
-        const float m_new = fmaxf(m, cmax);               // finite: the chunk holds >= 1 key
-        const float alpha = expf(m - m_new);              // m = -inf on the first chunk -> 0
-        const float p = (t < t_hi) ? expf(s - m_new) : 0.f;
-        float psum = p;
+    for (int r = 0; r < RPT; ++r) {
+        m[r] = -INFINITY;
+        l[r] = 0.f;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, off);
-        l = l * alpha + psum;
-        m = m_new;
-#pragma unroll
-        for (int c = 0; c < C; ++c) o[c] *= alpha;
-        const int cnt = (int)((t_hi - t0) < 32 ? (t_hi - t0) : 32);
-        for (int j = 0; j < cnt; ++j) {
-            const float pj = __shfl_sync(0xffffffffu, p, j);
-            const T* v = vbase + (t0 + j) * D;
-#pragma unroll
-            for (int c = 0; c < C; ++c) o[c] = fmaf(pj, to_float(v[lane + 32 * c]), o[c]);
-        }
+        for (int c = 0; c < 2 * NV; ++c) o[r][c] = 0ull;
     }
 
-    const long prow = ((long)split * a.Hkv + g) * R + r;
-    float* op = a.o_part + prow * D;
-    const float inv = (l > 0.f) ? 1.f / l : 0.f;
+    for (int j = 0; j < ntiles; ++j) {
+        ptx::cp_async_wait<1>();
+        __syncthreads();                                // Q and K_j are there
+        float s[RPT][4];
+        {
+            uint64_t acc[RPT][4];
 #pragma unroll
-    for (int c = 0; c < C; ++c) op[lane + 32 * c] = o[c] * inv;
-    if (lane == 0) a.lse_part[prow] = (l > 0.f) ? m + logf(l) : -INFINITY;
+            for (int r = 0; r < RPT; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[r][c] = 0ull;
+#pragma unroll kUnrollQ
+            for (int d = 0; d < D; d += 4) {
+                ulonglong2 k[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) k[c] = *reinterpret_cast<const ulonglong2*>(s_k + (tx + 16 * c) * QS + d);
+#pragma unroll
+                for (int r = 0; r < RPT; ++r) {
+                    const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(s_q + (r * TY + ty) * QS + d);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        acc[r][c] = ptx::fma2(q.x, k[c].x, acc[r][c]);
+                        acc[r][c] = ptx::fma2(q.y, k[c].y, acc[r][c]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < RPT; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    float lo, hi;
+                    ptx::unpack2(acc[r][c], lo, hi);
+                    s[r][c] = (lo + hi) * a.scale;
+                }
+        }
+        __syncthreads();                                // everyone is done with K_j
+        if (j + 1 < ntiles) fetch_k(j + 1);
+        ptx::cp_async_commit();
+
+        const int key0 = t_lo + j * BN + tx;
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            float mx = -INFINITY;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (key0 + 16 * c > bound[r] || key0 + 16 * c >= t_hi) s[r][c] = -INFINITY;
+                mx = fmaxf(mx, s[r][c]);
+            }
+#pragma unroll
+            for (int off = 8; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            const float m_new = fmaxf(m[r], mx);
+            const float ref = (m_new == -INFINITY) ? 0.f : m_new;      // a row that has seen no key yet: every p is 0
+            const float alpha = expf(m[r] - ref);                       // m = -inf: 0
+            m[r] = m_new;
+            float sum = 0.f;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float p = expf(s[r][c] - ref);
+                sum += p;
+                s_p[(r * TY + ty) * PS + tx + 16 * c] = p;
+            }
+            l[r] = l[r] * alpha + sum;
+            const uint64_t alpha2 = ptx::pack2(alpha, alpha);
+#pragma unroll
+            for (int c = 0; c < 2 * NV; ++c) o[r][c] = ptx::mul2(o[r][c], alpha2);
+        }
+        ptx::cp_async_wait<1>();
+        __syncthreads();                                // V_j is there (a row's P stays within its warp)
+#pragma unroll kUnrollV
+        for (int k = 0; k < BN; k += 4) {
+            float4 p[RPT];
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) p[r] = *reinterpret_cast<const float4*>(s_p + (r * TY + ty) * PS + k);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                ulonglong2 v[NV];
+#pragma unroll
+                for (int c = 0; c < NV; ++c) v[c] = *reinterpret_cast<const ulonglong2*>(s_v + (k + kk) * D + c * 64 + tx * 4);
+#pragma unroll
+                for (int r = 0; r < RPT; ++r) {
+                    const float x = kk == 0 ? p[r].x : kk == 1 ? p[r].y : kk == 2 ? p[r].z : p[r].w;
+                    const uint64_t x2 = ptx::pack2(x, x);
+#pragma unroll
+                    for (int c = 0; c < NV; ++c) {
+                        o[r][2 * c] = ptx::fma2(x2, v[c].x, o[r][2 * c]);
+                        o[r][2 * c + 1] = ptx::fma2(x2, v[c].y, o[r][2 * c + 1]);
+                    }
+                }
+            }
+        }
+        __syncthreads();                                // everyone is done with V_j
+        if (j + 1 < ntiles) fetch_v(j + 1);
+        ptx::cp_async_commit();
+    }
+
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+        float sum = l[r];
+#pragma unroll
+        for (int off = 8; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+        const int row = row0 + r * TY + ty;
+        if (row >= R) continue;
+        const long prow = ((long)split * a.Hkv + g) * R + row;
+        const float inv = (sum > 0.f) ? 1.f / sum : 0.f;
+#pragma unroll
+        for (int c = 0; c < NV; ++c) {
+            float4 v;
+            ptx::unpack2(o[r][2 * c], v.x, v.y);
+            ptx::unpack2(o[r][2 * c + 1], v.z, v.w);
+            *reinterpret_cast<float4*>(a.o_part + prow * D + c * 64 + tx * 4) = make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv);
+        }
+        if (tx == 0) a.lse_part[prow] = (sum > 0.f) ? m[r] + logf(sum) : -INFINITY;
+    }
 }
 
 }  // namespace evln

@@ -87,6 +87,34 @@ cudaError_t launch_pair_pdl(void (*kernel)(KArgs...), dim3 grid, size_t smem, cu
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+template <typename T, int D, int RPT>
+cudaError_t prepare_simt()
+{
+    return cudaFuncSetAttribute(attn_simt_kernel<T, D, RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt_smem_bytes<D, RPT>());
+}
+
+// Shared-memory limits of the kernels that take more than the default, on the current device.
+cudaError_t prepare_kernels()
+{
+    const std::pair<const void*, int> tc[4] = {{(const void*)attn_pair_kernel<false, NoLens>, kTcSmemBytes},
+                                               {(const void*)attn_pair_kernel<true, BatchLens>, kTcSmemBytes},
+                                               {(const void*)attn_solo_kernel, kSoloSmemBytes},
+                                               {(const void*)attn_tail_kernel, kTcSmemBytes}};
+    for (const auto& k : tc) {
+        cudaError_t e = cudaFuncSetAttribute(k.first, cudaFuncAttributeMaxDynamicSharedMemorySize, k.second);
+        if (e != cudaSuccess) return e;
+    }
+    cudaError_t e = prepare_simt<float, 128, 8>();
+    if (e == cudaSuccess) e = prepare_simt<float, 128, 2>();
+    if (e == cudaSuccess) e = prepare_simt<float, 64, 8>();
+    if (e == cudaSuccess) e = prepare_simt<float, 64, 2>();
+    if (e == cudaSuccess) e = prepare_simt<__nv_bfloat16, 128, 8>();
+    if (e == cudaSuccess) e = prepare_simt<__nv_bfloat16, 128, 2>();
+    if (e == cudaSuccess) e = prepare_simt<__nv_bfloat16, 64, 8>();
+    if (e == cudaSuccess) e = prepare_simt<__nv_bfloat16, 64, 2>();
+    return e;
+}
+
 // The attention kernels move registers between their warpgroups (setmaxnreg) inside the pool a CTA
 // gets at launch; a request the pool cannot serve would wait for ever.  The plan in attn_pair.cuh is
 // made for kRegsLaunch registers per thread: refuse to run a build that came out differently.
@@ -194,6 +222,45 @@ int choose_splits_solo(int Hkv, int R, int nkv, int num_sms)
     return best;
 }
 
+// Row tile and split count of the SIMT kernel (splits > 0: given), by a model of measured times at
+// head_dim 128 (head_dim 64: about half).  A block of 128 rows runs alone on its SM, 13.3 us per 64-key
+// tile and 7 us for its start and write-out; a block of 32 rows takes 6.3 us per tile and 5 us when it
+// has the SM to itself, 9.5 per tile when two share it.  So 128-row tiles are 1.4 times cheaper per row
+// where they fill the chip, 32-row tiles have twice the latency advantage where they would not.  A
+// split writes and re-reads a set of partials (about 5 TB/s out of L2).
+struct SimtSchedule {
+    int rows_per_thread, splits;
+};
+SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits)
+{
+    const int R = p->num_new * (p->num_q_heads / p->num_kv_heads);
+    const int tiles = ceil_div(p->cache_len + p->num_new, kSimtKeys);
+    const double d = p->head_dim / 128.0;
+    const double split_us = 0.3 + 2.0 * R * p->num_kv_heads * p->head_dim * 4 / 5e6;
+    SimtSchedule best = {8, splits > 0 ? splits : 1};
+    double best_cost = 1e30;
+    const int smax = tiles < kMaxSplits ? tiles : kMaxSplits;
+    for (int rpt = 8; rpt >= 2; rpt -= 6) {
+        const long row_blocks = (long)ceil_div(R, 16 * rpt) * p->num_kv_heads;
+        for (int s = splits > 0 ? splits : 1; s <= (splits > 0 ? splits : smax); ++s) {
+            const long blocks = row_blocks * s;
+            const long at_once = rpt == 8 || blocks <= h->num_sms ? h->num_sms : 2 * h->num_sms;
+            const double tile_us = rpt == 8 ? 13.3 : at_once == h->num_sms ? 6.3 : 9.5;
+            const double waves = (double)((blocks + at_once - 1) / at_once);
+            const double cost = waves * (ceil_div(tiles, s) * tile_us * d + (rpt == 8 ? 7.0 : 5.0)) + split_us * s;
+            if (cost < best_cost - 1e-9) { best_cost = cost; best = {rpt, s}; }
+        }
+    }
+    return best;
+}
+
+template <typename T, int D>
+void launch_simt(int rows_per_thread, dim3 grid, cudaStream_t st, const SimtAttnArgs& a)
+{
+    if (rows_per_thread == 8) launch_pdl(attn_simt_kernel<T, D, 8>, grid, dim3(kSimtThreads), simt_smem_bytes<D, 8>(), st, a);
+    else launch_pdl(attn_simt_kernel<T, D, 2>, grid, dim3(kSimtThreads), simt_smem_bytes<D, 2>(), st, a);
+}
+
 int resolve_splits(evlnHandle_t h, const evlnStepParams* p)
 {
     if (p->num_new == 0) return 1;
@@ -209,13 +276,7 @@ int resolve_splits(evlnHandle_t h, const evlnStepParams* p)
         const int nkv_min = unit_kv_tiles(p->cache_len, p->num_new, G, 0, kUnitRows);
         return choose_splits_tc(units * p->num_kv_heads, nkv_max, nkv_min, h->num_sms);
     }
-    const int blocks = ceil_div(R, 4) * p->num_kv_heads;
-    int s = ceil_div(2 * h->num_sms, blocks);
-    const int cap = ceil_div(T, 64);
-    if (s > cap) s = cap;
-    if (s > kMaxSplits) s = kMaxSplits;
-    if (s < 1) s = 1;
-    return s;
+    return simt_schedule(h, p, 0).splits;
 }
 
 size_t partial_bytes(int splits, int Hkv, long rows, int D)
@@ -428,16 +489,7 @@ evlnStatus_t evlnCreate(evlnHandle_t* handle, int device)
     h->encode = reinterpret_cast<EncodeTiledFn>(fn);
     e = cudaMalloc(&h->d_status, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(attn_pair_kernel<false, NoLens>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kTcSmemBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(attn_pair_kernel<true, BatchLens>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kTcSmemBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(attn_solo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSoloSmemBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(attn_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemBytes);
+    if (e == cudaSuccess) e = prepare_kernels();
     if (e == cudaSuccess && !attention_register_pool_ok()) {
         cudaFree(h->d_status);
         delete h;
@@ -667,16 +719,17 @@ evlnStatus_t evlnStepAttention(evlnHandle_t h, const evlnStepParams* p, const vo
         SimtAttnArgs a = {};
         a.q_rot = q_rot; a.k_cache = k_cache; a.v_cache = v_cache;
         a.o_part = o_part; a.lse_part = lse_part;
-        a.Hkv = p->num_kv_heads; a.G = G; a.D = D;
+        a.Hkv = p->num_kv_heads; a.G = G;
         a.cache_len = p->cache_len; a.num_new = p->num_new; a.cache_cap = p->cache_capacity;
         a.num_splits = S; a.scale = scale;
-        dim3 grid(ceil_div(R, 4), p->num_kv_heads, S);
+        const int rpt = simt_schedule(h, p, S).rows_per_thread;
+        dim3 grid(ceil_div(R, 16 * rpt), p->num_kv_heads, S);
         if (p->dtype == EVLN_BF16) {
-            if (D == 128) launch_pdl(attn_simt_kernel<__nv_bfloat16, 128>, dim3(grid), dim3(128), 0, st, a);
-            else launch_pdl(attn_simt_kernel<__nv_bfloat16, 64>, dim3(grid), dim3(128), 0, st, a);
+            if (D == 128) launch_simt<__nv_bfloat16, 128>(rpt, grid, st, a);
+            else launch_simt<__nv_bfloat16, 64>(rpt, grid, st, a);
         } else {
-            if (D == 128) launch_pdl(attn_simt_kernel<float, 128>, dim3(grid), dim3(128), 0, st, a);
-            else launch_pdl(attn_simt_kernel<float, 64>, dim3(grid), dim3(128), 0, st, a);
+            if (D == 128) launch_simt<float, 128>(rpt, grid, st, a);
+            else launch_simt<float, 64>(rpt, grid, st, a);
         }
     }
     cudaError_t e = cudaGetLastError();
@@ -1256,10 +1309,7 @@ evlnStatus_t noalloc_setup(int device, NoAllocDevice** out)
         cudaDriverEntryPointQueryResult qres;
         e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
         if (e != cudaSuccess || qres != cudaDriverEntryPointSuccess || !fn) return EVLN_CUDA_ERROR;
-        e = cudaFuncSetAttribute(attn_pair_kernel<false, NoLens>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kTcSmemBytes);
-        if (e != cudaSuccess) return EVLN_CUDA_ERROR;
-        e = cudaFuncSetAttribute(attn_solo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSoloSmemBytes);
+        e = prepare_kernels();
         if (e != cudaSuccess) return EVLN_CUDA_ERROR;
         if (!attention_register_pool_ok()) return EVLN_NOT_SUPPORTED;
         d->ctx.device = device;

@@ -338,6 +338,22 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
     asm("add.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// ---- cp.async: 16 bytes to shared memory, zeros when `valid` is false ----------------------
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 // Registers per thread of the executing warpgroup (all four warps execute it together): dec gives
 // registers back to the CTA's pool, inc takes from it and WAITS until the pool can serve it.
 template <int N> __device__ __forceinline__ void setmaxnreg_inc()
