@@ -67,8 +67,7 @@ gather_rope_kernel(const GatherArgs a, const __grid_constant__ SegList segs)
     constexpr int V = VecTraits<T>::kVec;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __shared__ double s_cos[64];
-    __shared__ double s_sin[64];
+    __shared__ typename Rotation<T>::Angle s_angle[72];                // angle j at j + j / 8: the 8 vectors of a half head in different banks
 
     const int pos = blockIdx.x;             // working slot = new position id
     const int D = a.D, half = D / 2;
@@ -82,8 +81,7 @@ gather_rope_kernel(const GatherArgs a, const __grid_constant__ SegList segs)
     if (threadIdx.x < half) {
         const int j = threadIdx.x;
         const double2 cs = a.table ? a.table[(long)(pos - a.table_first) * half + j] : rope_cos_sin(pos, j, D, a.log2_theta);
-        s_cos[j] = cs.x;
-        s_sin[j] = cs.y;
+        s_angle[j + (j >> 3)] = Rotation<T>::angle(cs);
     }
     __syncthreads();
 
@@ -105,11 +103,10 @@ gather_rope_kernel(const GatherArgs a, const __grid_constant__ SegList segs)
             T* out_hi = reinterpret_cast<T*>(&out_hi_raw);
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                // products and their difference in double, then one rounding to float and one to storage
-                const double c = s_cos[j0 + v], s = s_sin[j0 + v];
-                const double x0 = (double)to_float(xl[v]), x1 = (double)to_float(xh[v]);
-                from_float((float)(x0 * c - x1 * s), out_lo[v]);
-                from_float((float)(x1 * c + x0 * s), out_hi[v]);
+                float y0, y1;
+                Rotation<T>::turn(to_float(xl[v]), to_float(xh[v]), s_angle[j0 + (j0 >> 3) + v], y0, y1);
+                from_float(y0, out_lo[v]);
+                from_float(y1, out_hi[v]);
             }
             *reinterpret_cast<uint4*>(dst + j0) = out_lo_raw;
             *reinterpret_cast<uint4*>(dst + j0 + half) = out_hi_raw;

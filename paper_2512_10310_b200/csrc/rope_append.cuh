@@ -60,6 +60,58 @@ __device__ __forceinline__ double2 rope_cos_sin(long pos, int j, int D, double l
     return make_double2(c, s);
 }
 
+// The rotation itself.  Products and sums are formed with at least 47 bits, then rounded once to float and
+// once to the storage dtype (a float product would lose bits exactly where x0*c and x1*s cancel).
+//  - float: in double.
+//  - bf16: in pairs of floats.  A double operation and the conversions around it issue at a small
+//    fraction of the float rate (measured: 32 double operations and 32 conversions per vector pair kept
+//    an SM at ~7 per cycle; the rotation was most of the append and gather kernels' time), and a bf16
+//    value times a cosine split into two floats is exact up to 2^-48: p + e is the exact product with
+//    the high part (fma), the low part joins the residual, the two products are subtracted with the
+//    rounding error recovered (Knuth's two-sum).
+template <typename T> struct Rotation;
+template <> struct Rotation<float> {
+    typedef double2 Angle;                       // (cos, sin)
+    static __device__ __forceinline__ Angle angle(const double2& cs) { return cs; }
+    static __device__ __forceinline__ void turn(float x0, float x1, const Angle& a, float& y0, float& y1)
+    {
+        y0 = (float)((double)x0 * a.x - (double)x1 * a.y);
+        y1 = (float)((double)x1 * a.x + (double)x0 * a.y);
+    }
+};
+template <> struct Rotation<__nv_bfloat16> {
+    typedef float4 Angle;                        // cos high, cos low, sin high, sin low
+    static __device__ __forceinline__ Angle angle(const double2& cs)
+    {
+        const float ch = (float)cs.x, sh = (float)cs.y;
+        return make_float4(ch, (float)(cs.x - (double)ch), sh, (float)(cs.y - (double)sh));
+    }
+    // x * (hi + lo) as p + e
+    static __device__ __forceinline__ void product(float x, float hi, float lo, float& p, float& e)
+    {
+        p = __fmul_rn(x, hi);
+        e = __fmaf_rn(x, lo, __fmaf_rn(x, hi, -p));
+    }
+    static __device__ __forceinline__ float difference(float p, float e, float q, float f)
+    {
+        const float d = __fsub_rn(p, q);
+        const float b = __fsub_rn(d, p);
+        const float err = __fsub_rn(__fsub_rn(p, __fsub_rn(d, b)), __fadd_rn(q, b));
+        const float y = __fadd_rn(d, __fadd_rn(err, __fsub_rn(e, f)));
+        return fabsf(d) < INFINITY ? y : d;      // (an infinite or undefined result stays what it is)
+    }
+    static __device__ __forceinline__ void turn(float x0, float x1, const Angle& a, float& y0, float& y1)
+    {
+        float p, e, q, f;
+        product(x0, a.x, a.y, p, e);
+        product(x1, a.z, a.w, q, f);
+        y0 = difference(p, e, q, f);
+        product(x1, a.x, a.y, p, e);
+        product(x0, -a.z, -a.w, q, f);
+        y1 = difference(p, e, q, f);
+    }
+};
+
 // Position table: entry (p, j) = (cos, sin) of (first_pos + p) * theta^(-2j/D).
 __global__ void __launch_bounds__(128)
 rope_table_kernel(double2* table, int first_pos, int count, int D, double log2_theta)
@@ -85,8 +137,7 @@ __global__ void __launch_bounds__(kRopeThreadsMax)
 rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
 {
     constexpr int V = VecTraits<T>::kVec;
-    __shared__ double s_cos[128];
-    __shared__ double s_sin[128];
+    __shared__ typename Rotation<T>::Angle s_angle[72];                // angle j at j + j / 8: the 8 vectors of a half head in different banks
 
     const int tok = blockIdx.x;           // index into the packed new tokens
     const int D = a.D, half = D / 2;
@@ -113,8 +164,7 @@ rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
     if (threadIdx.x < half) {
         const int j = threadIdx.x;
         const double2 cs = trow ? trow[j] : rope_cos_sin(pos, j, D, a.log2_theta);
-        s_cos[j] = cs.x;
-        s_sin[j] = cs.y;
+        s_angle[j + (j >> 3)] = Rotation<T>::angle(cs);
     }
 
     // destination of this token's K/V row for kv head g (element offset)
@@ -181,12 +231,10 @@ rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
             T* out_hi = reinterpret_cast<T*>(&out_hi_raw);
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                // products and the difference in double (a float product loses bits exactly where
-                // x0*c and x1*s cancel), then one rounding to float and one to the storage dtype
-                const double c = s_cos[j0 + v], s = s_sin[j0 + v];
-                const double x0 = (double)to_float(lo[v]), x1 = (double)to_float(hi[v]);
-                from_float((float)(x0 * c - x1 * s), out_lo[v]);
-                from_float((float)(x1 * c + x0 * s), out_hi[v]);
+                float y0, y1;
+                Rotation<T>::turn(to_float(lo[v]), to_float(hi[v]), s_angle[j0 + (j0 >> 3) + v], y0, y1);
+                from_float(y0, out_lo[v]);
+                from_float(y1, out_hi[v]);
             }
             *reinterpret_cast<uint4*>(dst + j0) = out_lo_raw;
             *reinterpret_cast<uint4*>(dst + j0 + half) = out_hi_raw;
