@@ -15,6 +15,7 @@
 
 #include "attn_simt.cuh"
 #include "attn_pair.cuh"
+#include "attn_few.cuh"
 #include "combine.cuh"
 #include "gather_rope.cuh"
 #include "common.cuh"
@@ -33,6 +34,7 @@ struct evlnContext {
     int last_cuda_error;
     int* d_status;
     EncodeTiledFn encode;
+    int max_clusters[5];     // clusters of 1, 2, 4, 8, 16 blocks of the few-row kernel that fit the device at once
 };
 
 #ifdef EVLN_TIMELINE
@@ -93,6 +95,20 @@ cudaError_t prepare_simt()
     return cudaFuncSetAttribute(attn_simt_kernel<T, D, RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt_smem_bytes<D, RPT>());
 }
 
+template <int MT>
+cudaError_t prepare_few()
+{
+    const void* kernels[3] = {(const void*)attn_few_kernel<MT, false, false, NoLens>, (const void*)attn_few_kernel<MT, false, true, NoLens>,
+                              (const void*)attn_few_kernel<MT, true, false, BatchLens>};
+    for (int i = 0; i < 3; ++i) {
+        cudaError_t e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kFewMaxSmem);
+        if (e == cudaSuccess && i < 2) e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // Shared-memory limits of the kernels that take more than the default, on the current device.
 cudaError_t prepare_kernels()
 {
@@ -104,7 +120,9 @@ cudaError_t prepare_kernels()
         cudaError_t e = cudaFuncSetAttribute(k.first, cudaFuncAttributeMaxDynamicSharedMemorySize, k.second);
         if (e != cudaSuccess) return e;
     }
-    cudaError_t e = prepare_simt<float, 128, 8>();
+    cudaError_t e = prepare_few<1>();
+    if (e == cudaSuccess) e = prepare_few<2>();
+    if (e == cudaSuccess) e = prepare_simt<float, 128, 8>();
     if (e == cudaSuccess) e = prepare_simt<float, 128, 2>();
     if (e == cudaSuccess) e = prepare_simt<float, 64, 8>();
     if (e == cudaSuccess) e = prepare_simt<float, 64, 2>();
@@ -206,6 +224,95 @@ inline bool use_solo_kernel(const evlnStepParams* p)
     return use_tensor_kernel(p) && (long)p->num_new * (p->num_q_heads / p->num_kv_heads) <= kTileM;
 }
 
+// At most 32 rows per kv head (up to four action tokens with seven query heads per kv head): the kernel
+// whose products stay in registers (attn_few.cuh).
+inline bool use_few_kernel(const evlnStepParams* p)
+{
+    return use_tensor_kernel(p) && (long)p->num_new * (p->num_q_heads / p->num_kv_heads) <= kFewRows;
+}
+inline int few_row_tiles(int rows) { return rows <= 16 ? 1 : 2; }
+
+struct FewPlan {
+    int splits, cluster, stages;
+};
+// A block needs 0.40 us per 64-key stage (0.54 with two row tiles), all of them together what HBM needs;
+// clusters beyond those that fit the device at once wait for a whole round; a cluster costs 1 us of
+// exchange, splits a second launch that merges them (measured with 4 and 8 kv heads, 40 .. 32768 keys).
+FewPlan few_plan(evlnHandle_t h, const evlnStepParams* p)
+{
+    const int T = p->cache_len + p->num_new, ns = ceil_div(T, kFewKeys);
+    const int rows = p->num_new * (p->num_q_heads / p->num_kv_heads);
+    const double stage_us = few_row_tiles(rows) == 1 ? 0.40 : 0.54;
+    const double hbm_us = 512.0 * T * p->num_kv_heads / 6.2e6;
+    FewPlan best = {1, 1, 0};
+    double best_cost = 1e30;
+    for (int i = 0; i < 5; ++i) {
+        const int c = 1 << i;
+        for (int s = p->num_splits > 0 ? p->num_splits : 1; s <= (p->num_splits > 0 ? p->num_splits : 8); ++s) {
+            if ((c > 1 || s > 1) && c * s > ns && !(c == 1 && s == p->num_splits)) continue;
+            const long clusters = (long)p->num_kv_heads * s;
+            const int fit = h->max_clusters[i] > 0 ? h->max_clusters[i] : 0;
+            if (fit == 0) continue;
+            const double rounds = (double)((clusters + fit - 1) / fit);
+            const double work = rounds * ceil_div(ns, c * s) * stage_us;
+            const double cost = (work > hbm_us ? work : hbm_us) + rounds + (c > 1 ? 1.0 : 0.0) + (s > 1 ? 1.8 + 0.1 * s : 0.0);
+            if (cost < best_cost - 1e-9) { best_cost = cost; best.splits = s; best.cluster = c; }
+        }
+    }
+    best.stages = few_smem_bytes(kFewMaxStages, rows, best.cluster, true, p->num_new) <= kFewMaxSmem ? kFewMaxStages : kFewMinStages;
+    return best;
+}
+
+// How many clusters of each size of the largest few-row block the current device holds at once.
+cudaError_t query_few_clusters(int* max_clusters)
+{
+    for (int i = 0; i < 5; ++i) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1u << i);
+        cfg.blockDim = dim3(kFewThreads);
+        cfg.dynamicSmemBytes = kFewMaxSmem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1u << i;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        cudaError_t e = cudaOccupancyMaxActiveClusters(&n, attn_few_kernel<2, false, true, NoLens>, &cfg);
+        if (e != cudaSuccess) {
+            if (i == 0) return e;
+            cudaGetLastError();            // this cluster size is not available
+            n = 0;
+        }
+        max_clusters[i] = n;
+    }
+    return cudaSuccess;
+}
+
+template <bool FUSED>
+cudaError_t launch_few(const FewPlan& f, int rows, cudaStream_t st, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const FewArgs& a)
+{
+    cudaLaunchConfig_t cfg = {};
+    const int mt = few_row_tiles(rows);
+    cfg.gridDim = dim3(f.cluster, a.Hkv, f.splits);
+    cfg.blockDim = dim3(kFewThreads);
+    cfg.dynamicSmemBytes = few_smem_bytes(f.stages, rows, f.cluster, FUSED, a.num_new);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = f.cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = f.cluster > 1 ? 2 : 1;
+    const NoLens nl = {};
+    if (mt == 1) return cudaLaunchKernelEx(&cfg, attn_few_kernel<1, false, FUSED, NoLens>, tm_k, tm_v, a, nl);
+    return cudaLaunchKernelEx(&cfg, attn_few_kernel<2, false, FUSED, NoLens>, tm_k, tm_v, a, nl);
+}
+
 // Split schedule of the one-CTA-per-item kernel: the step is bound by streaming K/V once, so the
 // KV range is spread over all SMs; an item's fixed cost is about 3 tiles of streaming, and a split
 // adds a partial row set of R rows to merge.
@@ -268,6 +375,7 @@ int resolve_splits(evlnHandle_t h, const evlnStepParams* p)
     const int G = p->num_q_heads / p->num_kv_heads;
     const int R = p->num_new * G;
     const int T = p->cache_len + p->num_new;
+    if (use_few_kernel(p)) return few_plan(h, p).splits;
     if (use_solo_kernel(p))
         return choose_splits_solo(p->num_kv_heads, R, ceil_div(T, kTileN), h->num_sms);
     if (use_tensor_kernel(p)) {
@@ -325,7 +433,7 @@ inline int batch_kv_tiles(bool tail, int L, int n, int G, int u)
 }
 
 // Work-item size (KV tiles) and the largest split count of a batch.
-void batch_schedule(int num_sms, int G, int Hkv, int batch, const int* lens, const int* offs, bool tail,
+void batch_schedule(int num_sms, int G, int Hkv, int batch, const int* lens, const int* offs, bool tail, bool few,
                     int kv_chunk_tiles, int* chunk_tiles, int* max_splits, long* items)
 {
     long total = 0;
@@ -341,7 +449,12 @@ void batch_schedule(int num_sms, int G, int Hkv, int batch, const int* lens, con
     }
     total *= Hkv;
     int chunk = kv_chunk_tiles;
-    if (chunk <= 0) {
+    if (chunk <= 0 && few) {
+        // one block per item: four items per SM even out the lengths (16 ragged episodes of one token:
+        // 65 us with one per SM, 62 with four, 72 with six: every item pays its own start and merge)
+        chunk = (int)((total + (long)num_sms * 4 - 1) / ((long)num_sms * 4));
+        if (chunk < 2) chunk = 2;
+    } else if (chunk <= 0) {
         const long pairs = num_sms / 2 > 0 ? num_sms / 2 : 1;
         chunk = (int)((total + pairs * 4 - 1) / (pairs * 4));
         if (chunk < 8) chunk = 8;
@@ -358,11 +471,20 @@ void batch_schedule(int num_sms, int G, int Hkv, int batch, const int* lens, con
     *items = cnt * Hkv;
 }
 
+// A batch whose episodes all bring few rows (action tokens): the few-row kernel, one block per work item.
+bool paged_few(const evlnPagedParams* p, const int* offs)
+{
+    const int G = p->num_q_heads / p->num_kv_heads;
+    for (int b = 0; b < p->batch; ++b)
+        if ((long)(offs[b + 1] - offs[b]) * G > kFewRows) return false;
+    return true;
+}
+
 void paged_schedule(evlnHandle_t h, const evlnPagedParams* p, const int* lens, const int* offs,
                     int* chunk_tiles, int* max_splits, long* items)
 {
     batch_schedule(h->num_sms, p->num_q_heads / p->num_kv_heads, p->num_kv_heads, p->batch, lens, offs, false,
-                   p->kv_chunk_tiles, chunk_tiles, max_splits, items);
+                   paged_few(p, offs), p->kv_chunk_tiles, chunk_tiles, max_splits, items);
 }
 
 // chunk_tiles > 0: also the first attention work item of every episode (items are numbered
@@ -439,6 +561,63 @@ void launch_rope_append(evlnHandle_t h, const RopeArgs& a, int tokens, cudaStrea
     launch_pdl(rope_append_kernel<T, PAGED, LensT>, dim3(tokens), dim3(t), 0, st, a, lens);
 }
 
+// What the one-launch step adds to an attention call: the new tokens and where the results go (out null:
+// partials to the workspace, for the combine kernel).
+struct FewFused {
+    const void *q_new, *k_new, *v_new;
+    long q_stride, k_stride, v_stride;
+    void* q_rot;
+    void* out;
+    float* lse_out;
+};
+
+// Attention of few rows on a contiguous cache: the call's partials, or the whole step (fused not null).
+evlnStatus_t step_few(evlnHandle_t h, const evlnStepParams* p, const void* q_rot, const void* k_cache, const void* v_cache,
+                      float* o_part, float* lse_part, const FewFused* fused, cudaStream_t st)
+{
+    const int G = p->num_q_heads / p->num_kv_heads, R = p->num_new * G;
+    const FewPlan f = few_plan(h, p);
+    if (p->num_kv_heads > 65535) return EVLN_NOT_SUPPORTED;
+    CUtensorMap tm_k, tm_v;
+    {
+        // rows past L+n read as zeros, so stale slots never reach the tensor core
+        cuuint64_t dims[3] = {128, (cuuint64_t)(p->cache_len + p->num_new), (cuuint64_t)p->num_kv_heads};
+        cuuint64_t strides[2] = {256, (cuuint64_t)p->cache_capacity * 256};
+        cuuint32_t box[3] = {64, kFewKeys, 1};
+        if (!encode_map(h, &tm_k, k_cache, 3, dims, strides, box)) return EVLN_INVALID_VALUE;
+        if (!encode_map(h, &tm_v, v_cache, 3, dims, strides, box)) return EVLN_INVALID_VALUE;
+    }
+    FewArgs a = {};
+    a.o_part = o_part; a.lse_part = lse_part;
+    a.q_rot_in = (const __nv_bfloat16*)q_rot;
+    a.status = h->d_status;
+    a.Hkv = p->num_kv_heads; a.G = G; a.rows = R;
+    a.cache_len = p->cache_len; a.num_new = p->num_new; a.num_splits = f.splits;
+    a.stages = f.stages;
+    a.scale_log2 = (p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf(128.f)) * 1.4426950408889634f;
+    a.div_g = make_fast_div((uint32_t)G);
+    a.k_cache = (__nv_bfloat16*)const_cast<void*>(k_cache);
+    a.v_cache = (__nv_bfloat16*)const_cast<void*>(v_cache);
+    a.cache_cap = p->cache_capacity;
+    cudaError_t e;
+    if (fused) {
+        a.q_new = (const __nv_bfloat16*)fused->q_new;
+        a.k_new = (const __nv_bfloat16*)fused->k_new;
+        a.v_new = (const __nv_bfloat16*)fused->v_new;
+        a.q_stride = fused->q_stride; a.k_stride = fused->k_stride; a.v_stride = fused->v_stride;
+        a.q_rot = (__nv_bfloat16*)fused->q_rot;
+        a.out = (__nv_bfloat16*)fused->out;
+        a.lse_out = fused->lse_out;
+        a.log2_theta = log2(p->rope_theta);
+        a.table = (const double2*)p->rope_table;
+        a.table_first = p->rope_table_first_pos;
+        e = launch_few<true>(f, R, st, tm_k, tm_v, a);
+    } else {
+        e = launch_few<false>(f, R, st, tm_k, tm_v, a);
+    }
+    return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
+}
+
 evlnStatus_t noalloc_status_word(int** word);     // defined with the allocation-free variant below
 
 }  // namespace
@@ -490,6 +669,7 @@ evlnStatus_t evlnCreate(evlnHandle_t* handle, int device)
     e = cudaMalloc(&h->d_status, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int));
     if (e == cudaSuccess) e = prepare_kernels();
+    if (e == cudaSuccess) e = query_few_clusters(h->max_clusters);
     if (e == cudaSuccess && !attention_register_pool_ok()) {
         cudaFree(h->d_status);
         delete h;
@@ -610,13 +790,11 @@ evlnStatus_t evlnStepQRotSize(evlnHandle_t h, const evlnStepParams* p, size_t* b
     return EVLN_OK;
 }
 
-static evlnStatus_t rope_append_impl(evlnHandle_t h, const evlnStepParams* p, const void* q_new, const void* k_new,
-                                     const void* v_new, long q_stride_tok, long k_stride_tok, long v_stride_tok,
-                                     void* q_rot, void* k_cache, void* v_cache, void* stream, const PackedMap& map)
+// Argument checks of the append (the parameters themselves are checked, num_new > 0).
+static evlnStatus_t check_rope_append(evlnHandle_t h, const evlnStepParams* p, const void* q_new, const void* k_new,
+                                      const void* v_new, long q_stride_tok, long k_stride_tok, long v_stride_tok,
+                                      const void* q_rot, const void* k_cache, const void* v_cache)
 {
-    evlnStatus_t s = check_step_params(h, p);
-    if (s != EVLN_OK) return s;
-    if (p->num_new == 0) return EVLN_OK;
     if (!q_new || !k_new || !v_new || !q_rot || !k_cache || !v_cache) return EVLN_INVALID_VALUE;
     if (!aligned16(q_new) || !aligned16(k_new) || !aligned16(v_new) || !aligned16(q_rot) ||
         !aligned16(k_cache) || !aligned16(v_cache))
@@ -627,7 +805,18 @@ static evlnStatus_t rope_append_impl(evlnHandle_t h, const evlnStepParams* p, co
         v_stride_tok < (long)p->num_kv_heads * p->head_dim)
         return EVLN_INVALID_VALUE;
     if (q_stride_tok % vec || k_stride_tok % vec || v_stride_tok % vec) return EVLN_INVALID_VALUE;
+    return EVLN_OK;
+}
 
+static evlnStatus_t rope_append_impl(evlnHandle_t h, const evlnStepParams* p, const void* q_new, const void* k_new,
+                                     const void* v_new, long q_stride_tok, long k_stride_tok, long v_stride_tok,
+                                     void* q_rot, void* k_cache, void* v_cache, void* stream, const PackedMap& map)
+{
+    evlnStatus_t s = check_step_params(h, p);
+    if (s != EVLN_OK) return s;
+    if (p->num_new == 0) return EVLN_OK;
+    s = check_rope_append(h, p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, k_cache, v_cache);
+    if (s != EVLN_OK) return s;
     RopeArgs a = {};
     a.q_new = q_new; a.k_new = k_new; a.v_new = v_new;
     a.q_rot = q_rot; a.k_cache = k_cache; a.v_cache = v_cache;
@@ -678,7 +867,9 @@ evlnStatus_t evlnStepAttention(evlnHandle_t h, const evlnStepParams* p, const vo
     const float scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)D);
     cudaStream_t st = (cudaStream_t)stream;
 
-    if (use_tensor_kernel(p)) {
+    if (use_few_kernel(p)) {
+        return step_few(h, p, q_rot, k_cache, v_cache, o_part, lse_part, nullptr, st);
+    } else if (use_tensor_kernel(p)) {
         const int T = p->cache_len + p->num_new;
         CUtensorMap tm_q, tm_k, tm_v;
         {
@@ -778,6 +969,16 @@ evlnStatus_t evlnStep(evlnHandle_t h, const evlnStepParams* p, const void* q_new
     const long rows = (long)p->num_new * (p->num_q_heads / p->num_kv_heads);
     if (workspace_bytes < partial_bytes(resolve_splits(h, p), p->num_kv_heads, rows, p->head_dim))
         return EVLN_WORKSPACE_TOO_SMALL;
+    if (use_few_kernel(p) && p->num_new <= kFewFusedTokens) {
+        s = check_rope_append(h, p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, k_cache, v_cache);
+        if (s != EVLN_OK) return s;
+        const int S = resolve_splits(h, p);
+        float* o_part = (float*)workspace;
+        FewFused f = {q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, S == 1 ? out : nullptr, lse_out};
+        s = step_few(h, p, q_rot, k_cache, v_cache, o_part, o_part + (size_t)S * p->num_kv_heads * rows * 128, &f, (cudaStream_t)stream);
+        if (s != EVLN_OK || S == 1) return s;
+        return evlnStepCombine(h, p, workspace, out, lse_out, stream);
+    }
     s = evlnRopeAppend(h, p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, k_cache, v_cache,
                        stream);
     if (s != EVLN_OK) return s;
@@ -853,6 +1054,36 @@ evlnStatus_t evlnPagedStepAttention(evlnHandle_t h, const evlnPagedParams* p, co
     paged_schedule(h, p, h_cache_lens, h_new_offsets, &chunk, &smax, &items);
     if (workspace_bytes < partial_bytes(smax, p->num_kv_heads, rows, 128)) return EVLN_WORKSPACE_TOO_SMALL;
     if (items <= 0 || items > 0x3fffffffL) return EVLN_NOT_SUPPORTED;
+
+    if (paged_few(p, h_new_offsets)) {
+        CUtensorMap tm_k, tm_v;
+        cuuint64_t dims[4] = {128, 64, (cuuint64_t)p->num_kv_heads, (cuuint64_t)p->num_pages};
+        cuuint64_t strides[3] = {256, 64 * 256, (cuuint64_t)p->num_kv_heads * 64 * 256};
+        cuuint32_t box[4] = {64, kFewKeys, 1, 1};
+        if (!encode_map(h, &tm_k, k_pool, 4, dims, strides, box)) return EVLN_INVALID_VALUE;
+        if (!encode_map(h, &tm_v, v_pool, 4, dims, strides, box)) return EVLN_INVALID_VALUE;
+        int most = 0;
+        for (int b = 0; b < p->batch; ++b) most = h_new_offsets[b + 1] - h_new_offsets[b] > most ? h_new_offsets[b + 1] - h_new_offsets[b] : most;
+        FewArgs a = {};
+        a.o_part = (float*)workspace;
+        a.lse_part = a.o_part + (size_t)smax * p->num_kv_heads * rows * 128;
+        a.q_rot_in = (const __nv_bfloat16*)q_rot;
+        a.page_table = d_page_table; a.status = h->d_status;
+        a.Hkv = p->num_kv_heads; a.G = G; a.rows = (int)rows;
+        a.batch = p->batch; a.max_pages = p->max_pages_per_seq; a.chunk_tiles = chunk;
+        a.stages = kFewMaxStages;
+        a.scale_log2 = (p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf(128.f)) * 1.4426950408889634f;
+        a.div_g = make_fast_div((uint32_t)G);
+        BatchLens bl;
+        fill_lens(&bl, p, h_cache_lens, h_new_offsets, chunk);
+        if (bl.item_off[p->batch] != (int)items) return EVLN_INVALID_VALUE;
+        const size_t smem = few_smem_bytes(a.stages, most * G, 1, false, 0);
+        cudaStream_t st = (cudaStream_t)stream;
+        cudaError_t e = few_row_tiles(most * G) == 1
+                            ? launch_pdl(attn_few_kernel<1, true, false, BatchLens>, dim3((int)items), dim3(kFewThreads), smem, st, tm_k, tm_v, a, bl)
+                            : launch_pdl(attn_few_kernel<2, true, false, BatchLens>, dim3((int)items), dim3(kFewThreads), smem, st, tm_k, tm_v, a, bl);
+        return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
+    }
 
     CUtensorMap tm_q, tm_k, tm_v;
     {
@@ -986,7 +1217,7 @@ evlnStatus_t plan_packed(evlnHandle_t h, const evlnPackedParams* p, PackedPlan* 
     pl->chunk = pl->smax = 1;
     pl->items = 0;
     if (n_act > 0)
-        batch_schedule(h->num_sms, G, p->num_kv_heads, p->num_frames, pl->lens, pl->offs, true, p->kv_chunk_tiles,
+        batch_schedule(h->num_sms, G, p->num_kv_heads, p->num_frames, pl->lens, pl->offs, true, false, p->kv_chunk_tiles,
                        &pl->chunk, &pl->smax, &pl->items);
     size_t part_v = 0;
     if (n_vis > 0) {
@@ -1310,6 +1541,7 @@ evlnStatus_t noalloc_setup(int device, NoAllocDevice** out)
         e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
         if (e != cudaSuccess || qres != cudaDriverEntryPointSuccess || !fn) return EVLN_CUDA_ERROR;
         e = prepare_kernels();
+        if (e == cudaSuccess) e = query_few_clusters(d->ctx.max_clusters);
         if (e != cudaSuccess) return EVLN_CUDA_ERROR;
         if (!attention_register_pool_ok()) return EVLN_NOT_SUPPORTED;
         d->ctx.device = device;
