@@ -195,7 +195,8 @@ evlnStatus_t evlnStepCombine(evlnHandle_t handle, const evlnStepParams* params,
                              const void* workspace, void* out, float* lse_out, void* stream);
 
 /* The whole step in one call (Sec. 3.2): evlnRopeAppend, evlnStepAttention and evlnStepCombine
- * with the same arguments, enqueued back to back on `stream`; same results bit for bit.
+ * with the same arguments, enqueued on `stream`; same results bit for bit.  One launch instead of three for at most 32 query
+ * rows per kv head, two when the keys are not split.
  * All arguments are validated before the first launch; errors as for the three calls.          */
 evlnStatus_t evlnStep(evlnHandle_t handle, const evlnStepParams* params,
                       const void* q_new, const void* k_new, const void* v_new,
@@ -250,11 +251,12 @@ evlnStatus_t evlnPagedCheckTable(const evlnPagedParams* params, const int* h_cac
  * another chunk.  Position ids (the paper does not print them): the instruction and the visual
  * tokens are numbered contiguously as if no action token were there, chunk t continues after v_t.
  *
- * evlnPackedForward runs the whole sequence in one call and six launches, whatever N is: the
- * instruction and visual rows as ONE causal step on an empty cache (a query tile never loads a
- * KV tile beyond its own last token, and action tokens are not among its keys at all), then all
- * N action chunks as ONE batch whose items share prefixes of the cache just written and keep
- * their own rotated keys / values in a separate buffer.  No mask operand exists: the blocks the
+ * evlnPackedForward runs the whole sequence in one call and two launches, whatever N is: all tokens
+ * are rotated and stored, then the instruction and visual rows run as ONE causal step on an empty
+ * cache (a query tile never loads a KV tile beyond its own last token, and action tokens are not
+ * among its keys at all) beside all N action chunks, items that share prefixes of that cache and
+ * keep their own rotated keys / values in a separate buffer (a third launch merges them if
+ * kv_chunk_tiles cuts their keys).  No mask operand exists: the blocks the
  * mask removes are never loaded.
  *   q [T, Hq, D], k, v [T, Hkv, D]: the packed sequence, T = instr_len + N (frame_tokens +
  *       action_tokens), token strides in elements (multiples of 8);
@@ -273,7 +275,7 @@ typedef struct {
     int action_tokens;       /* |a|                                                          */
     int num_frames;          /* N                                                            */
     int cache_capacity;      /* token slots per kv head in k_cache / v_cache                 */
-    int kv_chunk_tiles;      /* max 128-key tiles per work item of the action batch; 0 = heuristic */
+    int kv_chunk_tiles;      /* max 128-key tiles per work item of the action batch; 0 = all */
     float softmax_scale;     /* 0 -> 1/sqrt(D)                                               */
     double rope_theta;
 } evlnPackedParams;

@@ -105,13 +105,29 @@ struct TcAttnArgs {
     int* status;              // device status word
     int Hkv, G;
     int rows;                 // packed rows per kv head over the whole call
-    int cache_len, num_new;   // contiguous only
+    int cache_len, num_new;   // contiguous (packed: the visual run)
     int num_splits;           // contiguous only
-    int units_per_head;       // contiguous only
+    int units_per_head;       // contiguous, packed
     int batch, max_pages, chunk_tiles;   // paged only
     float scale_log2;         // softmax scale * log2(e)
     FastDiv div_g;            // division by G
     FastDiv div_s;            // contiguous only: division by num_splits
+};
+
+// What a launch needs beyond that, for the set-up and the write-out only (apart from TcAttnArgs: in one
+// larger structure the pair kernel came out with 150 bytes of spills in its tile loop).
+struct TcOutArgs {
+    // Final output [n, Hq, 128] (+ log-sum-exps [n, Hq] or null) of rows whose keys are not split: their
+    // work item writes it itself.  Null: everything goes to o_part / lse_part.
+    __nv_bfloat16* out;
+    float* lse_out;
+    PackedMap map;            // where output token m goes (identity unless the call serves a packed sequence)
+    // packed sequence only: the action items come first (largest prefix first), then the units of the
+    // visual run (largest first), kv heads side by side
+    int act_items;            // work items of the action chunks
+    int act_split;            // some of them are splits: theirs go to o_part / lse_part
+    PackedMap act_map;
+    FastDiv div_hkv;
 };
 
 // --- descriptors --------------------------------------------------------------------------
@@ -263,23 +279,27 @@ struct WorkItem {
     int L, n;                 // episode lengths
     int row_base;             // first packed row of the episode within the kv head
     int j0, j1;               // KV tile range
+    bool visual;              // packed sequence: a unit of the visual run (else an action chunk's)
 };
 
-// Contiguous cache: the grid is (CTAS * units, kv heads, splits), so a CTA reads its work item off
+// Contiguous cache: the grid is (CTAS * kv heads, units, splits), so a CTA reads its work item off
 // its block index; the two divisions left (by G and by the split count) are multiplications by
-// constants the host prepared.  Batches (paged cache, or episodes sharing a cache prefix): items are
-// numbered episode by episode (kv head, unit, split inside), the host passes the first item of every
-// episode and the CTA searches that table.
+// constants the host prepared.  Units are taken from the last one down: where they do not all fit the
+// chip at once (a prefill), the ones with most keys start first and the last round is short.
+// Batches (paged cache, action chunks of a packed sequence): items are numbered episode by episode (kv
+// head, unit, split inside), the host passes the first item of every episode and the CTA searches that
+// table.
 template <bool PAGED, bool TAIL, typename LensT, int CTAS>
-__device__ __forceinline__ WorkItem decode_work(const TcAttnArgs& a, const LensT& lens)
+__device__ __forceinline__ WorkItem decode_work(const TcAttnArgs& a, const LensT& lens, const TcOutArgs& d)
 {
     constexpr int UNIT_ROWS = CTAS * kTileM;
     WorkItem w;
     if (!PAGED && !TAIL) {
         w.b = 0;
-        w.unit = CTAS == 2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-        w.g = (int)blockIdx.y;
+        w.unit = (int)(gridDim.y - 1 - blockIdx.y);
+        w.g = CTAS == 2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
         w.slot = (int)blockIdx.z;
+        w.visual = true;
         w.L = a.cache_len;
         w.n = a.num_new;
         w.row_base = 0;
@@ -287,7 +307,25 @@ __device__ __forceinline__ WorkItem decode_work(const TcAttnArgs& a, const LensT
         w.j0 = (int)fast_div((uint32_t)w.slot * nkv, a.div_s);
         w.j1 = (int)fast_div((uint32_t)(w.slot + 1) * nkv, a.div_s);
     } else {
-        const int item = (int)(blockIdx.x >> 1);
+        int item = (int)(blockIdx.x >> 1);
+        w.visual = TAIL && item >= d.act_items;
+        if (TAIL) {
+            if (w.visual) {
+                const uint32_t v = (uint32_t)(item - d.act_items), u = fast_div(v, d.div_hkv);
+                w.b = 0;
+                w.g = (int)(v - u * (uint32_t)a.Hkv);
+                w.unit = a.units_per_head - 1 - (int)u;
+                w.slot = 0;
+                w.L = 0;
+                w.n = a.num_new;
+                w.row_base = 0;
+                w.j0 = 0;
+                w.j1 = w.unit < 0 ? 0 : unit_kv_tiles_fast(0, w.n, a.div_g, w.unit, UNIT_ROWS);
+                if (w.unit < 0) w.b = -1;
+                return w;
+            }
+            item = d.act_items - 1 - item;
+        }
         int lo = 0, hi = a.batch;             // largest b with item_off[b] <= item
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
@@ -327,14 +365,15 @@ __device__ __forceinline__ WorkItem decode_work(const TcAttnArgs& a, const LensT
 // CTAS = 2: launched with a cluster of 2 CTAs along x: query tile = cluster rank.
 // CTAS = 1: no cluster; one query tile (all the rows of a kv head fit in it).
 
-// TAIL: a batch of items that share the first L_b tokens of ONE contiguous cache (every row sees all
-// of them) and bring their own n_b new tokens in a separate buffer (tm_kt / tm_vt, packed over the
-// batch; causal among themselves): the action chunks of a packed sequence (Sec. 3.3), each after
-// its own prefix of the visual tokens, none visible to another.
+// TAIL: a packed sequence (Sec. 3.3) in one launch.  Its visual run is an ordinary causal prefill on the
+// cache (tm_q, tm_k, tm_v).  Its action chunks are a batch of items that share the first L_b tokens of
+// that cache (every row sees all of them) and bring their own n_b new tokens in a separate buffer
+// (tm_qt / tm_kt / tm_vt, packed over the batch; causal among themselves), each after its own prefix of
+// the visual tokens, none visible to another.
 template <bool PAGED, bool TAIL, typename LensT, int CTAS>
 __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
-                                             const CUtensorMap* tm_kt, const CUtensorMap* tm_vt,
-                                             const TcAttnArgs& a, const LensT& lens)
+                                             const CUtensorMap* tm_qt, const CUtensorMap* tm_kt, const CUtensorMap* tm_vt,
+                                             const TcAttnArgs& a, const LensT& lens, const TcOutArgs& d)
 {
     static_assert(CTAS == 2 || !(PAGED || TAIL), "the batch kernels run on CTA pairs");
     static_assert(!(PAGED && TAIL), "one cache layout at a time");
@@ -380,13 +419,14 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
     const uint32_t rank = CTAS == 2 ? ptx::cluster_ctarank() : 0u;   // 0: issues the MMAs, owns the "(CTA 0)" barriers
     if (threadIdx.x == 0) EVLN_STAMP(0);
 
-    const WorkItem w = decode_work<PAGED, TAIL, LensT, CTAS>(a, lens);
+    const WorkItem w = decode_work<PAGED, TAIL, LensT, CTAS>(a, lens, d);
     if ((PAGED || TAIL) && w.b < 0) return;                      // both CTAs of the pair decode the same item
 
     const int rows_valid = w.n * a.G;                            // packed rows of this episode
     const int row0 = w.unit * kItemRows + (int)rank * kTileM;    // first row of this CTA's tile (episode-local)
     const int ntiles = w.j1 - w.j0;
-    const int nct = TAIL ? (w.L + kTileN - 1) / kTileN : 0;      // TAIL: tiles below nct come from the shared cache
+    // TAIL: tiles below nct come from the shared cache (all of a visual unit's)
+    const int nct = TAIL ? (w.visual ? 0x3fffffff : (w.L + kTileN - 1) / kTileN) : 0;
     // Lane quarters (32 rows each) of the tile that hold rows of the episode.  A CTA on its own lets
     // the softmax warps of the others sit out; a pair keeps all of them (both CTAs count alike).
     int quarters = 4;
@@ -416,6 +456,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
         ptx::prefetch_tensormap(&tm_k);
         ptx::prefetch_tensormap(&tm_v);
         if (TAIL) {
+            ptx::prefetch_tensormap(tm_qt);
             ptx::prefetch_tensormap(tm_kt);
             ptx::prefetch_tensormap(tm_vt);
         }
@@ -553,8 +594,9 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
                 const uint32_t dst = smem_base + kSmemQOff;
                 const int qrow = w.row_base + row0;
                 expect(q_full0, kTileBytes);
-                tma3(dst, &tm_q, q_full0, 0, qrow, w.g);
-                tma3(dst + kHalfBytes, &tm_q, q_full0, 64, qrow, w.g);
+                const CUtensorMap* map_q = TAIL && !w.visual ? tm_qt : &tm_q;
+                tma3(dst, map_q, q_full0, 0, qrow, w.g);
+                tma3(dst + kHalfBytes, map_q, q_full0, 64, qrow, w.g);
             }
         for (int jj = 0; jj < pre_k; ++jj) load_k(jj);
     }
@@ -675,8 +717,10 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
         // last visible key index; a padding row (beyond the episode's rows: its Q is zero fill or
         // another episode's) is never stored, so it takes everything unmasked rather than making its
         // warp mask every tile
-        // (TAIL: `bound` is the row's last visible token among the item's OWN tokens)
+        // (TAIL: `bound` is the row's last visible token among the item's OWN tokens, `cache_last` the last
+        // visible one of the cache)
         const int bound = row_valid ? (TAIL ? 0 : w.L) + (int)fast_div((uint32_t)r_local, a.div_g) : 0x3fffffff;
+        const int cache_last = w.visual ? bound : w.L - 1;
         const uint32_t t_lane = tmem + ((uint32_t)(quarter << 5) << 16);
         const uint32_t t_s = t_lane + (uint32_t)grp * 128 + (uint32_t)half * 64;          // its half of the group's score buffer
         const uint32_t t_p = t_lane + kColP + (uint32_t)grp * 64 + (uint32_t)half * 32;   // ... and of its P buffer
@@ -821,7 +865,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
             if (ok) {
                 ptx::fence_after_sync();
                 int lim0 = bound - w.j0 * kTileN;
-                if (TAIL) lim0 = w.j0 < nct ? w.L - 1 - w.j0 * kTileN : bound - (w.j0 - nct) * kTileN;
+                if (TAIL) lim0 = w.j0 < nct ? cache_last - w.j0 * kTileN : bound - (w.j0 - nct) * kTileN;
                 m_ref = first_block_reference(t_lane, lim0, a.scale_log2);
             }
         } else if (part != 0) {
@@ -857,7 +901,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
             int lim = bound - (w.j0 + jj) * kTileN - half * 64;
             if (TAIL) {
                 const int j = w.j0 + jj;
-                lim = (j < nct ? w.L - 1 - j * kTileN : bound - (j - nct) * kTileN) - half * 64;
+                lim = (j < nct ? cache_last - j * kTileN : bound - (j - nct) * kTileN) - half * 64;
             }
             if (!__all_sync(0xffffffffu, lim >= 63)) {
 #pragma unroll
@@ -970,12 +1014,40 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
             uint8_t* stage = smem_gen + kSmemKOff + (warp - 4) * (32 * 144);
             const int first_row = row0 + wrow0;                              // episode-local
             const int rows_here = rows_valid - first_row;                    // may be <= 0 or > 32
-            const long prow0 = ((long)w.slot * a.Hkv + w.g) * a.rows + w.row_base + first_row;
-            {
+            const bool direct = !PAGED && CTAS == 2 && d.out != nullptr && !(TAIL && !w.visual && d.act_split);
+            uint32_t regs[32];
+            ptx::tmem_ld32(t_o, regs);
+            ptx::tmem_ld_wait();
+            if (direct) {
+                // the row's only work item: round once to the storage dtype and write the output itself
+                auto out_row = [&](int rl) -> long {           // row of [n, Hq, 128] of the item's row rl
+                    const int tok = (int)fast_div((uint32_t)rl, a.div_g);
+                    const long t = TAIL ? packed_row(w.visual ? d.map : d.act_map, (w.visual ? 0 : (long)lens.new_off[w.b]) + tok)
+                                        : packed_row(d.map, tok);
+                    return t * (a.Hkv * a.G) + w.g * a.G + (rl - tok * a.G);
+                };
+                uint4* srow = reinterpret_cast<uint4*>(stage + lane * 80);
+#pragma unroll
+                for (int e = 0; e < 32; e += 8) {
+                    uint32_t v[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        v[c] = ptx::pack_bf16x2(__uint_as_float(regs[e + 2 * c]) * inv, __uint_as_float(regs[e + 2 * c + 1]) * inv);
+                    srow[e >> 3] = make_uint4(v[0], v[1], v[2], v[3]);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = i * 8 + (lane >> 2);
+                    if (r < rows_here)
+                        reinterpret_cast<uint4*>(d.out + out_row(first_row + r) * 128 + part * 32)[lane & 3] =
+                            *reinterpret_cast<const uint4*>(stage + r * 80 + (lane & 3) * 16);
+                }
+                if (d.lse_out && row_valid && part == 0)
+                    d.lse_out[out_row(r_local)] = (l > 0.f) ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
+            } else {
+                const long prow0 = ((long)w.slot * a.Hkv + w.g) * a.rows + w.row_base + first_row;
                 float* gbase = a.o_part + prow0 * 128 + part * 32;
-                uint32_t regs[32];
-                ptx::tmem_ld32(t_o, regs);
-                ptx::tmem_ld_wait();
                 float4* srow = reinterpret_cast<float4*>(stage + lane * 144);
 #pragma unroll
                 for (int e = 0; e < 32; e += 4)
@@ -990,9 +1062,9 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
                         *reinterpret_cast<float4*>(gbase + (long)r * 128 + (lane & 7) * 4) = v;
                     }
                 }
+                if (row_valid && part == 0)
+                    a.lse_part[prow0 + lane] = (l > 0.f) ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
             }
-            if (row_valid && part == 0)
-                a.lse_part[prow0 + lane] = (l > 0.f) ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
             if (warp == 4 && lane == 0) EVLN_STAMP(61);
         }
     }
@@ -1019,20 +1091,19 @@ template <bool PAGED, typename LensT>
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const TcAttnArgs a,
-                 const __grid_constant__ LensT lens)
+                 const __grid_constant__ LensT lens, const __grid_constant__ TcOutArgs d)
 {
-    attn_tc_body<PAGED, false, LensT, 2>(tm_q, tm_k, tm_v, nullptr, nullptr, a, lens);
+    attn_tc_body<PAGED, false, LensT, 2>(tm_q, tm_k, tm_v, nullptr, nullptr, nullptr, a, lens, d);
 }
 
-// CTA pairs over a batch of items that share a prefix of one contiguous cache and bring their own
-// new tokens in a separate buffer (the action chunks of a packed sequence, Sec. 3.3).
+// CTA pairs over a packed sequence (Sec. 3.3): the units of its visual run and its action chunks.
 __global__ void __launch_bounds__(kTcThreads, 1)
-attn_tail_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                 const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kt,
-                 const __grid_constant__ CUtensorMap tm_vt, const TcAttnArgs a,
-                 const __grid_constant__ BatchLens lens)
+attn_packed_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_qt,
+                   const __grid_constant__ CUtensorMap tm_kt, const __grid_constant__ CUtensorMap tm_vt, const TcAttnArgs a,
+                   const __grid_constant__ BatchLens lens, const __grid_constant__ TcOutArgs d)
 {
-    attn_tc_body<false, true, BatchLens, 2>(tm_q, tm_k, tm_v, &tm_kt, &tm_vt, a, lens);
+    attn_tc_body<false, true, BatchLens, 2>(tm_q, tm_k, tm_v, &tm_qt, &tm_kt, &tm_vt, a, lens, d);
 }
 
 // One CTA per work item, for steps whose rows per kv head fit one 128-row tile (the few action
@@ -1042,7 +1113,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 attn_solo_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const TcAttnArgs a)
 {
-    attn_tc_body<false, false, NoLens, 1>(tm_q, tm_k, tm_v, nullptr, nullptr, a, NoLens{});
+    attn_tc_body<false, false, NoLens, 1>(tm_q, tm_k, tm_v, nullptr, nullptr, nullptr, a, NoLens{}, TcOutArgs{});
 }
 
 }  // namespace evln

@@ -115,7 +115,7 @@ cudaError_t prepare_kernels()
     const std::pair<const void*, int> tc[4] = {{(const void*)attn_pair_kernel<false, NoLens>, kTcSmemBytes},
                                                {(const void*)attn_pair_kernel<true, BatchLens>, kTcSmemBytes},
                                                {(const void*)attn_solo_kernel, kSoloSmemBytes},
-                                               {(const void*)attn_tail_kernel, kTcSmemBytes}};
+                                               {(const void*)attn_packed_kernel, kTcSmemBytes}};
     for (const auto& k : tc) {
         cudaError_t e = cudaFuncSetAttribute(k.first, cudaFuncAttributeMaxDynamicSharedMemorySize, k.second);
         if (e != cudaSuccess) return e;
@@ -140,7 +140,7 @@ bool attention_register_pool_ok()
 {
     cudaFuncAttributes fa;
     const void* kernels[4] = {(const void*)attn_pair_kernel<false, NoLens>, (const void*)attn_pair_kernel<true, BatchLens>,
-                              (const void*)attn_solo_kernel, (const void*)attn_tail_kernel};
+                              (const void*)attn_solo_kernel, (const void*)attn_packed_kernel};
     for (const void* k : kernels) {
         if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return false;
         if (fa.numRegs != kRegsLaunch) return false;
@@ -545,20 +545,21 @@ void finish_rope_args(RopeArgs* a, int vec)
     while ((1 << a->page_shift) < a->page_size) ++a->page_shift;
 }
 
-// The append kernel for `tokens` tokens.  Few enough to be one wave of two blocks per SM: one thread
-// per work item (in whole warps, at most kRopeThreadsMax).  Else 256 threads.
+// Threads of the append kernels for `tokens` tokens.  Few enough to be one wave of two blocks per SM: one
+// thread per work item (in whole warps, at most kRopeThreadsMax).  Else 256 threads.
+int rope_threads(evlnHandle_t h, const RopeArgs& a, int tokens)
+{
+    if (tokens > 2 * h->num_sms) return kRopeThreads;
+    const int items = ((a.Hq + a.Hkv) << a.vph_shift) + (a.Hkv << (a.vph_shift + 1));
+    int t = (items + 31) / 32 * 32;
+    if (t > kRopeThreadsMax) t = kRopeThreadsMax;
+    return t < 64 ? 64 : t;
+}
+
 template <typename T, bool PAGED, typename LensT>
 void launch_rope_append(evlnHandle_t h, const RopeArgs& a, int tokens, cudaStream_t st, const LensT& lens)
 {
-    const bool few = tokens <= 2 * h->num_sms;
-    int t = kRopeThreads;
-    if (few) {
-        const int items = ((a.Hq + a.Hkv) << a.vph_shift) + (a.Hkv << (a.vph_shift + 1));
-        t = (items + 31) / 32 * 32;
-        if (t > kRopeThreadsMax) t = kRopeThreadsMax;
-        if (t < 64) t = 64;
-    }
-    launch_pdl(rope_append_kernel<T, PAGED, LensT>, dim3(tokens), dim3(t), 0, st, a, lens);
+    launch_pdl(rope_append_kernel<T, PAGED, LensT>, dim3(tokens), dim3(rope_threads(h, a, tokens)), 0, st, a, lens);
 }
 
 // What the one-launch step adds to an attention call: the new tokens and where the results go (out null:
@@ -808,9 +809,9 @@ static evlnStatus_t check_rope_append(evlnHandle_t h, const evlnStepParams* p, c
     return EVLN_OK;
 }
 
-static evlnStatus_t rope_append_impl(evlnHandle_t h, const evlnStepParams* p, const void* q_new, const void* k_new,
-                                     const void* v_new, long q_stride_tok, long k_stride_tok, long v_stride_tok,
-                                     void* q_rot, void* k_cache, void* v_cache, void* stream, const PackedMap& map)
+evlnStatus_t evlnRopeAppend(evlnHandle_t h, const evlnStepParams* p, const void* q_new, const void* k_new,
+                            const void* v_new, long q_stride_tok, long k_stride_tok, long v_stride_tok,
+                            void* q_rot, void* k_cache, void* v_cache, void* stream)
 {
     evlnStatus_t s = check_step_params(h, p);
     if (s != EVLN_OK) return s;
@@ -827,7 +828,6 @@ static evlnStatus_t rope_append_impl(evlnHandle_t h, const evlnStepParams* p, co
     a.log2_theta = log2(p->rope_theta);
     a.table = (const double2*)p->rope_table;
     a.table_first = p->rope_table_first_pos;
-    a.map = map;
     finish_rope_args(&a, p->dtype == EVLN_BF16 ? 8 : 4);
     NoLens nl = {};
     cudaStream_t st = (cudaStream_t)stream;
@@ -839,16 +839,15 @@ static evlnStatus_t rope_append_impl(evlnHandle_t h, const evlnStepParams* p, co
     return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
 }
 
-evlnStatus_t evlnRopeAppend(evlnHandle_t h, const evlnStepParams* p, const void* q_new, const void* k_new,
-                            const void* v_new, long q_stride_tok, long k_stride_tok, long v_stride_tok,
-                            void* q_rot, void* k_cache, void* v_cache, void* stream)
-{
-    return rope_append_impl(h, p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, k_cache,
-                            v_cache, stream, PackedMap{0, 0, 0, 0});
-}
-
-evlnStatus_t evlnStepAttention(evlnHandle_t h, const evlnStepParams* p, const void* q_rot, const void* k_cache,
-                               const void* v_cache, void* workspace, size_t workspace_bytes, void* stream)
+// Attention of a step.  `direct` (may be null): the step's final output; when the keys are not split and
+// the pair kernel runs, it writes that itself and `done` says that there is nothing left to combine.
+struct DirectOut {
+    void* out;
+    float* lse_out;
+    bool done;
+};
+static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, const void* q_rot, const void* k_cache,
+                                   const void* v_cache, void* workspace, size_t workspace_bytes, void* stream, DirectOut* direct)
 {
     evlnStatus_t s = check_step_params(h, p);
     if (s != EVLN_OK) return s;
@@ -900,12 +899,19 @@ evlnStatus_t evlnStepAttention(evlnHandle_t h, const evlnStepParams* p, const vo
         a.div_s = make_fast_div((uint32_t)S);
         NoLens nl = {};
         // one work item per (unit, kv head, split): the kernels read it off the block index
-        if (a.units_per_head > 32767 || p->num_kv_heads > 65535) return EVLN_NOT_SUPPORTED;
-        if (use_solo_kernel(p))
-            launch_pdl(attn_solo_kernel, dim3(1, p->num_kv_heads, S), dim3(kTcThreads), kSoloSmemBytes, st, tm_q, tm_k, tm_v, a);
-        else
-            launch_pair_pdl(attn_pair_kernel<false, NoLens>, dim3(2 * a.units_per_head, p->num_kv_heads, S), kTcSmemBytes, st,
-                            tm_q, tm_k, tm_v, a, nl);
+        if (a.units_per_head > 65535 || p->num_kv_heads > 65535) return EVLN_NOT_SUPPORTED;
+        if (use_solo_kernel(p)) {
+            launch_pdl(attn_solo_kernel, dim3(p->num_kv_heads, 1, S), dim3(kTcThreads), kSoloSmemBytes, st, tm_q, tm_k, tm_v, a);
+        } else {
+            TcOutArgs d = {};
+            if (direct && S == 1) {
+                d.out = (__nv_bfloat16*)direct->out;
+                d.lse_out = direct->lse_out;
+                direct->done = true;
+            }
+            launch_pair_pdl(attn_pair_kernel<false, NoLens>, dim3(2 * p->num_kv_heads, a.units_per_head, S), kTcSmemBytes, st,
+                            tm_q, tm_k, tm_v, a, nl, d);
+        }
     } else {
         SimtAttnArgs a = {};
         a.q_rot = q_rot; a.k_cache = k_cache; a.v_cache = v_cache;
@@ -928,8 +934,14 @@ evlnStatus_t evlnStepAttention(evlnHandle_t h, const evlnStepParams* p, const vo
 }
 
 
-static evlnStatus_t step_combine_impl(evlnHandle_t h, const evlnStepParams* p, const void* workspace, void* out,
-                                      float* lse_out, void* stream, const PackedMap& map)
+evlnStatus_t evlnStepAttention(evlnHandle_t h, const evlnStepParams* p, const void* q_rot, const void* k_cache,
+                               const void* v_cache, void* workspace, size_t workspace_bytes, void* stream)
+{
+    return step_attention(h, p, q_rot, k_cache, v_cache, workspace, workspace_bytes, stream, nullptr);
+}
+
+evlnStatus_t evlnStepCombine(evlnHandle_t h, const evlnStepParams* p, const void* workspace, void* out,
+                             float* lse_out, void* stream)
 {
     evlnStatus_t s = check_step_params(h, p);
     if (s != EVLN_OK) return s;
@@ -944,16 +956,9 @@ static evlnStatus_t step_combine_impl(evlnHandle_t h, const evlnStepParams* p, c
     a.lse_part = a.o_part + (size_t)S * p->num_kv_heads * R * p->head_dim;
     a.out = out; a.lse_out = lse_out;
     a.Hkv = p->num_kv_heads; a.G = G; a.D = p->head_dim; a.rows = R; a.num_splits = S;
-    a.map = map;
     cudaStream_t st = (cudaStream_t)stream;
     if (p->dtype == EVLN_BF16) return launch_combine<__nv_bfloat16>(h, a, p->head_dim, false, nullptr, st);
     return launch_combine<float>(h, a, p->head_dim, false, nullptr, st);
-}
-
-evlnStatus_t evlnStepCombine(evlnHandle_t h, const evlnStepParams* p, const void* workspace, void* out,
-                             float* lse_out, void* stream)
-{
-    return step_combine_impl(h, p, workspace, out, lse_out, stream, PackedMap{0, 0, 0, 0});
 }
 
 evlnStatus_t evlnStep(evlnHandle_t h, const evlnStepParams* p, const void* q_new, const void* k_new,
@@ -982,8 +987,9 @@ evlnStatus_t evlnStep(evlnHandle_t h, const evlnStepParams* p, const void* q_new
     s = evlnRopeAppend(h, p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, k_cache, v_cache,
                        stream);
     if (s != EVLN_OK) return s;
-    s = evlnStepAttention(h, p, q_rot, k_cache, v_cache, workspace, workspace_bytes, stream);
-    if (s != EVLN_OK) return s;
+    DirectOut direct = {out, lse_out, false};
+    s = step_attention(h, p, q_rot, k_cache, v_cache, workspace, workspace_bytes, stream, &direct);
+    if (s != EVLN_OK || direct.done) return s;
     return evlnStepCombine(h, p, workspace, out, lse_out, stream);
 }
 
@@ -1113,7 +1119,7 @@ evlnStatus_t evlnPagedStepAttention(evlnHandle_t h, const evlnPagedParams* p, co
     fill_lens(&bl, p, h_cache_lens, h_new_offsets, chunk);
     if (bl.item_off[p->batch] != (int)items) return EVLN_INVALID_VALUE;
     launch_pair_pdl(attn_pair_kernel<true, BatchLens>, dim3(2 * (int)items), kTcSmemBytes, (cudaStream_t)stream, tm_q, tm_k,
-                    tm_v, a, bl);
+                    tm_v, a, bl, TcOutArgs{});
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
 }
@@ -1177,7 +1183,6 @@ evlnStatus_t evlnPagedCheckTable(const evlnPagedParams* p, const int* h_cache_le
 namespace {
 struct PackedPlan {
     int n_vis, n_act;            // instruction + visual tokens; action tokens
-    evlnStepParams vis;          // the visual run as one step on an empty cache
     int lens[kMaxBatch];         // per action chunk: visible prefix of the cache
     int offs[kMaxBatch + 1];     // per action chunk: first own token
     int chunk, smax;             // KV tiles per work item of the action batch, its largest split count
@@ -1201,14 +1206,6 @@ evlnStatus_t plan_packed(evlnHandle_t h, const evlnPackedParams* p, PackedPlan* 
     if (n_vis > (long)p->cache_capacity) return EVLN_CACHE_FULL;
     pl->n_vis = (int)n_vis;
     pl->n_act = (int)n_act;
-    evlnStepParams& sp = pl->vis;
-    memset(&sp, 0, sizeof(sp));
-    sp.struct_size = sizeof(sp);
-    sp.dtype = EVLN_BF16;
-    sp.num_q_heads = p->num_q_heads; sp.num_kv_heads = p->num_kv_heads; sp.head_dim = 128;
-    sp.cache_len = 0; sp.num_new = (int)n_vis; sp.cache_capacity = p->cache_capacity;
-    sp.num_splits = 0; sp.kernel = EVLN_KERNEL_AUTO;
-    sp.softmax_scale = p->softmax_scale; sp.rope_theta = p->rope_theta;
     for (int t = 0; t < p->num_frames; ++t) {
         pl->lens[t] = p->instr_len + (t + 1) * p->frame_tokens;      // chunk t sees the instruction and v_1 .. v_{t+1}
         pl->offs[t] = t * p->action_tokens;
@@ -1216,22 +1213,18 @@ evlnStatus_t plan_packed(evlnHandle_t h, const evlnPackedParams* p, PackedPlan* 
     pl->offs[p->num_frames] = (int)n_act;
     pl->chunk = pl->smax = 1;
     pl->items = 0;
+    // an action chunk walks no more keys than the largest unit of the visual run beside it: not split
+    // unless the caller says so
     if (n_act > 0)
-        batch_schedule(h->num_sms, G, p->num_kv_heads, p->num_frames, pl->lens, pl->offs, true, false, p->kv_chunk_tiles,
-                       &pl->chunk, &pl->smax, &pl->items);
-    size_t part_v = 0;
-    if (n_vis > 0) {
-        evlnStatus_t s = check_step_params(h, &sp);
-        if (s != EVLN_OK) return s;
-        part_v = partial_bytes(resolve_splits(h, &sp), p->num_kv_heads, n_vis * G, 128);
-    }
-    const size_t part_a = n_act > 0 ? partial_bytes(pl->smax, p->num_kv_heads, n_act * G, 128) : 0;
+        batch_schedule(h->num_sms, G, p->num_kv_heads, p->num_frames, pl->lens, pl->offs, true, false,
+                       p->kv_chunk_tiles > 0 ? p->kv_chunk_tiles : 1 << 24, &pl->chunk, &pl->smax, &pl->items);
+    const size_t part_a = pl->smax > 1 ? partial_bytes(pl->smax, p->num_kv_heads, n_act * G, 128) : 0;
     size_t off = 0;
     pl->off_qv = off; off += round_up((size_t)n_vis * p->num_q_heads * 128 * 2, 256);
     pl->off_qa = off; off += round_up((size_t)n_act * p->num_q_heads * 128 * 2, 256);
     pl->off_tk = off; off += round_up((size_t)n_act * p->num_kv_heads * 128 * 2, 256);
     pl->off_tv = off; off += round_up((size_t)n_act * p->num_kv_heads * 128 * 2, 256);
-    pl->off_part = off; off += part_v > part_a ? part_v : part_a;
+    pl->off_part = off; off += part_a;
     pl->bytes = off > 256 ? off : 256;
     return EVLN_OK;
 }
@@ -1268,86 +1261,81 @@ extern "C" evlnStatus_t evlnPackedForward(evlnHandle_t h, const evlnPackedParams
     char* ws = (char*)workspace;
     cudaStream_t st = (cudaStream_t)stream;
     const int G = p->num_q_heads / p->num_kv_heads;
-    const PackedMap map_v{p->instr_len, p->frame_tokens, p->action_tokens, 0};
-    const PackedMap map_a{p->instr_len, p->frame_tokens, p->action_tokens, 1};
-
-    // the instruction and the visual tokens: ONE causal step on an empty cache; its query tiles never
-    // load a KV tile past their own last token, and no action token is among the keys at all
-    if (pl.n_vis > 0) {
-        s = rope_append_impl(h, &pl.vis, q, k, v, q_stride_tok, k_stride_tok, v_stride_tok, ws + pl.off_qv, k_cache, v_cache,
-                             stream, map_v);
-        if (s != EVLN_OK) return s;
-        const size_t part_v = partial_bytes(resolve_splits(h, &pl.vis), p->num_kv_heads, (long)pl.n_vis * G, 128);
-        s = evlnStepAttention(h, &pl.vis, ws + pl.off_qv, k_cache, v_cache, ws + pl.off_part, part_v, stream);
-        if (s != EVLN_OK) return s;
-        s = step_combine_impl(h, &pl.vis, ws + pl.off_part, out, lse_out, stream, map_v);
-        if (s != EVLN_OK) return s;
-    }
-    if (pl.n_act == 0) return EVLN_OK;
-
-    // all action chunks in one batch: chunk t sees the first lens[t] tokens of the cache just written
-    // and its own tokens, which live in a buffer of their own (nobody else's keys)
+    if ((long)ceil_div(pl.n_vis * G, kUnitRows) * p->num_kv_heads + pl.items > 0x3fffffffL) return EVLN_NOT_SUPPORTED;
     BatchLens bl;
     fill_batch_lens(&bl, G, p->num_kv_heads, p->num_frames, pl.lens, pl.offs, pl.chunk, true);
-    if (bl.item_off[p->num_frames] != (int)pl.items || pl.items <= 0 || pl.items > 0x3fffffffL) return EVLN_NOT_SUPPORTED;
+    if (bl.item_off[p->num_frames] != (int)pl.items) return EVLN_NOT_SUPPORTED;
+
+    // every token of the sequence: the visual run into the cache, the action tokens into buffers of their
+    // own (nobody else's keys)
     {
-        RopeArgs a = {};
-        a.q_new = q; a.k_new = k; a.v_new = v;
-        a.q_rot = ws + pl.off_qa; a.k_cache = ws + pl.off_tk; a.v_cache = ws + pl.off_tv; a.page_table = nullptr;
-        a.q_stride = q_stride_tok; a.k_stride = k_stride_tok; a.v_stride = v_stride_tok;
-        a.Hq = p->num_q_heads; a.Hkv = p->num_kv_heads; a.D = 128;
-        a.num_new = pl.n_act; a.batch = p->num_frames; a.page_size = 1; a.max_pages = 0;
-        a.log2_theta = log2(p->rope_theta);
-        a.tail = 1;
-        a.map = map_a;
-        finish_rope_args(&a, 8);
-        launch_rope_append<__nv_bfloat16, true, BatchLens>(h, a, pl.n_act, st, bl);
-        cudaError_t e = cudaGetLastError();
+        RopePackedArgs a = {};
+        a.r.q_new = q; a.r.k_new = k; a.r.v_new = v;
+        a.r.q_rot = ws + pl.off_qv; a.r.k_cache = k_cache; a.r.v_cache = v_cache;
+        a.r.q_stride = q_stride_tok; a.r.k_stride = k_stride_tok; a.r.v_stride = v_stride_tok;
+        a.r.Hq = p->num_q_heads; a.r.Hkv = p->num_kv_heads; a.r.D = 128;
+        a.r.num_new = pl.n_vis + pl.n_act; a.r.cache_cap = p->cache_capacity;
+        a.r.page_size = 1;
+        a.r.log2_theta = log2(p->rope_theta);
+        finish_rope_args(&a.r, 8);
+        a.num_visual = pl.n_vis; a.num_action = pl.n_act;
+        a.I = p->instr_len; a.F = p->frame_tokens; a.A = p->action_tokens;
+        a.div_f = make_fast_div((uint32_t)(p->frame_tokens > 0 ? p->frame_tokens : 1));
+        a.div_a = make_fast_div((uint32_t)(p->action_tokens > 0 ? p->action_tokens : 1));
+        a.q_rot_act = ws + pl.off_qa; a.k_act = ws + pl.off_tk; a.v_act = ws + pl.off_tv;
+        cudaError_t e = launch_pdl(rope_packed_kernel, dim3(a.r.num_new), dim3(rope_threads(h, a.r, a.r.num_new)), 0, st, a);
         if (e != cudaSuccess) return cuda_fail(h, e);
     }
-    const long rows = (long)pl.n_act * G;
+    // one launch: the visual run as one causal prefill (its query tiles never load a KV tile past their own
+    // last token, and no action token is among the keys at all), and beside it the action chunks, chunk t
+    // seeing the first lens[t] tokens of the cache and its own tokens
+    const long rows_a = (long)pl.n_act * G;
+    const bool split = pl.smax > 1;
     {
-        CUtensorMap tm_q, tm_k, tm_v, tm_kt, tm_vt;
-        cuuint32_t box_q[3] = {64, 128, 1}, box_k[3] = {64, 64, 1}, box_v[3] = {64, 128, 1};
-        {
-            cuuint64_t dims[3] = {128, (cuuint64_t)rows, (cuuint64_t)p->num_kv_heads};
-            cuuint64_t strides[2] = {256, (cuuint64_t)rows * 256};
-            if (!encode_map(h, &tm_q, ws + pl.off_qa, 3, dims, strides, box_q)) return EVLN_INVALID_VALUE;
+        CUtensorMap maps[6];              // visual q, k, v; action q, k, v
+        const cuuint32_t box_q[3] = {64, 128, 1}, box_k[3] = {64, 64, 1}, box_v[3] = {64, 128, 1};
+        const cuuint32_t* boxes[3] = {box_q, box_k, box_v};
+        const void* bases[6] = {ws + pl.off_qv, k_cache, v_cache, ws + pl.off_qa, ws + pl.off_tk, ws + pl.off_tv};
+        const long rows[6] = {(long)pl.n_vis * G, pl.n_vis, pl.n_vis, rows_a, pl.n_act, pl.n_act};
+        const long pitch[6] = {rows[0], p->cache_capacity, p->cache_capacity, rows_a, pl.n_act, pl.n_act};
+        for (int i = 0; i < 6; ++i) {
+            if (rows[i] == 0) continue;
+            cuuint64_t dims[3] = {128, (cuuint64_t)rows[i], (cuuint64_t)p->num_kv_heads};
+            cuuint64_t strides[2] = {256, (cuuint64_t)pitch[i] * 256};
+            if (!encode_map(h, &maps[i], bases[i], 3, dims, strides, boxes[i % 3])) return EVLN_INVALID_VALUE;
         }
-        {
-            cuuint64_t dims[3] = {128, (cuuint64_t)pl.n_vis, (cuuint64_t)p->num_kv_heads};
-            cuuint64_t strides[2] = {256, (cuuint64_t)p->cache_capacity * 256};
-            if (!encode_map(h, &tm_k, k_cache, 3, dims, strides, box_k)) return EVLN_INVALID_VALUE;
-            if (!encode_map(h, &tm_v, v_cache, 3, dims, strides, box_v)) return EVLN_INVALID_VALUE;
-        }
-        {
-            cuuint64_t dims[3] = {128, (cuuint64_t)pl.n_act, (cuuint64_t)p->num_kv_heads};
-            cuuint64_t strides[2] = {256, (cuuint64_t)pl.n_act * 256};
-            if (!encode_map(h, &tm_kt, ws + pl.off_tk, 3, dims, strides, box_k)) return EVLN_INVALID_VALUE;
-            if (!encode_map(h, &tm_vt, ws + pl.off_tv, 3, dims, strides, box_v)) return EVLN_INVALID_VALUE;
-        }
+        for (int i = 0; i < 6; ++i)       // a run without tokens loads nothing: any valid map will do
+            if (rows[i] == 0) maps[i] = maps[(i + 3) % 6];
         const float scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf(128.f);
         TcAttnArgs a = {};
         a.o_part = (float*)(ws + pl.off_part);
-        a.lse_part = a.o_part + (size_t)pl.smax * p->num_kv_heads * rows * 128;
-        a.page_table = nullptr; a.status = h->d_status;
-        a.Hkv = p->num_kv_heads; a.G = G; a.rows = (int)rows;
-        a.batch = p->num_frames; a.max_pages = 0; a.chunk_tiles = pl.chunk;
+        a.lse_part = a.o_part + (size_t)pl.smax * p->num_kv_heads * rows_a * 128;
+        a.status = h->d_status;
+        a.Hkv = p->num_kv_heads; a.G = G; a.rows = (int)rows_a;
+        a.num_new = pl.n_vis; a.units_per_head = ceil_div(pl.n_vis * G, kUnitRows);
+        a.batch = p->num_frames; a.chunk_tiles = pl.chunk;
         a.scale_log2 = scale * 1.4426950408889634f;
         a.div_g = make_fast_div((uint32_t)G);
         a.div_s = make_fast_div(1u);
-        launch_pair_pdl(attn_tail_kernel, dim3(2 * (int)pl.items), kTcSmemBytes, st, tm_q, tm_k, tm_v, tm_kt, tm_vt, a, bl);
-        cudaError_t e = cudaGetLastError();
+        TcOutArgs d = {};
+        d.out = (__nv_bfloat16*)out; d.lse_out = lse_out;
+        d.map = PackedMap{p->instr_len, p->frame_tokens, p->action_tokens, 0};
+        d.act_items = (int)pl.items; d.act_split = split;
+        d.act_map = PackedMap{p->instr_len, p->frame_tokens, p->action_tokens, 1};
+        d.div_hkv = make_fast_div((uint32_t)p->num_kv_heads);
+        cudaError_t e = launch_pair_pdl(attn_packed_kernel, dim3(2 * (unsigned)(pl.items + (long)a.units_per_head * p->num_kv_heads)),
+                                        kTcSmemBytes, st, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], a, bl, d);
         if (e != cudaSuccess) return cuda_fail(h, e);
     }
+    if (!split) return EVLN_OK;
     CombineArgs c = {};
     c.o_part = (const float*)(ws + pl.off_part);
-    c.lse_part = c.o_part + (size_t)pl.smax * p->num_kv_heads * rows * 128;
+    c.lse_part = c.o_part + (size_t)pl.smax * p->num_kv_heads * rows_a * 128;
     c.out = out; c.lse_out = lse_out;
-    c.Hkv = p->num_kv_heads; c.G = G; c.D = 128; c.rows = (int)rows; c.num_splits = pl.smax;
+    c.Hkv = p->num_kv_heads; c.G = G; c.D = 128; c.rows = (int)rows_a; c.num_splits = pl.smax;
     c.batch = p->num_frames; c.unit_rows = kUnitRows; c.chunk_tiles = pl.chunk;
     c.tail = 1;
-    c.map = map_a;
+    c.map = PackedMap{p->instr_len, p->frame_tokens, p->action_tokens, 1};
     return launch_combine<__nv_bfloat16>(h, c, 128, true, &bl, st);
 }
 
@@ -1582,8 +1570,9 @@ extern "C" evlnStatus_t evlnStepAttentionNoAlloc(const evlnStepParams* p, const 
     if (s != EVLN_OK) return s;
     if (need > (size_t)EVLN_NOALLOC_SCRATCH_BYTES) return EVLN_WORKSPACE_TOO_SMALL;
     if (p->num_new == 0) return EVLN_OK;
-    if (!out) return EVLN_INVALID_VALUE;
-    s = evlnStepAttention(h, p, q_rot, k_cache, v_cache, d->scratch, (size_t)EVLN_NOALLOC_SCRATCH_BYTES, stream);
-    if (s != EVLN_OK) return s;
+    if (!out || !aligned16(out)) return EVLN_INVALID_VALUE;
+    DirectOut direct = {out, lse_out, false};
+    s = step_attention(h, p, q_rot, k_cache, v_cache, d->scratch, (size_t)EVLN_NOALLOC_SCRATCH_BYTES, stream, &direct);
+    if (s != EVLN_OK || direct.done) return s;
     return evlnStepCombine(h, p, d->scratch, out, lse_out, stream);
 }

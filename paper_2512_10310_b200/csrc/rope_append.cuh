@@ -38,9 +38,6 @@ struct RopeArgs {
     double log2_theta;
     const double2* table;   // optional: (cos, sin) per (position - table_first, j), [count][D/2]
     int table_first;
-    int tail;               // batch mode without pages: K/V of new token m go to row m of k_cache / v_cache
-                            // = buffers [Hkv, total new tokens, D] (the items' own tokens, not a shared cache)
-    PackedMap map;          // where new token m sits in q_new / k_new / v_new (identity unless packed)
     // derived by the host (finish_rope_args): the threads decode their work with shifts and one
     // multiplication instead of integer divisions
     int G;                  // Hq / Hkv
@@ -132,66 +129,32 @@ rope_table_kernel(double2* table, int first_pos, int count, int D, double log2_t
 constexpr int kRopeThreadsMax = 384;
 constexpr int kRopeThreads = 256;
 
-template <typename T, bool PAGED, typename LensT>
-__global__ void __launch_bounds__(kRopeThreadsMax)
-rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
+// Where one new token comes from and goes to.
+template <typename T>
+struct TokenPlace {
+    long src_tok;            // its row of q_new / k_new / v_new
+    T* q_dst;                // its first query row of kv head 0, ...
+    long q_rows;             //   rows per kv head of that buffer
+    T* k_dst;                // its key / value row of kv head 0, ...
+    T* v_dst;
+    long kv_rows;            //   rows from one kv head to the next
+};
+
+// Rotates and stores one token with the whole block; the angles are in s_angle once the block has met.
+template <typename T>
+__device__ __forceinline__ void rope_token(const RopeArgs& a, const TokenPlace<T>& t, const typename Rotation<T>::Angle* s_angle)
 {
     constexpr int V = VecTraits<T>::kVec;
-    __shared__ typename Rotation<T>::Angle s_angle[72];                // angle j at j + j / 8: the 8 vectors of a half head in different banks
-
-    const int tok = blockIdx.x;           // index into the packed new tokens
-    const int D = a.D, half = D / 2;
-    const int G = a.G;
-
-    int b = 0, i = tok, L = a.cache_len, n_b = a.num_new;
-    if (PAGED) {
-        int lo = 0, hi = a.batch;         // largest b with new_off[b] <= tok
-        while (hi - lo > 1) {
-            int mid = (lo + hi) >> 1;
-            if (lens.new_off[mid] <= tok) lo = mid; else hi = mid;
-        }
-        b = lo;
-        i = tok - lens.new_off[b];
-        L = lens.cache_len[b];
-        n_b = lens.new_off[b + 1] - lens.new_off[b];
-    }
-    const long pos = (long)L + i;
-    // (so far launch parameters only; what follows reads memory that earlier kernels may have written)
-    asm volatile("griddepcontrol.wait;" ::: "memory");          // programmatic dependent launch: inputs ready
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const double2* trow = a.table ? a.table + (pos - a.table_first) * half : nullptr;
-
-    if (threadIdx.x < half) {
-        const int j = threadIdx.x;
-        const double2 cs = trow ? trow[j] : rope_cos_sin(pos, j, D, a.log2_theta);
-        s_angle[j + (j >> 3)] = Rotation<T>::angle(cs);
-    }
-
-    // destination of this token's K/V row for kv head g (element offset)
-    long page_base = 0;     // paged: (page_id * Hkv) * page_size * D, slot within page
-    int slot = 0;
-    if (PAGED && !a.tail) {
-        int pg = a.page_table[(long)b * a.max_pages + (int)(pos >> a.page_shift)];
-        slot = (int)(pos & (a.page_size - 1));
-        page_base = (long)pg * a.Hkv * a.page_size * D;
-    }
-    auto kv_row = [&](int g) -> long {
-        if (PAGED && a.tail) return ((long)g * lens.new_off[a.batch] + tok) * D;
-        if (PAGED) return page_base + ((long)g * a.page_size + slot) * D;
-        return ((long)g * a.cache_cap + pos) * D;
-    };
-
-    const long src_tok = packed_row(a.map, tok);
-    const T* q_tok = (const T*)a.q_new + src_tok * a.q_stride;
-    const T* k_tok = (const T*)a.k_new + src_tok * a.k_stride;
-    const T* v_tok = (const T*)a.v_new + src_tok * a.v_stride;
+    const int D = a.D, half = D / 2, G = a.G;
+    const T* q_tok = (const T*)a.q_new + t.src_tok * a.q_stride;
+    const T* k_tok = (const T*)a.k_new + t.src_tok * a.k_stride;
+    const T* v_tok = (const T*)a.v_new + t.src_tok * a.v_stride;
 
     const int vph = a.vph_shift, vpr = a.vph_shift + 1;       // vectors per half head vector / per head vector (log2)
     const int q_items = a.Hq << vph;
     const int k_items = a.Hkv << vph;
     const int v_items = a.Hkv << vpr;
     const int items = q_items + k_items + v_items;
-    const long rows_per_head = PAGED ? (long)lens.new_off[a.batch] * G : (long)a.num_new * G;
 
     // a thread's work item `it`: a pair of 16-byte vectors (j0.., j0+half..) of a query or key head,
     // or one 16-byte vector of a value head
@@ -220,9 +183,9 @@ rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
             T* dst;
             if (is_q) {
                 const int g = (int)fast_div((uint32_t)h, a.div_g);
-                dst = (T*)a.q_rot + ((long)g * rows_per_head + (long)tok * G + (h - g * G)) * D;
+                dst = t.q_dst + ((long)g * t.q_rows + (h - g * G)) * D;
             } else {
-                dst = (T*)a.k_cache + kv_row(h);
+                dst = t.k_dst + (long)h * t.kv_rows * D;
             }
             const T* lo = reinterpret_cast<const T*>(&lo_raw);
             const T* hi = reinterpret_cast<const T*>(&hi_raw);
@@ -242,20 +205,75 @@ rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
             const int e = it - q_items - k_items;
             const int g = e >> vpr;
             const int d0 = (e & ((1 << vpr) - 1)) * V;
-            *reinterpret_cast<uint4*>((T*)a.v_cache + kv_row(g) + d0) = lo_raw;
+            *reinterpret_cast<uint4*>(t.v_dst + (long)g * t.kv_rows * D + d0) = lo_raw;
         }
     };
 
     uint4 r0 = make_uint4(0u, 0u, 0u, 0u), r1 = r0;
-    if ((int)threadIdx.x < items) load_item(threadIdx.x, r0, r1);     // in flight while the cos/sin arrive
+    if ((int)threadIdx.x < items) load_item(threadIdx.x, r0, r1);     // in flight while the angles arrive
     __syncthreads();
     if ((int)threadIdx.x < items) finish_item(threadIdx.x, r0, r1);
     for (int it = threadIdx.x + blockDim.x; it < items; it += blockDim.x) {
         load_item(it, r0, r1);
         finish_item(it, r0, r1);
     }
+}
 
-    if (PAGED && !a.tail && i == n_b - 1 && slot + 1 < a.page_size) {
+// The angles of position `pos` into shared memory (angle j at j + j / 8: the 8 vectors of a half head in
+// different banks).
+template <typename T>
+__device__ __forceinline__ void load_angles(typename Rotation<T>::Angle* s_angle, const double2* table, long table_first, long pos,
+                                            int D, double log2_theta)
+{
+    const int j = threadIdx.x;
+    if (j < D / 2)
+        s_angle[j + (j >> 3)] = Rotation<T>::angle(table ? table[(pos - table_first) * (D / 2) + j] : rope_cos_sin(pos, j, D, log2_theta));
+}
+
+template <typename T, bool PAGED, typename LensT>
+__global__ void __launch_bounds__(kRopeThreadsMax)
+rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
+{
+    constexpr int V = VecTraits<T>::kVec;
+    __shared__ typename Rotation<T>::Angle s_angle[72];
+
+    const int tok = blockIdx.x;           // index into the packed new tokens
+    const int D = a.D;
+
+    int b = 0, i = tok, L = a.cache_len, n_b = a.num_new;
+    if (PAGED) {
+        int lo = 0, hi = a.batch;         // largest b with new_off[b] <= tok
+        while (hi - lo > 1) {
+            int mid = (lo + hi) >> 1;
+            if (lens.new_off[mid] <= tok) lo = mid; else hi = mid;
+        }
+        b = lo;
+        i = tok - lens.new_off[b];
+        L = lens.cache_len[b];
+        n_b = lens.new_off[b + 1] - lens.new_off[b];
+    }
+    const long pos = (long)L + i;
+    // (so far launch parameters only; what follows reads memory that earlier kernels may have written)
+    asm volatile("griddepcontrol.wait;" ::: "memory");          // programmatic dependent launch: inputs ready
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    load_angles<T>(s_angle, a.table, a.table_first, pos, D, a.log2_theta);
+
+    long page_base = 0;     // paged: first row of the page in the pool; slot within the page
+    int slot = 0;
+    if (PAGED) {
+        page_base = (long)a.page_table[(long)b * a.max_pages + (int)(pos >> a.page_shift)] * a.Hkv * a.page_size;
+        slot = (int)(pos & (a.page_size - 1));
+    }
+    TokenPlace<T> t;
+    t.src_tok = tok;
+    t.q_dst = (T*)a.q_rot + (long)tok * a.G * D;
+    t.q_rows = (long)a.num_new * a.G;
+    t.kv_rows = PAGED ? a.page_size : a.cache_cap;
+    t.k_dst = (T*)a.k_cache + (PAGED ? page_base + slot : pos) * D;
+    t.v_dst = (T*)a.v_cache + (PAGED ? page_base + slot : pos) * D;
+    rope_token<T>(a, t, s_angle);
+
+    if (PAGED && i == n_b - 1 && slot + 1 < a.page_size) {
         // the episode's last page is only partly filled: clear the value slots behind the last
         // token so that a tile load of the whole page never brings in stale bits
         const int tail = a.page_size - (slot + 1);
@@ -267,9 +285,54 @@ rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
             const int r = it % (tail * vec_per_row);
             const int s2 = slot + 1 + r / vec_per_row;
             const int d0 = (r % vec_per_row) * V;
-            *reinterpret_cast<uint4*>((T*)a.v_cache + page_base + ((long)g * a.page_size + s2) * D + d0) = zero;
+            *reinterpret_cast<uint4*>((T*)a.v_cache + (page_base + (long)g * a.page_size + s2) * D + d0) = zero;
         }
     }
+}
+
+// The tokens of a packed sequence I, v_1, a_1, ..., v_N, a_N in one launch (Sec. 3.3): the instruction and
+// visual tokens at contiguous positions into the cache, then the action tokens, chunk t at the positions
+// that continue v_t, into buffers of their own.
+struct RopePackedArgs {
+    RopeArgs r;              // visual run: q_rot, k_cache, v_cache, cache_cap; num_new = all tokens
+    int num_visual, num_action;
+    int I, F, A;
+    FastDiv div_f, div_a;
+    void* q_rot_act;         // [Hkv, num_action * G, D]
+    void* k_act;             // [Hkv, num_action, D]
+    void* v_act;
+};
+
+__global__ void __launch_bounds__(kRopeThreadsMax)
+rope_packed_kernel(const RopePackedArgs p)
+{
+    typedef __nv_bfloat16 T;
+    __shared__ typename Rotation<T>::Angle s_angle[72];
+    const RopeArgs& a = p.r;
+    const int tok = blockIdx.x;
+    const bool action = tok >= p.num_visual;
+    const int m = action ? tok - p.num_visual : tok;             // within its run
+    TokenPlace<T> t;
+    long pos;
+    if (action) {
+        const int c = (int)fast_div((uint32_t)m, p.div_a), i = m - c * p.A;
+        pos = (long)p.I + (long)(c + 1) * p.F + i;
+        t.src_tok = (long)p.I + (long)c * (p.F + p.A) + p.F + i;
+        t.kv_rows = p.num_action;
+    } else {
+        pos = m;
+        t.src_tok = m;
+        if (m >= p.I && p.F > 0) t.src_tok += (long)fast_div((uint32_t)(m - p.I), p.div_f) * p.A;
+        t.kv_rows = a.cache_cap;
+    }
+    t.q_dst = (T*)(action ? p.q_rot_act : a.q_rot) + (long)m * a.G * a.D;
+    t.q_rows = (long)(action ? p.num_action : p.num_visual) * a.G;
+    t.k_dst = (T*)(action ? p.k_act : a.k_cache) + (long)m * a.D;
+    t.v_dst = (T*)(action ? p.v_act : a.v_cache) + (long)m * a.D;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    load_angles<T>(s_angle, a.table, a.table_first, pos, a.D, a.log2_theta);
+    rope_token<T>(a, t, s_angle);
 }
 
 }  // namespace evln
