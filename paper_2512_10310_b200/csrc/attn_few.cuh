@@ -83,6 +83,7 @@ struct FewArgs {
 constexpr int kFewBarBytes = 256;
 constexpr int kFewStatBytes = 2 * kFewWarps * kFewRows * 4;
 constexpr int kFewRowBytes = kFewOStride * 4;           // a row in flight: 128 channels, reference, sum
+constexpr int kFewAngleBytes = Rotation<__nv_bfloat16>::kAngles * 16;
 constexpr int kFewMaxSmem = 227 * 1024;
 __host__ __device__ inline int few_cluster_bytes(int rows, int cluster)
 {
@@ -91,7 +92,7 @@ __host__ __device__ inline int few_cluster_bytes(int rows, int cluster)
 inline int few_smem_bytes(int stages, int rows, int cluster, bool fused, int num_new)
 {
     return 1024 + stages * kFewStageBytes + (rows + 15) / 16 * 16 * 256 + kFewBarBytes + kFewStatBytes + few_cluster_bytes(rows, cluster) +
-           (fused ? num_new * (1024 + 512) : 0);
+           (fused ? num_new * (kFewAngleBytes + 512) : 0);
 }
 static_assert(kFewMinStages * kFewStageBytes >= kFewWarps * 16 * kFewOStride * 4, "the outputs fit the stages");
 
@@ -138,8 +139,8 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
     float* s_l = s_m + kFewWarps * kFewRows;                               // ... and their sums
     float* s_in = s_l + kFewWarps * kFewRows;                              // [rows this block merges][cluster][kFewOStride]
     uint8_t* s_tail = smem_gen + stat_off + kFewStatBytes + (PAGED ? 0 : few_cluster_bytes(a.num_new * a.G, gridDim.x));
-    float4* s_cs = reinterpret_cast<float4*>(s_tail);                      // fused: [n][64]
-    uint8_t* s_new = s_tail + (FUSED ? a.num_new * 1024 : 0);              // fused: [n][K 256 B | V 256 B]
+    float4* s_cs = reinterpret_cast<float4*>(s_tail);                      // fused: [n][kAngles]
+    uint8_t* s_new = s_tail + (FUSED ? a.num_new * kFewAngleBytes : 0);              // fused: [n][K 256 B | V 256 B]
     const uint32_t bar_in = bar_full + 16 * kFewMaxStages + 8;             // the rows sent here have arrived
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -254,8 +255,8 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
         }
         for (int i = tid; i < n * 64; i += kFewThreads) {
             const int tok = i >> 6, j = i & 63;
-            s_cs[i] = Rotation<__nv_bfloat16>::angle(a.table ? a.table[((long)L + tok - a.table_first) * 64 + j]
-                                                             : rope_cos_sin((long)L + tok, j, 128, a.log2_theta));
+            Rotation<__nv_bfloat16>::put(s_cs + tok * Rotation<__nv_bfloat16>::kAngles, j,
+                                         a.table ? a.table[((long)L + tok - a.table_first) * 64 + j] : rope_cos_sin((long)L + tok, j, 128, a.log2_theta));
         }
         for (int i = rows * 16 + tid; i < MT * 16 * 16; i += kFewThreads) *q_slot(i >> 4, i & 15) = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
@@ -269,12 +270,9 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
             const int tok = is_q ? (int)fast_div((uint32_t)it, a.div_g) : is_v ? it - rows - n : it - rows;
             uint32_t x = lo, y = hi;
             if (!is_v) {
-                const float4* cs = s_cs + tok * 64 + 2 * lane;
-                float a0, a1, b0, b1;
-                Rotation<__nv_bfloat16>::turn(__uint_as_float(lo << 16), __uint_as_float(hi << 16), cs[0], a0, b0);
-                Rotation<__nv_bfloat16>::turn(__uint_as_float(lo & 0xffff0000u), __uint_as_float(hi & 0xffff0000u), cs[1], a1, b1);
-                x = ptx::pack_bf16x2(a0, a1);
-                y = ptx::pack_bf16x2(b0, b1);
+                typedef Rotation<__nv_bfloat16> R;
+                const float4* cs = s_cs + tok * R::kAngles + R::place(lane);
+                R::turn_pair(cs[0], cs[1], lo, hi, x, y);
             }
             if (is_q) {
                 reinterpret_cast<uint32_t*>(q_slot(it, lane >> 2))[lane & 3] = x;

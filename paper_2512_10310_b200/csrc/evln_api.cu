@@ -545,21 +545,18 @@ void finish_rope_args(RopeArgs* a, int vec)
     while ((1 << a->page_shift) < a->page_size) ++a->page_shift;
 }
 
-// Threads of the append kernels for `tokens` tokens.  Few enough to be one wave of two blocks per SM: one
-// thread per work item (in whole warps, at most kRopeThreadsMax).  Else 256 threads.
-int rope_threads(evlnHandle_t h, const RopeArgs& a, int tokens)
+// The append kernels: a block per token, one thread per work item of it.
+dim3 rope_block(const RopeArgs& a)
 {
-    if (tokens > 2 * h->num_sms) return kRopeThreads;
     const int items = ((a.Hq + a.Hkv) << a.vph_shift) + (a.Hkv << (a.vph_shift + 1));
-    int t = (items + 31) / 32 * 32;
-    if (t > kRopeThreadsMax) t = kRopeThreadsMax;
-    return t < 64 ? 64 : t;
+    const int t = (items + 31) / 32 * 32;
+    return dim3(t > kRopeThreadsMax ? kRopeThreadsMax : t < 64 ? 64 : t);
 }
 
 template <typename T, bool PAGED, typename LensT>
-void launch_rope_append(evlnHandle_t h, const RopeArgs& a, int tokens, cudaStream_t st, const LensT& lens)
+void launch_rope_append(const RopeArgs& a, int tokens, cudaStream_t st, const LensT& lens)
 {
-    launch_pdl(rope_append_kernel<T, PAGED, LensT>, dim3(tokens), dim3(rope_threads(h, a, tokens)), 0, st, a, lens);
+    launch_pdl(rope_append_kernel<T, PAGED, LensT>, dim3(tokens), rope_block(a), 0, st, a, lens);
 }
 
 // What the one-launch step adds to an attention call: the new tokens and where the results go (out null:
@@ -832,9 +829,9 @@ evlnStatus_t evlnRopeAppend(evlnHandle_t h, const evlnStepParams* p, const void*
     NoLens nl = {};
     cudaStream_t st = (cudaStream_t)stream;
     if (p->dtype == EVLN_BF16)
-        launch_rope_append<__nv_bfloat16, false, NoLens>(h, a, p->num_new, st, nl);
+        launch_rope_append<__nv_bfloat16, false, NoLens>(a, p->num_new, st, nl);
     else
-        launch_rope_append<float, false, NoLens>(h, a, p->num_new, st, nl);
+        launch_rope_append<float, false, NoLens>(a, p->num_new, st, nl);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
 }
@@ -1035,7 +1032,7 @@ evlnStatus_t evlnPagedRopeAppend(evlnHandle_t h, const evlnPagedParams* p, const
     finish_rope_args(&a, 8);
     BatchLens bl;
     fill_lens(&bl, p, h_cache_lens, h_new_offsets);
-    launch_rope_append<__nv_bfloat16, true, BatchLens>(h, a, total, (cudaStream_t)stream, bl);
+    launch_rope_append<__nv_bfloat16, true, BatchLens>(a, total, (cudaStream_t)stream, bl);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
 }
@@ -1283,7 +1280,7 @@ extern "C" evlnStatus_t evlnPackedForward(evlnHandle_t h, const evlnPackedParams
         a.div_f = make_fast_div((uint32_t)(p->frame_tokens > 0 ? p->frame_tokens : 1));
         a.div_a = make_fast_div((uint32_t)(p->action_tokens > 0 ? p->action_tokens : 1));
         a.q_rot_act = ws + pl.off_qa; a.k_act = ws + pl.off_tk; a.v_act = ws + pl.off_tv;
-        cudaError_t e = launch_pdl(rope_packed_kernel, dim3(a.r.num_new), dim3(rope_threads(h, a.r, a.r.num_new)), 0, st, a);
+        cudaError_t e = launch_pdl(rope_packed_kernel, dim3(a.r.num_new), rope_block(a.r), 0, st, a);
         if (e != cudaSuccess) return cuda_fail(h, e);
     }
     // one launch: the visual run as one causal prefill (its query tiles never load a KV tile past their own
@@ -1439,8 +1436,15 @@ extern "C" evlnStatus_t evlnGatherRope(evlnHandle_t h, const evlnGatherParams* p
     a.table = (const double2*)p->rope_table;
     a.table_first = p->rope_table_first_pos;
     cudaStream_t st = (cudaStream_t)stream;
-    if (p->dtype == EVLN_BF16) launch_pdl(gather_rope_kernel<__nv_bfloat16>, dim3((int)total), dim3(128), 0, st, a, segs);
-    else launch_pdl(gather_rope_kernel<float>, dim3((int)total), dim3(128), 0, st, a, segs);
+    const int vec = 16 / elem_bytes(p->dtype);
+    while ((1 << a.vph_shift) < a.D / 2 / vec) ++a.vph_shift;
+    a.k_chunks = ceil_div(a.Hkv << a.vph_shift, 32);
+    a.v_chunks = ceil_div(a.Hkv << (a.vph_shift + 1), 64);
+    a.div_chunks = make_fast_div((uint32_t)(a.k_chunks + a.v_chunks));
+    if (total * (a.k_chunks + a.v_chunks) > 0x7fffff00L) return EVLN_NOT_SUPPORTED;
+    const dim3 grid((unsigned)((total * (a.k_chunks + a.v_chunks) + kGatherWarps - 1) / kGatherWarps)), block(32 * kGatherWarps);
+    if (p->dtype == EVLN_BF16) launch_pdl(gather_rope_kernel<__nv_bfloat16>, grid, block, 0, st, a, segs);
+    else launch_pdl(gather_rope_kernel<float>, grid, block, 0, st, a, segs);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
 }

@@ -4,8 +4,7 @@
 //
 // store_append_kernel: the new frame's raw (un-rotated) K and V go to the store, head-major.
 // gather_rope_kernel: the kept segments of the store are laid out back to back in a working cache;
-// the token that lands in working slot p is rotated at position p (keys) or copied (values).  One
-// CTA per destination token; angles in double precision as in the append kernel (or from the
+// the token that lands in working slot p is rotated at position p (keys) or copied (values); angles in double precision as in the append kernel (or from the
 // caller's position table).  HBM-bound: every
 // kept element is read once and written once with 128-bit accesses.
 #pragma once
@@ -38,6 +37,9 @@ struct GatherArgs {
     double log2_theta;      // gather only
     const double2* table;   // gather only, optional: (cos, sin) per (position - table_first, j)
     int table_first;
+    // gather only, by the host: log2 of the 16-byte vectors per half head vector, chunks per token
+    int vph_shift, k_chunks, v_chunks;
+    FastDiv div_chunks;     // division by k_chunks + v_chunks
 };
 
 template <typename T>
@@ -60,62 +62,64 @@ store_append_kernel(const GatherArgs a)
     }
 }
 
+// A warp per chunk of a destination token: 32 vector pairs of its keys, or 64 vectors of its values.  Warps
+// do not wait for each other, so a call of a few thousand tokens is one wave of short chains (a block
+// per token, all of it behind the angles: 6.5 us for 3392 tokens of 4 kv heads; this: see launch_gather).
+constexpr int kGatherWarps = 8;
+
 template <typename T>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32 * kGatherWarps)
 gather_rope_kernel(const GatherArgs a, const __grid_constant__ SegList segs)
 {
     constexpr int V = VecTraits<T>::kVec;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __shared__ typename Rotation<T>::Angle s_angle[72];                // angle j at j + j / 8: the 8 vectors of a half head in different banks
-
-    const int pos = blockIdx.x;             // working slot = new position id
+    __shared__ typename Rotation<T>::Angle s_angles[kGatherWarps][Rotation<T>::kAngles];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t task = blockIdx.x * (uint32_t)kGatherWarps + (uint32_t)warp;
+    const int pos = (int)fast_div(task, a.div_chunks);     // working slot = new position id
+    const int chunk = (int)task - pos * (a.k_chunks + a.v_chunks);
     const int D = a.D, half = D / 2;
-    int lo = 0, hi = a.num_segments;        // largest s with dst_off[s] <= pos
+    int lo = 0, hi = a.num_segments;                       // largest s with dst_off[s] <= pos
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if (segs.dst_off[mid] <= pos) lo = mid; else hi = mid;
     }
-    const int src_slot = segs.src[lo] + (pos - segs.dst_off[lo]);
+    const long src_slot = segs.src[lo] + (pos - segs.dst_off[lo]);
+    // (so far launch parameters only)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (pos >= a.num_tokens) return;
 
-    if (threadIdx.x < half) {
-        const int j = threadIdx.x;
-        const double2 cs = a.table ? a.table[(long)(pos - a.table_first) * half + j] : rope_cos_sin(pos, j, D, a.log2_theta);
-        s_angle[j + (j >> 3)] = Rotation<T>::angle(cs);
-    }
-    __syncthreads();
-
-    const int vec_per_half = half / V;
-    const int k_items = a.Hkv * vec_per_half;
-    const int v_items = a.Hkv * (D / V);
-    for (int it = threadIdx.x; it < k_items + v_items; it += blockDim.x) {
-        if (it < k_items) {
-            const int g = it / vec_per_half;
-            const int j0 = (it % vec_per_half) * V;
-            const T* src = (const T*)a.k_src + ((long)g * a.src_cap + src_slot) * D;
-            T* dst = (T*)a.k_dst + ((long)g * a.dst_cap + pos) * D;
-            uint4 lo_raw = *reinterpret_cast<const uint4*>(src + j0);
-            uint4 hi_raw = *reinterpret_cast<const uint4*>(src + j0 + half);
-            const T* xl = reinterpret_cast<const T*>(&lo_raw);
-            const T* xh = reinterpret_cast<const T*>(&hi_raw);
-            uint4 out_lo_raw, out_hi_raw;
-            T* out_lo = reinterpret_cast<T*>(&out_lo_raw);
-            T* out_hi = reinterpret_cast<T*>(&out_hi_raw);
+    if (chunk < a.k_chunks) {
+        const int it = chunk * 32 + lane, k = it & ((1 << a.vph_shift) - 1), g = it >> a.vph_shift;
+        const bool mine = g < a.Hkv;
+        const T* src = (const T*)a.k_src + ((long)g * a.src_cap + src_slot) * D + k * V;
+        uint4 lo_raw = make_uint4(0u, 0u, 0u, 0u), hi_raw = lo_raw;
+        if (mine) {
+            lo_raw = *reinterpret_cast<const uint4*>(src);
+            hi_raw = *reinterpret_cast<const uint4*>(src + half);
+        }
+        for (int j = lane; j < half; j += 32)
+            Rotation<T>::put(s_angles[warp], j, a.table ? a.table[(long)(pos - a.table_first) * half + j] : rope_cos_sin(pos, j, D, a.log2_theta));
+        __syncwarp();
+        if (mine) {
+            uint4 out_lo, out_hi;
+            Rotation<T>::turn(s_angles[warp], k, lo_raw, hi_raw, out_lo, out_hi);
+            T* dst = (T*)a.k_dst + ((long)g * a.dst_cap + pos) * D + k * V;
+            *reinterpret_cast<uint4*>(dst) = out_lo;
+            *reinterpret_cast<uint4*>(dst + half) = out_hi;
+        }
+    } else {
+        uint4 x[2];
+        const int it = (chunk - a.k_chunks) * 64 + lane;
 #pragma unroll
-            for (int v = 0; v < V; ++v) {
-                float y0, y1;
-                Rotation<T>::turn(to_float(xl[v]), to_float(xh[v]), s_angle[j0 + (j0 >> 3) + v], y0, y1);
-                from_float(y0, out_lo[v]);
-                from_float(y1, out_hi[v]);
-            }
-            *reinterpret_cast<uint4*>(dst + j0) = out_lo_raw;
-            *reinterpret_cast<uint4*>(dst + j0 + half) = out_hi_raw;
-        } else {
-            const int e = it - k_items;
-            const int g = e / (D / V);
-            const int d0 = (e % (D / V)) * V;
-            *reinterpret_cast<uint4*>((T*)a.v_dst + ((long)g * a.dst_cap + pos) * D + d0) =
-                *reinterpret_cast<const uint4*>((const T*)a.v_src + ((long)g * a.src_cap + src_slot) * D + d0);
+        for (int i = 0; i < 2; ++i) {
+            const int d = (it + 32 * i) & ((2 << a.vph_shift) - 1), g = (it + 32 * i) >> (a.vph_shift + 1);
+            if (g < a.Hkv) x[i] = *reinterpret_cast<const uint4*>((const T*)a.v_src + ((long)g * a.src_cap + src_slot) * D + d * V);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int d = (it + 32 * i) & ((2 << a.vph_shift) - 1), g = (it + 32 * i) >> (a.vph_shift + 1);
+            if (g < a.Hkv) *reinterpret_cast<uint4*>((T*)a.v_dst + ((long)g * a.dst_cap + pos) * D + d * V) = x[i];
         }
     }
 }

@@ -1,23 +1,24 @@
 // Fused RoPE-rotate-and-append kernel (Sec. 3.2: contiguous position ids, rotation,
 // concatenation of the new frame with the reused cache).
 //
-// One CTA per new token.  Phase 1: D/2 threads get the token's cos/sin of phi_j = pos * theta^(-2j/D)
-// in double precision (pos reaches tens of thousands; a float angle would be off by ~1e-3 rad)
-// into shared memory for all heads: from the caller's position table when there is one (the
-// table depends on the positions only, so a model makes it once per navigation step for all its
-// layers: rope_table_kernel below), else formed on the spot.  Phase 2: every thread moves 16-byte
-// vectors (a work item is a pair of vectors (j.., j + D/2..) of a query or key head, or one vector
-// of a value head): rotated query halves to the kv-head-grouped q_rot scratch, rotated key halves
-// and the unchanged values to the token's cache slot; the loads of a thread's first item are issued
-// before the cos/sin are waited for.  HBM-bound by bytes (each element is read once and written
-// once with 128-bit accesses); at the sizes of a step it is one chain of latencies, which is why
-// nothing in it divides, and why a call of few tokens gets one thread per work item (all loads of
-// a token in flight at once).  (Letting every thread read the table entries of its own vector
-// instead of sharing them through shared memory was measured slower: 32 heads re-read the same 64
-// entries.)
+// One CTA per new token.  D/2 threads get the token's cos/sin of phi_j = pos * theta^(-2j/D) in double
+// precision (pos reaches tens of thousands; a float angle would be off by ~1e-3 rad) into shared memory
+// for all heads: from the caller's position table when there is one (the table depends on the positions
+// only, so a model makes it once per navigation step for all its layers: rope_table_kernel below), else
+// formed on the spot.  Every thread moves 16-byte vectors (a work item is a pair of vectors (j.., j + D/2..)
+// of a query or key head, or one vector of a value head): rotated query halves to the kv-head-grouped
+// q_rot scratch, rotated key halves and the unchanged values to the token's cache slot; the loads are
+// issued before the cos/sin are waited for.
+// Bound: a step's few hundred tokens are one chain of latencies (2.3 us for 196 tokens of the 7B shape,
+// 1.8 for one; 3.4 and 2.6 before the rotation was packed), thousands are bound by the instructions of
+// the rotation and then by HBM (each element read once and written once: 2048 tokens 9.8 us, 3136 paged
+// ones 17.6, 16 and 25 before; 6 and 9 us at the copy rate).
+// (Letting every thread read the table entries of its own vector instead of sharing them through shared
+// memory was measured slower: 32 heads re-read the same 64 entries.)
 #pragma once
 
 #include "common.cuh"
+#include "ptx_sm100.cuh"
 
 namespace evln {
 
@@ -47,65 +48,106 @@ struct RopeArgs {
 };
 
 // cos/sin of pos * theta^(-2j/D): the one definition the append, gather and table kernels share
-__device__ __forceinline__ double2 rope_cos_sin(long pos, int j, int D, double log2_theta)
+__device__ __forceinline__ double rope_omega(int j, int D, double log2_theta)
 {
-    const double omega = exp2(-(2.0 * (double)j / (double)D) * log2_theta);
+    return exp2(-(2.0 * (double)j / (double)D) * log2_theta);
+}
+__device__ __forceinline__ double2 rope_cos_sin_at(long pos, double omega)
+{
     double s, c;
     // sin/cos(pos * omega) through sincospi: its range reduction is exact and cheap, where a
     // plain sincos of an argument of thousands of radians takes the slow reduction path
     sincospi((double)pos * omega * 0.31830988618379067154, &s, &c);
     return make_double2(c, s);
 }
+__device__ __forceinline__ double2 rope_cos_sin(long pos, int j, int D, double log2_theta)
+{
+    return rope_cos_sin_at(pos, rope_omega(j, D, log2_theta));
+}
 
-// The rotation itself.  Products and sums are formed with at least 47 bits, then rounded once to float and
+// The rotation itself.  Products and sums are formed with at least 40 bits, then rounded once to float and
 // once to the storage dtype (a float product would lose bits exactly where x0*c and x1*s cancel).
 //  - float: in double.
-//  - bf16: in pairs of floats.  A double operation and the conversions around it issue at a small
-//    fraction of the float rate (measured: 32 double operations and 32 conversions per vector pair kept
-//    an SM at ~7 per cycle; the rotation was most of the append and gather kernels' time), and a bf16
-//    value times a cosine split into two floats is exact up to 2^-48: p + e is the exact product with
-//    the high part (fma), the low part joins the residual, the two products are subtracted with the
-//    rounding error recovered (Knuth's two-sum).
+//  - bf16: in pairs of floats, two channels per packed instruction.  A double operation and the
+//    conversions around it issue at a small fraction of the float rate (32 double operations and 32
+//    conversions per vector pair kept an SM at ~7 per cycle), and what bounds the append and gather
+//    kernels for thousands of tokens is the instructions they issue.  The angle is split into 16 bits and
+//    a float rest (40 bits), so a bf16 value times the first part is an exact float; the two exact products
+//    are added with the rounding error recovered (Knuth's two-sum), which the products with the rest join.
+// put(): angle j into a shared-memory array of kAngles; turn(): vector k (of a half head) of both halves.
 template <typename T> struct Rotation;
 template <> struct Rotation<float> {
-    typedef double2 Angle;                       // (cos, sin)
-    static __device__ __forceinline__ Angle angle(const double2& cs) { return cs; }
-    static __device__ __forceinline__ void turn(float x0, float x1, const Angle& a, float& y0, float& y1)
+    typedef double2 Angle;                       // (cos, sin); angle j at j + j / 8 (bank spread)
+    static constexpr int kAngles = 72;
+    static __device__ __forceinline__ void put(Angle* s, int j, const double2& cs) { s[j + (j >> 3)] = cs; }
+    static __device__ __forceinline__ void turn(const Angle* s, int k, const uint4& lo, const uint4& hi, uint4& out_lo, uint4& out_hi)
     {
-        y0 = (float)((double)x0 * a.x - (double)x1 * a.y);
-        y1 = (float)((double)x1 * a.x + (double)x0 * a.y);
+        const float* x0 = reinterpret_cast<const float*>(&lo);
+        const float* x1 = reinterpret_cast<const float*>(&hi);
+        float* y0 = reinterpret_cast<float*>(&out_lo);
+        float* y1 = reinterpret_cast<float*>(&out_hi);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int j = 4 * k + v;
+            const Angle a = s[j + (j >> 3)];
+            y0[v] = (float)((double)x0[v] * a.x - (double)x1[v] * a.y);
+            y1[v] = (float)((double)x1[v] * a.x + (double)x0[v] * a.y);
+        }
     }
 };
 template <> struct Rotation<__nv_bfloat16> {
-    typedef float4 Angle;                        // cos high, cos low, sin high, sin low
-    static __device__ __forceinline__ Angle angle(const double2& cs)
+    // a channel pair is two of these: (cos 16 bits of both, rest of both), (sin ..., ...); the pairs of a
+    // 16-byte vector take 9 places, so that the vectors of a half head start in different banks
+    typedef float4 Angle;
+    static constexpr int kAngles = 72;
+    static __device__ __forceinline__ int place(int pair) { return 2 * pair + (pair >> 2); }
+    static __device__ __forceinline__ void put(Angle* s, int j, const double2& cs)
     {
-        const float ch = (float)cs.x, sh = (float)cs.y;
-        return make_float4(ch, (float)(cs.x - (double)ch), sh, (float)(cs.y - (double)sh));
+        const float ch = __uint_as_float(__float_as_uint((float)cs.x) & 0xffffff00u);
+        const float sh = __uint_as_float(__float_as_uint((float)cs.y) & 0xffffff00u);
+        float* at = reinterpret_cast<float*>(s + place(j >> 1)) + (j & 1);
+        at[0] = ch;
+        at[2] = (float)(cs.x - (double)ch);
+        at[4] = sh;
+        at[6] = (float)(cs.y - (double)sh);
     }
-    // x * (hi + lo) as p + e
-    static __device__ __forceinline__ void product(float x, float hi, float lo, float& p, float& e)
+    // x * (ch + cl) + z * (sh + sl)
+    static __device__ __forceinline__ uint64_t combine(uint64_t x, uint64_t z, uint64_t ch, uint64_t cl, uint64_t sh, uint64_t sl)
     {
-        p = __fmul_rn(x, hi);
-        e = __fmaf_rn(x, lo, __fmaf_rn(x, hi, -p));
+        const uint64_t minus = ptx::pack2(-1.f, -1.f);
+        const uint64_t p = ptx::mul2(x, ch), q = ptx::mul2(z, sh);
+        const uint64_t d = ptx::add2(p, q);
+        const uint64_t nb = ptx::fma2(d, minus, p);                     // p - d: minus the part of q that d holds
+        const uint64_t err = ptx::add2(ptx::fma2(ptx::add2(d, nb), minus, p), ptx::add2(q, nb));
+        float r0, r1;
+        ptx::unpack2(ptx::fma2(z, sl, ptx::fma2(x, cl, err)), r0, r1);
+        // (an infinite or undefined d stays what it is: its rest is undefined, and min() drops that)
+        return ptx::add2(d, ptx::pack2(fminf(r0, 3.0e38f), fminf(r1, 3.0e38f)));
     }
-    static __device__ __forceinline__ float difference(float p, float e, float q, float f)
+    // a channel pair: words of the lower and the upper half
+    static __device__ __forceinline__ void turn_pair(const Angle& c, const Angle& s, uint32_t lo, uint32_t hi, uint32_t& out_lo,
+                                                     uint32_t& out_hi)
     {
-        const float d = __fsub_rn(p, q);
-        const float b = __fsub_rn(d, p);
-        const float err = __fsub_rn(__fsub_rn(p, __fsub_rn(d, b)), __fadd_rn(q, b));
-        const float y = __fadd_rn(d, __fadd_rn(err, __fsub_rn(e, f)));
-        return fabsf(d) < INFINITY ? y : d;      // (an infinite or undefined result stays what it is)
+        const uint32_t nhi = hi ^ 0x80008000u;
+        const uint64_t x0 = ptx::pack2(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u));
+        const uint64_t x1 = ptx::pack2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+        const uint64_t n1 = ptx::pack2(__uint_as_float(nhi << 16), __uint_as_float(nhi & 0xffff0000u));
+        const uint64_t ch = ptx::pack2(c.x, c.y), cl = ptx::pack2(c.z, c.w), sh = ptx::pack2(s.x, s.y), sl = ptx::pack2(s.z, s.w);
+        float a, b;
+        ptx::unpack2(combine(x0, n1, ch, cl, sh, sl), a, b);
+        out_lo = ptx::pack_bf16x2(a, b);
+        ptx::unpack2(combine(x1, x0, ch, cl, sh, sl), a, b);
+        out_hi = ptx::pack_bf16x2(a, b);
     }
-    static __device__ __forceinline__ void turn(float x0, float x1, const Angle& a, float& y0, float& y1)
+    static __device__ __forceinline__ void turn(const Angle* s, int k, const uint4& lo, const uint4& hi, uint4& out_lo, uint4& out_hi)
     {
-        float p, e, q, f;
-        product(x0, a.x, a.y, p, e);
-        product(x1, a.z, a.w, q, f);
-        y0 = difference(p, e, q, f);
-        product(x1, a.x, a.y, p, e);
-        product(x0, -a.z, -a.w, q, f);
-        y1 = difference(p, e, q, f);
+        const Angle* a = s + place(4 * k);
+        const uint32_t x0[4] = {lo.x, lo.y, lo.z, lo.w}, x1[4] = {hi.x, hi.y, hi.z, hi.w};
+        uint32_t y0[4], y1[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) turn_pair(a[2 * i], a[2 * i + 1], x0[i], x1[i], y0[i], y1[i]);
+        out_lo = make_uint4(y0[0], y0[1], y0[2], y0[3]);
+        out_hi = make_uint4(y1[0], y1[1], y1[2], y1[3]);
     }
 };
 
@@ -124,57 +166,63 @@ rope_table_kernel(double2* table, int first_pos, int count, int D, double log2_t
 
 // LensT is BatchLens for the paged kernel and NoLens (a stub) for the contiguous one.
 
-// Block size: calls of few tokens (one wave of blocks) get one thread per work item, in whole warps,
-// at most kRopeThreadsMax; batches of thousands of tokens are bound by throughput and take 256.
-constexpr int kRopeThreadsMax = 384;
-constexpr int kRopeThreads = 256;
+// A block per token with one thread per work item (in whole warps, at most kRopeThreadsMax): every load of
+// the token is in flight at once, and the other blocks of the SM hide its chain.  (Blocks that run through
+// several tokens and prefetch the next one's vectors were measured slower, 10.3 against 9.8 us for 2048
+// tokens and 19 against 17.6 for 3136 paged ones: what counts is warps, i.e. registers.)
+constexpr int kRopeThreadsMax = 448;
 
 // Where one new token comes from and goes to.
-template <typename T>
 struct TokenPlace {
-    long src_tok;            // its row of q_new / k_new / v_new
-    T* q_dst;                // its first query row of kv head 0, ...
-    long q_rows;             //   rows per kv head of that buffer
-    T* k_dst;                // its key / value row of kv head 0, ...
-    T* v_dst;
-    long kv_rows;            //   rows from one kv head to the next
+    int src_tok;             // its row of q_new / k_new / v_new
+    int m;                   // its number in its run: query rows m * G ..
+    int episode;             // paged: its episode; packed: 1 for an action token
+    long kv_row;             // its key / value row of kv head 0
+};
+// The buffers a token's run goes to.
+template <typename T>
+struct TokenRun {
+    T* q;                    // [Hkv, q_rows, D]
+    T* k;                    // rows of kv head g start kv_rows * g behind those of head 0
+    T* v;
+    long q_rows, kv_rows;
 };
 
-// Rotates and stores one token with the whole block; the angles are in s_angle once the block has met.
-template <typename T>
-__device__ __forceinline__ void rope_token(const RopeArgs& a, const TokenPlace<T>& t, const typename Rotation<T>::Angle* s_angle)
+// Rotates and stores token blockIdx.x with the whole block.  place(token, t) fills in the token's place and
+// returns its position, run(t) says which buffers it goes to, done(token, t) follows its stores.
+template <typename T, typename Place, typename Run, typename Done>
+__device__ __forceinline__ void rope_token(const RopeArgs& a, Place&& place, Run&& run, Done&& done)
 {
     constexpr int V = VecTraits<T>::kVec;
+    typedef typename Rotation<T>::Angle Angle;
+    __shared__ Angle s_angle[Rotation<T>::kAngles];
     const int D = a.D, half = D / 2, G = a.G;
-    const T* q_tok = (const T*)a.q_new + t.src_tok * a.q_stride;
-    const T* k_tok = (const T*)a.k_new + t.src_tok * a.k_stride;
-    const T* v_tok = (const T*)a.v_new + t.src_tok * a.v_stride;
-
     const int vph = a.vph_shift, vpr = a.vph_shift + 1;       // vectors per half head vector / per head vector (log2)
     const int q_items = a.Hq << vph;
     const int k_items = a.Hkv << vph;
     const int v_items = a.Hkv << vpr;
     const int items = q_items + k_items + v_items;
 
-    // a thread's work item `it`: a pair of 16-byte vectors (j0.., j0+half..) of a query or key head,
-    // or one 16-byte vector of a value head
-    auto load_item = [&](int it, uint4& r0, uint4& r1) {
+    // a work item `it` of a token: a pair of 16-byte vectors (j0.., j0+half..) of a query or key head, or one
+    // 16-byte vector of a value head
+    auto load_item = [&](const TokenPlace& t, int it, uint4& r0, uint4& r1) {
         if (it < q_items + k_items) {
             const bool is_q = it < q_items;
             const int e = is_q ? it : it - q_items;
             const int h = e >> vph;
             const int j0 = (e & ((1 << vph) - 1)) * V;
-            const T* src = (is_q ? q_tok : k_tok) + (long)h * D;
+            const T* src = (is_q ? (const T*)a.q_new + t.src_tok * a.q_stride : (const T*)a.k_new + t.src_tok * a.k_stride) + (long)h * D;
             r0 = *reinterpret_cast<const uint4*>(src + j0);
             r1 = *reinterpret_cast<const uint4*>(src + j0 + half);
         } else {
             const int e = it - q_items - k_items;
             const int g = e >> vpr;
             const int d0 = (e & ((1 << vpr) - 1)) * V;
-            r0 = *reinterpret_cast<const uint4*>(v_tok + (long)g * D + d0);
+            r0 = *reinterpret_cast<const uint4*>((const T*)a.v_new + t.src_tok * a.v_stride + (long)g * D + d0);
         }
     };
-    auto finish_item = [&](int it, const uint4& lo_raw, const uint4& hi_raw) {
+    auto finish_item = [&](const TokenPlace& t, const Angle* s_angle, int it, const uint4& lo_raw, const uint4& hi_raw) {
+        const TokenRun<T> to = run(t);
         if (it < q_items + k_items) {
             const bool is_q = it < q_items;
             const int e = is_q ? it : it - q_items;
@@ -183,97 +231,77 @@ __device__ __forceinline__ void rope_token(const RopeArgs& a, const TokenPlace<T
             T* dst;
             if (is_q) {
                 const int g = (int)fast_div((uint32_t)h, a.div_g);
-                dst = t.q_dst + ((long)g * t.q_rows + (h - g * G)) * D;
+                dst = to.q + ((long)g * to.q_rows + (long)t.m * G + (h - g * G)) * D;
             } else {
-                dst = t.k_dst + (long)h * t.kv_rows * D;
+                dst = to.k + ((long)h * to.kv_rows + t.kv_row) * D;
             }
-            const T* lo = reinterpret_cast<const T*>(&lo_raw);
-            const T* hi = reinterpret_cast<const T*>(&hi_raw);
             uint4 out_lo_raw, out_hi_raw;
-            T* out_lo = reinterpret_cast<T*>(&out_lo_raw);
-            T* out_hi = reinterpret_cast<T*>(&out_hi_raw);
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                float y0, y1;
-                Rotation<T>::turn(to_float(lo[v]), to_float(hi[v]), s_angle[j0 + (j0 >> 3) + v], y0, y1);
-                from_float(y0, out_lo[v]);
-                from_float(y1, out_hi[v]);
-            }
+            Rotation<T>::turn(s_angle, e & ((1 << vph) - 1), lo_raw, hi_raw, out_lo_raw, out_hi_raw);
             *reinterpret_cast<uint4*>(dst + j0) = out_lo_raw;
             *reinterpret_cast<uint4*>(dst + j0 + half) = out_hi_raw;
         } else {
             const int e = it - q_items - k_items;
             const int g = e >> vpr;
             const int d0 = (e & ((1 << vpr) - 1)) * V;
-            *reinterpret_cast<uint4*>(t.v_dst + (long)g * t.kv_rows * D + d0) = lo_raw;
+            *reinterpret_cast<uint4*>(to.v + ((long)g * to.kv_rows + t.kv_row) * D + d0) = lo_raw;
         }
     };
 
-    uint4 r0 = make_uint4(0u, 0u, 0u, 0u), r1 = r0;
-    if ((int)threadIdx.x < items) load_item(threadIdx.x, r0, r1);     // in flight while the angles arrive
-    __syncthreads();
-    if ((int)threadIdx.x < items) finish_item(threadIdx.x, r0, r1);
-    for (int it = threadIdx.x + blockDim.x; it < items; it += blockDim.x) {
-        load_item(it, r0, r1);
-        finish_item(it, r0, r1);
-    }
-}
-
-// The angles of position `pos` into shared memory (angle j at j + j / 8: the 8 vectors of a half head in
-// different banks).
-template <typename T>
-__device__ __forceinline__ void load_angles(typename Rotation<T>::Angle* s_angle, const double2* table, long table_first, long pos,
-                                            int D, double log2_theta)
-{
     const int j = threadIdx.x;
-    if (j < D / 2)
-        s_angle[j + (j >> 3)] = Rotation<T>::angle(table ? table[(pos - table_first) * (D / 2) + j] : rope_cos_sin(pos, j, D, log2_theta));
+    // without a table: the thread's frequency, once (j / D as in rope_cos_sin)
+    const double omega = !a.table && j < half ? rope_omega(j, D, a.log2_theta) : 0.0;
+    auto angle_of = [&](long pos) -> double2 {
+        return a.table ? a.table[(pos - a.table_first) * half + j] : rope_cos_sin_at(pos, omega);
+    };
+
+    const int tok = blockIdx.x;
+    TokenPlace t;
+    const long pos = place(tok, t);
+    uint4 r0 = make_uint4(0u, 0u, 0u, 0u), r1 = r0;
+    if (j < items) load_item(t, j, r0, r1);           // in flight while the angles arrive
+    if (j < half) Rotation<T>::put(s_angle, j, angle_of(pos));
+    __syncthreads();
+    if (j < items) finish_item(t, s_angle, j, r0, r1);
+    for (int it = j + blockDim.x; it < items; it += blockDim.x) {
+        load_item(t, it, r0, r1);
+        finish_item(t, s_angle, it, r0, r1);
+    }
+    done(tok, t);
 }
 
 template <typename T, bool PAGED, typename LensT>
-__global__ void __launch_bounds__(kRopeThreadsMax)
+__global__ void __launch_bounds__(kRopeThreadsMax, PAGED ? 3 : 1)
 rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
 {
     constexpr int V = VecTraits<T>::kVec;
-    __shared__ typename Rotation<T>::Angle s_angle[72];
-
-    const int tok = blockIdx.x;           // index into the packed new tokens
     const int D = a.D;
-
-    int b = 0, i = tok, L = a.cache_len, n_b = a.num_new;
+    int b = 0;                                    // the token's episode
     if (PAGED) {
-        int lo = 0, hi = a.batch;         // largest b with new_off[b] <= tok
-        while (hi - lo > 1) {
-            int mid = (lo + hi) >> 1;
-            if (lens.new_off[mid] <= tok) lo = mid; else hi = mid;
+        int hi = a.batch;                         // largest b with new_off[b] <= tok
+        while (hi - b > 1) {
+            const int mid = (b + hi) >> 1;
+            if (lens.new_off[mid] <= (int)blockIdx.x) b = mid; else hi = mid;
         }
-        b = lo;
-        i = tok - lens.new_off[b];
-        L = lens.cache_len[b];
-        n_b = lens.new_off[b + 1] - lens.new_off[b];
     }
-    const long pos = (long)L + i;
     // (so far launch parameters only; what follows reads memory that earlier kernels may have written)
     asm volatile("griddepcontrol.wait;" ::: "memory");          // programmatic dependent launch: inputs ready
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    load_angles<T>(s_angle, a.table, a.table_first, pos, D, a.log2_theta);
-
-    long page_base = 0;     // paged: first row of the page in the pool; slot within the page
-    int slot = 0;
-    if (PAGED) {
-        page_base = (long)a.page_table[(long)b * a.max_pages + (int)(pos >> a.page_shift)] * a.Hkv * a.page_size;
-        slot = (int)(pos & (a.page_size - 1));
-    }
-    TokenPlace<T> t;
-    t.src_tok = tok;
-    t.q_dst = (T*)a.q_rot + (long)tok * a.G * D;
-    t.q_rows = (long)a.num_new * a.G;
-    t.kv_rows = PAGED ? a.page_size : a.cache_cap;
-    t.k_dst = (T*)a.k_cache + (PAGED ? page_base + slot : pos) * D;
-    t.v_dst = (T*)a.v_cache + (PAGED ? page_base + slot : pos) * D;
-    rope_token<T>(a, t, s_angle);
-
-    if (PAGED && i == n_b - 1 && slot + 1 < a.page_size) {
+    auto place = [&](int tok, TokenPlace& t) -> long {          // tok: index into the packed new tokens
+        t.src_tok = t.m = tok;
+        if (!PAGED) return t.kv_row = (long)a.cache_len + tok;
+        const int pos = lens.cache_len[b] + tok - lens.new_off[b];
+        t.episode = b;
+        t.kv_row = (long)a.page_table[(long)b * a.max_pages + (pos >> a.page_shift)] * a.Hkv * a.page_size + (pos & (a.page_size - 1));
+        return pos;
+    };
+    auto run = [&](const TokenPlace&) -> TokenRun<T> {
+        return {(T*)a.q_rot, (T*)a.k_cache, (T*)a.v_cache, (long)a.num_new * a.G, PAGED ? (long)a.page_size : (long)a.cache_cap};
+    };
+    rope_token<T>(a, place, run, [&](int tok, const TokenPlace& t) {
+        if (!PAGED) return;
+        if (tok + 1 != lens.new_off[t.episode + 1]) return;
+        const int slot = (lens.cache_len[t.episode] + tok - lens.new_off[t.episode]) & (a.page_size - 1);
+        if (slot + 1 >= a.page_size) return;
         // the episode's last page is only partly filled: clear the value slots behind the last
         // token so that a tile load of the whole page never brings in stale bits
         const int tail = a.page_size - (slot + 1);
@@ -283,11 +311,9 @@ rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
         for (int it = threadIdx.x; it < total; it += blockDim.x) {
             const int g = it / (tail * vec_per_row);
             const int r = it % (tail * vec_per_row);
-            const int s2 = slot + 1 + r / vec_per_row;
-            const int d0 = (r % vec_per_row) * V;
-            *reinterpret_cast<uint4*>((T*)a.v_cache + (page_base + (long)g * a.page_size + s2) * D + d0) = zero;
+            *reinterpret_cast<uint4*>((T*)a.v_cache + (t.kv_row + (long)g * a.page_size + 1 + r / vec_per_row) * D + (r % vec_per_row) * V) = zero;
         }
-    }
+    });
 }
 
 // The tokens of a packed sequence I, v_1, a_1, ..., v_N, a_N in one launch (Sec. 3.3): the instruction and
@@ -303,36 +329,35 @@ struct RopePackedArgs {
     void* v_act;
 };
 
-__global__ void __launch_bounds__(kRopeThreadsMax)
+__global__ void __launch_bounds__(kRopeThreadsMax, 3)
 rope_packed_kernel(const RopePackedArgs p)
 {
     typedef __nv_bfloat16 T;
-    __shared__ typename Rotation<T>::Angle s_angle[72];
     const RopeArgs& a = p.r;
-    const int tok = blockIdx.x;
-    const bool action = tok >= p.num_visual;
-    const int m = action ? tok - p.num_visual : tok;             // within its run
-    TokenPlace<T> t;
-    long pos;
-    if (action) {
-        const int c = (int)fast_div((uint32_t)m, p.div_a), i = m - c * p.A;
-        pos = (long)p.I + (long)(c + 1) * p.F + i;
-        t.src_tok = (long)p.I + (long)c * (p.F + p.A) + p.F + i;
-        t.kv_rows = p.num_action;
-    } else {
-        pos = m;
-        t.src_tok = m;
-        if (m >= p.I && p.F > 0) t.src_tok += (long)fast_div((uint32_t)(m - p.I), p.div_f) * p.A;
-        t.kv_rows = a.cache_cap;
-    }
-    t.q_dst = (T*)(action ? p.q_rot_act : a.q_rot) + (long)m * a.G * a.D;
-    t.q_rows = (long)(action ? p.num_action : p.num_visual) * a.G;
-    t.k_dst = (T*)(action ? p.k_act : a.k_cache) + (long)m * a.D;
-    t.v_dst = (T*)(action ? p.v_act : a.v_cache) + (long)m * a.D;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    load_angles<T>(s_angle, a.table, a.table_first, pos, a.D, a.log2_theta);
-    rope_token<T>(a, t, s_angle);
+    auto place = [&](int tok, TokenPlace& t) -> long {
+        const bool action = tok >= p.num_visual;
+        const int m = action ? tok - p.num_visual : tok;             // within its run
+        long pos = m;
+        t.src_tok = m;
+        if (action) {
+            const int c = (int)fast_div((uint32_t)m, p.div_a), i = m - c * p.A;
+            pos = (long)p.I + (long)(c + 1) * p.F + i;
+            t.src_tok = p.I + c * (p.F + p.A) + p.F + i;
+        } else if (m >= p.I && p.F > 0) {
+            t.src_tok += (int)fast_div((uint32_t)(m - p.I), p.div_f) * p.A;
+        }
+        t.m = m;
+        t.kv_row = m;
+        t.episode = action;
+        return pos;
+    };
+    auto run = [&](const TokenPlace& t) -> TokenRun<T> {
+        if (t.episode) return {(T*)p.q_rot_act, (T*)p.k_act, (T*)p.v_act, (long)p.num_action * a.G, p.num_action};
+        return {(T*)a.q_rot, (T*)a.k_cache, (T*)a.v_cache, (long)p.num_visual * a.G, a.cache_cap};
+    };
+    rope_token<T>(a, place, run, [](int, const TokenPlace&) {});
 }
 
 }  // namespace evln
