@@ -118,10 +118,11 @@ struct TcAttnArgs {
 // larger structure the pair kernel came out with 150 bytes of spills in its tile loop).
 struct TcOutArgs {
     // Final output [n, Hq, 128] (+ log-sum-exps [n, Hq] or null) of rows whose keys are not split: their
-    // work item writes it itself.  Null: everything goes to o_part / lse_part.
+    // work item writes it itself (to the workspace when the caller's buffer comes with the combine call).
+    // Null: everything goes to o_part / lse_part.
     __nv_bfloat16* out;
     float* lse_out;
-    PackedMap map;            // where output token m goes (identity unless the call serves a packed sequence)
+    PackedMap map;            // packed sequence only: where output token m goes
     // packed sequence only: the action items come first (largest prefix first), then the units of the
     // visual run (largest first), kv heads side by side
     int act_items;            // work items of the action chunks
@@ -331,15 +332,16 @@ __device__ __forceinline__ WorkItem decode_work(const TcAttnArgs& a, const LensT
             const int mid = (lo + hi) >> 1;
             if (lens.item_off[mid] <= item) lo = mid; else hi = mid;
         }
-        const int b = lo;
+        int b = lo;
+        if constexpr (PAGED) b = lens.order[lo];
         w.b = b;
         w.L = lens.cache_len[b];
         w.n = lens.new_off[b + 1] - lens.new_off[b];
         w.row_base = lens.new_off[b] * a.G;
         w.g = w.unit = w.slot = 0;
         w.j0 = w.j1 = 0;
-        const int per_head = (lens.item_off[b + 1] - lens.item_off[b]) / a.Hkv;
-        int rem = item - lens.item_off[b];
+        const int per_head = (lens.item_off[lo + 1] - lens.item_off[lo]) / a.Hkv;
+        int rem = item - lens.item_off[lo];
         if (item >= lens.item_off[a.batch] || per_head <= 0) { w.b = -1; return w; }
         w.g = rem / per_head;
         rem -= w.g * per_head;
@@ -1014,7 +1016,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
             uint8_t* stage = smem_gen + kSmemKOff + (warp - 4) * (32 * 144);
             const int first_row = row0 + wrow0;                              // episode-local
             const int rows_here = rows_valid - first_row;                    // may be <= 0 or > 32
-            const bool direct = !PAGED && CTAS == 2 && d.out != nullptr && !(TAIL && !w.visual && d.act_split);
+            const bool direct = CTAS == 2 && d.out != nullptr && !(TAIL && !w.visual && d.act_split);
             uint32_t regs[32];
             ptx::tmem_ld32(t_o, regs);
             ptx::tmem_ld_wait();
@@ -1023,7 +1025,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
                 auto out_row = [&](int rl) -> long {           // row of [n, Hq, 128] of the item's row rl
                     const int tok = (int)fast_div((uint32_t)rl, a.div_g);
                     const long t = TAIL ? packed_row(w.visual ? d.map : d.act_map, (w.visual ? 0 : (long)lens.new_off[w.b]) + tok)
-                                        : packed_row(d.map, tok);
+                                        : PAGED ? (long)lens.new_off[w.b] + tok : (long)tok;
                     return t * (a.Hkv * a.G) + w.g * a.G + (rl - tok * a.G);
                 };
                 uint4* srow = reinterpret_cast<uint4*>(stage + lane * 80);

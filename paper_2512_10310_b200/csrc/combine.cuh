@@ -145,4 +145,35 @@ combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
     if (a.lse_out && lane == 0) a.lse_out[tok * Hq + h] = (wsum > 0.f) ? M + logf(wsum) : -INFINITY;
 }
 
+// Rows whose keys were not split are final (rounded, in output order) in the workspace: n * Hq rows of
+// 16-byte vectors and their log-sum-exps go to the caller's buffers.  HBM/L2-bound: a third of the bytes
+// that one set of fp32 partials would move.
+struct CopyOutArgs {
+    const uint4* src;
+    uint4* dst;
+    const float* lse_src;
+    float* lse_dst;          // or null
+    long vectors, rows;
+};
+constexpr int kCopyVectors = 4;      // per thread, all in flight
+
+__global__ void __launch_bounds__(256)
+copy_out_kernel(const CopyOutArgs a)
+{
+    const long i0 = (long)blockIdx.x * (256 * kCopyVectors) + threadIdx.x;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    uint4 v[kCopyVectors];
+#pragma unroll
+    for (int k = 0; k < kCopyVectors; ++k)
+        if (i0 + 256 * k < a.vectors) v[k] = a.src[i0 + 256 * k];
+#pragma unroll
+    for (int k = 0; k < kCopyVectors; ++k)
+        if (i0 + 256 * k < a.vectors) a.dst[i0 + 256 * k] = v[k];
+    if (a.lse_dst) {                 // 16 vectors per row
+        const long r = (long)blockIdx.x * (256 * kCopyVectors / 16) + threadIdx.x;
+        if (threadIdx.x < 256 * kCopyVectors / 16 && r < a.rows) a.lse_dst[r] = a.lse_src[r];
+    }
+}
+
 }  // namespace evln

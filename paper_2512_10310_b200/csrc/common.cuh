@@ -34,6 +34,12 @@ struct BatchLens {
     int item_off[kMaxBatch + 1];   // first work item of the attention kernel per episode
 };
 
+// The same for the pair kernel: work items are numbered over the episodes in the order `order` (item_off
+// is indexed by place in that order): longest first, so that the last round of items is a short one.
+struct PagedLens : BatchLens {
+    unsigned char order[kMaxBatch];
+};
+
 template <typename T> struct VecTraits;
 template <> struct VecTraits<__nv_bfloat16> { static constexpr int kVec = 8; };
 template <> struct VecTraits<float> { static constexpr int kVec = 4; };

@@ -8,6 +8,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <new>
 #include <utility>
@@ -113,7 +114,7 @@ cudaError_t prepare_few()
 cudaError_t prepare_kernels()
 {
     const std::pair<const void*, int> tc[4] = {{(const void*)attn_pair_kernel<false, NoLens>, kTcSmemBytes},
-                                               {(const void*)attn_pair_kernel<true, BatchLens>, kTcSmemBytes},
+                                               {(const void*)attn_pair_kernel<true, PagedLens>, kTcSmemBytes},
                                                {(const void*)attn_solo_kernel, kSoloSmemBytes},
                                                {(const void*)attn_packed_kernel, kTcSmemBytes}};
     for (const auto& k : tc) {
@@ -139,7 +140,7 @@ cudaError_t prepare_kernels()
 bool attention_register_pool_ok()
 {
     cudaFuncAttributes fa;
-    const void* kernels[4] = {(const void*)attn_pair_kernel<false, NoLens>, (const void*)attn_pair_kernel<true, BatchLens>,
+    const void* kernels[4] = {(const void*)attn_pair_kernel<false, NoLens>, (const void*)attn_pair_kernel<true, PagedLens>,
                               (const void*)attn_solo_kernel, (const void*)attn_packed_kernel};
     for (const void* k : kernels) {
         if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return false;
@@ -230,6 +231,7 @@ inline bool use_few_kernel(const evlnStepParams* p)
 {
     return use_tensor_kernel(p) && (long)p->num_new * (p->num_q_heads / p->num_kv_heads) <= kFewRows;
 }
+inline bool use_pair_kernel(const evlnStepParams* p) { return use_tensor_kernel(p) && !use_solo_kernel(p); }
 inline int few_row_tiles(int rows) { return rows <= 16 ? 1 : 2; }
 
 struct FewPlan {
@@ -432,9 +434,74 @@ inline int batch_kv_tiles(bool tail, int L, int n, int G, int u)
     return tail ? tail_kv_tiles(L, n, G, u, kUnitRows) : unit_kv_tiles(L, n, G, u, kUnitRows);
 }
 
+// Episodes by length, longest first (equal lengths in the caller's order).
+void longest_first(int batch, const int* lens, const int* offs, int* order)
+{
+    for (int b = 0; b < batch; ++b) order[b] = b;
+    std::stable_sort(order, order + batch, [&](int x, int y) {
+        return lens[x] + offs[x + 1] - offs[x] > lens[y] + offs[y + 1] - offs[y];
+    });
+}
+
+// When the last of `pairs` CTA pairs is done (in KV tiles) if each takes the next work item as it becomes free,
+// episodes in the order given, items of at most `chunk` tiles.  The pairs are kept as runs of equal load, so
+// an episode costs a few steps however many items it has.
+double finish_time(int pairs, int G, int Hkv, int batch, const int* lens, const int* offs, const int* order, int chunk)
+{
+    struct Run { double load; int count; };
+    std::vector<Run> runs(1, Run{0.0, pairs});        // ascending loads
+    double last = 0.0;
+    for (int i = 0; i < batch; ++i) {
+        const int b = order[i], n = offs[b + 1] - offs[b];
+        if (n == 0) continue;
+        const int units = ceil_div(n * G, kUnitRows);
+        const int nkv = unit_kv_tiles(lens[b], n, G, units - 1, kUnitRows), splits = ceil_div(nkv, chunk);
+        // set-up, first-tile latency, write-out and teardown of an item cost about as much as 7 KV tiles
+        const double cost = (double)nkv / splits + 7.0;
+        for (long left = (long)units * Hkv * splits; left > 0;) {
+            const int take = left < runs[0].count ? (int)left : runs[0].count;
+            const double load = runs[0].load + cost;
+            runs[0].count -= take;
+            if (runs[0].count == 0) runs.erase(runs.begin());
+            size_t at = 0;
+            while (at < runs.size() && runs[at].load < load) ++at;
+            if (at < runs.size() && runs[at].load == load) runs[at].count += take;
+            else runs.insert(runs.begin() + at, Run{load, take});
+            if (load > last) last = load;
+            left -= take;
+        }
+    }
+    return last;
+}
+
+// Work-item size of a batch on CTA pairs.  Not splitting saves the partials (an fp32 row set per split written
+// and read again against one rounded row set) and the items' fixed costs; splitting evens out the pairs.  Many
+// items even out by themselves (longest first); else the estimate above decides between a few sizes.  16
+// ragged episodes of one frame (384 unsplit items): see the paged batch in the measured table.
+int choose_chunk(int pairs, int G, int Hkv, int batch, const int* lens, const int* offs, const int* order, long total, int nkv_max)
+{
+    long unsplit = 0;
+    for (int b = 0; b < batch; ++b) unsplit += (long)ceil_div((offs[b + 1] - offs[b]) * G, kUnitRows) * Hkv;
+    if (unsplit >= 8L * pairs) return nkv_max;
+    const double rows = (double)offs[batch] * G * Hkv;
+    int best = nkv_max;
+    double best_cost = 1e30;
+    for (int k = 0; k <= 4; ++k) {
+        int chunk = k == 0 ? nkv_max : (int)((total + (long)pairs * k - 1) / ((long)pairs * k));
+        if (chunk < 4) chunk = 4;
+        if (chunk < ceil_div(nkv_max, kMaxSplits)) chunk = ceil_div(nkv_max, kMaxSplits);
+        if (chunk > nkv_max) chunk = nkv_max;
+        const double splits = chunk == nkv_max ? 0.5 : ceil_div(nkv_max, chunk);      // (row sets moved, in fp32 units)
+        // a KV tile takes a pair about 0.55 us; partials move at about 5.5 TB/s, each row written and read
+        const double cost = finish_time(pairs, G, Hkv, batch, lens, offs, order, chunk) + rows * splits * 1024.0 / 5.5e6 / 0.55;
+        if (cost < best_cost - 1e-9) { best_cost = cost; best = chunk; }
+    }
+    return best;
+}
+
 // Work-item size (KV tiles) and the largest split count of a batch.
-void batch_schedule(int num_sms, int G, int Hkv, int batch, const int* lens, const int* offs, bool tail, bool few,
-                    int kv_chunk_tiles, int* chunk_tiles, int* max_splits, long* items)
+void batch_schedule(int num_sms, int G, int Hkv, int batch, const int* lens, const int* offs, const int* order, bool tail,
+                    bool few, int kv_chunk_tiles, int* chunk_tiles, int* max_splits, long* items)
 {
     long total = 0;
     int nkv_max = 1;
@@ -455,9 +522,7 @@ void batch_schedule(int num_sms, int G, int Hkv, int batch, const int* lens, con
         chunk = (int)((total + (long)num_sms * 4 - 1) / ((long)num_sms * 4));
         if (chunk < 2) chunk = 2;
     } else if (chunk <= 0) {
-        const long pairs = num_sms / 2 > 0 ? num_sms / 2 : 1;
-        chunk = (int)((total + pairs * 4 - 1) / (pairs * 4));
-        if (chunk < 8) chunk = 8;
+        chunk = choose_chunk(num_sms / 2 > 0 ? num_sms / 2 : 1, G, Hkv, batch, lens, offs, order, total, nkv_max);
     }
     if (chunk < ceil_div(nkv_max, kMaxSplits)) chunk = ceil_div(nkv_max, kMaxSplits);
     long cnt = 0;
@@ -483,8 +548,10 @@ bool paged_few(const evlnPagedParams* p, const int* offs)
 void paged_schedule(evlnHandle_t h, const evlnPagedParams* p, const int* lens, const int* offs,
                     int* chunk_tiles, int* max_splits, long* items)
 {
-    batch_schedule(h->num_sms, p->num_q_heads / p->num_kv_heads, p->num_kv_heads, p->batch, lens, offs, false,
-                   paged_few(p, offs), p->kv_chunk_tiles, chunk_tiles, max_splits, items);
+    int order[kMaxBatch];
+    const bool few = paged_few(p, offs);
+    if (!few) longest_first(p->batch, lens, offs, order);
+    batch_schedule(h->num_sms, p->num_q_heads / p->num_kv_heads, p->num_kv_heads, p->batch, lens, offs, order, false, few, p->kv_chunk_tiles, chunk_tiles, max_splits, items);
 }
 
 // chunk_tiles > 0: also the first attention work item of every episode (items are numbered
@@ -531,6 +598,19 @@ evlnStatus_t launch_combine(evlnHandle_t h, const CombineArgs& args, int D, bool
         else launch_pdl(combine_kernel<T, 64, false, NoLens>, dim3(grid), dim3(128), 0, st, a, nl);
     }
     cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
+}
+
+// The combine step of rows that the attention kernel left final in the workspace (see CopyOutArgs).
+evlnStatus_t launch_copy_out(evlnHandle_t h, const CombineArgs& c, cudaStream_t st)
+{
+    CopyOutArgs a;
+    a.rows = (long)c.rows * c.Hkv;
+    a.vectors = a.rows * 16;
+    a.src = (const uint4*)c.o_part; a.dst = (uint4*)c.out;
+    a.lse_src = c.lse_part; a.lse_dst = c.lse_out;
+    const long blocks = (a.vectors + 256 * kCopyVectors - 1) / (256 * kCopyVectors);
+    cudaError_t e = launch_pdl(copy_out_kernel, dim3((unsigned)blocks), dim3(256), 0, st, a);
     return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
 }
 
@@ -901,10 +981,10 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
             launch_pdl(attn_solo_kernel, dim3(p->num_kv_heads, 1, S), dim3(kTcThreads), kSoloSmemBytes, st, tm_q, tm_k, tm_v, a);
         } else {
             TcOutArgs d = {};
-            if (direct && S == 1) {
-                d.out = (__nv_bfloat16*)direct->out;
-                d.lse_out = direct->lse_out;
-                direct->done = true;
+            if (S == 1) {                          // final rows: to the caller, or for the combine call to copy
+                d.out = direct ? (__nv_bfloat16*)direct->out : (__nv_bfloat16*)workspace;
+                d.lse_out = direct ? direct->lse_out : lse_part;
+                if (direct) direct->done = true;
             }
             launch_pair_pdl(attn_pair_kernel<false, NoLens>, dim3(2 * p->num_kv_heads, a.units_per_head, S), kTcSmemBytes, st,
                             tm_q, tm_k, tm_v, a, nl, d);
@@ -954,6 +1034,7 @@ evlnStatus_t evlnStepCombine(evlnHandle_t h, const evlnStepParams* p, const void
     a.out = out; a.lse_out = lse_out;
     a.Hkv = p->num_kv_heads; a.G = G; a.D = p->head_dim; a.rows = R; a.num_splits = S;
     cudaStream_t st = (cudaStream_t)stream;
+    if (S == 1 && use_pair_kernel(p)) return launch_copy_out(h, a, st);
     if (p->dtype == EVLN_BF16) return launch_combine<__nv_bfloat16>(h, a, p->head_dim, false, nullptr, st);
     return launch_combine<float>(h, a, p->head_dim, false, nullptr, st);
 }
@@ -1112,11 +1193,28 @@ evlnStatus_t evlnPagedStepAttention(evlnHandle_t h, const evlnPagedParams* p, co
     a.scale_log2 = scale * 1.4426950408889634f;
     a.div_g = make_fast_div((uint32_t)G);
     a.div_s = make_fast_div(1u);
-    BatchLens bl;
-    fill_lens(&bl, p, h_cache_lens, h_new_offsets, chunk);
-    if (bl.item_off[p->batch] != (int)items) return EVLN_INVALID_VALUE;
-    launch_pair_pdl(attn_pair_kernel<true, BatchLens>, dim3(2 * (int)items), kTcSmemBytes, (cudaStream_t)stream, tm_q, tm_k,
-                    tm_v, a, bl, TcOutArgs{});
+    PagedLens bl;
+    fill_lens(&bl, p, h_cache_lens, h_new_offsets);
+    {
+        int order[kMaxBatch];
+        longest_first(p->batch, h_cache_lens, h_new_offsets, order);
+        int item = 0;
+        for (int i = 0; i <= kMaxBatch; ++i) {
+            bl.item_off[i] = item;
+            if (i >= p->batch) continue;
+            const int b = order[i], n = h_new_offsets[b + 1] - h_new_offsets[b], units = ceil_div(n * G, kUnitRows);
+            bl.order[i] = (unsigned char)b;
+            for (int u = 0; u < units; ++u) item += ceil_div(unit_kv_tiles(h_cache_lens[b], n, G, u, kUnitRows), chunk) * p->num_kv_heads;
+        }
+        if (item != (int)items) return EVLN_INVALID_VALUE;
+    }
+    TcOutArgs d = {};
+    if (smax == 1) {
+        d.out = (__nv_bfloat16*)workspace;
+        d.lse_out = a.lse_part;
+    }
+    launch_pair_pdl(attn_pair_kernel<true, PagedLens>, dim3(2 * (int)items), kTcSmemBytes, (cudaStream_t)stream, tm_q, tm_k,
+                    tm_v, a, bl, d);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
 }
@@ -1142,6 +1240,7 @@ evlnStatus_t evlnPagedStepCombine(evlnHandle_t h, const evlnPagedParams* p, cons
     a.out = out; a.lse_out = lse_out;
     a.Hkv = p->num_kv_heads; a.G = G; a.D = 128; a.rows = (int)rows; a.num_splits = smax;
     a.batch = p->batch; a.unit_rows = kUnitRows; a.chunk_tiles = chunk;
+    if (smax == 1 && !paged_few(p, h_new_offsets)) return launch_copy_out(h, a, (cudaStream_t)stream);
     BatchLens bl;
     fill_lens(&bl, p, h_cache_lens, h_new_offsets);
     return launch_combine<__nv_bfloat16>(h, a, 128, true, &bl, (cudaStream_t)stream);
@@ -1213,7 +1312,7 @@ evlnStatus_t plan_packed(evlnHandle_t h, const evlnPackedParams* p, PackedPlan* 
     // an action chunk walks no more keys than the largest unit of the visual run beside it: not split
     // unless the caller says so
     if (n_act > 0)
-        batch_schedule(h->num_sms, G, p->num_kv_heads, p->num_frames, pl->lens, pl->offs, true, false,
+        batch_schedule(h->num_sms, G, p->num_kv_heads, p->num_frames, pl->lens, pl->offs, nullptr, true, false,
                        p->kv_chunk_tiles > 0 ? p->kv_chunk_tiles : 1 << 24, &pl->chunk, &pl->smax, &pl->items);
     const size_t part_a = pl->smax > 1 ? partial_bytes(pl->smax, p->num_kv_heads, n_act * G, 128) : 0;
     size_t off = 0;
