@@ -444,41 +444,59 @@ void longest_first(int batch, const int* lens, const int* offs, int* order)
 }
 
 // When the last of `pairs` CTA pairs is done (in KV tiles) if each takes the next work item as it becomes free,
-// episodes in the order given, items of at most `chunk` tiles.  The pairs are kept as runs of equal load, so
-// an episode costs a few steps however many items it has.
+// episodes in the order given, items of at most `chunk` tiles.  The pairs are kept as runs of equal load
+// (ascending), so an episode costs a few steps however many items it has.
+constexpr int kMaxPairs = 128;
+constexpr double kItemTiles = 10.0;      // an item's launch, set-up, first tile and write-out, in KV tiles (measured)
 double finish_time(int pairs, int G, int Hkv, int batch, const int* lens, const int* offs, const int* order, int chunk)
 {
-    struct Run { double load; int count; };
-    std::vector<Run> runs(1, Run{0.0, pairs});        // ascending loads
-    double last = 0.0;
+    struct Run { double load; int count; } runs[kMaxPairs];
+    int num = 1;
+    runs[0] = Run{0.0, pairs < kMaxPairs ? pairs : kMaxPairs};
     for (int i = 0; i < batch; ++i) {
         const int b = order[i], n = offs[b + 1] - offs[b];
         if (n == 0) continue;
         const int units = ceil_div(n * G, kUnitRows);
         const int nkv = unit_kv_tiles(lens[b], n, G, units - 1, kUnitRows), splits = ceil_div(nkv, chunk);
-        // set-up, first-tile latency, write-out and teardown of an item cost about as much as 7 KV tiles
-        const double cost = (double)nkv / splits + 7.0;
+        const double cost = (double)nkv / splits + kItemTiles;
         for (long left = (long)units * Hkv * splits; left > 0;) {
             const int take = left < runs[0].count ? (int)left : runs[0].count;
             const double load = runs[0].load + cost;
-            runs[0].count -= take;
-            if (runs[0].count == 0) runs.erase(runs.begin());
-            size_t at = 0;
-            while (at < runs.size() && runs[at].load < load) ++at;
-            if (at < runs.size() && runs[at].load == load) runs[at].count += take;
-            else runs.insert(runs.begin() + at, Run{load, take});
-            if (load > last) last = load;
             left -= take;
+            runs[0].count -= take;
+            int at = 0;
+            if (runs[0].count == 0) {              // the lowest run moves up: close its place while looking
+                --num;
+                for (; at < num && runs[at + 1].load < load; ++at) runs[at] = runs[at + 1];
+                if (at < num && runs[at + 1].load == load) {
+                    runs[at + 1].count += take;
+                    for (int k = at; k < num; ++k) runs[k] = runs[k + 1];
+                } else {
+                    runs[at] = Run{load, take};
+                    ++num;
+                }
+            } else {
+                while (at < num && runs[at].load < load) ++at;
+                if (at < num && runs[at].load == load) {
+                    runs[at].count += take;
+                } else {
+                    for (int k = num; k > at; --k) runs[k] = runs[k - 1];
+                    runs[at] = Run{load, take};
+                    ++num;
+                }
+            }
         }
     }
-    return last;
+    return runs[num - 1].load;
 }
 
 // Work-item size of a batch on CTA pairs.  Not splitting saves the partials (an fp32 row set per split written
 // and read again against one rounded row set) and the items' fixed costs; splitting evens out the pairs.  Many
-// items even out by themselves (longest first); else the estimate above decides between a few sizes.  16
-// ragged episodes of one frame (384 unsplit items): see the paged batch in the measured table.
-int choose_chunk(int pairs, int G, int Hkv, int batch, const int* lens, const int* offs, const int* order, long total, int nkv_max)
+// items even out by themselves (longest first); else the estimate above decides how often the longest
+// episode is split.  Measured: 16 ragged episodes of one frame (384 unsplit items) 480 us with items of a quarter
+// of a pair's share, 428 unsplit; episodes of 4000 and 1000 tokens 42 us, 28 with the longer one split in two;
+// of 16384 and 8000 tokens 104 and 91 (three and two ways).
+int choose_chunk(int pairs, int G, int Hkv, int batch, const int* lens, const int* offs, const int* order, int nkv_max)
 {
     long unsplit = 0;
     for (int b = 0; b < batch; ++b) unsplit += (long)ceil_div((offs[b + 1] - offs[b]) * G, kUnitRows) * Hkv;
@@ -486,14 +504,11 @@ int choose_chunk(int pairs, int G, int Hkv, int batch, const int* lens, const in
     const double rows = (double)offs[batch] * G * Hkv;
     int best = nkv_max;
     double best_cost = 1e30;
-    for (int k = 0; k <= 4; ++k) {
-        int chunk = k == 0 ? nkv_max : (int)((total + (long)pairs * k - 1) / ((long)pairs * k));
-        if (chunk < 4) chunk = 4;
-        if (chunk < ceil_div(nkv_max, kMaxSplits)) chunk = ceil_div(nkv_max, kMaxSplits);
-        if (chunk > nkv_max) chunk = nkv_max;
-        const double splits = chunk == nkv_max ? 0.5 : ceil_div(nkv_max, chunk);      // (row sets moved, in fp32 units)
-        // a KV tile takes a pair about 0.55 us; partials move at about 5.5 TB/s, each row written and read
-        const double cost = finish_time(pairs, G, Hkv, batch, lens, offs, order, chunk) + rows * splits * 1024.0 / 5.5e6 / 0.55;
+    for (int splits = 1; splits <= 8 && splits <= nkv_max; ++splits) {
+        const int chunk = ceil_div(nkv_max, splits);
+        // a KV tile takes a pair about 0.63 us; partials move at about 5.5 TB/s, each row written and read
+        const double moved = rows * (splits == 1 ? 0.5 : splits) * 1024.0 / 5.5e6 / 0.63;
+        const double cost = finish_time(pairs, G, Hkv, batch, lens, offs, order, chunk) + moved;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = chunk; }
     }
     return best;
@@ -522,7 +537,7 @@ void batch_schedule(int num_sms, int G, int Hkv, int batch, const int* lens, con
         chunk = (int)((total + (long)num_sms * 4 - 1) / ((long)num_sms * 4));
         if (chunk < 2) chunk = 2;
     } else if (chunk <= 0) {
-        chunk = choose_chunk(num_sms / 2 > 0 ? num_sms / 2 : 1, G, Hkv, batch, lens, offs, order, total, nkv_max);
+        chunk = choose_chunk(num_sms / 2 > 0 ? num_sms / 2 : 1, G, Hkv, batch, lens, offs, order, nkv_max);
     }
     if (chunk < ceil_div(nkv_max, kMaxSplits)) chunk = ceil_div(nkv_max, kMaxSplits);
     long cnt = 0;
