@@ -58,13 +58,17 @@ constexpr int kParts = 4;                             // softmax threads per que
 constexpr int kTileBytes = kTileM * 128 * 2;          // Q tile: 128 rows x 128 channels x bf16
 constexpr int kHalfBytes = kTileBytes / 2;            // 16 KB: a 64-channel half of Q; a K or V half tile
 constexpr int kSmemBarBytes = 384;
-constexpr int kSmemXchBytes = 128 * 4 + 2 * kParts * 128 * 4 + 128;
+constexpr int kSmemXchBytes = 128 * 4 + 3 * kParts * 128 * 4 + 2 * 128 * 4 + 128;
+constexpr int kPairItems = 32;                        // most work items of a persistent pair in one launch
 
 // Shared-memory plan of a CTA.  CTAS = 2: the CTA of a pair stages half tiles (16 KB) through two
 // 5-deep rings.  CTAS = 1: a CTA on its own stages whole K / V tiles (32 KB: two 64-channel blocks
 // of 128 keys) through a 3-deep K ring and a 2-deep V ring.
-template <int CTAS>
+template <int CTAS, bool PERSIST>
 struct SmemPlan {
+    // The epilogue's rows: in the K ring when the kernel ends with its item (all 32 rows of a warp at once),
+    // in an area of their own when the ring already holds the next item's keys.
+    static constexpr int kRowStageBytes = PERSIST ? 8 * 144 + 128 : 32 * 144;
     static constexpr int kKStages = CTAS == 2 ? 5 : 3;
     static constexpr int kVStages = CTAS == 2 ? 5 : 2;
     static constexpr int kStageBytes = CTAS == 2 ? kHalfBytes : kTileBytes;
@@ -73,15 +77,19 @@ struct SmemPlan {
     static constexpr int kVOff = kKOff + kKStages * kStageBytes;
     static constexpr int kBarOff = kVOff + kVStages * kStageBytes;
     static constexpr int kRefOff = kBarOff + kSmemBarBytes;          // float [128 rows]: published references
-    static constexpr int kSumOff = kRefOff + 128 * 4;                // float [kParts][128 rows]: row-sum shares
-    static constexpr int kCandOff = kSumOff + kParts * 128 * 4;      // float [kParts][128 rows]: reference requests
+    static constexpr int kSumOff = kRefOff + 128 * 4;                // float [2][kParts][128 rows]: row-sum shares, items in turn
+    static constexpr int kDoneOff = kSumOff + 2 * kParts * 128 * 4;  // float [2][128 rows]: references of finished items
+    static constexpr int kCandOff = kDoneOff + 2 * 128 * 4;          // float [kParts][128 rows]: reference requests
     static constexpr int kReqOff = kCandOff + kParts * 128 * 4;      // int [4] request flags, int [4][kParts] released tiles
-    static constexpr int kBytes = kRefOff + kSmemXchBytes + 1024;    // + slack to align to 1024
-    static_assert(kKStages * kStageBytes >= 16 * 32 * 144, "the epilogue stages its rows in the K ring");
+    static constexpr int kStageOff = PERSIST ? kRefOff + kSmemXchBytes : kKOff;
+    static constexpr int kItemsOff = kRefOff + kSmemXchBytes + (PERSIST ? 16 * kRowStageBytes : 0);   // the pair's items
+    static constexpr int kBytes = kItemsOff + (PERSIST ? kPairItems * 48 : 0) + 1024;    // + slack to align to 1024
+    static_assert(PERSIST || kKStages * kStageBytes >= 16 * kRowStageBytes, "the epilogue stages its rows in the K ring");
     static_assert(kBytes <= 227 * 1024, "shared memory per CTA");
 };
-constexpr int kTcSmemBytes = SmemPlan<2>::kBytes;
-constexpr int kSoloSmemBytes = SmemPlan<1>::kBytes;
+constexpr int kTcSmemBytes = SmemPlan<2, false>::kBytes;
+constexpr int kPersistSmemBytes = SmemPlan<2, true>::kBytes;
+constexpr int kSoloSmemBytes = SmemPlan<1, false>::kBytes;
 constexpr long long kWaitLimitCycles = 2000000000LL;  // ~1 s at boost clocks
 constexpr int kScoreBufs = 2;
 // Registers per thread after the set-up.  setmaxnreg moves registers inside the pool the CTA got at
@@ -128,7 +136,8 @@ struct TcOutArgs {
     int act_items;            // work items of the action chunks
     int act_split;            // some of them are splits: theirs go to o_part / lse_part
     PackedMap act_map;
-    FastDiv div_hkv;
+    FastDiv div_hkv, div_units;
+    int first_item, num_items;   // persistent kernels only: the launch serves items first_item .. num_items-1
 };
 
 // --- descriptors --------------------------------------------------------------------------
@@ -275,7 +284,7 @@ __device__ __noinline__ float first_block_reference(uint32_t taddr, int lim, flo
 
 // --- work decoding ------------------------------------------------------------------------
 
-struct WorkItem {
+struct __align__(16) WorkItem {
     int b, g, unit, slot;     // episode, kv head, unit within the episode, partial slot
     int L, n;                 // episode lengths
     int row_base;             // first packed row of the episode within the kv head
@@ -290,16 +299,24 @@ struct WorkItem {
 // Batches (paged cache, action chunks of a packed sequence): items are numbered episode by episode (kv
 // head, unit, split inside), the host passes the first item of every episode and the CTA searches that
 // table.
-template <bool PAGED, bool TAIL, typename LensT, int CTAS>
-__device__ __forceinline__ WorkItem decode_work(const TcAttnArgs& a, const LensT& lens, const TcOutArgs& d)
+template <bool PAGED, bool TAIL, bool PERSIST, typename LensT, int CTAS>
+__device__ __forceinline__ WorkItem decode_work(const TcAttnArgs& a, const LensT& lens, const TcOutArgs& d, int item)
 {
     constexpr int UNIT_ROWS = CTAS * kTileM;
     WorkItem w;
     if (!PAGED && !TAIL) {
         w.b = 0;
-        w.unit = (int)(gridDim.y - 1 - blockIdx.y);
-        w.g = CTAS == 2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-        w.slot = (int)blockIdx.z;
+        if (PERSIST) {
+            // split by split, so that the units that read the same keys run side by side
+            const uint32_t su = fast_div((uint32_t)item, d.div_hkv), slot = fast_div(su, d.div_units);
+            w.unit = a.units_per_head - 1 - (int)(su - slot * (uint32_t)a.units_per_head);
+            w.g = item - (int)su * a.Hkv;
+            w.slot = (int)slot;
+        } else {
+            w.unit = (int)(gridDim.y - 1 - blockIdx.y);
+            w.g = CTAS == 2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+            w.slot = (int)blockIdx.z;
+        }
         w.visual = true;
         w.L = a.cache_len;
         w.n = a.num_new;
@@ -308,7 +325,6 @@ __device__ __forceinline__ WorkItem decode_work(const TcAttnArgs& a, const LensT
         w.j0 = (int)fast_div((uint32_t)w.slot * nkv, a.div_s);
         w.j1 = (int)fast_div((uint32_t)(w.slot + 1) * nkv, a.div_s);
     } else {
-        int item = (int)(blockIdx.x >> 1);
         w.visual = TAIL && item >= d.act_items;
         if (TAIL) {
             if (w.visual) {
@@ -363,6 +379,85 @@ __device__ __forceinline__ WorkItem decode_work(const TcAttnArgs& a, const LensT
     return w;
 }
 
+// --- the write-out of an item's rows ----------------------------------------------------------
+// One warp: the 32 rows of its lane quarter, its 32 channels of O (at t_o), scaled by each lane's `inv`.  They
+// go out through shared memory, as many rows at a time as `stage` holds, so that global stores are whole
+// sectors of few lines (straight from the registers, a line per lane, they took 1 us longer).
+template <bool PAGED, bool TAIL, bool PERSIST, typename LensT, int CTAS>
+__device__ __forceinline__ void write_rows(const TcAttnArgs& a, const LensT& lens, const TcOutArgs& d, const WorkItem& w, uint32_t rank,
+                                           int quarter, int part, float inv, float lse, uint32_t t_o, uint8_t* stage, uint32_t o_free0)
+{
+    const int lane = threadIdx.x & 31;
+    const int rows_valid = w.n * a.G;
+    const int first_row = w.unit * (CTAS * kTileM) + (int)rank * kTileM + (quarter << 5);   // episode-local
+    const int r_local = first_row + lane;
+    const int rows_here = rows_valid - first_row;                    // may be <= 0 or > 32
+    const bool direct = CTAS == 2 && d.out != nullptr && !(TAIL && !w.visual && d.act_split);
+    uint32_t regs[32];
+    ptx::tmem_ld32(t_o, regs);
+    ptx::tmem_ld_wait();
+    if (PERSIST) {
+        ptx::fence_before_sync();
+        if (ptx::elect_one()) ptx::mbar_arrive_cluster(o_free0);
+    }
+    if (direct) {
+        // the row's only work item: round once to the storage dtype and write the output itself
+        auto out_row = [&](int rl) -> long {           // row of [n, Hq, 128] of the item's row rl
+            const int tok = (int)fast_div((uint32_t)rl, a.div_g);
+            const long t = TAIL ? packed_row(w.visual ? d.map : d.act_map, (w.visual ? 0 : lens.new_off[w.b]) + tok)
+                                : PAGED ? (long)lens.new_off[w.b] + tok : (long)tok;
+            return t * (a.Hkv * a.G) + w.g * a.G + (rl - tok * a.G);
+        };
+        uint32_t v[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e)
+            v[e] = ptx::pack_bf16x2(__uint_as_float(regs[2 * e]) * inv, __uint_as_float(regs[2 * e + 1]) * inv);
+        constexpr int kRows = SmemPlan<CTAS, PERSIST>::kRowStageBytes >= 32 * 80 ? 32 : 16;      // 80 bytes apart
+#pragma unroll
+        for (int h = 0; h < 32; h += kRows) {
+            if (lane >= h && lane < h + kRows) {
+                uint4* srow = reinterpret_cast<uint4*>(stage + (lane - h) * 80);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) srow[e] = make_uint4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < kRows; i += 8) {
+                const int r = i + (lane >> 2);
+                if (h + r < rows_here)
+                    reinterpret_cast<uint4*>(d.out + out_row(first_row + h + r) * 128 + part * 32)[lane & 3] =
+                        *reinterpret_cast<const uint4*>(stage + r * 80 + (lane & 3) * 16);
+            }
+            __syncwarp();
+        }
+        if (d.lse_out && part == 0 && r_local < rows_valid) d.lse_out[out_row(r_local)] = lse;
+    } else {
+        const long prow0 = ((long)w.slot * a.Hkv + w.g) * a.rows + w.row_base + first_row;
+        float* gbase = a.o_part + prow0 * 128 + part * 32;
+        constexpr int kRows = SmemPlan<CTAS, PERSIST>::kRowStageBytes / 144;    // rows at a time, 144 bytes apart
+#pragma unroll
+        for (int h = 0; h < 32; h += kRows) {
+            if (lane >= h && lane < h + kRows) {
+                float4* srow = reinterpret_cast<float4*>(stage + (lane - h) * 144);
+#pragma unroll
+                for (int e = 0; e < 32; e += 4)
+                    srow[e >> 2] = make_float4(__uint_as_float(regs[e]) * inv, __uint_as_float(regs[e + 1]) * inv,
+                                               __uint_as_float(regs[e + 2]) * inv, __uint_as_float(regs[e + 3]) * inv);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < kRows; i += 4) {
+                const int r = i + (lane >> 3);
+                if (h + r < rows_here)
+                    *reinterpret_cast<float4*>(gbase + (long)(h + r) * 128 + (lane & 7) * 4) =
+                        *reinterpret_cast<const float4*>(stage + r * 144 + (lane & 7) * 16);
+            }
+            __syncwarp();
+        }
+        if (part == 0 && r_local < rows_valid) a.lse_part[prow0 + lane] = lse;
+    }
+}
+
 // --- the kernel ---------------------------------------------------------------------------
 // CTAS = 2: launched with a cluster of 2 CTAs along x: query tile = cluster rank.
 // CTAS = 1: no cluster; one query tile (all the rows of a kv head fit in it).
@@ -372,14 +467,14 @@ __device__ __forceinline__ WorkItem decode_work(const TcAttnArgs& a, const LensT
 // that cache (every row sees all of them) and bring their own n_b new tokens in a separate buffer
 // (tm_qt / tm_kt / tm_vt, packed over the batch; causal among themselves), each after its own prefix of
 // the visual tokens, none visible to another.
-template <bool PAGED, bool TAIL, typename LensT, int CTAS>
+template <bool PAGED, bool TAIL, bool PERSIST, typename LensT, int CTAS, typename TableT>
 __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                                              const CUtensorMap* tm_qt, const CUtensorMap* tm_kt, const CUtensorMap* tm_vt,
-                                             const TcAttnArgs& a, const LensT& lens, const TcOutArgs& d)
+                                             const TcAttnArgs& a, const LensT& lens, const TcOutArgs& d, const TableT& table)
 {
     static_assert(CTAS == 2 || !(PAGED || TAIL), "the batch kernels run on CTA pairs");
     static_assert(!(PAGED && TAIL), "one cache layout at a time");
-    using Plan = SmemPlan<CTAS>;
+    using Plan = SmemPlan<CTAS, PERSIST>;
     constexpr int kKStages = Plan::kKStages, kVStages = Plan::kVStages, kStageBytes = Plan::kStageBytes;
     constexpr int kSmemQOff = Plan::kQOff, kSmemKOff = Plan::kKOff, kSmemVOff = Plan::kVOff;
     constexpr int kItemRows = CTAS * kTileM;           // query rows of a work item
@@ -402,17 +497,20 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
     const uint32_t bar_ref = bar_o_full + 8;                     // [4] the rows' references are published
     const uint32_t bar_xch = bar_ref + 32;                       // [4] the four warps of a lane quarter meet here (row sums)
     const uint32_t bar_rare = bar_xch + 32;                      // [4] ... and here when a row's reference has to move
-    const uint32_t tmem_slot = bar_rare + 32;                    // uint32
+    const uint32_t bar_q_free = bar_rare + 32;                   // last score MMA of the item: Q may be overwritten
+    const uint32_t bar_o_free = bar_q_free + 8;                  // (CTA 0) both CTAs' softmax has read O
+    const uint32_t tmem_slot = bar_o_free + 8;                   // uint32
     constexpr int kBarsCtas = 1 + kKStages + kVStages;                                 // arrival count CTAS
     constexpr int kBarsSoft = 2 * kScoreBufs;                                          // one per softmax warp of the tile
     constexpr int kBarsOne = kKStages + kVStages + kScoreBufs + 4 + 1 + 4;             // count 1
-    constexpr int kNumBars = kBarsCtas + kBarsSoft + kBarsOne + 8;                     // + xch, rare: kParts
+    constexpr int kNumBars = kBarsCtas + kBarsSoft + kBarsOne + 8 + 2;                 // + xch, rare: kParts; q_free, o_free
     static_assert(8 * kNumBars + 8 <= kSmemBarBytes, "barrier area");
     static_assert(kNumBars <= 64, "one thread of warps 2-3 per barrier");
     volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(smem_gen + (tmem_slot - smem_base));
     volatile int* s_abort = reinterpret_cast<volatile int*>(smem_gen + (tmem_slot - smem_base) + 4);
     float* s_ref = reinterpret_cast<float*>(smem_gen + Plan::kRefOff);
     float* s_sum = reinterpret_cast<float*>(smem_gen + Plan::kSumOff);
+    float* s_done = reinterpret_cast<float*>(smem_gen + Plan::kDoneOff);
     float* s_cand = reinterpret_cast<float*>(smem_gen + Plan::kCandOff);
     volatile int* s_req = reinterpret_cast<volatile int*>(smem_gen + Plan::kReqOff);        // [4]
     volatile int* s_rel = reinterpret_cast<volatile int*>(smem_gen + Plan::kReqOff) + 4;    // [4][kParts]
@@ -421,14 +519,47 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
     const uint32_t rank = CTAS == 2 ? ptx::cluster_ctarank() : 0u;   // 0: issues the MMAs, owns the "(CTA 0)" barriers
     if (threadIdx.x == 0) EVLN_STAMP(0);
 
-    const WorkItem w = decode_work<PAGED, TAIL, LensT, CTAS>(a, lens, d);
+    // A persistent pair takes the items the host's table gives it, or else pair, 2 P - 1 - pair, 2 P + pair, ... (P
+    // pairs; the items come longest first, so going back and forth evens the pairs out).  All barriers and
+    // buffers run on across items: `base` counts the KV tiles of the items before this one, `turn` the items.
+    const int pair = (int)(blockIdx.x >> 1), pairs = (int)(gridDim.x >> 1);
+    auto item_number = [&](int turn) -> int {
+        if constexpr (PERSIST) {
+            if (table.count > 0) {
+                const int at = turn * pairs + pair;
+                return at < table.count && table.item[at] != kNoItem ? (int)table.item[at] : 0x7fffffff;
+            }
+        }
+        return (PERSIST ? d.first_item : 0) + turn * pairs + ((turn & 1) ? pairs - 1 - pair : pair);
+    };
+    // Decoding an item takes a few integer divisions (1-2 K cycles), and every role of the pair needs every
+    // item: warp 3 decodes them into shared memory, a lane each, while the pair sets up (so a launch has at most
+    // kPairItems items per pair).
+    WorkItem* s_items = reinterpret_cast<WorkItem*>(smem_gen + Plan::kItemsOff);
+    static_assert(sizeof(WorkItem) == 48, "place of an item");
+    auto item_of = [&](int turn) -> WorkItem { return s_items[turn]; };
+    WorkItem w = decode_work<PAGED, TAIL, PERSIST, LensT, CTAS>(a, lens, d, item_number(0));
     if ((PAGED || TAIL) && w.b < 0) return;                      // both CTAs of the pair decode the same item
 
-    const int rows_valid = w.n * a.G;                            // packed rows of this episode
-    const int row0 = w.unit * kItemRows + (int)rank * kTileM;    // first row of this CTA's tile (episode-local)
-    const int ntiles = w.j1 - w.j0;
-    // TAIL: tiles below nct come from the shared cache (all of a visual unit's)
-    const int nct = TAIL ? (w.visual ? 0x3fffffff : (w.L + kTileN - 1) / kTileN) : 0;
+    int rows_valid, row0, ntiles, nct;
+    auto set_item = [&]() {
+        rows_valid = w.n * a.G;                                  // packed rows of this episode
+        row0 = w.unit * kItemRows + (int)rank * kTileM;          // first row of this CTA's tile (episode-local)
+        ntiles = w.j1 - w.j0;
+        // TAIL: tiles below nct come from the shared cache (all of a visual unit's)
+        nct = TAIL ? (w.visual ? 0x3fffffff : (w.L + kTileN - 1) / kTileN) : 0;
+    };
+    set_item();
+    int base = 0, turn = 0;
+    // the next item of the pair, if there is one (every role goes through the items on its own)
+    auto next_item = [&]() -> bool {
+        if (!PERSIST) return false;
+        base += ntiles;
+        if (item_number(++turn) >= d.num_items) return false;
+        w = item_of(turn);
+        set_item();
+        return true;
+    };
     // Lane quarters (32 rows each) of the tile that hold rows of the episode.  A CTA on its own lets
     // the softmax warps of the others sit out; a pair keeps all of them (both CTAs count alike).
     int quarters = 4;
@@ -483,12 +614,15 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
             if (i < kBarsCtas) count = CTAS;                                   // q_full, k_full, v_full
             else if (i < kBarsCtas + kBarsSoft) count = CTAS * quarters * 2;   // s_free, p_full: the tile's softmax warps
             else if (i < kBarsCtas + kBarsSoft + kBarsOne) count = 1;          // k_empty .. ref
-            else count = kParts;                                               // xch, rare
+            else if (i < kNumBars - 2) count = kParts;                         // xch, rare
+            else if (i == kNumBars - 1) count = CTAS * quarters * kParts;      // o_free (q_free: 1)
             ptx::mbar_init(bar_base + 8 * i, count);
             ptx::fence_barrier_init();
         }
         if (i < 4) s_req[i] = 0;
         if (i == 0) *s_abort = 0;
+        if (PERSIST && warp == 3 && item_number(lane) < d.num_items)
+            s_items[lane] = decode_work<PAGED, TAIL, PERSIST, LensT, CTAS>(a, lens, d, item_number(lane));
     }
     if (warp == 1) {
         if (CTAS == 2) {
@@ -525,9 +659,9 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
             // K tile j.  Pair: this CTA's half, keys [128 j + 64 rank, +64), all channels (two 64-channel
             // blocks of 64 keys).  Alone: the whole tile (two 64-channel blocks of 128 keys).
             auto load_k = [&](int jj) {
-                const int stage = jj % kKStages;
-                if (jj >= kKStages)
-                    ok_prod = wait_bounded(bar_k_empty + 8 * stage, ((jj / kKStages) & 1) ^ 1, kDevTimeoutProducer, a.status, s_abort);
+                const int gj = base + jj, stage = gj % kKStages;
+                if (gj >= kKStages)
+                    ok_prod = wait_bounded(bar_k_empty + 8 * stage, ((gj / kKStages) & 1) ^ 1, kDevTimeoutProducer, a.status, s_abort);
                 if (!ok_prod) return;
                 const uint32_t dst = smem_base + kSmemKOff + stage * kStageBytes;
                 const uint32_t bar = on_cta0(bar_k_full + 8 * stage);
@@ -558,9 +692,9 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
             };
             // V tile j, all 128 keys.  Pair: channels [64 rank, +64).  Alone: both 64-channel blocks.
             auto load_v = [&](int jj) {
-                const int stage = jj % kVStages;
-                if (jj >= kVStages)
-                    ok_prod = wait_bounded(bar_v_empty + 8 * stage, ((jj / kVStages) & 1) ^ 1, kDevTimeoutProducer, a.status, s_abort);
+                const int gj = base + jj, stage = gj % kVStages;
+                if (gj >= kVStages)
+                    ok_prod = wait_bounded(bar_v_empty + 8 * stage, ((gj / kVStages) & 1) ^ 1, kDevTimeoutProducer, a.status, s_abort);
                 if (!ok_prod) return;
                 const uint32_t dst = smem_base + kSmemVOff + stage * kStageBytes;
                 const uint32_t bar = on_cta0(bar_v_full + 8 * stage);
@@ -583,24 +717,26 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
                 }
             };
 
-    // The producer's first loads (Q, then the K tiles of the first scores) go out before the warps
-    // change their register shares: that hand-over is a rendezvous of the whole warpgroup, and the
-    // loads' latency is the longest item on the way to the first MMA.
-    const int pre_k = ntiles < kScoreBufs ? ntiles : kScoreBufs;
+    // the item's Q tile, then the K tiles of its first scores
+    auto load_first = [&]() {
+        const uint32_t q_full0 = on_cta0(bar_q_full);
+        const uint32_t dst = smem_base + kSmemQOff;
+        const int qrow = w.row_base + row0;
+        const CUtensorMap* map_q = TAIL && !w.visual ? tm_qt : &tm_q;
+        expect(q_full0, kTileBytes);
+        tma3(dst, map_q, q_full0, 0, qrow, w.g);
+        tma3(dst + kHalfBytes, map_q, q_full0, 64, qrow, w.g);
+        for (int jj = 0; jj < kScoreBufs && jj < ntiles && ok_prod; ++jj) load_k(jj);
+    };
+
+    // The producer's first loads go out before the warps change their register shares: that hand-over is
+    // a rendezvous of the whole warpgroup, and the loads' latency is the longest item on the way to the
+    // first MMA.
     if (warp == 0 && lane == 0) {
         // everything this CTA reads or writes in global memory follows this thread's loads, so
         // one wait here orders the whole CTA after the kernels it depends on
         ptx::grid_dependency_wait();
-            {
-                const uint32_t q_full0 = on_cta0(bar_q_full);
-                const uint32_t dst = smem_base + kSmemQOff;
-                const int qrow = w.row_base + row0;
-                expect(q_full0, kTileBytes);
-                const CUtensorMap* map_q = TAIL && !w.visual ? tm_qt : &tm_q;
-                tma3(dst, map_q, q_full0, 0, qrow, w.g);
-                tma3(dst + kHalfBytes, map_q, q_full0, 64, qrow, w.g);
-            }
-        for (int jj = 0; jj < pre_k; ++jj) load_k(jj);
+        load_first();
     }
     __syncwarp();            // (the register hand-over below wants whole warps)
 
@@ -612,9 +748,15 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
         // ================= TMA producer =================
         if (lane == 0) {
             // in the order the MMAs consume them: (K_0, K_1 are on their way,) then V_j, K_{j+2}
-            for (int jj = 0; jj < ntiles && ok_prod; ++jj) {
-                load_v(jj);
-                if (ok_prod && jj + kScoreBufs < ntiles) load_k(jj + kScoreBufs);
+            for (;;) {
+                for (int jj = 0; jj < ntiles && ok_prod; ++jj) {
+                    load_v(jj);
+                    if (ok_prod && jj + kScoreBufs < ntiles) load_k(jj + kScoreBufs);
+                }
+                if (!ok_prod || !next_item()) break;
+                ok_prod = wait_bounded(bar_q_free, (turn - 1) & 1, kDevTimeoutProducer, a.status, s_abort);
+                if (!ok_prod) break;
+                load_first();
             }
             if (!ok_prod || *s_abort) {
                 // give this CTA's loads in flight time to land before the pair may leave
@@ -629,25 +771,28 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
         // descriptors differ only in their address field (units of 16 bytes): build them once
         const uint64_t qdesc0 = make_sdesc(smem_base + kSmemQOff, 16, 1024);
         const uint64_t kdesc0 = make_sdesc(smem_base + kSmemKOff, 16, 1024);            // K-major; 64 (pair) or 128 keys per CTA
-        bool ok = warp_wait(bar_q_full, 0, kDevTimeoutMmaQ, a.status, s_abort, lane);
+        bool ok = true;
+        do {
+        ok = warp_wait(bar_q_full, turn & 1, kDevTimeoutMmaQ, a.status, s_abort, lane);
         for (int jj = 0; jj < ntiles && ok; ++jj) {
+            const int gj = base + jj;
             // K_jj landed; the softmax has read tile jj - 2 out of this score buffer.  A wait costs
             // ~150 cycles even on a completed barrier, so two lanes take one each.
             {
-                uint32_t bar = bar_k_full + 8 * (jj % kKStages), parity = (jj / kKStages) & 1;
+                uint32_t bar = bar_k_full + 8 * (gj % kKStages), parity = (gj / kKStages) & 1;
                 int code = kDevTimeoutMmaKV;
-                if (lane == 1) { bar = bar_s_free + 8 * (jj & 1); parity = ((jj >> 1) - 1) & 1; code = kDevTimeoutMmaP; }
+                if (lane == 1) { bar = bar_s_free + 8 * (gj & 1); parity = ((gj >> 1) - 1) & 1; code = kDevTimeoutMmaP; }
                 bool mine = true;
-                if (lane == 0 || (lane == 1 && jj >= kScoreBufs)) mine = wait_bounded(bar, parity, code, a.status, s_abort);
+                if (lane == 0 || (lane == 1 && gj >= kScoreBufs)) mine = wait_bounded(bar, parity, code, a.status, s_abort);
                 if (lane < 2 && jj < 9) EVLN_STAMP(20 + 9 * lane + jj);
                 ok = __all_sync(0xffffffffu, mine);
             }
             if (!ok) break;
             ptx::fence_after_sync();
             if (ptx::elect_one()) {
-                const int stage = jj % kKStages;
+                const int stage = gj % kKStages;
                 const uint64_t kd = kdesc0 + (uint64_t)((stage * kStageBytes) >> 4);
-                const uint32_t d = tmem + (uint32_t)(jj & 1) * 128;
+                const uint32_t d = tmem + (uint32_t)(gj & 1) * 128;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
                     const uint64_t qoff = (uint64_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4);
@@ -656,54 +801,61 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
                     else ptx::mma_ss(d, qdesc0 + qoff, kd + koff, idesc_s, ks > 0);
                 }
                 if (CTAS == 2) {
-                    ptx::mma_commit_pair(bar_s_full + 8 * (jj & 1), (uint16_t)3);
+                    ptx::mma_commit_pair(bar_s_full + 8 * (gj & 1), (uint16_t)3);
                     ptx::mma_commit_pair(bar_k_empty + 8 * stage, (uint16_t)3);
+                    if (PERSIST && jj == ntiles - 1) ptx::mma_commit_pair(bar_q_free, (uint16_t)3);
                 } else {
-                    ptx::mma_commit(bar_s_full + 8 * (jj & 1));
+                    ptx::mma_commit(bar_s_full + 8 * (gj & 1));
                     ptx::mma_commit(bar_k_empty + 8 * stage);
                 }
             }
             if (lane == 0 && jj < 9) EVLN_STAMP(38 + jj);
             __syncwarp();
         }
+        } while (ok && next_item());
     } else if (warp == 2 && rank == 0) {
         // ================= product issuer (CTA 0 of the pair): O (+)= P_jj V_jj =================
         const uint32_t idesc_pv = make_idesc(true, CTAS * kTileM, 128);
         const uint64_t vdesc0 = make_sdesc(smem_base + kSmemVOff, kHalfBytes, 1024);    // MN-major; 64-channel blocks 16 KB apart
         bool ok = true;
+        do {
         for (int jj = 0; jj < ntiles && ok; ++jj) {
+            const int gj = base + jj;
             {
-                uint32_t bar = bar_v_full + 8 * (jj % kVStages), parity = (jj / kVStages) & 1;
+                uint32_t bar = bar_v_full + 8 * (gj % kVStages), parity = (gj / kVStages) & 1;
                 int code = kDevTimeoutMmaKV;
-                if (lane == 1) { bar = bar_p_full + 8 * (jj & 1); parity = (jj >> 1) & 1; code = kDevTimeoutMmaP; }
+                if (lane == 1) { bar = bar_p_full + 8 * (gj & 1); parity = (gj >> 1) & 1; code = kDevTimeoutMmaP; }
+                // the item's first product overwrites O: the previous item's has been read
+                if (PERSIST && lane == 2) { bar = bar_o_free; parity = (turn - 1) & 1; code = kDevTimeoutMmaP; }
                 bool mine = true;
-                if (lane < 2) mine = wait_bounded(bar, parity, code, a.status, s_abort);
+                if (lane < 2 || (PERSIST && lane == 2 && jj == 0 && turn > 0)) mine = wait_bounded(bar, parity, code, a.status, s_abort);
                 ok = __all_sync(0xffffffffu, mine);
             }
             if (!ok) break;
             if (lane == 0 && jj < 9) EVLN_STAMP(47 + jj);
             ptx::fence_after_sync();
             if (ptx::elect_one()) {
-                const int stage = jj % kVStages;
+                const int stage = gj % kVStages;
                 const uint64_t vd = vdesc0 + (uint64_t)((stage * kStageBytes) >> 4);
-                const uint32_t p = tmem + kColP + (uint32_t)(jj & 1) * 64;
+                const uint32_t p = tmem + kColP + (uint32_t)(gj & 1) * 64;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
                     if (CTAS == 2) ptx::mma_ts_pair(tmem + kColO, p + ks * 8, vd + (uint64_t)((ks * 2048) >> 4), idesc_pv, jj > 0 || ks > 0);
                     else ptx::mma_ts(tmem + kColO, p + ks * 8, vd + (uint64_t)((ks * 2048) >> 4), idesc_pv, jj > 0 || ks > 0);
                 }
                 if (CTAS == 2) {
-                    ptx::mma_commit_pair(bar_pv_done + 8 * (jj & 3), (uint16_t)3);
+                    ptx::mma_commit_pair(bar_pv_done + 8 * (gj & 3), (uint16_t)3);
                     ptx::mma_commit_pair(bar_v_empty + 8 * stage, (uint16_t)3);
                     if (jj == ntiles - 1) ptx::mma_commit_pair(bar_o_full, (uint16_t)3);
                 } else {
-                    ptx::mma_commit(bar_pv_done + 8 * (jj & 3));
+                    ptx::mma_commit(bar_pv_done + 8 * (gj & 3));
                     ptx::mma_commit(bar_v_empty + 8 * stage);
                     if (jj == ntiles - 1) ptx::mma_commit(bar_o_full);
                 }
             }
             __syncwarp();
         }
+        } while (ok && next_item());
     }
     } else {
     ptx::setmaxnreg_inc<kRegsSoftmax>();
@@ -714,15 +866,6 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
         const int grp = part >> 1;                         // its KV tiles: grp, grp + 2, ...
         const int half = part & 1;                         // its score columns: [64 half, +64), two blocks of 32
         const int r_tile = (quarter << 5) + lane;          // row within the tile = TMEM lane
-        const int r_local = row0 + r_tile;                 // packed row within the episode
-        const bool row_valid = r_local < rows_valid;
-        // last visible key index; a padding row (beyond the episode's rows: its Q is zero fill or
-        // another episode's) is never stored, so it takes everything unmasked rather than making its
-        // warp mask every tile
-        // (TAIL: `bound` is the row's last visible token among the item's OWN tokens, `cache_last` the last
-        // visible one of the cache)
-        const int bound = row_valid ? (TAIL ? 0 : w.L) + (int)fast_div((uint32_t)r_local, a.div_g) : 0x3fffffff;
-        const int cache_last = w.visual ? bound : w.L - 1;
         const uint32_t t_lane = tmem + ((uint32_t)(quarter << 5) << 16);
         const uint32_t t_s = t_lane + (uint32_t)grp * 128 + (uint32_t)half * 64;          // its half of the group's score buffer
         const uint32_t t_p = t_lane + kColP + (uint32_t)grp * 64 + (uint32_t)half * 32;   // ... and of its P buffer
@@ -730,8 +873,35 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
         const uint32_t s_free0 = on_cta0(bar_s_free + 8 * grp);
         const uint32_t p_full0 = on_cta0(bar_p_full + 8 * grp);
 
-        float m_ref = -INFINITY;      // reference maximum (log2 domain) the exponentials use
-        float l = 0.f;                // this thread's share of the running sum of exponentials
+        // of the item at hand (set_rows):
+        int first = 0, last;          // its tiles: numbers first .. last-1 over the pair's items
+        int lim;                      // columns 0 .. lim of this thread's 64 of its next tile are visible
+        int bound, own_from;          // TAIL: the row's last own token; the first tile of the item's own tokens
+        int rgrp, rpart;              // grp and part counted from the group of the item's first tile
+        float m_ref;                  // reference maximum (log2 domain) the exponentials use
+        float l;                      // this thread's share of the running sum of exponentials
+        bool sum_published;           // this thread's share of the row sum is out for the final exchange
+        auto set_rows = [&]() {
+            WorkItem it = w;
+            if (PERSIST) it = item_of(turn);
+            const int r_local = it.unit * kItemRows + (int)rank * kTileM + r_tile;      // packed row within the episode
+            const bool row_valid = r_local < it.n * a.G;
+            // the row's last visible key; a padding row (beyond the episode's rows: its Q is zero fill or
+            // another episode's) is never stored, so it takes everything unmasked rather than making its
+            // warp mask every tile
+            // (TAIL, action chunk: keys of the cache up to L-1, own tokens up to `bound`)
+            const int own = row_valid ? (int)fast_div((uint32_t)r_local, a.div_g) : 0x3f000000;
+            const bool chunk = TAIL && !it.visual;
+            last = first + it.j1 - it.j0;
+            bound = own;
+            own_from = chunk ? first + (it.L + kTileN - 1) / kTileN - it.j0 : 0x3fffffff;
+            rgrp = grp ^ (first & 1);
+            rpart = 2 * rgrp + half;
+            lim = (chunk ? it.L - 1 : it.L + own) - (it.j0 + rgrp) * kTileN - half * 64;
+            m_ref = -INFINITY;
+            l = 0.f;
+            sum_published = false;
+        };
         bool ok = true;
         const uint64_t scale2 = ptx::pack2(a.scale_log2, a.scale_log2);
         // Meeting of the four warps of this lane quarter (one phase of their barrier each): what any of
@@ -785,7 +955,6 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
         // reference (a power-of-two factor, exact): running sum, their channels of O, and their P
         // tile if it is written but not yet consumed.
         int nrare = 0;                // meetings on bar_rare so far
-        bool sum_published = false;   // this thread's share of the row sum is out for the final exchange
         auto move_reference = [&](int released, bool mine, float want) -> bool {
             s_cand[part * 128 + r_tile] = mine ? want : m_ref;
             if (lane == 0) s_rel[quarter * kParts + part] = released;
@@ -813,12 +982,12 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
             }
             const bool any_change = __any_sync(0xffffffffu, alpha != 1.f);
             if (any_change) {
-                if (r_min > 0) {
+                if (r_min > first) {
                     // PV(r_min - 1) must have landed.  Every tile below r_min is handed over, tile r_min
                     // is not, and the products are issued in order: PV(r_min + 3) cannot have been
                     // issued, so barrier (r_min - 1) % 4 has seen (r_min - 1) / 4 phases or one more.
-                    if (!warp_wait(bar_pv_done + 8 * ((r_min - 1) & 3), ((r_min - 1) >> 2) & 1, kDevTimeoutSoftmaxO, a.status,
-                                   s_abort, lane))
+                    const int last_pv = r_min - 1;
+                    if (!warp_wait(bar_pv_done + 8 * (last_pv & 3), (last_pv >> 2) & 1, kDevTimeoutSoftmaxO, a.status, s_abort, lane))
                         return false;
                     ptx::fence_after_sync();
                     uint32_t regs[32];              // this thread's 32 of the row's 128 channels
@@ -850,68 +1019,88 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
                 ptx::fence_before_sync();
             }
             m_ref = m_new;
-            if (sum_published) s_sum[part * 128 + r_tile] = l;    // (ordered by the meeting below)
+            if (sum_published) {                                  // (ordered by the meeting below)
+                s_sum[((turn & 1) * kParts + part) * 128 + r_tile] = l;
+                if (PERSIST && part == 0) s_done[(turn & 1) * 128 + r_tile] = m_ref;
+            }
             return meet(bar_rare, nrare++);
         };
 
+        // A persistent pair writes an item's rows out after each warp's first tile of the next item: while the last
+        // products of the one run, the first probabilities of the next are computed, and the tensor core waits
+        // for one softmax chain at the boundary instead of a write-out and a chain.
+        auto flush = [&](int done) {                  // the item of turn `done`
+            ok = warp_wait(bar_o_full, done & 1, kDevTimeoutSoftmaxO, a.status, s_abort, lane);
+            if (!ok) return;
+            ptx::fence_after_sync();
+            if (warp == 4 && lane == 0) EVLN_STAMP(60);
+            const float* sums = s_sum + (done & 1) * kParts * 128 + r_tile;
+            const float sum = (sums[0] + sums[128]) + (sums[256] + sums[384]);
+            const float inv = (sum > 0.f) ? 1.f / sum : 0.f;
+            const float ref = PERSIST ? s_done[(done & 1) * 128 + r_tile] : m_ref;
+            const float lse = (sum > 0.f) ? (ref + log2f(sum)) * 0.6931471805599453f : -INFINITY;
+            write_rows<PAGED, TAIL, PERSIST, LensT, CTAS>(a, lens, d, PERSIST ? item_of(done) : w, rank, quarter, part, inv, lse, t_o,
+                                                          smem_gen + Plan::kStageOff + (warp - 4) * Plan::kRowStageBytes, on_cta0(bar_o_free));
+            if (warp == 4 && lane == 0) EVLN_STAMP(61);
+        };
+        for (;;) {
+        set_rows();
         // The row's reference: the largest of its first 32 scores of the item's first tile (-inf: the
         // row sees no key of this split, since the visible keys of a row are a prefix).  The
         // thread that owns those columns reads it off and publishes it; nobody can ask for a new
         // reference before, so the other threads of the row simply wait for it.
-        if (part == 1 && ntiles > 0) {
+        if (rpart == 1) {
             // The other half of the first tile's group does not wait for the publisher: it reads the
             // same 32 scores itself (the buffer is not given back before all of the group's warps
             // have arrived) and gets the same maximum, ~1 K cycles before the published one could
             // reach it: the first product starts that much earlier.
-            ok = warp_wait(bar_s_full, 0, kDevTimeoutSoftmaxS, a.status, s_abort, lane);
+            ok = warp_wait(bar_s_full + 8 * grp, (first >> 1) & 1, kDevTimeoutSoftmaxS, a.status, s_abort, lane);
             if (ok) {
                 ptx::fence_after_sync();
-                int lim0 = bound - w.j0 * kTileN;
-                if (TAIL) lim0 = w.j0 < nct ? cache_last - w.j0 * kTileN : bound - (w.j0 - nct) * kTileN;
-                m_ref = first_block_reference(t_lane, lim0, a.scale_log2);
+                int lim0 = lim + 64;                       // (rpart 1: the second half of the first tile)
+                if (TAIL && first >= own_from) lim0 = bound - (first - own_from) * kTileN;
+                m_ref = first_block_reference(t_lane + (uint32_t)grp * 128, lim0, a.scale_log2);
             }
-        } else if (part != 0) {
-            ok = warp_wait(bar_ref + 8 * quarter, 0, kDevTimeoutSoftmaxX, a.status, s_abort, lane);
+        } else if (rpart != 0) {
+            ok = warp_wait(bar_ref + 8 * quarter, turn & 1, kDevTimeoutSoftmaxX, a.status, s_abort, lane);
             if (ok) m_ref = s_ref[r_tile];
         }
 
-        for (int jj = grp; jj < ntiles && ok; jj += 2) {
-            const uint32_t use = (uint32_t)(jj >> 1);           // how often this group's buffers were used before
+        for (int gj = first + rgrp; gj < last && ok; gj += 2) {
+            const uint32_t use = (uint32_t)(gj >> 1);           // how often this group's buffers were used before
             while (ok) {
-                const int r = (jj == 0 && part == 0)
-                                  ? (warp_wait(bar_s_full, 0, kDevTimeoutSoftmaxS, a.status, s_abort, lane) ? 0 : 2)
+                const int r = (gj == first && rpart == 0)
+                                  ? (warp_wait(bar_s_full + 8 * grp, use & 1, kDevTimeoutSoftmaxS, a.status, s_abort, lane) ? 0 : 2)
                                   : wait_or_request(bar_s_full + 8 * grp, use & 1, kDevTimeoutSoftmaxS);
                 if (r == 0) break;
-                ok = (r == 1) && move_reference(jj, false, 0.f);
+                ok = (r == 1) && move_reference(gj, false, 0.f);
             }
             if (!ok) break;
             ptx::fence_after_sync();
-            if (quarter == 0 && half == 0 && lane == 0 && jj < 9) EVLN_STAMP(2 + jj);
+            if (quarter == 0 && half == 0 && lane == 0 && gj < 9) EVLN_STAMP(2 + gj);
 
             // this thread's 64 scores of the row into registers; the score buffer goes back to the tensor core
             uint32_t s[64];
 #pragma unroll
             for (int blk = 0; blk < 2; ++blk) ptx::tmem_ld32(t_s + blk * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[blk * 32]));
             ptx::tmem_ld_wait();
-            if (quarter == 0 && half == 0 && lane == 0 && jj == 4) EVLN_STAMP(56);
+            if (quarter == 0 && half == 0 && lane == 0 && gj == 4) EVLN_STAMP(56);
             ptx::fence_before_sync();
             if (ptx::elect_one()) {
                 if (CTAS == 2) ptx::mbar_arrive_cluster(s_free0); else ptx::mbar_arrive(s_free0);
             }
 
-            // columns 0..lim of this thread's 64 are visible
-            int lim = bound - (w.j0 + jj) * kTileN - half * 64;
-            if (TAIL) {
-                const int j = w.j0 + jj;
-                lim = (j < nct ? cache_last - j * kTileN : bound - (j - nct) * kTileN) - half * 64;
-            }
-            if (!__all_sync(0xffffffffu, lim >= 63)) {
+            // columns 0..seen of this thread's 64 are visible
+            int seen = lim;
+            if (TAIL && gj >= own_from) seen = bound - (gj - own_from) * kTileN - half * 64;
+            lim -= 2 * kTileN;
+            if (!__all_sync(0xffffffffu, seen >= 63)) {
 #pragma unroll
-                for (int blk = 0; blk < 2; ++blk) mask32(&s[blk * 32], lim - blk * 32);   // -inf: masked keys (and stale slots) drop out
+                for (int blk = 0; blk < 2; ++blk) mask32(&s[blk * 32], seen - blk * 32);   // -inf: masked keys (and stale slots) drop out
             }
             float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
             rowmax32(&s[0], mx0, mx1, mx2, mx3);
-            if (jj == 0 && part == 0) {
+            if (gj == first && rpart == 0) {
                 m_ref = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * a.scale_log2;   // scale > 0
                 s_ref[r_tile] = m_ref;
                 __syncwarp();
@@ -921,14 +1110,14 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
             const float tmax = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * a.scale_log2;
             bool over = tmax > m_ref + kRefHeadroom;
             while (ok && __any_sync(0xffffffffu, over)) {
-                ok = move_reference(jj, over, tmax);
+                ok = move_reference(gj, over, tmax);
                 over = tmax > m_ref + kRefHeadroom;
             }
             if (!ok) break;
-            if (quarter == 0 && half == 0 && lane == 0 && jj == 4) EVLN_STAMP(57);
+            if (quarter == 0 && half == 0 && lane == 0 && gj == 4) EVLN_STAMP(57);
 
             // P = 2^(s*scale_log2 - m_ref) (packed FMA), row sum (packed add), bf16 P.  The P buffer is
-            // free once the product of tile jj - 2 has landed: this thread handed that tile over only a
+            // free once the product of tile gj - 2 has landed: this thread handed that tile over only a
             // moment ago, so it asks after the first block of exponentials, not before.
             const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
             const uint64_t negm2 = ptx::pack2(neg_m, neg_m);
@@ -936,13 +1125,13 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
             {
                 uint32_t pk[16];
                 exp32(&s[0], pk, scale2, negm2, sum2a, sum2b);
-                while (ok && jj >= 2) {
-                    const int r = wait_or_request(bar_pv_done + 8 * ((jj - 2) & 3), ((jj - 2) >> 2) & 1, kDevTimeoutSoftmaxO);
+                while (ok && gj >= 2) {
+                    const int r = wait_or_request(bar_pv_done + 8 * ((gj - 2) & 3), ((gj - 2) >> 2) & 1, kDevTimeoutSoftmaxO);
                     if (r == 0) break;
                     // (the meeting moves what is written and handed over; this block is still in
                     // registers, so it follows by the same power of two)
                     const float m_old = m_ref;
-                    ok = (r == 1) && move_reference(jj, false, 0.f);
+                    ok = (r == 1) && move_reference(gj, false, 0.f);
                     if (ok && m_ref != m_old) {
                         const float alpha = (m_old == -INFINITY) ? 0.f : ptx::ex2(m_old - m_ref);
 #pragma unroll
@@ -960,7 +1149,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
                 }
                 if (!ok) break;
                 ptx::fence_after_sync();
-                if (quarter == 0 && half == 0 && lane == 0 && jj == 4) EVLN_STAMP(58);
+                if (quarter == 0 && half == 0 && lane == 0 && gj == 4) EVLN_STAMP(58);
                 ptx::tmem_st16(t_p, pk);
             }
             {
@@ -977,97 +1166,46 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
                 ptx::unpack2(sum2b, b0, b1);
                 l += (a0 + a1) + (b0 + b1);
             }
-            if (quarter == 0 && half == 0 && lane == 0 && jj == 4) EVLN_STAMP(59);
+            if (quarter == 0 && half == 0 && lane == 0 && gj == 4) EVLN_STAMP(59);
             ptx::tmem_st_wait();
             ptx::fence_before_sync();
-            if (quarter == 0 && half == 0 && lane == 0 && jj == 4) EVLN_STAMP(63);
+            if (quarter == 0 && half == 0 && lane == 0 && gj == 4) EVLN_STAMP(63);
             if (ptx::elect_one()) {
                 if (CTAS == 2) ptx::mbar_arrive_cluster(p_full0); else ptx::mbar_arrive(p_full0);
             }
-            if (quarter == 0 && half == 0 && lane == 0 && jj < 9) EVLN_STAMP(11 + jj);
+            if (quarter == 0 && half == 0 && lane == 0 && gj < 9) EVLN_STAMP(11 + gj);
+            if (PERSIST && turn > 0 && gj < first + 2) flush(turn - 1);
         }
+        if (PERSIST && ok && turn > 0 && first + rgrp >= last) flush(turn - 1);      // (no tile for this warp's group)
 
         // All tiles handed over.  The row sum is the sum of the row's four threads (same reference in
         // all): they exchange it while the last product is still running.  A slower warp of the
         // quarter may still ask for a new reference until it arrives here too; a warp that serves such
         // a request after publishing its share publishes the rescaled share again (inside move_reference).
         if (ok) {
-            s_sum[part * 128 + r_tile] = l;
+            s_sum[((turn & 1) * kParts + part) * 128 + r_tile] = l;
+            if (PERSIST && part == 0) s_done[(turn & 1) * 128 + r_tile] = m_ref;
             sum_published = true;
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(bar_xch + 8 * quarter);
         }
         while (ok) {
-            const int r = wait_or_request(bar_xch + 8 * quarter, 0, kDevTimeoutSoftmaxX);
+            const int r = wait_or_request(bar_xch + 8 * quarter, turn & 1, kDevTimeoutSoftmaxX);
             if (r == 0) break;
-            ok = (r == 1) && move_reference(ntiles, false, 0.f);
+            ok = (r == 1) && move_reference(last, false, 0.f);
         }
-        // nobody of the quarter can ask any more; the last product
-        if (ok) ok = warp_wait(bar_o_full, 0, kDevTimeoutSoftmaxO, a.status, s_abort, lane);
-        if (ok) {
-            ptx::fence_after_sync();
-            if (warp == 4 && lane == 0) EVLN_STAMP(60);
-            l = (s_sum[r_tile] + s_sum[128 + r_tile]) + (s_sum[256 + r_tile] + s_sum[384 + r_tile]);
-            // Epilogue: O/l goes out through shared memory so that global stores are whole
-            // 128-byte lines.  The K ring is dead (its last consumer has completed); each warp
-            // stages its 32 rows x 32 channels there, rows 144 bytes apart.
-            const float inv = (l > 0.f) ? 1.f / l : 0.f;
-            const int wrow0 = quarter << 5;
-            uint8_t* stage = smem_gen + kSmemKOff + (warp - 4) * (32 * 144);
-            const int first_row = row0 + wrow0;                              // episode-local
-            const int rows_here = rows_valid - first_row;                    // may be <= 0 or > 32
-            const bool direct = CTAS == 2 && d.out != nullptr && !(TAIL && !w.visual && d.act_split);
-            uint32_t regs[32];
-            ptx::tmem_ld32(t_o, regs);
-            ptx::tmem_ld_wait();
-            if (direct) {
-                // the row's only work item: round once to the storage dtype and write the output itself
-                auto out_row = [&](int rl) -> long {           // row of [n, Hq, 128] of the item's row rl
-                    const int tok = (int)fast_div((uint32_t)rl, a.div_g);
-                    const long t = TAIL ? packed_row(w.visual ? d.map : d.act_map, (w.visual ? 0 : (long)lens.new_off[w.b]) + tok)
-                                        : PAGED ? (long)lens.new_off[w.b] + tok : (long)tok;
-                    return t * (a.Hkv * a.G) + w.g * a.G + (rl - tok * a.G);
-                };
-                uint4* srow = reinterpret_cast<uint4*>(stage + lane * 80);
-#pragma unroll
-                for (int e = 0; e < 32; e += 8) {
-                    uint32_t v[4];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        v[c] = ptx::pack_bf16x2(__uint_as_float(regs[e + 2 * c]) * inv, __uint_as_float(regs[e + 2 * c + 1]) * inv);
-                    srow[e >> 3] = make_uint4(v[0], v[1], v[2], v[3]);
-                }
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int r = i * 8 + (lane >> 2);
-                    if (r < rows_here)
-                        reinterpret_cast<uint4*>(d.out + out_row(first_row + r) * 128 + part * 32)[lane & 3] =
-                            *reinterpret_cast<const uint4*>(stage + r * 80 + (lane & 3) * 16);
-                }
-                if (d.lse_out && row_valid && part == 0)
-                    d.lse_out[out_row(r_local)] = (l > 0.f) ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
-            } else {
-                const long prow0 = ((long)w.slot * a.Hkv + w.g) * a.rows + w.row_base + first_row;
-                float* gbase = a.o_part + prow0 * 128 + part * 32;
-                float4* srow = reinterpret_cast<float4*>(stage + lane * 144);
-#pragma unroll
-                for (int e = 0; e < 32; e += 4)
-                    srow[e >> 2] = make_float4(__uint_as_float(regs[e]) * inv, __uint_as_float(regs[e + 1]) * inv,
-                                               __uint_as_float(regs[e + 2]) * inv, __uint_as_float(regs[e + 3]) * inv);
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int r = i * 4 + (lane >> 3);
-                    if (r < rows_here) {
-                        const float4 v = *reinterpret_cast<const float4*>(stage + r * 144 + (lane & 7) * 16);
-                        *reinterpret_cast<float4*>(gbase + (long)r * 128 + (lane & 7) * 4) = v;
-                    }
-                }
-                if (row_valid && part == 0)
-                    a.lse_part[prow0 + lane] = (l > 0.f) ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
-            }
-            if (warp == 4 && lane == 0) EVLN_STAMP(61);
+        // nobody of the quarter can ask any more
+        if (!ok) break;
+        if (!PERSIST) {
+            flush(0);
+            break;
+        }
+        first = last;
+        ++turn;
+        if (item_number(turn) >= d.num_items) {
+            flush(turn - 1);
+            break;
+        }
         }
     }
     }
@@ -1088,24 +1226,35 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
     }
 }
 
-// One CTA pair per work item (256 query rows): any number of rows, contiguous or paged cache.
-template <bool PAGED, typename LensT>
+// A CTA pair per work item (256 query rows) of one episode on a contiguous cache.
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                 const __grid_constant__ CUtensorMap tm_v, const TcAttnArgs a,
-                 const __grid_constant__ LensT lens, const __grid_constant__ TcOutArgs d)
+                 const __grid_constant__ CUtensorMap tm_v, const TcAttnArgs a, const __grid_constant__ NoLens lens,
+                 const __grid_constant__ TcOutArgs d)
 {
-    attn_tc_body<PAGED, false, LensT, 2>(tm_q, tm_k, tm_v, nullptr, nullptr, nullptr, a, lens, d);
+    attn_tc_body<false, false, false, NoLens, 2, NoTable>(tm_q, tm_k, tm_v, nullptr, nullptr, nullptr, a, lens, d, NoTable{});
 }
 
-// CTA pairs over a packed sequence (Sec. 3.3): the units of its visual run and its action chunks.
+// At most one CTA pair per two SMs, each going through several work items: more items than pairs on a
+// contiguous cache, or a batch of paged episodes.
+template <bool PAGED, typename LensT>
+__global__ void __launch_bounds__(kTcThreads, 1)
+attn_persistent_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                       const __grid_constant__ CUtensorMap tm_v, const TcAttnArgs a, const __grid_constant__ LensT lens,
+                       const __grid_constant__ TcOutArgs d, const __grid_constant__ ItemTable table)
+{
+    attn_tc_body<PAGED, false, true, LensT, 2, ItemTable>(tm_q, tm_k, tm_v, nullptr, nullptr, nullptr, a, lens, d, table);
+}
+
+// Persistent CTA pairs over a packed sequence (Sec. 3.3): the units of its visual run and its action chunks.
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_packed_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_qt,
                    const __grid_constant__ CUtensorMap tm_kt, const __grid_constant__ CUtensorMap tm_vt, const TcAttnArgs a,
-                   const __grid_constant__ BatchLens lens, const __grid_constant__ TcOutArgs d)
+                   const __grid_constant__ BatchLens lens, const __grid_constant__ TcOutArgs d,
+                   const __grid_constant__ ItemTable table)
 {
-    attn_tc_body<false, true, BatchLens, 2>(tm_q, tm_k, tm_v, &tm_qt, &tm_kt, &tm_vt, a, lens, d);
+    attn_tc_body<false, true, true, BatchLens, 2, ItemTable>(tm_q, tm_k, tm_v, &tm_qt, &tm_kt, &tm_vt, a, lens, d, table);
 }
 
 // One CTA per work item, for steps whose rows per kv head fit one 128-row tile (the few action
@@ -1115,7 +1264,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 attn_solo_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const TcAttnArgs a)
 {
-    attn_tc_body<false, false, NoLens, 1>(tm_q, tm_k, tm_v, nullptr, nullptr, nullptr, a, NoLens{}, TcOutArgs{});
+    attn_tc_body<false, false, false, NoLens, 1, NoTable>(tm_q, tm_k, tm_v, nullptr, nullptr, nullptr, a, NoLens{}, TcOutArgs{}, NoTable{});
 }
 
 }  // namespace evln

@@ -136,7 +136,7 @@ combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
     }
     const float inv = (wsum > 0.f) ? 1.f / wsum : 0.f;
 
-    const long tok = packed_row(a.map, (long)row_tok);
+    const long tok = packed_row(a.map, (int)row_tok);
     const int h = g * a.G + row_head;
     const int Hq = a.Hkv * a.G;
     T* dst = (T*)a.out + (tok * Hq + h) * D + lane * C;

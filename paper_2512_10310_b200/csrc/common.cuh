@@ -40,6 +40,15 @@ struct PagedLens : BatchLens {
     unsigned char order[kMaxBatch];
 };
 
+// Work items of a persistent launch by pair: entry turn * pairs + pair, kNoItem where a pair has no more.
+constexpr int kTableItems = 1024;
+constexpr int kNoItem = 0xffff;
+struct ItemTable {
+    int count;                         // entries, 0: no table
+    unsigned short item[kTableItems];
+};
+struct NoTable {};
+
 template <typename T> struct VecTraits;
 template <> struct VecTraits<__nv_bfloat16> { static constexpr int kVec = 8; };
 template <> struct VecTraits<float> { static constexpr int kVec = 4; };
@@ -111,16 +120,22 @@ __host__ __device__ inline int tail_kv_tiles_fast(int L, int n, FastDiv div_g, i
 
 // Where token m of a dense run of tokens sits in a PACKED sequence I, v_1, a_1, ..., v_N, a_N
 // (Sec. 3.3): `action` = 0 maps the run instruction + visual tokens, 1 the run of action tokens.
-// F = 0 means "not packed": the identity.
+// F = A = 0 means "not packed": the identity.
 struct PackedMap {
     int I, F, A, action;
+    FastDiv div;             // by A (action) or F
 };
-__host__ __device__ inline long packed_row(const PackedMap& pm, long m)
+inline PackedMap make_packed_map(int I, int F, int A, int action)
+{
+    const int by = action ? A : F;
+    return PackedMap{I, F, A, action, make_fast_div((uint32_t)(by > 0 ? by : 1))};
+}
+__device__ __forceinline__ int packed_row(const PackedMap& pm, int m)
 {
     if (pm.F <= 0 && pm.A <= 0) return m;
-    if (pm.action) return pm.I + (m / pm.A) * (long)(pm.F + pm.A) + pm.F + m % pm.A;
+    if (pm.action) return pm.I + m + ((int)fast_div((uint32_t)m, pm.div) + 1) * pm.F;
     if (m < pm.I || pm.F <= 0) return m;
-    return pm.I + ((m - pm.I) / pm.F) * (long)(pm.F + pm.A) + (m - pm.I) % pm.F;
+    return m + (int)fast_div((uint32_t)(m - pm.I), pm.div) * pm.A;
 }
 
 // Stub lengths for the kernels that serve one episode.

@@ -113,10 +113,11 @@ cudaError_t prepare_few()
 // Shared-memory limits of the kernels that take more than the default, on the current device.
 cudaError_t prepare_kernels()
 {
-    const std::pair<const void*, int> tc[4] = {{(const void*)attn_pair_kernel<false, NoLens>, kTcSmemBytes},
-                                               {(const void*)attn_pair_kernel<true, PagedLens>, kTcSmemBytes},
+    const std::pair<const void*, int> tc[5] = {{(const void*)attn_pair_kernel, kTcSmemBytes},
+                                               {(const void*)attn_persistent_kernel<false, NoLens>, kPersistSmemBytes},
+                                               {(const void*)attn_persistent_kernel<true, PagedLens>, kPersistSmemBytes},
                                                {(const void*)attn_solo_kernel, kSoloSmemBytes},
-                                               {(const void*)attn_packed_kernel, kTcSmemBytes}};
+                                               {(const void*)attn_packed_kernel, kPersistSmemBytes}};
     for (const auto& k : tc) {
         cudaError_t e = cudaFuncSetAttribute(k.first, cudaFuncAttributeMaxDynamicSharedMemorySize, k.second);
         if (e != cudaSuccess) return e;
@@ -140,7 +141,7 @@ cudaError_t prepare_kernels()
 bool attention_register_pool_ok()
 {
     cudaFuncAttributes fa;
-    const void* kernels[4] = {(const void*)attn_pair_kernel<false, NoLens>, (const void*)attn_pair_kernel<true, PagedLens>,
+    const void* kernels[5] = {(const void*)attn_pair_kernel, (const void*)attn_persistent_kernel<false, NoLens>, (const void*)attn_persistent_kernel<true, PagedLens>,
                               (const void*)attn_solo_kernel, (const void*)attn_packed_kernel};
     for (const void* k : kernels) {
         if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return false;
@@ -447,7 +448,7 @@ void longest_first(int batch, const int* lens, const int* offs, int* order)
 // episodes in the order given, items of at most `chunk` tiles.  The pairs are kept as runs of equal load
 // (ascending), so an episode costs a few steps however many items it has.
 constexpr int kMaxPairs = 128;
-constexpr double kItemTiles = 10.0;      // an item's launch, set-up, first tile and write-out, in KV tiles (measured)
+constexpr int kNextItemTiles = 5;        // from a pair's last product of an item to the first of its next one, in KV tiles
 double finish_time(int pairs, int G, int Hkv, int batch, const int* lens, const int* offs, const int* order, int chunk)
 {
     struct Run { double load; int count; } runs[kMaxPairs];
@@ -458,7 +459,7 @@ double finish_time(int pairs, int G, int Hkv, int batch, const int* lens, const 
         if (n == 0) continue;
         const int units = ceil_div(n * G, kUnitRows);
         const int nkv = unit_kv_tiles(lens[b], n, G, units - 1, kUnitRows), splits = ceil_div(nkv, chunk);
-        const double cost = (double)nkv / splits + kItemTiles;
+        const double cost = (double)nkv / splits + kNextItemTiles;
         for (long left = (long)units * Hkv * splits; left > 0;) {
             const int take = left < runs[0].count ? (int)left : runs[0].count;
             const double load = runs[0].load + cost;
@@ -652,6 +653,68 @@ template <typename T, bool PAGED, typename LensT>
 void launch_rope_append(const RopeArgs& a, int tokens, cudaStream_t st, const LensT& lens)
 {
     launch_pdl(rope_append_kernel<T, PAGED, LensT>, dim3(tokens), rope_block(a), 0, st, a, lens);
+}
+
+// CTA pairs of a persistent launch: one per two SMs, no more than there are items.
+inline unsigned persistent_pairs(evlnHandle_t h, long items)
+{
+    const long pairs = h->num_sms / 2 > 0 ? h->num_sms / 2 : 1;
+    return (unsigned)(items < pairs ? items : pairs);
+}
+
+// Gives every work item, longest first, to the pair that is done first so far.  next() returns the items in that
+// order with their KV tiles; false: no table (one item per pair, or more than the table holds).
+struct CostedItem {
+    int number, tiles;
+};
+template <typename Next>
+bool assign_items(int pairs, long items, Next&& next, ItemTable* table)
+{
+    table->count = 0;
+    if (items <= pairs || items > kTableItems - pairs || pairs > kMaxPairs) return false;
+    struct Load { int tiles, pair; } heap[kMaxPairs];         // the least loaded pair on top
+    int turns[kMaxPairs];
+    for (int i = 0; i < pairs; ++i) { heap[i] = Load{0, i}; turns[i] = 0; }
+    memset(table->item, 0xff, sizeof(table->item));
+    int count = 0;
+    for (long k = 0; k < items; ++k) {
+        const CostedItem it = next();
+        Load l = heap[0];
+        const int at = turns[l.pair]++ * pairs + l.pair;
+        if (at >= kTableItems || turns[l.pair] > kPairItems) return false;
+        table->item[at] = (unsigned short)it.number;
+        if (at >= count) count = at + 1;
+        l.tiles += it.tiles + kNextItemTiles;
+        int i = 0;
+        for (int c; (c = 2 * i + 1) < pairs; i = c) {
+            if (c + 1 < pairs && heap[c + 1].tiles < heap[c].tiles) ++c;
+            if (heap[c].tiles >= l.tiles) break;
+            heap[i] = heap[c];
+        }
+        heap[i] = l;
+    }
+    table->count = count;
+    return true;
+}
+
+// Launches a persistent kernel on `items` work items (several times when a pair would get more than it keeps).
+template <typename Launch>
+evlnStatus_t launch_persistent(evlnHandle_t h, long items, TcOutArgs& d, const ItemTable& table, Launch&& launch)
+{
+    if (table.count > 0) {
+        d.first_item = 0;
+        d.num_items = (int)items;
+        cudaError_t e = launch(dim3(2 * persistent_pairs(h, items)));
+        return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
+    }
+    const long most = (long)persistent_pairs(h, items) * kPairItems;
+    for (long first = 0; first < items; first += most) {
+        d.first_item = (int)first;
+        d.num_items = (int)(first + most < items ? first + most : items);
+        cudaError_t e = launch(dim3(2 * persistent_pairs(h, d.num_items - first)));
+        if (e != cudaSuccess) return cuda_fail(h, e);
+    }
+    return EVLN_OK;
 }
 
 // What the one-launch step adds to an attention call: the new tokens and where the results go (out null:
@@ -1001,8 +1064,21 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
                 d.lse_out = direct ? direct->lse_out : lse_part;
                 if (direct) direct->done = true;
             }
-            launch_pair_pdl(attn_pair_kernel<false, NoLens>, dim3(2 * p->num_kv_heads, a.units_per_head, S), kTcSmemBytes, st,
-                            tm_q, tm_k, tm_v, a, nl, d);
+            const long items = (long)p->num_kv_heads * a.units_per_head * S;
+            if (items > persistent_pairs(h, items) && items <= 0x3fffffffL) {
+                d.div_hkv = make_fast_div((uint32_t)p->num_kv_heads);
+                d.div_units = make_fast_div((uint32_t)a.units_per_head);
+                ItemTable table;
+                int k = 0;
+                assign_items((int)persistent_pairs(h, items), items, [&]() -> CostedItem {
+                    const int unit = a.units_per_head - 1 - k / a.Hkv % a.units_per_head;
+                    return CostedItem{k++, unit_kv_tiles(p->cache_len, p->num_new, G, unit, kUnitRows) / S};
+                }, &table);
+                return launch_persistent(h, items, d, table, [&](dim3 grid) {
+                    return launch_pair_pdl(attn_persistent_kernel<false, NoLens>, grid, kPersistSmemBytes, st, tm_q, tm_k, tm_v, a, nl, d, table);
+                });
+            }
+            launch_pair_pdl(attn_pair_kernel, dim3(2 * p->num_kv_heads, a.units_per_head, S), kTcSmemBytes, st, tm_q, tm_k, tm_v, a, nl, d);
         }
     } else {
         SimtAttnArgs a = {};
@@ -1228,10 +1304,17 @@ evlnStatus_t evlnPagedStepAttention(evlnHandle_t h, const evlnPagedParams* p, co
         d.out = (__nv_bfloat16*)workspace;
         d.lse_out = a.lse_part;
     }
-    launch_pair_pdl(attn_pair_kernel<true, PagedLens>, dim3(2 * (int)items), kTcSmemBytes, (cudaStream_t)stream, tm_q, tm_k,
-                    tm_v, a, bl, d);
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
+    ItemTable table;
+    int k = 0, place = 0;
+    assign_items((int)persistent_pairs(h, items), items, [&]() -> CostedItem {
+        while (bl.item_off[place + 1] <= k) ++place;
+        const int b = bl.order[place], n = h_new_offsets[b + 1] - h_new_offsets[b];
+        const int nkv = unit_kv_tiles(h_cache_lens[b], n, G, ceil_div(n * G, kUnitRows) - 1, kUnitRows);
+        return CostedItem{k++, nkv / ceil_div(nkv, chunk)};
+    }, &table);
+    return launch_persistent(h, items, d, table, [&](dim3 grid) {
+        return launch_pair_pdl(attn_persistent_kernel<true, PagedLens>, grid, kPersistSmemBytes, (cudaStream_t)stream, tm_q, tm_k, tm_v, a, bl, d, table);
+    });
 }
 
 evlnStatus_t evlnPagedStepCombine(evlnHandle_t h, const evlnPagedParams* p, const void* workspace,
@@ -1430,13 +1513,29 @@ extern "C" evlnStatus_t evlnPackedForward(evlnHandle_t h, const evlnPackedParams
         a.div_s = make_fast_div(1u);
         TcOutArgs d = {};
         d.out = (__nv_bfloat16*)out; d.lse_out = lse_out;
-        d.map = PackedMap{p->instr_len, p->frame_tokens, p->action_tokens, 0};
+        d.map = make_packed_map(p->instr_len, p->frame_tokens, p->action_tokens, 0);
         d.act_items = (int)pl.items; d.act_split = split;
-        d.act_map = PackedMap{p->instr_len, p->frame_tokens, p->action_tokens, 1};
+        d.act_map = make_packed_map(p->instr_len, p->frame_tokens, p->action_tokens, 1);
         d.div_hkv = make_fast_div((uint32_t)p->num_kv_heads);
-        cudaError_t e = launch_pair_pdl(attn_packed_kernel, dim3(2 * (unsigned)(pl.items + (long)a.units_per_head * p->num_kv_heads)),
-                                        kTcSmemBytes, st, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], a, bl, d);
-        if (e != cudaSuccess) return cuda_fail(h, e);
+        // both runs of items come longest first: merge them
+        const long items = pl.items + (long)a.units_per_head * p->num_kv_heads;
+        ItemTable table;
+        int act = 0, vis = 0, chunk_of = p->num_frames - 1;
+        assign_items((int)persistent_pairs(h, items), items, [&]() -> CostedItem {
+            int act_tiles = -1, vis_tiles = -1;
+            if (act < (int)pl.items) {
+                while (bl.item_off[chunk_of] > (int)pl.items - 1 - act) --chunk_of;
+                const int nkv = tail_kv_tiles(pl.lens[chunk_of], p->action_tokens, G, 0, kUnitRows);
+                act_tiles = nkv / ceil_div(nkv, pl.chunk);
+            }
+            if (vis < a.units_per_head * a.Hkv) vis_tiles = unit_kv_tiles(0, pl.n_vis, G, a.units_per_head - 1 - vis / a.Hkv, kUnitRows);
+            if (act_tiles >= vis_tiles) return CostedItem{act++, act_tiles};
+            return CostedItem{(int)pl.items + vis++, vis_tiles};
+        }, &table);
+        s = launch_persistent(h, items, d, table, [&](dim3 grid) {
+            return launch_pair_pdl(attn_packed_kernel, grid, kPersistSmemBytes, st, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], a, bl, d, table);
+        });
+        if (s != EVLN_OK) return s;
     }
     if (!split) return EVLN_OK;
     CombineArgs c = {};
@@ -1446,7 +1545,7 @@ extern "C" evlnStatus_t evlnPackedForward(evlnHandle_t h, const evlnPackedParams
     c.Hkv = p->num_kv_heads; c.G = G; c.D = 128; c.rows = (int)rows_a; c.num_splits = pl.smax;
     c.batch = p->num_frames; c.unit_rows = kUnitRows; c.chunk_tiles = pl.chunk;
     c.tail = 1;
-    c.map = PackedMap{p->instr_len, p->frame_tokens, p->action_tokens, 1};
+    c.map = make_packed_map(p->instr_len, p->frame_tokens, p->action_tokens, 1);
     return launch_combine<__nv_bfloat16>(h, c, 128, true, &bl, st);
 }
 
