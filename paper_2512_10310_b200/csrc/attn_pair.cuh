@@ -70,7 +70,8 @@ struct SmemPlan {
     // in an area of their own when the ring already holds the next item's keys.
     static constexpr int kRowStageBytes = PERSIST ? 8 * 144 + 128 : 32 * 144;
     static constexpr int kKStages = CTAS == 2 ? 5 : 3;
-    static constexpr int kVStages = CTAS == 2 ? 5 : 2;
+    // (persistent: a shallower V ring leaves the L1 cache 20 KB for the few registers that kernel spills)
+    static constexpr int kVStages = CTAS == 2 ? (PERSIST ? 4 : 5) : 2;
     static constexpr int kStageBytes = CTAS == 2 ? kHalfBytes : kTileBytes;
     static constexpr int kQOff = 0;
     static constexpr int kKOff = kTileBytes;
@@ -292,10 +293,10 @@ struct __align__(16) WorkItem {
     bool visual;              // packed sequence: a unit of the visual run (else an action chunk's)
 };
 
-// Contiguous cache: the grid is (CTAS * kv heads, units, splits), so a CTA reads its work item off
-// its block index; the two divisions left (by G and by the split count) are multiplications by
-// constants the host prepared.  Units are taken from the last one down: where they do not all fit the
-// chip at once (a prefill), the ones with most keys start first and the last round is short.
+// Contiguous cache: the grid is (CTAS * units, kv heads, splits), so a CTA reads its work item off its
+// block index and neighbouring pairs read the same keys (kv heads first was 1 % slower at 26 K keys of 8
+// kv heads); the divisions left (by G and by the split count) are multiplications by constants the host
+// prepared.  Persistent pairs: items count kv heads first, then units from the last one (most keys) down.
 // Batches (paged cache, action chunks of a packed sequence): items are numbered episode by episode (kv
 // head, unit, split inside), the host passes the first item of every episode and the CTA searches that
 // table.
@@ -313,8 +314,8 @@ __device__ __forceinline__ WorkItem decode_work(const TcAttnArgs& a, const LensT
             w.g = item - (int)su * a.Hkv;
             w.slot = (int)slot;
         } else {
-            w.unit = (int)(gridDim.y - 1 - blockIdx.y);
-            w.g = CTAS == 2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+            w.unit = CTAS == 2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+            w.g = (int)blockIdx.y;
             w.slot = (int)blockIdx.z;
         }
         w.visual = true;

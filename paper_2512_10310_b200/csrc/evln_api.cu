@@ -1054,9 +1054,9 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
         a.div_s = make_fast_div((uint32_t)S);
         NoLens nl = {};
         // one work item per (unit, kv head, split): the kernels read it off the block index
-        if (a.units_per_head > 65535 || p->num_kv_heads > 65535) return EVLN_NOT_SUPPORTED;
+        if (p->num_kv_heads > 65535) return EVLN_NOT_SUPPORTED;
         if (use_solo_kernel(p)) {
-            launch_pdl(attn_solo_kernel, dim3(p->num_kv_heads, 1, S), dim3(kTcThreads), kSoloSmemBytes, st, tm_q, tm_k, tm_v, a);
+            launch_pdl(attn_solo_kernel, dim3(1, p->num_kv_heads, S), dim3(kTcThreads), kSoloSmemBytes, st, tm_q, tm_k, tm_v, a);
         } else {
             TcOutArgs d = {};
             if (S == 1) {                          // final rows: to the caller, or for the combine call to copy
@@ -1065,7 +1065,11 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
                 if (direct) direct->done = true;
             }
             const long items = (long)p->num_kv_heads * a.units_per_head * S;
-            if (items > persistent_pairs(h, items) && items <= 0x3fffffffL) {
+            // More items than pairs: persistent pairs where items are short (a prefill).  From about 32 KV tiles per
+            // item on, what the boundaries save is lost to the spills of that kernel's tile loop (140 items of 78
+            // tiles: 168 us against 158; 112 items of up to 8: 22.6 against 25.3).
+            const int tiles = unit_kv_tiles(p->cache_len, p->num_new, G, a.units_per_head - 1, kUnitRows) / S;
+            if (items > persistent_pairs(h, items) && tiles <= 32 && items <= 0x3fffffffL) {
                 d.div_hkv = make_fast_div((uint32_t)p->num_kv_heads);
                 d.div_units = make_fast_div((uint32_t)a.units_per_head);
                 ItemTable table;
@@ -1078,7 +1082,7 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
                     return launch_pair_pdl(attn_persistent_kernel<false, NoLens>, grid, kPersistSmemBytes, st, tm_q, tm_k, tm_v, a, nl, d, table);
                 });
             }
-            launch_pair_pdl(attn_pair_kernel, dim3(2 * p->num_kv_heads, a.units_per_head, S), kTcSmemBytes, st, tm_q, tm_k, tm_v, a, nl, d);
+            launch_pair_pdl(attn_pair_kernel, dim3(2 * a.units_per_head, p->num_kv_heads, S), kTcSmemBytes, st, tm_q, tm_k, tm_v, a, nl, d);
         }
     } else {
         SimtAttnArgs a = {};
