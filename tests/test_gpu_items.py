@@ -1,0 +1,42 @@
+"""Paged batches at the edges of how the persistent attention launch deals work items to CTA pairs,
+against the oracle."""
+import dataclasses
+
+import pytest
+import torch
+
+from oracle import step_oracle as so
+from paper_2512_10310_b200 import binding as B
+from paper_2512_10310_b200 import workloads as W
+from tests.helpers import check_output, f64
+from tests.test_gpu_paged import _check_pools, _gpu_paged
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def handle():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    h = B.evlnCreate(0)
+    yield h
+    B.evlnDestroy(h)
+
+
+@pytest.mark.parametrize("batch", [
+    4,       # 64 work items: fewer than SM pairs
+    20,      # 320: dealt to the pairs by the item table
+    64,      # 1024: more than the table holds, dealt in turn
+    160,     # 2560: more than the pairs keep, two launches
+])
+def test_paged_batch_of_many_work_items(handle, batch):
+    # one query head per kv head and 33 tokens: one unit per (episode, kv head) for the tile kernel
+    cfg = dataclasses.replace(W.PAGED_B16, name=f"many_{batch}", num_q_heads=16, num_kv_heads=16, batch=batch, seed=90 + batch)
+    lens = [(37 * b) % 301 for b in range(batch)]
+    x = W.make_paged_inputs(cfg, lens, [33] * batch)
+    out, lse, k_pool, v_pool = _gpu_paged(handle, cfg, x)
+    okp, ovp = f64(x["k_pool"]), f64(x["v_pool"])
+    ref_out, ref_lse = so.step_paged(f64(x["q_new"]), f64(x["k_new"]), f64(x["v_new"]), okp, ovp, x["page_table"], lens,
+                                     x["new_offsets"], cfg.rope_theta, storage="bf16")
+    check_output("bf16", out, lse, ref_out, ref_lse)
+    _check_pools(x, cfg, k_pool, v_pool, okp, ovp)
