@@ -642,17 +642,21 @@ void finish_rope_args(RopeArgs* a, int vec)
 }
 
 // The append kernels: a block per token, one thread per work item of it.
-dim3 rope_block(const RopeArgs& a)
+inline int rope_items(const RopeArgs& a) { return ((a.Hq + a.Hkv) << a.vph_shift) + (a.Hkv << (a.vph_shift + 1)); }
+dim3 rope_block(int items)
 {
-    const int items = ((a.Hq + a.Hkv) << a.vph_shift) + (a.Hkv << (a.vph_shift + 1));
     const int t = (items + 31) / 32 * 32;
     return dim3(t > kRopeThreadsMax ? kRopeThreadsMax : t < 64 ? 64 : t);
 }
 
+// Few tokens with more work items than a block has threads (64 query heads): several blocks per token, so that
+// no thread starts its second item after its first.  Many tokens fill the SMs as they are, and every block of a
+// token computes all of its angles.
 template <typename T, bool PAGED, typename LensT>
 void launch_rope_append(const RopeArgs& a, int tokens, cudaStream_t st, const LensT& lens)
 {
-    launch_pdl(rope_append_kernel<T, PAGED, LensT>, dim3(tokens), rope_block(a), 0, st, a, lens);
+    const int items = rope_items(a), parts = tokens <= kRopeFewTokens ? ceil_div(items, kRopeThreadsMax) : 1;
+    launch_pdl(rope_append_kernel<T, PAGED, LensT>, dim3(tokens + (PAGED ? a.batch : 0), parts), rope_block(ceil_div(items, parts)), 0, st, a, lens);
 }
 
 // CTA pairs of a persistent launch: one per two SMs, no more than there are items.
@@ -1481,7 +1485,7 @@ extern "C" evlnStatus_t evlnPackedForward(evlnHandle_t h, const evlnPackedParams
         a.div_f = make_fast_div((uint32_t)(p->frame_tokens > 0 ? p->frame_tokens : 1));
         a.div_a = make_fast_div((uint32_t)(p->action_tokens > 0 ? p->action_tokens : 1));
         a.q_rot_act = ws + pl.off_qa; a.k_act = ws + pl.off_tk; a.v_act = ws + pl.off_tv;
-        cudaError_t e = launch_pdl(rope_packed_kernel, dim3(a.r.num_new), rope_block(a.r), 0, st, a);
+        cudaError_t e = launch_pdl(rope_packed_kernel, dim3(a.r.num_new), rope_block(rope_items(a.r)), 0, st, a);
         if (e != cudaSuccess) return cuda_fail(h, e);
     }
     // one launch: the visual run as one causal prefill (its query tiles never load a KV tile past their own

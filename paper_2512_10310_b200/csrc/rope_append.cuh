@@ -171,6 +171,7 @@ rope_table_kernel(double2* table, int first_pos, int count, int D, double log2_t
 // several tokens and prefetch the next one's vectors were measured slower, 10.3 against 9.8 us for 2048
 // tokens and 19 against 17.6 for 3136 paged ones: what counts is warps, i.e. registers.)
 constexpr int kRopeThreadsMax = 448;
+constexpr int kRopeFewTokens = 256;      // (64 query heads: 8 tokens 27.2 us a step, 25.7 with two blocks each; 256 tokens 38.7 and 37.3)
 
 // Where one new token comes from and goes to.
 struct TokenPlace {
@@ -188,10 +189,10 @@ struct TokenRun {
     long q_rows, kv_rows;
 };
 
-// Rotates and stores token blockIdx.x with the whole block.  place(token, t) fills in the token's place and
-// returns its position, run(t) says which buffers it goes to, done(token, t) follows its stores.
-template <typename T, typename Place, typename Run, typename Done>
-__device__ __forceinline__ void rope_token(const RopeArgs& a, Place&& place, Run&& run, Done&& done)
+// Rotates and stores token blockIdx.x with the whole block (gridDim.y > 1: a share of its work items).  place(token, t) fills in the token's place and
+// returns its position, run(t) says which buffers it goes to.
+template <typename T, typename Place, typename Run>
+__device__ __forceinline__ void rope_token(const RopeArgs& a, Place&& place, Run&& run)
 {
     constexpr int V = VecTraits<T>::kVec;
     typedef typename Rotation<T>::Angle Angle;
@@ -258,15 +259,15 @@ __device__ __forceinline__ void rope_token(const RopeArgs& a, Place&& place, Run
     TokenPlace t;
     const long pos = place(tok, t);
     uint4 r0 = make_uint4(0u, 0u, 0u, 0u), r1 = r0;
-    if (j < items) load_item(t, j, r0, r1);           // in flight while the angles arrive
+    const int first = j + (int)(blockIdx.y * blockDim.x);
+    if (first < items) load_item(t, first, r0, r1);   // in flight while the angles arrive
     if (j < half) Rotation<T>::put(s_angle, j, angle_of(pos));
     __syncthreads();
-    if (j < items) finish_item(t, s_angle, j, r0, r1);
-    for (int it = j + blockDim.x; it < items; it += blockDim.x) {
+    if (first < items) finish_item(t, s_angle, first, r0, r1);
+    for (int it = first + (int)(gridDim.y * blockDim.x); it < items; it += (int)(gridDim.y * blockDim.x)) {
         load_item(t, it, r0, r1);
         finish_item(t, s_angle, it, r0, r1);
     }
-    done(tok, t);
 }
 
 template <typename T, bool PAGED, typename LensT>
@@ -276,6 +277,23 @@ rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
     constexpr int V = VecTraits<T>::kVec;
     const int D = a.D;
     int b = 0;                                    // the token's episode
+    if (PAGED && (int)blockIdx.x >= a.num_new) {
+        // An episode's last page is only partly filled: clear the value slots behind its last token so that a
+        // tile load of the whole page never brings in stale bits.  (A block per episode: behind the stores of
+        // the last token's block it was the longest chain of the launch, 4.65 us for 16 episodes of one token.)
+        b = blockIdx.x - a.num_new;
+        const int len = lens.cache_len[b] + lens.new_off[b + 1] - lens.new_off[b], used = len & (a.page_size - 1);
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (lens.new_off[b + 1] == lens.new_off[b] || used == 0) return;
+        const long row = (long)a.page_table[(long)b * a.max_pages + (len >> a.page_shift)] * a.Hkv * a.page_size + used;
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        for (int g = blockIdx.y; g < a.Hkv; g += gridDim.y) {
+            uint4* dst = reinterpret_cast<uint4*>((T*)a.v_cache + (row + (long)g * a.page_size) * D);
+            for (int it = threadIdx.x; it < (a.page_size - used) * (D / V); it += blockDim.x) dst[it] = zero;
+        }
+        return;
+    }
     if (PAGED) {
         int hi = a.batch;                         // largest b with new_off[b] <= tok
         while (hi - b > 1) {
@@ -297,23 +315,7 @@ rope_append_kernel(const RopeArgs a, const __grid_constant__ LensT lens)
     auto run = [&](const TokenPlace&) -> TokenRun<T> {
         return {(T*)a.q_rot, (T*)a.k_cache, (T*)a.v_cache, (long)a.num_new * a.G, PAGED ? (long)a.page_size : (long)a.cache_cap};
     };
-    rope_token<T>(a, place, run, [&](int tok, const TokenPlace& t) {
-        if (!PAGED) return;
-        if (tok + 1 != lens.new_off[t.episode + 1]) return;
-        const int slot = (lens.cache_len[t.episode] + tok - lens.new_off[t.episode]) & (a.page_size - 1);
-        if (slot + 1 >= a.page_size) return;
-        // the episode's last page is only partly filled: clear the value slots behind the last
-        // token so that a tile load of the whole page never brings in stale bits
-        const int tail = a.page_size - (slot + 1);
-        const int vec_per_row = D / V;
-        const int total = a.Hkv * tail * vec_per_row;
-        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-        for (int it = threadIdx.x; it < total; it += blockDim.x) {
-            const int g = it / (tail * vec_per_row);
-            const int r = it % (tail * vec_per_row);
-            *reinterpret_cast<uint4*>((T*)a.v_cache + (t.kv_row + (long)g * a.page_size + 1 + r / vec_per_row) * D + (r % vec_per_row) * V) = zero;
-        }
-    });
+    rope_token<T>(a, place, run);
 }
 
 // The tokens of a packed sequence I, v_1, a_1, ..., v_N, a_N in one launch (Sec. 3.3): the instruction and
@@ -357,7 +359,7 @@ rope_packed_kernel(const RopePackedArgs p)
         if (t.episode) return {(T*)p.q_rot_act, (T*)p.k_act, (T*)p.v_act, (long)p.num_action * a.G, p.num_action};
         return {(T*)a.q_rot, (T*)a.k_cache, (T*)a.v_cache, (long)p.num_visual * a.G, a.cache_cap};
     };
-    rope_token<T>(a, place, run, [](int, const TokenPlace&) {});
+    rope_token<T>(a, place, run);
 }
 
 }  // namespace evln
