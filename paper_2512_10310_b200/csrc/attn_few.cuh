@@ -10,7 +10,11 @@
 // 16 KB, TMA, 128-byte swizzle; a 64-token page is exactly one stage).  With MT 16-row tiles of queries
 // (1 or 2), four warps share a stage (16 MT keys x 16 rows each) and the two groups of four take the stages
 // in turn; every warp keeps a running maximum, sum and output of its own.
-// The warps' results are merged in shared memory; contiguous caches spread a kv head's keys over a
+// The warps' results are merged in shared memory.  Paged: one block per SM, each with an equal share of the
+// batch's stages, walked in episode order; a share goes through the ends of units (episode, kv head) with the
+// ring running on, and a unit is split where the shares meet.  (One block per work item of a quarter of an
+// SM's share, until then: 16 ragged episodes of one token 61.6 us, 8 episodes of up to 4096 tokens 22.4.  Items
+// in whole numbers left SMs idle at the end, and every item paid a start of about 3 us.)  Contiguous caches spread a kv head's keys over a
 // cluster of up to 16 blocks, which send each row to the block that merges it (distributed shared memory,
 // st.async on that block's barrier: one way, no cluster-wide meeting at the end), so that a whole
 // step leaves one (normalised) result per head, or per split when the caller asks for splits.
@@ -34,7 +38,6 @@ constexpr int kFewRows = 32;                  // most packed query rows per kv h
 constexpr int kFewFusedTokens = 16;           // most new tokens of a fused step
 constexpr int kFewWarps = 8;                  // compute warps
 constexpr int kFewThreads = 32 * (kFewWarps + 1);
-constexpr int kFewKeys = 64;                  // keys per stage
 constexpr int kFewStageBytes = 2 * kFewKeys * 256;
 constexpr int kFewGroups = 2;                 // groups of warps that take the stages in turn
 // Ring depth: a multiple of the number of groups, so that a slot is always consumed by the same group.
@@ -43,6 +46,9 @@ constexpr int kFewGroups = 2;                 // groups of warps that take the s
 // 64 blocks need to draw the full HBM rate (with four, 71 GB/s per SM).
 constexpr int kFewMaxStages = 6, kFewMinStages = 4;
 static_assert(kFewMaxStages % kFewGroups == 0 && kFewMinStages % kFewGroups == 0, "a slot belongs to one group");
+// Paged: four, beside them the warps' outputs have a place of their own, so that the ring goes on filling while a
+// unit's results are merged.  148 blocks draw the full HBM rate with half of that.
+constexpr int kFewPagedStages = 4;
 constexpr int kFewMaxCluster = 16;
 constexpr int kFewOStride = 132;              // floats per row of a warp's output in shared memory
 
@@ -58,6 +64,8 @@ struct FewArgs {
     int num_splits;           // contiguous only
     int stages;               // ring depth
     int batch, max_pages, chunk_tiles;   // paged only
+    int share;                // paged only: stages per block, 0: work items of chunk_tiles tiles
+    FastDiv div_share;
     float scale_log2;         // softmax scale * log2(e)
     FastDiv div_g;            // division by G
     // contiguous only: the cache, for prefetches into L2 and for the fused append
@@ -79,12 +87,13 @@ struct FewArgs {
 
 // Shared memory, from a 1024-byte boundary: stages | Q [16 MT][256 B] | barriers | weights | rows the cluster's
 // blocks send here | fused: angles, new K/V rows.  After the last stage has been consumed the ring holds
-// the warps' outputs.
+// the warps' outputs (paged: they lie behind the weights).
 constexpr int kFewBarBytes = 256;
 constexpr int kFewStatBytes = 2 * kFewWarps * kFewRows * 4;
 constexpr int kFewRowBytes = kFewOStride * 4;           // a row in flight: 128 channels, reference, sum
 constexpr int kFewAngleBytes = Rotation<__nv_bfloat16>::kAngles * 16;
 constexpr int kFewMaxSmem = 227 * 1024;
+constexpr int kFewOutBytes = kFewWarps * 16 * kFewOStride * 4;      // the warps' outputs (paged: behind the statistics)
 __host__ __device__ inline int few_cluster_bytes(int rows, int cluster)
 {
     return cluster > 1 ? (rows + cluster - 1) / cluster * cluster * kFewRowBytes : 0;
@@ -94,7 +103,7 @@ inline int few_smem_bytes(int stages, int rows, int cluster, bool fused, int num
     return 1024 + stages * kFewStageBytes + (rows + 15) / 16 * 16 * 256 + kFewBarBytes + kFewStatBytes + few_cluster_bytes(rows, cluster) +
            (fused ? num_new * (kFewAngleBytes + 512) : 0);
 }
-static_assert(kFewMinStages * kFewStageBytes >= kFewWarps * 16 * kFewOStride * 4, "the outputs fit the stages");
+static_assert(kFewMinStages * kFewStageBytes >= kFewOutBytes, "the outputs fit the stages");
 
 // Bytes of (row, 16-byte chunk) in a 64-channel block of 128-byte swizzled rows.
 __device__ __forceinline__ uint32_t swz(int row, int chunk) { return (uint32_t)(row * 128 + ((chunk ^ (row & 7)) << 4)); }
@@ -120,7 +129,7 @@ __device__ __forceinline__ void few_write_row(const FewArgs& a, const float4& ac
 }
 
 // MT: 16-row tiles of the queries.  Contiguous cache: grid (cluster, kv heads, splits);
-// PAGED: one block per work item, numbered as in the pair kernel.
+// PAGED: one block per share of the stages, or per work item, numbered as in the pair kernel.
 template <int MT, bool PAGED, bool FUSED, typename LensT>
 __global__ void __launch_bounds__(kFewThreads)
 attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const FewArgs a,
@@ -132,7 +141,8 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem_gen = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
-    const int q_off = a.stages * kFewStageBytes, bar_off = q_off + MT * 16 * 256, stat_off = bar_off + kFewBarBytes;
+    const int stages = PAGED ? kFewPagedStages : a.stages;
+    const int q_off = stages * kFewStageBytes, bar_off = q_off + MT * 16 * 256, stat_off = bar_off + kFewBarBytes;
     const uint32_t bar_full = smem_base + bar_off, bar_empty = bar_full + 8 * kFewMaxStages;
     volatile int* s_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 16 * kFewMaxStages);
     float* s_m = reinterpret_cast<float*>(smem_gen + stat_off);            // [kFewWarps][64] reference of each warp's rows
@@ -147,7 +157,16 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
 
     // ---- the block's share: keys of stages [st0, st1) ----
     int g, slot, L, n, row_base = 0, b = 0, st0, st1;
+    int left = 0;                                      // paged: stages of the block's share behind this unit
     uint32_t rank = 0, csize = 1;
+    auto episode = [&](int e) {
+        if constexpr (PAGED) {
+            b = e;
+            L = lens.cache_len[b];
+            n = lens.new_off[b + 1] - lens.new_off[b];
+            row_base = lens.new_off[b] * a.G;
+        }
+    };
     if (!PAGED) {
         csize = gridDim.x;                             // the cluster spans x
         rank = blockIdx.x;
@@ -160,30 +179,52 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
         st0 = lo + (int)rank * len / (int)csize;
         st1 = lo + ((int)rank + 1) * len / (int)csize;
     } else {
-        const int item = (int)blockIdx.x;
-        int lo = 0, hi = a.batch;                      // largest b with item_off[b] <= item
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (lens.item_off[mid] <= item) lo = mid; else hi = mid;
+        if constexpr (PAGED) {
+            const int item = (int)blockIdx.x, first = a.share > 0 ? item * a.share : item;
+            int lo = 0, hi = a.batch;                  // largest b with item_off[b] <= first
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (lens.item_off[mid] <= first) lo = mid; else hi = mid;
+            }
+            episode(lo);
+            const int end = lens.item_off[a.batch], rem = first - lens.item_off[b];
+            if (first >= end || n <= 0) return;
+            const int ns = (L + n + kFewKeys - 1) / kFewKeys;
+            if (a.share > 0) {
+                g = (int)((unsigned)rem / (unsigned)ns);
+                st0 = rem - g * ns;
+                left = min(a.share, end - first);
+                st1 = min(ns, st0 + left);
+                left -= st1 - st0;
+                slot = item - (int)fast_div((uint32_t)(first - st0), a.div_share);      // shares that the unit met before
+            } else {
+                const int per_head = (int)((unsigned)(lens.item_off[b + 1] - lens.item_off[b]) / (unsigned)a.Hkv);    // one row unit: the split count
+                g = (int)((unsigned)rem / (unsigned)per_head);
+                slot = rem - g * per_head;
+                const int nkv = (L + n + kTileN - 1) / kTileN;                           // work items are cut at 128-key tiles
+                st0 = 2 * (int)((unsigned)slot * (unsigned)nkv / (unsigned)per_head);
+                st1 = min(2 * (int)((unsigned)(slot + 1) * (unsigned)nkv / (unsigned)per_head), ns);
+            }
         }
-        b = lo;
-        L = lens.cache_len[b];
-        n = lens.new_off[b + 1] - lens.new_off[b];
-        row_base = lens.new_off[b] * a.G;
-        const int per_head = (lens.item_off[b + 1] - lens.item_off[b]) / a.Hkv;      // one row unit: the split count
-        if (item >= lens.item_off[a.batch] || per_head <= 0) return;
-        const int rem = item - lens.item_off[b];
-        g = rem / per_head;
-        slot = rem - g * per_head;
-        const int nkv = (L + n + kTileN - 1) / kTileN;                               // work items are cut at 128-key tiles
-        st0 = 2 * (int)((unsigned)slot * (unsigned)nkv / (unsigned)per_head);
-        st1 = min(2 * (int)((unsigned)(slot + 1) * (unsigned)nkv / (unsigned)per_head), (L + n + kFewKeys - 1) / kFewKeys);
     }
-    const int rows = n * a.G;
-    const int count = st1 - st0;
+    auto next_unit = [&]() {                           // the share goes on at the start of the next (episode, kv head)
+        if constexpr (PAGED) {
+            if (++g == a.Hkv) {
+                g = 0;
+                int e = b;
+                do ++e; while (lens.new_off[e + 1] == lens.new_off[e]);
+                episode(e);
+            }
+            slot = st0 = 0;
+            st1 = min((L + n + kFewKeys - 1) / kFewKeys, left);
+            left -= st1;
+        }
+    };
+    int rows = n * a.G;
+    int count = st1 - st0;
 
     if (tid == 0) {
-        for (int i = 0; i < a.stages; ++i) {
+        for (int i = 0; i < stages; ++i) {
             ptx::mbar_init(bar_full + 8 * i, 1);
             ptx::mbar_init(bar_empty + 8 * i, kFewWarps / kFewGroups);
         }
@@ -202,12 +243,11 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
     ptx::grid_dependency_wait();
 
     // stages are taken from the last key backwards: the new tokens' stage is the first to land
-    auto load_stage = [&](int i) {
-        const int s = st1 - 1 - i, at = i % a.stages;
+    auto load_stage = [&](int i, int at, int pg) {
+        const int s = st1 - 1 - i;
         const uint32_t dst = smem_base + at * kFewStageBytes, bar = bar_full + 8 * at;
         ptx::mbar_expect_tx(bar, kFewStageBytes);
         if (PAGED) {
-            const int pg = a.page_table[(long)b * a.max_pages + s];
             ptx::tma_load_4d(dst, &tm_k, bar, 0, 0, g, pg);
             ptx::tma_load_4d(dst + 8192, &tm_k, bar, 64, 0, g, pg);
             ptx::tma_load_4d(dst + 16384, &tm_v, bar, 0, 0, g, pg);
@@ -220,19 +260,67 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
             ptx::tma_load_3d(dst + 24576, &tm_v, bar, 64, key0, g);
         }
     };
-    if (warp == kFewWarps && lane == 0)
-        for (int i = 0; i < count && i < a.stages; ++i) load_stage(i);
+    if (!PAGED && warp == kFewWarps && lane == 0)
+        for (int i = 0; i < count && i < stages; ++i) load_stage(i, i, 0);
+    bool ok = true;
+    if (PAGED && warp == kFewWarps) {
+        // ================= producer =================
+        // (the whole warp: a page number costs a round trip to L2, so the lanes fetch 32 of them at once)
+        int at = 0;
+        uint32_t phase = 1;                            // of the ring's first turn: its slots are free
+        for (;;) {
+            const int* pages = a.page_table + (long)b * a.max_pages + st1 - 1;
+            int pg = 0;
+            for (int i = 0; i < st1 - st0 && ok; ++i) {
+                if ((i & 31) == 0) pg = i + lane < st1 - st0 ? pages[-(i + lane)] : 0;
+                const int page = __shfl_sync(0xffffffffu, pg, i & 31);
+                if (lane == 0) {
+                    ok = wait_bounded(bar_empty + 8 * at, phase, kDevTimeoutProducer, a.status, s_abort);
+                    if (ok) load_stage(i, at, page);
+                }
+                ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+                if (++at == stages) { at = 0; phase ^= 1; }
+            }
+            if (!ok || left == 0) break;
+            next_unit();
+        }
+        if (lane == 0 && (!ok || *s_abort)) {
+            const long long t0 = clock64();            // loads in flight land before the block may leave
+            while (clock64() - t0 < 400000) { }
+        }
+        return;
+    }
+    // the compute warps of a paged block go from unit to unit on a barrier of their own
+    auto sync = [&]() {
+        if (PAGED) asm volatile("bar.sync 1, %0;" :: "n"(32 * kFewWarps) : "memory");
+        else __syncthreads();
+    };
+    constexpr int kTeam = kFewWarps + (PAGED ? 0 : 1);                     // warps that share the work around the products
+    constexpr int kQPer = (MT * 16 * 16 + 32 * kTeam - 1) / (32 * kTeam);
+    constexpr bool kAhead = PAGED && MT == 1;          // the next unit's are requested before this one is merged (two row
+                                                       // tiles leave no registers for them: 69 us against 64)
+    uint4 qx[kQPer];                                   // the unit's queries on their way to shared memory
+    auto load_q = [&]() {
+#pragma unroll
+        for (int k = 0; k < kQPer; ++k) {
+            const int i = tid + k * 32 * kTeam, r = i >> 4;
+            qx[k] = make_uint4(0u, 0u, 0u, 0u);
+            if (i < MT * 16 * 16 && r < n * a.G) qx[k] = reinterpret_cast<const uint4*>(a.q_rot_in + ((long)g * a.rows + row_base + r) * 128)[i & 15];
+        }
+    };
+    int i0 = 0;                                        // ring index of the unit's first stage
+    for (;;) {
 
     // ---- queries into shared memory (rows past the last one are zeros) ----
     auto q_slot = [&](int r, int chunk) -> uint4* {    // 16-byte chunk 0..15 of row r: two 64-channel blocks
         return reinterpret_cast<uint4*>(smem_gen + q_off + (chunk >> 3) * (MT * 16 * 128) + swz(r, chunk & 7));
     };
     if (!FUSED) {
-        for (int i = tid; i < MT * 16 * 16; i += kFewThreads) {
-            const int r = i >> 4, c = i & 15;
-            uint4 x = make_uint4(0u, 0u, 0u, 0u);
-            if (r < rows) x = reinterpret_cast<const uint4*>(a.q_rot_in + ((long)g * a.rows + row_base + r) * 128)[c];
-            *q_slot(r, c) = x;
+        if (!kAhead || i0 == 0) load_q();
+#pragma unroll
+        for (int k = 0; k < kQPer; ++k) {
+            const int i = tid + k * 32 * kTeam;
+            if (i < MT * 16 * 16) *q_slot(i >> 4, i & 15) = qx[k];
         }
     } else {
         // a warp per head vector, two channel pairs per lane: rows 0 .. rows-1 are queries, then the new
@@ -312,15 +400,14 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
             ptx::fence_proxy_async();                  // a later load into these stages comes after these writes
         }
     }
-    __syncthreads();
+    sync();
 
-    bool ok = true;
-    if (warp == kFewWarps) {
+    if (!PAGED && warp == kFewWarps) {
         // ================= producer =================
         if (lane == 0) {
-            for (int i = a.stages; i < count && ok; ++i) {
-                ok = wait_bounded(bar_empty + 8 * (i % a.stages), ((i / a.stages) & 1) ^ 1, kDevTimeoutProducer, a.status, s_abort);
-                if (ok) load_stage(i);
+            for (int i = stages; i < count && ok; ++i) {
+                ok = wait_bounded(bar_empty + 8 * (i % stages), ((i / stages) & 1) ^ 1, kDevTimeoutProducer, a.status, s_abort);
+                if (ok) load_stage(i, i % stages, 0);
             }
             if (!ok || *s_abort) {
                 const long long t0 = clock64();        // loads in flight land before the block may leave
@@ -377,9 +464,10 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
         };
         // Two warps per scheduler: an iteration is a chain of latencies (barrier, fragments, scores,
         // exponentials, products), so all fragments are requested ahead of the products that need them.
-        int at = group;                                // slot of stage i, and its phase
-        uint32_t phase = 0;
-        for (int i = group; i < count && ok; i += kFewGroups) {
+        const int skip = (group ^ i0) & 1;             // slots belong to the groups, whichever stage they hold
+        int at = PAGED ? (i0 + skip) % kFewPagedStages : group;            // slot of stage i, and its phase
+        uint32_t phase = PAGED ? ((i0 + skip) / kFewPagedStages) & 1 : 0;
+        for (int i = skip; i < count && ok; i += kFewGroups) {
             ok = wait_bounded(bar_full + 8 * at, phase, kDevTimeoutMmaKV, a.status, s_abort);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -461,15 +549,22 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(bar_empty + 8 * at);
             at += kFewGroups;
-            if (at >= a.stages) { at -= a.stages; phase ^= 1; }
+            if (at >= stages) { at -= stages; phase ^= 1; }
         }
         m[0] *= a.scale_log2;                          // (log2 units from here on)
         m[1] *= a.scale_log2;
     }
 
-    // ---- the warps' results into shared memory (the ring is dead: every stage has been consumed) ----
-    __syncthreads();
-    float* s_o = reinterpret_cast<float*>(smem_gen);                                  // [kFewWarps][16][kFewOStride]
+    // ---- the warps' results into shared memory (not paged: where the ring was, every stage has been consumed) ----
+    if (!PAGED) __syncthreads();
+    const int done_g = g, done_slot = slot, done_base = row_base;
+    const bool more = PAGED && left > 0;
+    if (more) {
+        i0 += count;
+        next_unit();
+        if (kAhead) load_q();
+    }
+    float* s_o = reinterpret_cast<float*>(PAGED ? s_tail : smem_gen);                 // [kFewWarps][16][kFewOStride]
     if (warp < kFewWarps) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -488,9 +583,9 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
         }
     }
     if (csize > 1) ptx::cluster_wait();                // every block of the cluster has set up its barriers
-    __syncthreads();
+    sync();
     // merge the WK shares of every row: a warp per row, 4 channels per lane
-    for (int r = warp; r < rows; r += kFewWarps + 1) {
+    for (int r = warp; r < rows; r += kTeam) {
         float M = -INFINITY;
 #pragma unroll
         for (int w = 0; w < WK; ++w) M = fmaxf(M, s_m[w * kFewRows + r]);
@@ -513,8 +608,13 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
             ptx::st_async_f32x4(ptx::map_to_cta(at + lane * 16, owner), acc, bar);
             if (lane == 0) ptx::st_async_f32x2(ptx::map_to_cta(at + 512, owner), M, sum, bar);
         } else {
-            few_write_row(a, acc, M, sum, g, slot, row_base, r, lane);
+            few_write_row(a, acc, M, sum, done_g, done_slot, done_base, r, lane);
         }
+    }
+    if (more) {
+        rows = n * a.G;
+        count = st1 - st0;
+        continue;
     }
     if (csize > 1 && (int)rank < rows) {
         // merge the cluster's contributions to this block's rows
@@ -552,6 +652,8 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
             }
             few_write_row(a, acc, M, sum, g, slot, row_base, (int)rank + k * (int)csize, lane);
         }
+    }
+    break;
     }
 }
 

@@ -26,6 +26,8 @@ struct CombineArgs {
     FastDiv div_g;           // division by G, by the work-item size in KV tiles (chunk_tiles, at least 1):
     FastDiv div_chunk;       //   a row's warp decodes its place with multiplications (an integer division costs
                              //   as much as the rest of the merge)
+    int share;               // batches whose blocks took equal shares of the 64-key stages (item_off counts them):
+    FastDiv div_share;       //   the shares that met a row's keys are its splits; 0: work items of chunk_tiles
     PackedMap map;           // where output token m goes (identity unless the call serves a packed sequence)
 };
 
@@ -51,11 +53,16 @@ combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
         }
         const int b = lo;
         const int n_b = lens.new_off[b + 1] - lens.new_off[b];
-        const int local_row = (int)row - lens.new_off[b] * a.G;
-        const int unit = local_row / kUnitRows;                  // (a power of two)
-        const int nkv = a.tail ? tail_kv_tiles_fast(lens.cache_len[b], n_b, a.div_g, unit, kUnitRows)
-                               : unit_kv_tiles_fast(lens.cache_len[b], n_b, a.div_g, unit, kUnitRows);
-        S = (int)fast_div((uint32_t)(nkv + a.chunk_tiles - 1), a.div_chunk);
+        if (a.share > 0) {
+            const uint32_t ns = (uint32_t)(lens.cache_len[b] + n_b + kFewKeys - 1) / kFewKeys, at = (uint32_t)lens.item_off[b] + g * ns;
+            S = (int)(fast_div(at + ns - 1, a.div_share) - fast_div(at, a.div_share)) + 1;
+        } else {
+            const int local_row = (int)row - lens.new_off[b] * a.G;
+            const int unit = local_row / kUnitRows;                  // (a power of two)
+            const int nkv = a.tail ? tail_kv_tiles_fast(lens.cache_len[b], n_b, a.div_g, unit, kUnitRows)
+                                   : unit_kv_tiles_fast(lens.cache_len[b], n_b, a.div_g, unit, kUnitRows);
+            S = (int)fast_div((uint32_t)(nkv + a.chunk_tiles - 1), a.div_chunk);
+        }
     }
 
     const long stride_s = (long)a.Hkv * a.rows;           // rows between consecutive splits

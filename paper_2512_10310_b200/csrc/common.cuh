@@ -12,6 +12,7 @@ constexpr int kMaxBatch = 256;     // paged calls carry per-episode lengths as l
 constexpr int kMaxSplits = 32;     // a warp merges one split per lane
 constexpr int kTileM = 128;        // query rows per MMA tile
 constexpr int kTileN = 128;        // keys per KV tile
+constexpr int kFewKeys = 64;       // keys per stage of the few-row kernel
 constexpr int kUnitRows = 2 * kTileM;  // one CTA of the tensor-core kernel owns two query tiles
 
 // Device status codes written by kernels whose bounded waits expire.

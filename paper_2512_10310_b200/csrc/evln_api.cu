@@ -517,27 +517,19 @@ int choose_chunk(int pairs, int G, int Hkv, int batch, const int* lens, const in
 
 // Work-item size (KV tiles) and the largest split count of a batch.
 void batch_schedule(int num_sms, int G, int Hkv, int batch, const int* lens, const int* offs, const int* order, bool tail,
-                    bool few, int kv_chunk_tiles, int* chunk_tiles, int* max_splits, long* items)
+                    int kv_chunk_tiles, int* chunk_tiles, int* max_splits, long* items)
 {
-    long total = 0;
     int nkv_max = 1;
     for (int b = 0; b < batch; ++b) {
         const int n = offs[b + 1] - offs[b];
         const int units = ceil_div(n * G, kUnitRows);
         for (int u = 0; u < units; ++u) {
             const int nkv = batch_kv_tiles(tail, lens[b], n, G, u);
-            total += nkv;
             if (nkv > nkv_max) nkv_max = nkv;
         }
     }
-    total *= Hkv;
     int chunk = kv_chunk_tiles;
-    if (chunk <= 0 && few) {
-        // one block per item: four items per SM even out the lengths (16 ragged episodes of one token:
-        // 65 us with one per SM, 62 with four, 72 with six: every item pays its own start and merge)
-        chunk = (int)((total + (long)num_sms * 4 - 1) / ((long)num_sms * 4));
-        if (chunk < 2) chunk = 2;
-    } else if (chunk <= 0) {
+    if (chunk <= 0) {
         chunk = choose_chunk(num_sms / 2 > 0 ? num_sms / 2 : 1, G, Hkv, batch, lens, offs, order, nkv_max);
     }
     if (chunk < ceil_div(nkv_max, kMaxSplits)) chunk = ceil_div(nkv_max, kMaxSplits);
@@ -552,6 +544,9 @@ void batch_schedule(int num_sms, int G, int Hkv, int batch, const int* lens, con
     *items = cnt * Hkv;
 }
 
+// Stages of one kv head of an episode in the few-row kernel (none without new tokens).
+inline int few_stages(int L, int n) { return n > 0 ? ceil_div(L + n, kFewKeys) : 0; }
+
 // A batch whose episodes all bring few rows (action tokens): the few-row kernel, one block per work item.
 bool paged_few(const evlnPagedParams* p, const int* offs)
 {
@@ -561,13 +556,38 @@ bool paged_few(const evlnPagedParams* p, const int* offs)
     return true;
 }
 
-void paged_schedule(evlnHandle_t h, const evlnPagedParams* p, const int* lens, const int* offs,
-                    int* chunk_tiles, int* max_splits, long* items)
+struct PagedPlan {
+    int chunk, share;        // KV tiles per work item, or (share > 0) 64-key stages per block
+    int splits;              // most partials of a row
+    long items;              // work items, or blocks
+};
+PagedPlan paged_schedule(evlnHandle_t h, const evlnPagedParams* p, const int* lens, const int* offs)
 {
+    PagedPlan plan = {1, 0, 1, 0};
+    const int Hkv = p->num_kv_heads;
+    if (paged_few(p, offs) && p->kv_chunk_tiles == 0) {
+        // An equal share of all stages for every SM, but no row in more parts than a warp merges, nor in more
+        // than the merge is worth: a stage takes about 0.41 us, another part of the longest row 0.2.
+        long total = 0;
+        int ns_max = 1;
+        for (int b = 0; b < p->batch; ++b) {
+            const int ns = few_stages(lens[b], offs[b + 1] - offs[b]);
+            total += (long)ns * Hkv;
+            if (ns > ns_max) ns_max = ns;
+        }
+        long share = (total + h->num_sms - 1) / h->num_sms;
+        while (2 * share * share < ns_max) ++share;
+        if (share < ceil_div(ns_max, kMaxSplits - 1)) share = ceil_div(ns_max, kMaxSplits - 1);
+        plan.share = (int)share;
+        plan.splits = ceil_div(ns_max - 1, plan.share) + 1;
+        plan.items = (total + share - 1) / share;
+        return plan;
+    }
     int order[kMaxBatch];
-    const bool few = paged_few(p, offs);
-    if (!few) longest_first(p->batch, lens, offs, order);
-    batch_schedule(h->num_sms, p->num_q_heads / p->num_kv_heads, p->num_kv_heads, p->batch, lens, offs, order, false, few, p->kv_chunk_tiles, chunk_tiles, max_splits, items);
+    longest_first(p->batch, lens, offs, order);
+    batch_schedule(h->num_sms, p->num_q_heads / Hkv, Hkv, p->batch, lens, offs, order, false, p->kv_chunk_tiles, &plan.chunk, &plan.splits,
+                   &plan.items);
+    return plan;
 }
 
 // chunk_tiles > 0: also the first attention work item of every episode (items are numbered
@@ -592,9 +612,16 @@ void fill_batch_lens(BatchLens* bl, int G, int Hkv, int batch, const int* lens, 
     }
 }
 
-void fill_lens(BatchLens* bl, const evlnPagedParams* p, const int* lens, const int* offs, int chunk_tiles = 0)
+void fill_lens(BatchLens* bl, const evlnPagedParams* p, const int* lens, const int* offs, int chunk_tiles = 0, int share = 0)
 {
     fill_batch_lens(bl, p->num_q_heads / p->num_kv_heads, p->num_kv_heads, p->batch, lens, offs, chunk_tiles, false);
+    if (share > 0) {                     // the stages before every episode
+        int at = 0;
+        for (int b = 0; b <= kMaxBatch; ++b) {
+            bl->item_off[b] = at;
+            if (b < p->batch) at += few_stages(lens[b], offs[b + 1] - offs[b]) * p->num_kv_heads;
+        }
+    }
 }
 
 template <typename T>
@@ -1178,11 +1205,8 @@ evlnStatus_t evlnPagedWorkspaceSize(evlnHandle_t h, const evlnPagedParams* p, co
     evlnStatus_t s = check_paged_params(h, p, h_cache_lens, h_new_offsets);
     if (s != EVLN_OK) return s;
     if (!bytes) return EVLN_INVALID_VALUE;
-    int chunk, smax;
-    long items;
-    paged_schedule(h, p, h_cache_lens, h_new_offsets, &chunk, &smax, &items);
     const long rows = (long)h_new_offsets[p->batch] * (p->num_q_heads / p->num_kv_heads);
-    *bytes = partial_bytes(smax, p->num_kv_heads, rows, p->head_dim);
+    *bytes = partial_bytes(paged_schedule(h, p, h_cache_lens, h_new_offsets).splits, p->num_kv_heads, rows, p->head_dim);
     return EVLN_OK;
 }
 
@@ -1232,11 +1256,11 @@ evlnStatus_t evlnPagedStepAttention(evlnHandle_t h, const evlnPagedParams* p, co
     if (!device_is_current(h)) return EVLN_INVALID_VALUE;
     const int G = p->num_q_heads / p->num_kv_heads;
     const long rows = (long)total * G;
-    int chunk, smax;
-    long items;
-    paged_schedule(h, p, h_cache_lens, h_new_offsets, &chunk, &smax, &items);
+    const PagedPlan plan = paged_schedule(h, p, h_cache_lens, h_new_offsets);
+    const int chunk = plan.chunk, smax = plan.splits;
+    const long items = plan.items;
     if (workspace_bytes < partial_bytes(smax, p->num_kv_heads, rows, 128)) return EVLN_WORKSPACE_TOO_SMALL;
-    if (items <= 0 || items > 0x3fffffffL) return EVLN_NOT_SUPPORTED;
+    if (items <= 0 || items * (plan.share > 0 ? plan.share : 1) > 0x3fffffffL) return EVLN_NOT_SUPPORTED;
 
     if (paged_few(p, h_new_offsets)) {
         CUtensorMap tm_k, tm_v;
@@ -1254,13 +1278,14 @@ evlnStatus_t evlnPagedStepAttention(evlnHandle_t h, const evlnPagedParams* p, co
         a.page_table = d_page_table; a.status = h->d_status;
         a.Hkv = p->num_kv_heads; a.G = G; a.rows = (int)rows;
         a.batch = p->batch; a.max_pages = p->max_pages_per_seq; a.chunk_tiles = chunk;
-        a.stages = kFewMaxStages;
+        a.share = plan.share;
+        a.div_share = make_fast_div((uint32_t)(plan.share > 0 ? plan.share : 1));
         a.scale_log2 = (p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf(128.f)) * 1.4426950408889634f;
         a.div_g = make_fast_div((uint32_t)G);
         BatchLens bl;
-        fill_lens(&bl, p, h_cache_lens, h_new_offsets, chunk);
-        if (bl.item_off[p->batch] != (int)items) return EVLN_INVALID_VALUE;
-        const size_t smem = few_smem_bytes(a.stages, most * G, 1, false, 0);
+        fill_lens(&bl, p, h_cache_lens, h_new_offsets, chunk, plan.share);
+        if (plan.share == 0 && bl.item_off[p->batch] != (int)items) return EVLN_INVALID_VALUE;
+        const size_t smem = few_smem_bytes(kFewPagedStages, most * G, 1, false, 0) + kFewOutBytes;
         cudaStream_t st = (cudaStream_t)stream;
         cudaError_t e = few_row_tiles(most * G) == 1
                             ? launch_pdl(attn_few_kernel<1, true, false, BatchLens>, dim3((int)items), dim3(kFewThreads), smem, st, tm_k, tm_v, a, bl)
@@ -1337,9 +1362,8 @@ evlnStatus_t evlnPagedStepCombine(evlnHandle_t h, const evlnPagedParams* p, cons
     if (!device_is_current(h)) return EVLN_INVALID_VALUE;
     const int G = p->num_q_heads / p->num_kv_heads;
     const long rows = (long)total * G;
-    int chunk, smax;
-    long items;
-    paged_schedule(h, p, h_cache_lens, h_new_offsets, &chunk, &smax, &items);
+    const PagedPlan plan = paged_schedule(h, p, h_cache_lens, h_new_offsets);
+    const int chunk = plan.chunk, smax = plan.splits;
     CombineArgs a = {};
     a.o_part = (const float*)workspace;
     a.lse_part = a.o_part + (size_t)smax * p->num_kv_heads * rows * 128;
@@ -1347,8 +1371,10 @@ evlnStatus_t evlnPagedStepCombine(evlnHandle_t h, const evlnPagedParams* p, cons
     a.Hkv = p->num_kv_heads; a.G = G; a.D = 128; a.rows = (int)rows; a.num_splits = smax;
     a.batch = p->batch; a.unit_rows = kUnitRows; a.chunk_tiles = chunk;
     if (smax == 1 && !paged_few(p, h_new_offsets)) return launch_copy_out(h, a, (cudaStream_t)stream);
+    a.share = plan.share;
+    a.div_share = make_fast_div((uint32_t)(plan.share > 0 ? plan.share : 1));
     BatchLens bl;
-    fill_lens(&bl, p, h_cache_lens, h_new_offsets);
+    fill_lens(&bl, p, h_cache_lens, h_new_offsets, 0, plan.share);
     return launch_combine<__nv_bfloat16>(h, a, 128, true, &bl, (cudaStream_t)stream);
 }
 
@@ -1418,7 +1444,7 @@ evlnStatus_t plan_packed(evlnHandle_t h, const evlnPackedParams* p, PackedPlan* 
     // an action chunk walks no more keys than the largest unit of the visual run beside it: not split
     // unless the caller says so
     if (n_act > 0)
-        batch_schedule(h->num_sms, G, p->num_kv_heads, p->num_frames, pl->lens, pl->offs, nullptr, true, false,
+        batch_schedule(h->num_sms, G, p->num_kv_heads, p->num_frames, pl->lens, pl->offs, nullptr, true,
                        p->kv_chunk_tiles > 0 ? p->kv_chunk_tiles : 1 << 24, &pl->chunk, &pl->smax, &pl->items);
     const size_t part_a = pl->smax > 1 ? partial_bytes(pl->smax, p->num_kv_heads, n_act * G, 128) : 0;
     size_t off = 0;

@@ -1,4 +1,4 @@
-"""Paged batches at the edges of how the persistent attention launch deals work items to CTA pairs,
+"""Paged batches at the edges of how their work is dealt out (work items to CTA pairs, equal shares to blocks),
 against the oracle."""
 import dataclasses
 
@@ -34,6 +34,24 @@ def test_paged_batch_of_many_work_items(handle, batch):
     cfg = dataclasses.replace(W.PAGED_B16, name=f"many_{batch}", num_q_heads=16, num_kv_heads=16, batch=batch, seed=90 + batch)
     lens = [(37 * b) % 301 for b in range(batch)]
     x = W.make_paged_inputs(cfg, lens, [33] * batch)
+    out, lse, k_pool, v_pool = _gpu_paged(handle, cfg, x)
+    okp, ovp = f64(x["k_pool"]), f64(x["v_pool"])
+    ref_out, ref_lse = so.step_paged(f64(x["q_new"]), f64(x["k_new"]), f64(x["v_new"]), okp, ovp, x["page_table"], lens,
+                                     x["new_offsets"], cfg.rope_theta, storage="bf16")
+    check_output("bf16", out, lse, ref_out, ref_lse)
+    _check_pools(x, cfg, k_pool, v_pool, okp, ovp)
+
+
+@pytest.mark.parametrize("hq,hkv,lens,new", [
+    (28, 4, [5], [1]),                                        # shares of one stage
+    (28, 4, [64, 0, 700, 63, 4000], [0, 2, 0, 1, 4]),         # shares go over episodes without new tokens; two row tiles
+    (7, 1, [32000], [1]),                                     # a row in as many parts as a warp merges
+    (64, 8, [900, 2000, 130], [4, 1, 3]),                     # more work items per token than a block has threads
+    (4, 4, [(53 * b) % 190 for b in range(200)], [1] * 200),  # shares of many short units
+])
+def test_paged_batch_of_few_rows_in_equal_shares(handle, hq, hkv, lens, new):
+    cfg = dataclasses.replace(W.PAGED_B16, name="shares", num_q_heads=hq, num_kv_heads=hkv, batch=len(lens), seed=120 + len(lens))
+    x = W.make_paged_inputs(cfg, lens, new)
     out, lse, k_pool, v_pool = _gpu_paged(handle, cfg, x)
     okp, ovp = f64(x["k_pool"]), f64(x["v_pool"])
     ref_out, ref_lse = so.step_paged(f64(x["q_new"]), f64(x["k_new"]), f64(x["v_new"]), okp, ovp, x["page_table"], lens,
