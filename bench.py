@@ -414,7 +414,7 @@ def measure_widening(B, handle, cfg, dev, barrier, peaks):
     kind_flops = 4 * D * Hq * (n_vis * (n_vis + 1) // 2 + sum(A * (I + (t + 1) * F) + A * (A + 1) // 2 for t in range(N)))
     res["packed_forward"] = {
         "workload": f"packed sequence: instruction {I}, {N} frames x ({F} visual + {A} action tokens), {T} tokens",
-        "one_call_us": r3(t1["median"]), "one_call_p10": r3(t1["p10"]), "one_call_p90": r3(t1["p90"]), "launches_one_call": 6,
+        "one_call_us": r3(t1["median"]), "one_call_p10": r3(t1["p10"]), "one_call_p90": r3(t1["p90"]), "launches_one_call": 2,
         "step_loop_us": r3(t2["median"]), "launches_step_loop": 3 * len(calls), "speedup": round(t2["median"] / t1["median"], 2),
         "tflops_one_call": round(kind_flops / t1["median"] / 1e6, 1)}
     del g1, g2, packs
