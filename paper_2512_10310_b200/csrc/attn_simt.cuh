@@ -17,7 +17,13 @@
 // RPT = 8 (128 rows): each vector from shared memory feeds 8 rows, the FMA pipes are the limit.
 // RPT = 2 (32 rows): a quarter of the work per block, for calls whose 128-row tiles would leave SMs
 // idle; shared-memory reads bound it at about the same rate per row (K and V vectors feed 2 rows).
+// TilesT = SimtTiles (RPT = 8): one block per SM with an equal share of all visible (row block, key tile)
+// pairs instead of (row block, kv head, split) blocks, whose whole numbers left SMs idle (196 tokens of the 7B
+// shape over 1024 cached: 44 row blocks in three splits kept 132 SMs busy for up to 7 tiles each, now 148 for
+// 6: 108.5 and 96.4 us a step).  A share goes through the ends of row blocks; a row is split where two shares meet.
 #pragma once
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "ptx_sm100.cuh"
@@ -33,6 +39,7 @@ struct SimtAttnArgs {
     int Hkv, G;
     int cache_len, num_new, cache_cap;
     int num_splits;
+    int share;             // key tiles per block, 0: a block per (row block, kv head, split)
     float scale;
 };
 
@@ -58,10 +65,12 @@ __device__ __forceinline__ void simt_fetch(float* dst, const T* base, int row, i
     }
 }
 
-template <typename T, int D, int RPT, int NT = 256>
-__global__ void __launch_bounds__(NT)
-attn_simt_kernel(const SimtAttnArgs a)
+template <typename T, int D, int RPT, typename TilesT>
+__global__ void __launch_bounds__(kSimtThreads)
+attn_simt_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
 {
+    constexpr bool SHARE = std::is_same<TilesT, SimtTiles>::value;
+    constexpr int NT = kSimtThreads;
     constexpr int TY = NT / 16, BM = TY * RPT, BN = kSimtKeys, QS = D + 4, PS = kSimtPStride;
     constexpr int kUnrollQ = RPT >= 8 ? 4 : 8, kUnrollV = RPT >= 8 ? 2 : 4;   // loads in flight ahead of the products
     constexpr int NV = D / 64;                          // 4-channel groups of O per thread
@@ -74,16 +83,37 @@ attn_simt_kernel(const SimtAttnArgs a)
 
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int R = a.num_new * a.G;
-    const int row0 = blockIdx.x * BM;
-    const int g = blockIdx.y, split = blockIdx.z;
     const int total = a.cache_len + a.num_new;
-    // splits are whole key tiles
-    const int all_tiles = (total + BN - 1) / BN;
-    const int t_lo = (int)((long)split * all_tiles / a.num_splits) * BN;
-    int t_hi = min(total, (int)((long)(split + 1) * all_tiles / a.num_splits) * BN);
-    // keys past the tile's last token are visible to none of its rows
+    int rb, g, split, j_lo, j_hi;                       // the row block and its key tiles
+    int left = 0;                                       // tiles of the block's share behind them
+    if constexpr (SHARE) {
+        const int per_head = tiles.off[kSimtShareBlocks], first = blockIdx.x * a.share;
+        g = first / per_head;
+        const int rem = first - g * per_head;
+        rb = 0;
+        while (tiles.off[rb + 1] <= rem) ++rb;
+        j_lo = rem - tiles.off[rb];
+        left = min(a.share, per_head * a.Hkv - first);
+        j_hi = min(tiles.off[rb + 1] - tiles.off[rb], j_lo + left);
+        left -= j_hi - j_lo;
+        split = blockIdx.x - (first - j_lo) / a.share;  // shares that the row block met before
+    } else {
+        rb = blockIdx.x;
+        g = blockIdx.y;
+        split = blockIdx.z;
+        const int all_tiles = (total + BN - 1) / BN;    // splits are whole key tiles
+        j_lo = (int)((long)split * all_tiles / a.num_splits);
+        j_hi = (int)((long)(split + 1) * all_tiles / a.num_splits);
+    }
+
+    ptx::grid_dependency_wait();                        // programmatic dependent launch: inputs ready
+    ptx::grid_launch_dependents();
+    for (;;) {
+    const int row0 = rb * BM;
+    const int t_lo = j_lo * BN;
+    // keys past the row block's last token are visible to none of its rows
     const int last_row = min(row0 + BM, R) - 1;
-    t_hi = min(t_hi, a.cache_len + last_row / a.G + 1);
+    const int t_hi = min(min(total, j_hi * BN), a.cache_len + last_row / a.G + 1);
     int bound[RPT];                                     // last visible key of the thread's rows
 #pragma unroll
     for (int r = 0; r < RPT; ++r) bound[r] = a.cache_len + (row0 + r * TY + ty) / a.G;
@@ -102,8 +132,6 @@ attn_simt_kernel(const SimtAttnArgs a)
             simt_fetch(s_v + (i / kVec) * D + (i % kVec) * 4, vb, j * BN + i / kVec, keys, D, (i % kVec) * 4);
     };
 
-    ptx::grid_dependency_wait();                        // programmatic dependent launch: inputs ready
-    ptx::grid_launch_dependents();
     if (ntiles > 0) {
         for (int i = tid; i < BM * kVec; i += NT)
             simt_fetch(s_q + (i / kVec) * QS + (i % kVec) * 4, qb, i / kVec, R - row0, D, (i % kVec) * 4);
@@ -234,6 +262,23 @@ attn_simt_kernel(const SimtAttnArgs a)
             *reinterpret_cast<float4*>(a.o_part + prow * D + c * 64 + tx * 4) = make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv);
         }
         if (tx == 0) a.lse_part[prow] = (sum > 0.f) ? m[r] + logf(sum) : -INFINITY;
+    }
+    // (everyone is done with the tiles in shared memory since the last key tile's final meeting)
+    if constexpr (SHARE) {
+        if (left > 0) {
+            if (tiles.off[rb + 1] == tiles.off[kSimtShareBlocks]) {       // the kv head's last row block
+                rb = 0;
+                ++g;
+            } else {
+                ++rb;
+            }
+            split = j_lo = 0;
+            j_hi = min(tiles.off[rb + 1] - tiles.off[rb], left);
+            left -= j_hi;
+            continue;
+        }
+    }
+    break;
     }
 }
 

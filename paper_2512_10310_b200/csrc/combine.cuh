@@ -8,6 +8,8 @@
 // token-major [n, Hq, D] output.  HBM/L2-bound: S*(D+1) floats in, D elements out per row.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace evln {
@@ -26,7 +28,7 @@ struct CombineArgs {
     FastDiv div_g;           // division by G, by the work-item size in KV tiles (chunk_tiles, at least 1):
     FastDiv div_chunk;       //   a row's warp decodes its place with multiplications (an integer division costs
                              //   as much as the rest of the merge)
-    int share;               // batches whose blocks took equal shares of the 64-key stages (item_off counts them):
+    int share;               // fp32 kernel: key tiles per block of equal shares; batches whose blocks took equal shares of the 64-key stages (item_off counts them):
     FastDiv div_share;       //   the shares that met a row's keys are its splits; 0: work items of chunk_tiles
     PackedMap map;           // where output token m goes (identity unless the call serves a packed sequence)
 };
@@ -44,7 +46,7 @@ combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
     const int row_head = (int)(row - row_tok * (uint32_t)a.G);  // ... and its query head within the group
 
     int S = a.num_splits;
-    if (PAGED) {
+    if constexpr (PAGED) {
         const int tok = (int)row_tok;
         int lo = 0, hi = a.batch;
         while (hi - lo > 1) {
@@ -63,6 +65,12 @@ combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
                                    : unit_kv_tiles_fast(lens.cache_len[b], n_b, a.div_g, unit, kUnitRows);
             S = (int)fast_div((uint32_t)(nkv + a.chunk_tiles - 1), a.div_chunk);
         }
+    }
+
+    if constexpr (std::is_same<LensT, SimtTiles>::value) {
+        const int rb = (int)row >> 7;
+        const uint32_t at = (uint32_t)(g * lens.off[kSimtShareBlocks] + lens.off[rb]), tiles = (uint32_t)(lens.off[rb + 1] - lens.off[rb]);
+        S = (int)(fast_div(at + tiles - 1, a.div_share) - fast_div(at, a.div_share)) + 1;
     }
 
     const long stride_s = (long)a.Hkv * a.rows;           // rows between consecutive splits

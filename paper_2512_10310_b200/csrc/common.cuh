@@ -139,6 +139,13 @@ __device__ __forceinline__ int packed_row(const PackedMap& pm, int m)
     return m + (int)fast_div((uint32_t)(m - pm.I), pm.div) * pm.A;
 }
 
+// Key tiles before each 128-row block of a kv head in the fp32 kernel, where its blocks take equal shares of them
+// (entries behind the last block: all of the kv head's).
+constexpr int kSimtShareBlocks = 64;
+struct SimtTiles {
+    int off[kSimtShareBlocks + 1];
+};
+
 // Stub lengths for the kernels that serve one episode.
 struct NoLens {
     int cache_len[1];

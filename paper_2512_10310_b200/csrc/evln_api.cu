@@ -93,7 +93,10 @@ cudaError_t launch_pair_pdl(void (*kernel)(KArgs...), dim3 grid, size_t smem, cu
 template <typename T, int D, int RPT>
 cudaError_t prepare_simt()
 {
-    return cudaFuncSetAttribute(attn_simt_kernel<T, D, RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt_smem_bytes<D, RPT>());
+    cudaError_t e = cudaFuncSetAttribute(attn_simt_kernel<T, D, RPT, NoTable>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt_smem_bytes<D, RPT>());
+    if (RPT == 8 && e == cudaSuccess)
+        e = cudaFuncSetAttribute(attn_simt_kernel<T, D, 8, SimtTiles>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt_smem_bytes<D, 8>());
+    return e;
 }
 
 template <int MT>
@@ -332,6 +335,11 @@ int choose_splits_solo(int Hkv, int R, int nkv, int num_sms)
     return best;
 }
 
+size_t partial_bytes(int splits, int Hkv, long rows, int D)
+{
+    return round_up((size_t)splits * Hkv * rows * (D + 1) * sizeof(float), 256);
+}
+
 // Row tile and split count of the SIMT kernel (splits > 0: given), by a model of measured times at
 // head_dim 128 (head_dim 64: about half).  A block of 128 rows runs alone on its SM, 13.3 us per 64-key
 // tile and 7 us for its start and write-out; a block of 32 rows takes 6.3 us per tile and 5 us when it
@@ -340,14 +348,25 @@ int choose_splits_solo(int Hkv, int R, int nkv, int num_sms)
 // split writes and re-reads a set of partials (about 5 TB/s out of L2).
 struct SimtSchedule {
     int rows_per_thread, splits;
+    int share;               // > 0: one block per SM, each that many key tiles of 128-row blocks (see attn_simt.cuh)
 };
+// The row blocks' key tiles, at most kSimtShareBlocks blocks.
+void fill_simt_tiles(const evlnStepParams* p, SimtTiles* t)
+{
+    const int G = p->num_q_heads / p->num_kv_heads, R = p->num_new * G, blocks = ceil_div(R, 128);
+    t->off[0] = 0;
+    for (int rb = 0; rb < kSimtShareBlocks; ++rb) {
+        const int last = 128 * (rb + 1) < R ? 128 * (rb + 1) - 1 : R - 1;
+        t->off[rb + 1] = t->off[rb] + (rb < blocks ? ceil_div(p->cache_len + last / G + 1, kSimtKeys) : 0);
+    }
+}
 SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits)
 {
     const int R = p->num_new * (p->num_q_heads / p->num_kv_heads);
     const int tiles = ceil_div(p->cache_len + p->num_new, kSimtKeys);
     const double d = p->head_dim / 128.0;
     const double split_us = 0.3 + 2.0 * R * p->num_kv_heads * p->head_dim * 4 / 5e6;
-    SimtSchedule best = {8, splits > 0 ? splits : 1};
+    SimtSchedule best = {8, splits > 0 ? splits : 1, 0};
     double best_cost = 1e30;
     const int smax = tiles < kMaxSplits ? tiles : kMaxSplits;
     for (int rpt = 8; rpt >= 2; rpt -= 6) {
@@ -358,17 +377,41 @@ SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits)
             const double tile_us = rpt == 8 ? 13.3 : at_once == h->num_sms ? 6.3 : 9.5;
             const double waves = (double)((blocks + at_once - 1) / at_once);
             const double cost = waves * (ceil_div(tiles, s) * tile_us * d + (rpt == 8 ? 7.0 : 5.0)) + split_us * s;
-            if (cost < best_cost - 1e-9) { best_cost = cost; best = {rpt, s}; }
+            if (cost < best_cost - 1e-9) { best_cost = cost; best = {rpt, s, 0}; }
         }
+    }
+    if (splits == 0 && ceil_div(R, 128) <= kSimtShareBlocks && (long)ceil_div(R, 128) * p->num_kv_heads * tiles > h->num_sms) {
+        // equal shares: no block waits for another's last tile, but most go over the end of a row block (start and
+        // write-out of another one) and a row gets up to one split more
+        SimtTiles t;
+        fill_simt_tiles(p, &t);
+        const int per_head = t.off[kSimtShareBlocks], blocks = ceil_div(R, 128), most = t.off[blocks] - t.off[blocks - 1];
+        int share = ceil_div(per_head * p->num_kv_heads, h->num_sms);
+        if (share < ceil_div(most, kMaxSplits - 1)) share = ceil_div(most, kMaxSplits - 1);
+        const int s = ceil_div(most - 1, share) + 1;
+        const double cost = share * 13.3 * d + 7.0 + 4.0 * ceil_div(share, t.off[1]) + split_us * (1.0 + (double)most / share);
+        // (a step that fits the scratch of the allocation-free call goes on fitting it)
+        const size_t limit = EVLN_NOALLOC_SCRATCH_BYTES;
+        const bool fits = partial_bytes(s, p->num_kv_heads, R, p->head_dim) <= limit ||
+                          partial_bytes(best.splits, p->num_kv_heads, R, p->head_dim) > limit;
+        if (fits && cost < best_cost - 1e-9) best = {8, s, share};
     }
     return best;
 }
 
 template <typename T, int D>
-void launch_simt(int rows_per_thread, dim3 grid, cudaStream_t st, const SimtAttnArgs& a)
+void launch_simt(const SimtSchedule& plan, const evlnStepParams* p, dim3 grid, cudaStream_t st, const SimtAttnArgs& a)
 {
-    if (rows_per_thread == 8) launch_pdl(attn_simt_kernel<T, D, 8>, grid, dim3(kSimtThreads), simt_smem_bytes<D, 8>(), st, a);
-    else launch_pdl(attn_simt_kernel<T, D, 2>, grid, dim3(kSimtThreads), simt_smem_bytes<D, 2>(), st, a);
+    if (plan.share > 0) {
+        SimtTiles t;
+        fill_simt_tiles(p, &t);
+        const int blocks = ceil_div(t.off[kSimtShareBlocks] * p->num_kv_heads, plan.share);
+        launch_pdl(attn_simt_kernel<T, D, 8, SimtTiles>, dim3(blocks), dim3(kSimtThreads), simt_smem_bytes<D, 8>(), st, a, t);
+    } else if (plan.rows_per_thread == 8) {
+        launch_pdl(attn_simt_kernel<T, D, 8, NoTable>, grid, dim3(kSimtThreads), simt_smem_bytes<D, 8>(), st, a, NoTable{});
+    } else {
+        launch_pdl(attn_simt_kernel<T, D, 2, NoTable>, grid, dim3(kSimtThreads), simt_smem_bytes<D, 2>(), st, a, NoTable{});
+    }
 }
 
 int resolve_splits(evlnHandle_t h, const evlnStepParams* p)
@@ -388,11 +431,6 @@ int resolve_splits(evlnHandle_t h, const evlnStepParams* p)
         return choose_splits_tc(units * p->num_kv_heads, nkv_max, nkv_min, h->num_sms);
     }
     return simt_schedule(h, p, 0).splits;
-}
-
-size_t partial_bytes(int splits, int Hkv, long rows, int D)
-{
-    return round_up((size_t)splits * Hkv * rows * (D + 1) * sizeof(float), 256);
 }
 
 bool encode_map(evlnHandle_t h, CUtensorMap* map, const void* base, int rank, const cuuint64_t* dims,
@@ -626,7 +664,7 @@ void fill_lens(BatchLens* bl, const evlnPagedParams* p, const int* lens, const i
 
 template <typename T>
 evlnStatus_t launch_combine(evlnHandle_t h, const CombineArgs& args, int D, bool paged, const BatchLens* bl,
-                            cudaStream_t st)
+                            cudaStream_t st, const SimtTiles* shares = nullptr)
 {
     CombineArgs a = args;
     a.div_g = make_fast_div((uint32_t)a.G);
@@ -635,6 +673,9 @@ evlnStatus_t launch_combine(evlnHandle_t h, const CombineArgs& args, int D, bool
     if (paged) {
         if (D == 128) launch_pdl(combine_kernel<T, 128, true, BatchLens>, dim3(grid), dim3(128), 0, st, a, *bl);
         else return EVLN_NOT_SUPPORTED;
+    } else if (shares) {
+        if (D == 128) launch_pdl(combine_kernel<T, 128, false, SimtTiles>, dim3(grid), dim3(128), 0, st, a, *shares);
+        else launch_pdl(combine_kernel<T, 64, false, SimtTiles>, dim3(grid), dim3(128), 0, st, a, *shares);
     } else {
         NoLens nl = {};
         if (D == 128) launch_pdl(combine_kernel<T, 128, false, NoLens>, dim3(grid), dim3(128), 0, st, a, nl);
@@ -1045,7 +1086,9 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
     const int G = p->num_q_heads / p->num_kv_heads;
     const int R = p->num_new * G;
     const int D = p->head_dim;
-    const int S = resolve_splits(h, p);
+    const bool simt = !use_tensor_kernel(p);
+    const SimtSchedule plan = simt ? simt_schedule(h, p, p->num_splits) : SimtSchedule{};
+    const int S = simt ? plan.splits : resolve_splits(h, p);
     if (workspace_bytes < partial_bytes(S, p->num_kv_heads, R, D)) return EVLN_WORKSPACE_TOO_SMALL;
     float* o_part = (float*)workspace;
     float* lse_part = o_part + (size_t)S * p->num_kv_heads * R * D;
@@ -1122,14 +1165,14 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
         a.Hkv = p->num_kv_heads; a.G = G;
         a.cache_len = p->cache_len; a.num_new = p->num_new; a.cache_cap = p->cache_capacity;
         a.num_splits = S; a.scale = scale;
-        const int rpt = simt_schedule(h, p, S).rows_per_thread;
-        dim3 grid(ceil_div(R, 16 * rpt), p->num_kv_heads, S);
+        a.share = plan.share;
+        dim3 grid(ceil_div(R, 16 * plan.rows_per_thread), p->num_kv_heads, S);
         if (p->dtype == EVLN_BF16) {
-            if (D == 128) launch_simt<__nv_bfloat16, 128>(rpt, grid, st, a);
-            else launch_simt<__nv_bfloat16, 64>(rpt, grid, st, a);
+            if (D == 128) launch_simt<__nv_bfloat16, 128>(plan, p, grid, st, a);
+            else launch_simt<__nv_bfloat16, 64>(plan, p, grid, st, a);
         } else {
-            if (D == 128) launch_simt<float, 128>(rpt, grid, st, a);
-            else launch_simt<float, 64>(rpt, grid, st, a);
+            if (D == 128) launch_simt<float, 128>(plan, p, grid, st, a);
+            else launch_simt<float, 64>(plan, p, grid, st, a);
         }
     }
     cudaError_t e = cudaGetLastError();
@@ -1153,7 +1196,9 @@ evlnStatus_t evlnStepCombine(evlnHandle_t h, const evlnStepParams* p, const void
     if (!device_is_current(h)) return EVLN_INVALID_VALUE;
     const int G = p->num_q_heads / p->num_kv_heads;
     const int R = p->num_new * G;
-    const int S = resolve_splits(h, p);
+    const bool simt = !use_tensor_kernel(p);
+    const SimtSchedule plan = simt ? simt_schedule(h, p, p->num_splits) : SimtSchedule{};
+    const int S = simt ? plan.splits : resolve_splits(h, p);
     CombineArgs a = {};
     a.o_part = (const float*)workspace;
     a.lse_part = a.o_part + (size_t)S * p->num_kv_heads * R * p->head_dim;
@@ -1161,8 +1206,16 @@ evlnStatus_t evlnStepCombine(evlnHandle_t h, const evlnStepParams* p, const void
     a.Hkv = p->num_kv_heads; a.G = G; a.D = p->head_dim; a.rows = R; a.num_splits = S;
     cudaStream_t st = (cudaStream_t)stream;
     if (S == 1 && use_pair_kernel(p)) return launch_copy_out(h, a, st);
-    if (p->dtype == EVLN_BF16) return launch_combine<__nv_bfloat16>(h, a, p->head_dim, false, nullptr, st);
-    return launch_combine<float>(h, a, p->head_dim, false, nullptr, st);
+    SimtTiles tiles;
+    const SimtTiles* shares = nullptr;
+    if (plan.share > 0) {
+        a.share = plan.share;
+        a.div_share = make_fast_div((uint32_t)a.share);
+        fill_simt_tiles(p, &tiles);
+        shares = &tiles;
+    }
+    if (p->dtype == EVLN_BF16) return launch_combine<__nv_bfloat16>(h, a, p->head_dim, false, nullptr, st, shares);
+    return launch_combine<float>(h, a, p->head_dim, false, nullptr, st, shares);
 }
 
 evlnStatus_t evlnStep(evlnHandle_t h, const evlnStepParams* p, const void* q_new, const void* k_new,

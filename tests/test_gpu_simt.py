@@ -31,6 +31,10 @@ def handle():
     ("f32", 14, 2, 128, 5, 300, 3),        # mostly causal: whole key ranges invisible to early rows
     ("bf16", 14, 2, 64, 321, 70, 0),       # bf16 of head_dim 64 runs here too
     ("bf16", 28, 4, 64, 1500, 196, 0),
+    ("f32", 28, 4, 128, 1024, 196, 0),     # equal shares of the key tiles, each over the end of a row block
+    ("f32", 8, 1, 64, 5000, 64, 0),        # ... of two or three tiles: a row in many parts
+    ("f32", 7, 1, 128, 40, 1170, 0),       # ... of the most row blocks, short ones first
+    ("f32", 7, 1, 64, 40, 1172, 0),        # one row block more: no shares
 ])
 def test_simt_step_against_oracle(handle, dtype, hq, hkv, d, L, n, splits):
     # unit-variance inputs in fp32 (softmax far from uniform); 0.3 in bf16, where the operands' rounding
