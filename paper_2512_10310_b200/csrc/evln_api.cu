@@ -205,7 +205,10 @@ inline bool use_tensor_kernel(const evlnStepParams* p)
 
 // Cost model of the split-KV schedule of the tensor-core kernel: work items (unit x split) run
 // in waves of one CTA pair per two SMs, each walks ceil(nkv / S) KV tiles plus a fixed
-// prologue/epilogue; every extra split adds combine traffic.
+// prologue/epilogue; every split adds combine traffic, the first one the combine itself: unsplit rows are
+// written by the attention kernel.  (Measured over 256 .. 32768 cached keys, 64 .. 256 new tokens, three head shapes:
+// within 2 % of the best split count everywhere.  Without the price of the combine up to 28 % off at short
+// caches: 196 tokens over 256 13.1 us in two splits, 11.0 in one.)
 int choose_splits_tc(int units_total, int nkv_max, int nkv_min, int num_sms)
 {
     int best = 1;
@@ -216,7 +219,7 @@ int choose_splits_tc(int units_total, int nkv_max, int nkv_min, int num_sms)
         const double waves = ceil((double)units_total * s / pairs);
         // per work item: set-up, first-tile latency, partial write-out and teardown cost about as
         // much as 7 KV tiles (measured); every split adds about half a tile of combine work
-        const double cost = waves * (ceil((double)nkv_max / s) + 7.0) + 0.5 * s;
+        const double cost = waves * (ceil((double)nkv_max / s) + 7.0) + (s > 1 ? 4.0 : 0.0) + 0.5 * s;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = s; }
     }
     return best;
@@ -230,10 +233,15 @@ inline bool use_solo_kernel(const evlnStepParams* p)
 }
 
 // At most 32 rows per kv head (up to four action tokens with seven query heads per kv head): the kernel
-// whose products stay in registers (attn_few.cuh).
+// whose products stay in registers (attn_few.cuh).  Not with two row tiles and long caches of eight or more kv
+// heads: clusters of 16 blocks for all heads do not fit the device at once, and mma.sync on half of the SMs is
+// slower than the one-CTA kernel on all of them (32 rows, 8 heads, 4292 keys 14.6 us against 12.3, 20656 keys
+// 25.2 against 23.0; 1500 keys 9.7 against 10.0; 4 heads 9.8 against 10.8 and 17.4 against 17.3).
 inline bool use_few_kernel(const evlnStepParams* p)
 {
-    return use_tensor_kernel(p) && (long)p->num_new * (p->num_q_heads / p->num_kv_heads) <= kFewRows;
+    const long rows = (long)p->num_new * (p->num_q_heads / p->num_kv_heads);
+    if (!use_tensor_kernel(p) || rows > kFewRows) return false;
+    return rows <= 16 || p->num_kv_heads < 8 || p->cache_len + p->num_new < 3072 || p->num_splits > 0;
 }
 inline bool use_pair_kernel(const evlnStepParams* p) { return use_tensor_kernel(p) && !use_solo_kernel(p); }
 inline int few_row_tiles(int rows) { return rows <= 16 ? 1 : 2; }
@@ -319,17 +327,21 @@ cudaError_t launch_few(const FewPlan& f, int rows, cudaStream_t st, const CUtens
     return cudaLaunchKernelEx(&cfg, attn_few_kernel<2, false, FUSED, NoLens>, tm_k, tm_v, a, nl);
 }
 
-// Split schedule of the one-CTA-per-item kernel: the step is bound by streaming K/V once, so the
-// KV range is spread over all SMs; an item's fixed cost is about 3 tiles of streaming, and a split
-// adds a partial row set of R rows to merge.
-int choose_splits_solo(int Hkv, int R, int nkv, int num_sms)
+// Split schedule of the one-CTA-per-item kernel, in microseconds: a CTA takes 0.9 per KV tile unless HBM (all
+// of K and V at most of its rate) takes longer, and a split adds partials of every row to write and merge.
+// (Measured over 500 .. 32000 cached keys, 4 and 8 kv heads, 35 .. 128 rows each: within 3 % of the best split
+// count everywhere, 0.2 % on average.  Spreading over as many SMs as there are cost up to 19 % with 8 kv
+// heads: 8 tokens over 4292 keys 15.1 us with 18 splits, 12.7 with 12.)
+int choose_splits_solo(int Hkv, int R, int T, int num_sms)
 {
+    const int nkv = ceil_div(T, kTileN);
+    const double hbm_us = 512.0 * T * Hkv / 6.4e6, split_us = 0.1 + 1e-4 * R * Hkv;
     int best = 1;
     double best_cost = 1e30;
     const int smax = nkv < kMaxSplits ? (nkv < 1 ? 1 : nkv) : kMaxSplits;
     for (int s = 1; s <= smax; ++s) {
-        const double waves = ceil((double)Hkv * s / num_sms);
-        const double cost = waves * (ceil((double)nkv / s) + 3.0) + 0.5 * s * R / 256.0;
+        const double waves = ceil((double)Hkv * s / num_sms), work = 0.9 * waves * ceil_div(nkv, s);
+        const double cost = (work > 0.8 * hbm_us ? work : 0.8 * hbm_us) + split_us * s;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = s; }
     }
     return best;
@@ -423,7 +435,7 @@ int resolve_splits(evlnHandle_t h, const evlnStepParams* p)
     const int T = p->cache_len + p->num_new;
     if (use_few_kernel(p)) return few_plan(h, p).splits;
     if (use_solo_kernel(p))
-        return choose_splits_solo(p->num_kv_heads, R, ceil_div(T, kTileN), h->num_sms);
+        return choose_splits_solo(p->num_kv_heads, R, T, h->num_sms);
     if (use_tensor_kernel(p)) {
         const int units = ceil_div(R, kUnitRows);
         const int nkv_max = unit_kv_tiles(p->cache_len, p->num_new, G, units - 1, kUnitRows);

@@ -33,6 +33,7 @@ def handle():
     (2, 2, 700, 17, 0),           # one more: the three launches
     (32, 8, 5000, 4, 0),          # 16 rows, eight kv heads
     (64, 8, 3000, 4, 0),          # 32 rows: the most
+    (64, 8, 3068, 4, 0),          # 32 rows over a longer cache of eight kv heads: the one-CTA kernel
     (28, 4, 9000, 3, 0),          # more stages per block than the ring holds
     (7, 1, 20000, 1, 0),          # one kv head: the library splits
     (28, 4, 500, 1, 5),           # splits of one and two stages: clusters of one block
