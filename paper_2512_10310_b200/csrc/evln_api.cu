@@ -508,32 +508,36 @@ double finish_time(int pairs, int G, int Hkv, int batch, const int* lens, const 
         const int b = order[i], n = offs[b + 1] - offs[b];
         if (n == 0) continue;
         const int units = ceil_div(n * G, kUnitRows);
-        const int nkv = unit_kv_tiles(lens[b], n, G, units - 1, kUnitRows), splits = ceil_div(nkv, chunk);
-        const double cost = (double)nkv / splits + kNextItemTiles;
-        for (long left = (long)units * Hkv * splits; left > 0;) {
-            const int take = left < runs[0].count ? (int)left : runs[0].count;
-            const double load = runs[0].load + cost;
-            left -= take;
-            runs[0].count -= take;
-            int at = 0;
-            if (runs[0].count == 0) {              // the lowest run moves up: close its place while looking
-                --num;
-                for (; at < num && runs[at + 1].load < load; ++at) runs[at] = runs[at + 1];
-                if (at < num && runs[at + 1].load == load) {
-                    runs[at + 1].count += take;
-                    for (int k = at; k < num; ++k) runs[k] = runs[k + 1];
+        // (a row unit further on may need a tile more, and by that a split more)
+        for (int u = 0, same; u < units; u += same) {
+            const int nkv = unit_kv_tiles(lens[b], n, G, u, kUnitRows), splits = ceil_div(nkv, chunk);
+            for (same = 1; u + same < units && unit_kv_tiles(lens[b], n, G, u + same, kUnitRows) == nkv;) ++same;
+            const double cost = (double)nkv / splits + kNextItemTiles;
+            for (long left = (long)same * Hkv * splits; left > 0;) {
+                const int take = left < runs[0].count ? (int)left : runs[0].count;
+                const double load = runs[0].load + cost;
+                left -= take;
+                runs[0].count -= take;
+                int at = 0;
+                if (runs[0].count == 0) {              // the lowest run moves up: close its place while looking
+                    --num;
+                    for (; at < num && runs[at + 1].load < load; ++at) runs[at] = runs[at + 1];
+                    if (at < num && runs[at + 1].load == load) {
+                        runs[at + 1].count += take;
+                        for (int k = at; k < num; ++k) runs[k] = runs[k + 1];
+                    } else {
+                        runs[at] = Run{load, take};
+                        ++num;
+                    }
                 } else {
-                    runs[at] = Run{load, take};
-                    ++num;
-                }
-            } else {
-                while (at < num && runs[at].load < load) ++at;
-                if (at < num && runs[at].load == load) {
-                    runs[at].count += take;
-                } else {
-                    for (int k = num; k > at; --k) runs[k] = runs[k - 1];
-                    runs[at] = Run{load, take};
-                    ++num;
+                    while (at < num && runs[at].load < load) ++at;
+                    if (at < num && runs[at].load == load) {
+                        runs[at].count += take;
+                    } else {
+                        for (int k = num; k > at; --k) runs[k] = runs[k - 1];
+                        runs[at] = Run{load, take};
+                        ++num;
+                    }
                 }
             }
         }
@@ -546,7 +550,7 @@ double finish_time(int pairs, int G, int Hkv, int batch, const int* lens, const 
 // items even out by themselves (longest first); else the estimate above decides how often the longest
 // episode is split.  Measured: 16 ragged episodes of one frame (384 unsplit items) 480 us with items of a quarter
 // of a pair's share, 428 unsplit; episodes of 4000 and 1000 tokens 42 us, 28 with the longer one split in two;
-// of 16384 and 8000 tokens 104 and 91 (three and two ways).
+// of 16384 and 8000 tokens 104 and 91 (three and two ways); four of 4000 .. 16000 tokens 128 unsplit, 105 in up to four.
 int choose_chunk(int pairs, int G, int Hkv, int batch, const int* lens, const int* offs, const int* order, int nkv_max)
 {
     long unsplit = 0;
@@ -557,8 +561,9 @@ int choose_chunk(int pairs, int G, int Hkv, int batch, const int* lens, const in
     double best_cost = 1e30;
     for (int splits = 1; splits <= 8 && splits <= nkv_max; ++splits) {
         const int chunk = ceil_div(nkv_max, splits);
-        // a KV tile takes a pair about 0.63 us; partials move at about 5.5 TB/s, each row written and read
-        const double moved = rows * (splits == 1 ? 0.5 : splits) * 1024.0 / 5.5e6 / 0.63;
+        // a KV tile takes a pair about 0.87 us with all of them at work; partials move at about 5.5 TB/s, each row
+        // written and read
+        const double moved = rows * (splits == 1 ? 0.5 : splits) * 1024.0 / 5.5e6 / 0.87;
         const double cost = finish_time(pairs, G, Hkv, batch, lens, offs, order, chunk) + moved;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = chunk; }
     }
@@ -1403,12 +1408,22 @@ evlnStatus_t evlnPagedStepAttention(evlnHandle_t h, const evlnPagedParams* p, co
         d.lse_out = a.lse_part;
     }
     ItemTable table;
-    int k = 0, place = 0;
+    int k = 0, place = -1, unit = 0, units = 0, slot = 0, splits = 0, tiles = 0;     // in the order decode_work numbers them
     assign_items((int)persistent_pairs(h, items), items, [&]() -> CostedItem {
-        while (bl.item_off[place + 1] <= k) ++place;
-        const int b = bl.order[place], n = h_new_offsets[b + 1] - h_new_offsets[b];
-        const int nkv = unit_kv_tiles(h_cache_lens[b], n, G, ceil_div(n * G, kUnitRows) - 1, kUnitRows);
-        return CostedItem{k++, nkv / ceil_div(nkv, chunk)};
+        if (slot == splits) {
+            slot = 0;
+            if (++unit >= units) unit = 0;                                           // the next kv head
+            if (place < 0 || bl.item_off[place + 1] <= k) {
+                do ++place; while (bl.item_off[place + 1] <= k);
+                units = ceil_div((h_new_offsets[bl.order[place] + 1] - h_new_offsets[bl.order[place]]) * G, kUnitRows);
+                unit = 0;
+            }
+            const int b = bl.order[place], nkv = unit_kv_tiles(h_cache_lens[b], h_new_offsets[b + 1] - h_new_offsets[b], G, unit, kUnitRows);
+            splits = ceil_div(nkv, chunk);
+            tiles = nkv / splits;
+        }
+        ++slot;
+        return CostedItem{k++, tiles};
     }, &table);
     return launch_persistent(h, items, d, table, [&](dim3 grid) {
         return launch_pair_pdl(attn_persistent_kernel<true, PagedLens>, grid, kPersistSmemBytes, (cudaStream_t)stream, tm_q, tm_k, tm_v, a, bl, d, table);
