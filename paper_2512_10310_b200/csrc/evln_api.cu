@@ -1159,8 +1159,11 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
             // More items than pairs: persistent pairs where items are short (a prefill).  From about 32 KV tiles per
             // item on, what the boundaries save is lost to the spills of that kernel's tile loop (140 items of 78
             // tiles: 168 us against 158; 112 items of up to 8: 22.6 against 25.3).
+            // Not with more splits than the first unit has tiles (the caller's choice only): a persistent pair ends at
+            // an item without tiles, the other kernel writes its empty partial.
             const int tiles = unit_kv_tiles(p->cache_len, p->num_new, G, a.units_per_head - 1, kUnitRows) / S;
-            if (items > persistent_pairs(h, items) && tiles <= 32 && items <= 0x3fffffffL) {
+            const bool none_empty = S <= unit_kv_tiles(p->cache_len, p->num_new, G, 0, kUnitRows);
+            if (items > persistent_pairs(h, items) && none_empty && tiles <= 32 && items <= 0x3fffffffL) {
                 d.div_hkv = make_fast_div((uint32_t)p->num_kv_heads);
                 d.div_units = make_fast_div((uint32_t)a.units_per_head);
                 ItemTable table;

@@ -42,3 +42,22 @@ def test_unsplit_step_writes_the_output_directly(handle, L, n, splits):
         check_output("bf16", g["out"], g["lse"], r["out"], r["lse"])
         bits.append((g["out"].view(torch.int16), g["lse"]))
     assert all(torch.equal(a, b) for a, b in zip(*bits))
+
+
+@pytest.mark.parametrize("L,n,splits", [
+    (1000, 256, 3),     # 84 work items of three or four tiles: persistent pairs that keep their place among the splits
+    (0, 256, 3),        # 84 items again, but the units have one or two tiles: empty splits
+    (0, 400, 32),       # nearly all of them empty
+    (130, 700, 2),      # the first unit has just as many tiles as there are splits
+])
+def test_more_split_items_than_pairs(handle, L, n, splits):
+    cfg = dataclasses.replace(W.STEP_7B, name=f"split_items_{L}_{n}", cache_len=L, num_new=n, seed=900 + L + n)
+    x = W.make_step_inputs(cfg)
+    r = oracle_step("bf16", x["k_cache"], x["v_cache"], x["q_new"], x["k_new"], x["v_new"], L, cfg.rope_theta)
+    for fused in (True, False):
+        gs = GpuStep(handle, "bf16", 28, 4, 128, L + n + 3, cfg.rope_theta, n, num_splits=splits, fused=fused)
+        gs.load_cache(x["k_cache"], x["v_cache"])
+        g = gs.step(L, x["q_new"], x["k_new"], x["v_new"])         # (checks the device status)
+        assert g["splits"] == splits
+        check_cache(gs, r, L, n)
+        check_output("bf16", g["out"], g["lse"], r["out"], r["lse"])
