@@ -65,6 +65,38 @@ __device__ __forceinline__ void simt_fetch(float* dst, const T* base, int row, i
     }
 }
 
+// One row over the `keys` keys from kb / vb on that it sees, by one warp, key after key: see the end of the kernel.
+// (Out of line and with plain arguments, so that the tile loop keeps its registers: inlined, 97.2 us instead of
+// 94.9 for 196 tokens of the 7B shape over 1024 cached.)
+template <typename T, int D>
+__device__ __noinline__ void simt_row(const T* q, const T* kb, const T* vb, float* op, float* lp, float scale, int keys)
+{
+    constexpr int C = D / 32;
+    const int lane = threadIdx.x & 31;
+    q += lane * C;
+    float m = -INFINITY, l = 0.f, o[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) o[c] = 0.f;
+    for (int t = 0; t < keys; ++t) {
+        float s = 0.f;
+#pragma unroll
+        for (int c = 0; c < C; ++c) s = fmaf(to_float(q[c]), to_float(kb[(long)t * D + lane * C + c]), s);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        s *= scale;
+        const float m_new = fmaxf(m, s), ref = (m_new == -INFINITY) ? 0.f : m_new;
+        const float alpha = expf(m - ref), p = expf(s - ref);
+        m = m_new;
+        l = l * alpha + p;
+#pragma unroll
+        for (int c = 0; c < C; ++c) o[c] = fmaf(p, to_float(vb[(long)t * D + lane * C + c]), o[c] * alpha);
+    }
+    const float inv = (l > 0.f) ? 1.f / l : 0.f;
+#pragma unroll
+    for (int c = 0; c < C; ++c) op[lane * C + c] = o[c] * inv;
+    if (lane == 0) *lp = (l > 0.f) ? m + logf(l) : -INFINITY;
+}
+
 template <typename T, int D, int RPT, typename TilesT>
 __global__ void __launch_bounds__(kSimtThreads)
 attn_simt_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
@@ -245,23 +277,40 @@ attn_simt_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
         ptx::cp_async_commit();
     }
 
+    // A masked key's probability is 0, but 0 times an infinite or undefined value is not: a row block whose results
+    // are not all finite is done again row by row, each over the keys it sees.
+    uint64_t zero = 0ull;                               // ... or undefined
 #pragma unroll
-    for (int r = 0; r < RPT; ++r) {
-        float sum = l[r];
+    for (int r = 0; r < RPT; ++r)
 #pragma unroll
-        for (int off = 8; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-        const int row = row0 + r * TY + ty;
-        if (row >= R) continue;
-        const long prow = ((long)split * a.Hkv + g) * R + row;
-        const float inv = (sum > 0.f) ? 1.f / sum : 0.f;
+        for (int c = 0; c < 2 * NV; ++c) zero = ptx::fma2(o[r][c], 0ull, zero);
+    float z0, z1;
+    ptx::unpack2(zero, z0, z1);
+    if (__syncthreads_and(z0 + z1 == 0.f)) {
 #pragma unroll
-        for (int c = 0; c < NV; ++c) {
-            float4 v;
-            ptx::unpack2(o[r][2 * c], v.x, v.y);
-            ptx::unpack2(o[r][2 * c + 1], v.z, v.w);
-            *reinterpret_cast<float4*>(a.o_part + prow * D + c * 64 + tx * 4) = make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv);
+        for (int r = 0; r < RPT; ++r) {
+            float sum = l[r];
+#pragma unroll
+            for (int off = 8; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            const int row = row0 + r * TY + ty;
+            if (row >= R) continue;
+            const long prow = ((long)split * a.Hkv + g) * R + row;
+            const float inv = (sum > 0.f) ? 1.f / sum : 0.f;
+#pragma unroll
+            for (int c = 0; c < NV; ++c) {
+                float4 v;
+                ptx::unpack2(o[r][2 * c], v.x, v.y);
+                ptx::unpack2(o[r][2 * c + 1], v.z, v.w);
+                *reinterpret_cast<float4*>(a.o_part + prow * D + c * 64 + tx * 4) = make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv);
+            }
+            if (tx == 0) a.lse_part[prow] = (sum > 0.f) ? m[r] + logf(sum) : -INFINITY;
         }
-        if (tx == 0) a.lse_part[prow] = (sum > 0.f) ? m[r] + logf(sum) : -INFINITY;
+    } else {
+        for (int row = row0 + (tid >> 5); row <= last_row; row += NT / 32)
+        {
+            const long prow = ((long)split * a.Hkv + g) * R + row;
+            simt_row<T, D>(qb + (long)(row - row0) * D, kb, vb, a.o_part + prow * D, a.lse_part + prow, a.scale, min(keys, a.cache_len + row / a.G + 1 - t_lo));
+        }
     }
     // (everyone is done with the tiles in shared memory since the last key tile's final meeting)
     if constexpr (SHARE) {

@@ -47,3 +47,25 @@ def test_simt_step_against_oracle(handle, dtype, hq, hkv, d, L, n, splits):
     r = oracle_step(dtype, x["k_cache"], x["v_cache"], x["q_new"], x["k_new"], x["v_new"], L, cfg.rope_theta)
     check_cache(gs, r, L, n)
     check_output(dtype, g["out"], g["lse"], r["out"], r["lse"])
+
+
+@pytest.mark.parametrize("dtype,hq,hkv,d,L,n", [
+    ("f32", 2, 1, 64, 100, 20),            # 32-row blocks
+    ("f32", 28, 4, 128, 1024, 196),        # equal shares of 128-row blocks
+    ("f32", 8, 8, 64, 0, 700),             # several key tiles that rows of the same block see in part
+    ("bf16", 14, 2, 64, 321, 70),
+])
+def test_values_of_keys_a_row_does_not_see(handle, dtype, hq, hkv, d, L, n):
+    # infinite and undefined values at token `bad` reach the rows of the tokens from `bad` on, and no others
+    cfg = W.StepConfig("unseen", dtype, hq, hkv, d, L, n, 1e4, 1.0 if dtype == "f32" else 0.3, 90 + L + n)
+    x = W.make_step_inputs(cfg)
+    r = oracle_step(dtype, x["k_cache"], x["v_cache"], x["q_new"], x["k_new"], x["v_new"], L, cfg.rope_theta)
+    bad = n * 2 // 3
+    v = x["v_new"].clone()
+    v[bad, :, :d // 2] = float("inf")
+    v[bad, :, d // 2:] = float("nan")
+    gs = GpuStep(handle, dtype, hq, hkv, d, L + n + 5, cfg.rope_theta, n)
+    gs.load_cache(x["k_cache"], x["v_cache"])
+    g = gs.step(L, x["q_new"], x["k_new"], v)
+    check_output(dtype, g["out"][:bad], g["lse"][:bad], r["out"][:bad], r["lse"][:bad])
+    assert not bool(torch.isfinite(g["out"][bad:]).any())
