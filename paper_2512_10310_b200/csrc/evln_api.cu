@@ -155,6 +155,11 @@ bool attention_register_pool_ok()
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+inline bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes)
+{
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return a_bytes > 0 && b_bytes > 0 && x < y + b_bytes && y < x + a_bytes;
+}
 inline int elem_bytes(int dtype) { return dtype == EVLN_BF16 ? 2 : 4; }
 
 evlnStatus_t cuda_fail(evlnHandle_t h, cudaError_t e)
@@ -1083,6 +1088,31 @@ evlnStatus_t evlnRopeAppend(evlnHandle_t h, const evlnStepParams* p, const void*
     return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
 }
 
+// Buffers a caller shares between the arguments of a step.  Launch by launch that is sound: q_rot over q_new (rotation
+// in place) or the output over anything but the cache and the workspace.  A launch that does two of the three calls'
+// work has no order among its blocks: one block may write what another has still to read.
+static bool output_over_q_rot(const evlnStepParams* p, const void* q_rot, const void* out, const float* lse_out)
+{
+    const size_t rows = (size_t)p->num_new * p->num_q_heads, bytes = rows * p->head_dim * elem_bytes(p->dtype);
+    return overlap(out, bytes, q_rot, bytes) || (lse_out && overlap(lse_out, rows * sizeof(float), q_rot, bytes));
+}
+static bool step_buffers_shared(const evlnStepParams* p, const void* q_new, const void* k_new, const void* v_new, long q_stride,
+                                long k_stride, long v_stride, const void* q_rot, const void* out, const float* lse_out)
+{
+    const size_t e = elem_bytes(p->dtype), rows = (size_t)p->num_new * p->num_q_heads, q_row = (size_t)p->num_q_heads * p->head_dim;
+    const size_t kv_row = (size_t)p->num_kv_heads * p->head_dim, before_last = (size_t)(p->num_new - 1);
+    const struct { const void* at; size_t bytes; } in[3] = {{q_new, (before_last * q_stride + q_row) * e},
+                                                            {k_new, (before_last * k_stride + kv_row) * e},
+                                                            {v_new, (before_last * v_stride + kv_row) * e}};
+    for (const auto& x : in) {
+        if (overlap(q_rot, rows * p->head_dim * e, x.at, x.bytes)) return true;
+        // (the output in the very place of the queries: a head's are read by the blocks that write its output, before)
+        if (x.at == q_new && out == q_new && q_stride == (long)q_row) continue;
+        if (overlap(out, rows * p->head_dim * e, x.at, x.bytes) || (lse_out && overlap(lse_out, rows * sizeof(float), x.at, x.bytes))) return true;
+    }
+    return output_over_q_rot(p, q_rot, out, lse_out);
+}
+
 // Attention of a step.  `direct` (may be null): the step's final output; when the keys are not split and
 // the pair kernel runs, it writes that itself and `done` says that there is nothing left to combine.
 struct DirectOut {
@@ -1251,7 +1281,8 @@ evlnStatus_t evlnStep(evlnHandle_t h, const evlnStepParams* p, const void* q_new
     const long rows = (long)p->num_new * (p->num_q_heads / p->num_kv_heads);
     if (workspace_bytes < partial_bytes(resolve_splits(h, p), p->num_kv_heads, rows, p->head_dim))
         return EVLN_WORKSPACE_TOO_SMALL;
-    if (use_few_kernel(p) && p->num_new <= kFewFusedTokens) {
+    if (use_few_kernel(p) && p->num_new <= kFewFusedTokens &&
+        !step_buffers_shared(p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, out, lse_out)) {
         s = check_rope_append(h, p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, k_cache, v_cache);
         if (s != EVLN_OK) return s;
         const int S = resolve_splits(h, p);
@@ -1265,7 +1296,8 @@ evlnStatus_t evlnStep(evlnHandle_t h, const evlnStepParams* p, const void* q_new
                        stream);
     if (s != EVLN_OK) return s;
     DirectOut direct = {out, lse_out, false};
-    s = step_attention(h, p, q_rot, k_cache, v_cache, workspace, workspace_bytes, stream, &direct);
+    s = step_attention(h, p, q_rot, k_cache, v_cache, workspace, workspace_bytes, stream,
+                       output_over_q_rot(p, q_rot, out, lse_out) ? nullptr : &direct);
     if (s != EVLN_OK || direct.done) return s;
     return evlnStepCombine(h, p, workspace, out, lse_out, stream);
 }
@@ -1906,7 +1938,8 @@ extern "C" evlnStatus_t evlnStepAttentionNoAlloc(const evlnStepParams* p, const 
     if (p->num_new == 0) return EVLN_OK;
     if (!out || !aligned16(out)) return EVLN_INVALID_VALUE;
     DirectOut direct = {out, lse_out, false};
-    s = step_attention(h, p, q_rot, k_cache, v_cache, d->scratch, (size_t)EVLN_NOALLOC_SCRATCH_BYTES, stream, &direct);
+    s = step_attention(h, p, q_rot, k_cache, v_cache, d->scratch, (size_t)EVLN_NOALLOC_SCRATCH_BYTES, stream,
+                       output_over_q_rot(p, q_rot, out, lse_out) ? nullptr : &direct);
     if (s != EVLN_OK || direct.done) return s;
     return evlnStepCombine(h, p, d->scratch, out, lse_out, stream);
 }
