@@ -248,7 +248,6 @@ inline bool use_few_kernel(const evlnStepParams* p)
     if (!use_tensor_kernel(p) || rows > kFewRows) return false;
     return rows <= 16 || p->num_kv_heads < 8 || p->cache_len + p->num_new < 3072 || p->num_splits > 0;
 }
-inline bool use_pair_kernel(const evlnStepParams* p) { return use_tensor_kernel(p) && !use_solo_kernel(p); }
 inline int few_row_tiles(int rows) { return rows <= 16 ? 1 : 2; }
 
 struct FewPlan {
@@ -1180,10 +1179,10 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
             launch_pdl(attn_solo_kernel, dim3(1, p->num_kv_heads, S), dim3(kTcThreads), kSoloSmemBytes, st, tm_q, tm_k, tm_v, a);
         } else {
             TcOutArgs d = {};
-            if (S == 1) {                          // final rows: to the caller, or for the combine call to copy
-                d.out = direct ? (__nv_bfloat16*)direct->out : (__nv_bfloat16*)workspace;
-                d.lse_out = direct ? direct->lse_out : lse_part;
-                if (direct) direct->done = true;
+            if (S == 1 && direct) {                // final rows, straight to the caller
+                d.out = (__nv_bfloat16*)direct->out;
+                d.lse_out = direct->lse_out;
+                direct->done = true;
             }
             const long items = (long)p->num_kv_heads * a.units_per_head * S;
             // More items than pairs: persistent pairs where items are short (a prefill).  From about 32 KV tiles per
@@ -1255,7 +1254,6 @@ evlnStatus_t evlnStepCombine(evlnHandle_t h, const evlnStepParams* p, const void
     a.out = out; a.lse_out = lse_out;
     a.Hkv = p->num_kv_heads; a.G = G; a.D = p->head_dim; a.rows = R; a.num_splits = S;
     cudaStream_t st = (cudaStream_t)stream;
-    if (S == 1 && use_pair_kernel(p)) return launch_copy_out(h, a, st);
     SimtTiles tiles;
     const SimtTiles* shares = nullptr;
     if (plan.share > 0) {

@@ -1,5 +1,5 @@
 """Steps whose keys are not split: the one-call form writes the output from the attention kernel, the three
-calls go through the workspace.  Same bits, and both against the oracle; sizes at the edges of the
+calls go through the workspace, whose partials are part of the contract.  Same bits, and both against the oracle; sizes at the edges of the
 256-row units (several of them start largest first)."""
 import dataclasses
 
@@ -61,3 +61,33 @@ def test_more_split_items_than_pairs(handle, L, n, splits):
         assert g["splits"] == splits
         check_cache(gs, r, L, n)
         check_output("bf16", g["out"], g["lse"], r["out"], r["lse"])
+
+
+@pytest.mark.parametrize("dtype,hq,hkv,d,L,n,splits", [
+    ("bf16", 28, 4, 128, 0, 256, 1),       # unsplit on CTA pairs
+    ("bf16", 28, 4, 128, 500, 1100, 1),    # ... on persistent ones
+    ("bf16", 28, 4, 128, 1000, 196, 3),
+    ("bf16", 28, 4, 128, 900, 10, 4),      # the one-CTA kernel
+    ("bf16", 28, 4, 128, 900, 1, 1),       # few rows
+    ("f32", 4, 2, 64, 300, 40, 2),
+])
+def test_workspace_holds_the_partials(handle, dtype, hq, hkv, d, L, n, splits):
+    # what evlnStepAttention leaves is documented: [S, Hkv, n G, D] outputs, then [S, Hkv, n G] log-sum-exps, all
+    # float.  A caller's own merge of them is what evlnStepCombine gives, up to its fp32 sums and one rounding.
+    cfg = W.StepConfig("partials", dtype, hq, hkv, d, L, n, 1e6, 0.5, 60 + L + n)
+    x = W.make_step_inputs(cfg)
+    gs = GpuStep(handle, dtype, hq, hkv, d, L + n, cfg.rope_theta, n, num_splits=splits)
+    gs.load_cache(x["k_cache"], x["v_cache"])
+    g = gs.step(L, x["q_new"], x["k_new"], x["v_new"])
+    p, rows = gs.params(L, n), n * hq // hkv
+    q_rot = g["q_rot"].reshape(n, hkv, hq // hkv, d).permute(1, 0, 2, 3).contiguous()
+    ws = torch.full((B.evlnStepWorkspaceSize(handle, p) // 4,), float("nan"), device="cuda:0")
+    B.evlnStepAttention(handle, p, q_rot, gs.k_cache, gs.v_cache, ws)
+    o = ws[:splits * hkv * rows * d].view(splits, hkv, rows, d).double()
+    lse = ws[splits * hkv * rows * d:][:splits * hkv * rows].view(splits, hkv, rows).double()
+    total = torch.logsumexp(lse, 0)
+    out = (torch.exp(lse - total).unsqueeze(-1) * o).sum(0)
+    to_tokens = lambda t: t.reshape(hkv, n, hq // hkv, -1).permute(1, 0, 2, 3).reshape(n, hq, -1)
+    eps = 2.0 ** -8 if dtype == "bf16" else 1e-6           # half a unit of the storage type, and the sums' last bits
+    assert bool(((g["out"].double() - to_tokens(out)).abs() <= eps * to_tokens(out).abs() + 1e-6).all())
+    assert float((g["lse"].double() - to_tokens(total)[..., 0]).abs().max()) <= 1e-5
