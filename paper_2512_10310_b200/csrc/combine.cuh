@@ -160,7 +160,52 @@ combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
     if (a.lse_out && lane == 0) a.lse_out[tok * Hq + h] = (wsum > 0.f) ? M + logf(wsum) : -INFINITY;
 }
 
-// Rows whose keys were not split are final (rounded, in output order) in the workspace: n * Hq rows of
+// The combine step of rows whose keys were not split: the one partial of a row is its output, rounded and put in its
+// place.  Same bits as the merge above (weight and sum are 1), without its chain of loads and shuffles.  Bound by the
+// boundary between two launches and then by L2.
+constexpr int kRoundVectors = 2;      // 16-byte vectors of the output per thread, all in flight
+
+template <typename T, int D>
+__global__ void __launch_bounds__(256)
+round_out_kernel(const CombineArgs a)
+{
+    constexpr int V = VecTraits<T>::kVec, kPerRow = D / V;
+    const int g = blockIdx.y;
+    const uint32_t i0 = blockIdx.x * (256u * kRoundVectors) + threadIdx.x;      // (rows per kv head are at most 2^24)
+    const float* part = a.o_part + (long)g * a.rows * D;
+    const int Hq = a.Hkv * a.G;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    float4 x[kRoundVectors][V / 4];
+    float lse[kRoundVectors];
+#pragma unroll
+    for (int k = 0; k < kRoundVectors; ++k) {
+        const uint32_t i = i0 + 256u * k, row = i / kPerRow;
+        if (row >= (uint32_t)a.rows) continue;
+#pragma unroll
+        for (int c = 0; c < V / 4; ++c) x[k][c] = *reinterpret_cast<const float4*>(part + (long)i * V + 4 * c);
+        if (a.lse_out && i % kPerRow == 0) lse[k] = a.lse_part[(long)g * a.rows + row];
+    }
+#pragma unroll
+    for (int k = 0; k < kRoundVectors; ++k) {
+        const uint32_t i = i0 + 256u * k, row = i / kPerRow;
+        if (row >= (uint32_t)a.rows) continue;
+        const uint32_t tok = fast_div(row, a.div_g);
+        const long at = (long)tok * Hq + g * a.G + (int)(row - tok * (uint32_t)a.G);
+        __align__(16) T y[V];
+#pragma unroll
+        for (int c = 0; c < V / 4; ++c) {
+            from_float(x[k][c].x, y[4 * c]);
+            from_float(x[k][c].y, y[4 * c + 1]);
+            from_float(x[k][c].z, y[4 * c + 2]);
+            from_float(x[k][c].w, y[4 * c + 3]);
+        }
+        *reinterpret_cast<uint4*>((T*)a.out + at * D + (i % kPerRow) * V) = *reinterpret_cast<const uint4*>(y);
+        if (a.lse_out && i % kPerRow == 0) a.lse_out[at] = lse[k];
+    }
+}
+
+// Unsplit paged batches: the rows are final (rounded, in output order) in the workspace: n * Hq rows of
 // 16-byte vectors and their log-sum-exps go to the caller's buffers.  HBM/L2-bound: a third of the bytes
 // that one set of fp32 partials would move.
 struct CopyOutArgs {

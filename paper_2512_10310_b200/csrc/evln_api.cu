@@ -706,6 +706,19 @@ evlnStatus_t launch_combine(evlnHandle_t h, const CombineArgs& args, int D, bool
     return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
 }
 
+// The combine step of an unsplit step on a contiguous cache.
+template <typename T>
+evlnStatus_t launch_round_out(evlnHandle_t h, const CombineArgs& args, int D, cudaStream_t st)
+{
+    CombineArgs a = args;
+    a.div_g = make_fast_div((uint32_t)a.G);
+    const long vectors = (long)a.rows * D / VecTraits<T>::kVec;
+    const dim3 grid((unsigned)((vectors + 256 * kRoundVectors - 1) / (256 * kRoundVectors)), a.Hkv);
+    const cudaError_t e = D == 128 ? launch_pdl(round_out_kernel<T, 128>, grid, dim3(256), 0, st, a)
+                                   : launch_pdl(round_out_kernel<T, 64>, grid, dim3(256), 0, st, a);
+    return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
+}
+
 // The combine step of rows that the attention kernel left final in the workspace (see CopyOutArgs).
 evlnStatus_t launch_copy_out(evlnHandle_t h, const CombineArgs& c, cudaStream_t st)
 {
@@ -1254,6 +1267,8 @@ evlnStatus_t evlnStepCombine(evlnHandle_t h, const evlnStepParams* p, const void
     a.out = out; a.lse_out = lse_out;
     a.Hkv = p->num_kv_heads; a.G = G; a.D = p->head_dim; a.rows = R; a.num_splits = S;
     cudaStream_t st = (cudaStream_t)stream;
+    if (S == 1 && p->dtype == EVLN_BF16) return launch_round_out<__nv_bfloat16>(h, a, p->head_dim, st);
+    if (S == 1) return launch_round_out<float>(h, a, p->head_dim, st);
     SimtTiles tiles;
     const SimtTiles* shares = nullptr;
     if (plan.share > 0) {
