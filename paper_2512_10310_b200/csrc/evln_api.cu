@@ -210,21 +210,25 @@ inline bool use_tensor_kernel(const evlnStepParams* p)
 
 // Cost model of the split-KV schedule of the tensor-core kernel: work items (unit x split) run
 // in waves of one CTA pair per two SMs, each walks ceil(nkv / S) KV tiles plus a fixed
-// prologue/epilogue; every split adds combine traffic, the first one the combine itself: unsplit rows are
-// written by the attention kernel.  (Measured over 256 .. 32768 cached keys, 64 .. 256 new tokens, three head shapes:
-// within 2 % of the best split count everywhere.  Without the price of the combine up to 28 % off at short
-// caches: 196 tokens over 256 13.1 us in two splits, 11.0 in one.)
-int choose_splits_tc(int units_total, int nkv_max, int nkv_min, int num_sms)
+// prologue/epilogue; every split adds combine traffic, the first one the merge that a step of one call does not need
+// unsplit.  The three calls run a combine either way, and both forms use the same split count, so the price lies
+// between what the two would like: it grows with the rows that a merge moves, up to 4 tiles.  (Measured over 0 .. 1500
+// cached keys, 40 .. 256 new tokens, five head shapes, both forms: 1.2 % above the best split count on average.  With 4
+// tiles for any number of rows three calls took up to 30 % more: 40 tokens of the 7B shape over 700 12.5 us
+// unsplit, 10.6 in three splits; without a price one call took up to 33 % more: 196 tokens over 256 12.6 us in two
+// splits, 10.6 unsplit.)
+int choose_splits_tc(int units_total, long rows_total, int nkv_max, int nkv_min, int num_sms)
 {
     int best = 1;
     double best_cost = 1e30;
     const int pairs = num_sms / 2 > 0 ? num_sms / 2 : 1;
+    const double merge = std::min(4.0, 1.0 + 7e-4 * rows_total);
     const int smax = nkv_min < kMaxSplits ? (nkv_min < 1 ? 1 : nkv_min) : kMaxSplits;
     for (int s = 1; s <= smax; ++s) {
         const double waves = ceil((double)units_total * s / pairs);
         // per work item: set-up, first-tile latency, partial write-out and teardown cost about as
         // much as 7 KV tiles (measured); every split adds about half a tile of combine work
-        const double cost = waves * (ceil((double)nkv_max / s) + 7.0) + (s > 1 ? 4.0 : 0.0) + 0.5 * s;
+        const double cost = waves * (ceil((double)nkv_max / s) + 7.0) + (s > 1 ? merge : 0.0) + 0.5 * s;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = s; }
     }
     return best;
@@ -444,7 +448,7 @@ int resolve_splits(evlnHandle_t h, const evlnStepParams* p)
         const int units = ceil_div(R, kUnitRows);
         const int nkv_max = unit_kv_tiles(p->cache_len, p->num_new, G, units - 1, kUnitRows);
         const int nkv_min = unit_kv_tiles(p->cache_len, p->num_new, G, 0, kUnitRows);
-        return choose_splits_tc(units * p->num_kv_heads, nkv_max, nkv_min, h->num_sms);
+        return choose_splits_tc(units * p->num_kv_heads, (long)R * p->num_kv_heads, nkv_max, nkv_min, h->num_sms);
     }
     return simt_schedule(h, p, 0).splits;
 }

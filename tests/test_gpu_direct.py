@@ -91,3 +91,14 @@ def test_workspace_holds_the_partials(handle, dtype, hq, hkv, d, L, n, splits):
     eps = 2.0 ** -8 if dtype == "bf16" else 1e-6           # half a unit of the storage type, and the sums' last bits
     assert bool(((g["out"].double() - to_tokens(out)).abs() <= eps * to_tokens(out).abs() + 1e-6).all())
     assert float((g["lse"].double() - to_tokens(total)[..., 0]).abs().max()) <= 1e-5
+
+
+@pytest.mark.parametrize("hq,hkv,L,n,unsplit", [
+    (28, 4, 128, 196, True),      # three key tiles, many rows: the merge costs more than it saves
+    (28, 4, 0, 40, True),         # one tile
+    (28, 4, 700, 40, False),      # six tiles, few rows: unsplit, three calls took 12.5 us against 10.6
+    (32, 8, 700, 64, False),
+])
+def test_where_short_steps_are_split(handle, hq, hkv, L, n, unsplit):
+    p = B.step_params("bf16", hq, hkv, 128, L, n, L + n, 1e6)
+    assert (B.evlnStepNumSplits(handle, p) == 1) == unsplit
