@@ -318,7 +318,8 @@ evlnStatus_t evlnPackedForward(evlnHandle_t handle, const evlnPackedParams* para
  * clears it for the current device.
  * Limits and errors: parameters whose split workspace (evlnStepWorkspaceSize) exceeds
  * EVLN_NOALLOC_SCRATCH_BYTES are rejected with EVLN_WORKSPACE_TOO_SMALL and nothing is
- * launched; other errors as for evlnStepAttention / evlnStepCombine.
+ * launched, except that the SIMT kernel with num_splits = 0 takes as many splits as fit
+ * (rejected only if one does not); other errors as for evlnStepAttention / evlnStepCombine.
  * Sharing: every call on a device uses the same scratch array, which keeps the previous
  * call's contents (each call overwrites every partial it later reads, so nothing needs
  * clearing).  Two such calls that overlap on the GPU (different streams, or different host

@@ -380,7 +380,8 @@ void fill_simt_tiles(const evlnStepParams* p, SimtTiles* t)
         t->off[rb + 1] = t->off[rb] + (rb < blocks ? ceil_div(p->cache_len + last / G + 1, kSimtKeys) : 0);
     }
 }
-SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits)
+// (most_splits: bound on the splits of the library's own choice)
+SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits, int most_splits = kMaxSplits)
 {
     const int R = p->num_new * (p->num_q_heads / p->num_kv_heads);
     const int tiles = ceil_div(p->cache_len + p->num_new, kSimtKeys);
@@ -388,7 +389,7 @@ SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits)
     const double split_us = 0.3 + 2.0 * R * p->num_kv_heads * p->head_dim * 4 / 5e6;
     SimtSchedule best = {8, splits > 0 ? splits : 1, 0};
     double best_cost = 1e30;
-    const int smax = tiles < kMaxSplits ? tiles : kMaxSplits;
+    const int smax = tiles < most_splits ? tiles : most_splits;
     for (int rpt = 8; rpt >= 2; rpt -= 6) {
         const long row_blocks = (long)ceil_div(R, 16 * rpt) * p->num_kv_heads;
         for (int s = splits > 0 ? splits : 1; s <= (splits > 0 ? splits : smax); ++s) {
@@ -410,11 +411,7 @@ SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits)
         if (share < ceil_div(most, kMaxSplits - 1)) share = ceil_div(most, kMaxSplits - 1);
         const int s = ceil_div(most - 1, share) + 1;
         const double cost = share * 13.3 * d + 7.0 + 4.0 * ceil_div(share, t.off[1]) + split_us * (1.0 + (double)most / share);
-        // (a step that fits the scratch of the allocation-free call goes on fitting it)
-        const size_t limit = EVLN_NOALLOC_SCRATCH_BYTES;
-        const bool fits = partial_bytes(s, p->num_kv_heads, R, p->head_dim) <= limit ||
-                          partial_bytes(best.splits, p->num_kv_heads, R, p->head_dim) > limit;
-        if (fits && cost < best_cost - 1e-9) best = {8, s, share};
+        if (s <= most_splits && cost < best_cost - 1e-9) best = {8, s, share};
     }
     return best;
 }
@@ -1951,8 +1948,17 @@ extern "C" evlnStatus_t evlnStepAttentionNoAlloc(const evlnStepParams* p, const 
     size_t need = 0;
     s = evlnStepWorkspaceSize(h, p, &need);
     if (s != EVLN_OK) return s;
-    if (need > (size_t)EVLN_NOALLOC_SCRATCH_BYTES) return EVLN_WORKSPACE_TOO_SMALL;
     if (p->num_new == 0) return EVLN_OK;
+    evlnStepParams fitting = *p;
+    if (need > (size_t)EVLN_NOALLOC_SCRATCH_BYTES) {
+        // The fp32 kernel splits to fill the chip, up to 2.3 times faster than what fits here for large steps, so it is
+        // this call that makes do with fewer splits.  (The schedules of the other kernels take about as few as they can.)
+        const size_t one = partial_bytes(1, p->num_kv_heads, (long)p->num_new * (p->num_q_heads / p->num_kv_heads), p->head_dim);
+        const int fit = (int)(EVLN_NOALLOC_SCRATCH_BYTES / one);
+        if (p->num_splits > 0 || use_tensor_kernel(p) || fit < 1) return EVLN_WORKSPACE_TOO_SMALL;
+        fitting.num_splits = simt_schedule(h, p, 0, fit).splits;
+        p = &fitting;
+    }
     if (!out || !aligned16(out)) return EVLN_INVALID_VALUE;
     DirectOut direct = {out, lse_out, false};
     s = step_attention(h, p, q_rot, k_cache, v_cache, d->scratch, (size_t)EVLN_NOALLOC_SCRATCH_BYTES, stream,

@@ -87,3 +87,38 @@ def test_no_alloc_rejects_oversized_problems():
     with pytest.raises(B.EvlnError) as e:
         B.evlnStepAttentionNoAlloc(p, buf, buf, buf, buf, None)
     assert e.value.status == B.EVLN_WORKSPACE_TOO_SMALL
+
+
+@pytest.mark.parametrize("hq,hkv,d,L,n", [
+    (4, 1, 128, 2441, 3561),      # with a workspace five splits, 36.7 MB; one split is 7.3 MB
+    (16, 1, 64, 18, 2974),        # three of 12.4 MB
+    (32, 16, 128, 100, 2000),     # 33.0 MB in one split: just inside
+])
+def test_no_alloc_takes_the_splits_that_fit(hq, hkv, d, L, n):
+    # steps of the SIMT kernel whose own split count needs more than the built-in scratch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    dev = "cuda:0"
+    torch.cuda.set_device(0)
+    handle = B.evlnCreate(0)
+    try:
+        gen = torch.Generator(device=dev).manual_seed(L + n)
+        p = B.step_params("f32", hq, hkv, d, L, n, L + n, 1e4)
+        assert B.evlnStepWorkspaceSize(handle, p) > 32 << 20
+        kc, vc = (torch.randn((hkv, L + n, d), generator=gen, device=dev) for _ in range(2))
+        q_rot = torch.randn((hkv, n * hq // hkv, d), generator=gen, device=dev)
+        ws = torch.empty(B.evlnStepWorkspaceSize(handle, p), dtype=torch.uint8, device=dev)
+        want, out = (torch.full((n, hq, d), float("nan"), device=dev) for _ in range(2))
+        want_lse, lse = (torch.full((n, hq), float("nan"), device=dev) for _ in range(2))
+        B.evlnStepAttention(handle, p, q_rot, kc, vc, ws)
+        B.evlnStepCombine(handle, p, ws, want, want_lse)
+        B.evlnStepAttentionNoAlloc(p, q_rot, kc, vc, out, lse)
+        torch.cuda.synchronize()
+        # (two fp32 evaluations of the same step: each within the 1e-5 of the fp32 gates)
+        assert (out - want).abs().max().item() <= 2e-5 and (lse - want_lse).abs().max().item() <= 2e-5
+        p = B.step_params("f32", hq, hkv, d, L, n, L + n, 1e4, num_splits=32)
+        with pytest.raises(B.EvlnError) as e:                 # an explicit split count is taken as it is
+            B.evlnStepAttentionNoAlloc(p, q_rot, kc, vc, out, lse)
+        assert e.value.status == B.EVLN_WORKSPACE_TOO_SMALL
+    finally:
+        B.evlnDestroy(handle)
