@@ -241,16 +241,46 @@ inline bool use_solo_kernel(const evlnStepParams* p)
     return use_tensor_kernel(p) && (long)p->num_new * (p->num_q_heads / p->num_kv_heads) <= kTileM;
 }
 
-// At most 32 rows per kv head (up to four action tokens with seven query heads per kv head): the kernel
-// whose products stay in registers (attn_few.cuh).  Not with two row tiles and long caches of eight or more kv
-// heads: clusters of 16 blocks for all heads do not fit the device at once, and mma.sync on half of the SMs is
-// slower than the one-CTA kernel on all of them (32 rows, 8 heads, 4292 keys 14.6 us against 12.3, 20656 keys
-// 25.2 against 23.0; 1500 keys 9.7 against 10.0; 4 heads 9.8 against 10.8 and 17.4 against 17.3).
-inline bool use_few_kernel(const evlnStepParams* p)
+// Split schedule of the one-CTA-per-item kernel, in microseconds: a CTA takes 0.9 per KV tile unless HBM (all
+// of K and V at most of its rate) takes longer, and a split adds partials of every row to write and merge.
+// (Measured over 500 .. 32000 cached keys, 4 and 8 kv heads, 35 .. 128 rows each: within 3 % of the best split
+// count everywhere, 0.2 % on average.  Spreading over as many SMs as there are cost up to 19 % with 8 kv
+// heads: 8 tokens over 4292 keys 15.1 us with 18 splits, 12.7 with 12.)
+int choose_splits_solo(int Hkv, int R, int T, int num_sms)
 {
-    const long rows = (long)p->num_new * (p->num_q_heads / p->num_kv_heads);
+    const int nkv = ceil_div(T, kTileN);
+    const double hbm_us = 512.0 * T * Hkv / 6.4e6, split_us = 0.1 + 1e-4 * R * Hkv;
+    int best = 1;
+    double best_cost = 1e30;
+    const int smax = nkv < kMaxSplits ? (nkv < 1 ? 1 : nkv) : kMaxSplits;
+    for (int s = 1; s <= smax; ++s) {
+        const double waves = ceil((double)Hkv * s / num_sms), work = 0.9 * waves * ceil_div(nkv, s);
+        const double cost = (work > 0.8 * hbm_us ? work : 0.8 * hbm_us) + split_us * s;
+        if (cost < best_cost - 1e-9) { best_cost = cost; best = s; }
+    }
+    return best;
+}
+
+// At most 32 rows per kv head (up to four action tokens with seven query heads per kv head): the kernel
+// whose products stay in registers (attn_few.cuh).  Not with two row tiles where clusters of 16 blocks for all heads do
+// not fit the device at once, or do not cover it: mma.sync on half of the SMs is slower than the one-CTA kernel on all of
+// them.  Eight and more kv heads, from 3072 keys on: 32 rows of 8 heads 4292 keys 12.4 us against 11.4 (of 16 heads
+// 14.9 and 13.3), 20656 keys 21.3 and 19.3; 1500 keys 9.5 and 9.9.  From 24576 keys on also four heads with more than 24
+// rows (28 rows, 32768 keys 19.3 and 18.0; 21 rows, 28000 keys 16.0 and 16.6; seven heads 21.9 and 22.8), and
+// four to seven heads with too many tokens for the one-launch step (17 rows of 6 heads, 32768 keys 25.4 and 22.9).
+// A caller who passes on the split count that evlnStepNumSplits reports gets the library's own kernel; one who asks
+// for so few that they leave half of the SMs idle gets the few-row kernel, whose clusters fill them (64 query heads, 4
+// tokens over 9000 keys in one split 16.2 us against 59.6; 8 tokens of 32 query heads over 8000 keys in 12 splits 15.3
+// and 14.3).
+inline bool use_few_kernel(evlnHandle_t h, const evlnStepParams* p)
+{
+    const int Hkv = p->num_kv_heads, keys = p->cache_len + p->num_new;
+    const long rows = (long)p->num_new * (p->num_q_heads / Hkv);
     if (!use_tensor_kernel(p) || rows > kFewRows) return false;
-    return rows <= 16 || p->num_kv_heads < 8 || p->cache_len + p->num_new < 3072 || p->num_splits > 0;
+    if (rows <= 16 || Hkv < 4 || keys < (Hkv >= 8 ? 3072 : 24576)) return true;
+    if (Hkv < 8 && p->num_new <= kFewFusedTokens && (Hkv > 4 || rows <= 24)) return true;
+    return p->num_splits > 0 && (long)p->num_splits * Hkv <= h->num_sms / 2 &&
+           p->num_splits < choose_splits_solo(Hkv, (int)rows, keys, h->num_sms);
 }
 inline int few_row_tiles(int rows) { return rows <= 16 ? 1 : 2; }
 
@@ -333,26 +363,6 @@ cudaError_t launch_few(const FewPlan& f, int rows, cudaStream_t st, const CUtens
     const NoLens nl = {};
     if (mt == 1) return cudaLaunchKernelEx(&cfg, attn_few_kernel<1, false, FUSED, NoLens>, tm_k, tm_v, a, nl);
     return cudaLaunchKernelEx(&cfg, attn_few_kernel<2, false, FUSED, NoLens>, tm_k, tm_v, a, nl);
-}
-
-// Split schedule of the one-CTA-per-item kernel, in microseconds: a CTA takes 0.9 per KV tile unless HBM (all
-// of K and V at most of its rate) takes longer, and a split adds partials of every row to write and merge.
-// (Measured over 500 .. 32000 cached keys, 4 and 8 kv heads, 35 .. 128 rows each: within 3 % of the best split
-// count everywhere, 0.2 % on average.  Spreading over as many SMs as there are cost up to 19 % with 8 kv
-// heads: 8 tokens over 4292 keys 15.1 us with 18 splits, 12.7 with 12.)
-int choose_splits_solo(int Hkv, int R, int T, int num_sms)
-{
-    const int nkv = ceil_div(T, kTileN);
-    const double hbm_us = 512.0 * T * Hkv / 6.4e6, split_us = 0.1 + 1e-4 * R * Hkv;
-    int best = 1;
-    double best_cost = 1e30;
-    const int smax = nkv < kMaxSplits ? (nkv < 1 ? 1 : nkv) : kMaxSplits;
-    for (int s = 1; s <= smax; ++s) {
-        const double waves = ceil((double)Hkv * s / num_sms), work = 0.9 * waves * ceil_div(nkv, s);
-        const double cost = (work > 0.8 * hbm_us ? work : 0.8 * hbm_us) + split_us * s;
-        if (cost < best_cost - 1e-9) { best_cost = cost; best = s; }
-    }
-    return best;
 }
 
 size_t partial_bytes(int splits, int Hkv, long rows, int D)
@@ -438,7 +448,7 @@ int resolve_splits(evlnHandle_t h, const evlnStepParams* p)
     const int G = p->num_q_heads / p->num_kv_heads;
     const int R = p->num_new * G;
     const int T = p->cache_len + p->num_new;
-    if (use_few_kernel(p)) return few_plan(h, p).splits;
+    if (use_few_kernel(h, p)) return few_plan(h, p).splits;
     if (use_solo_kernel(p))
         return choose_splits_solo(p->num_kv_heads, R, T, h->num_sms);
     if (use_tensor_kernel(p)) {
@@ -1155,7 +1165,7 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
     const float scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)D);
     cudaStream_t st = (cudaStream_t)stream;
 
-    if (use_few_kernel(p)) {
+    if (use_few_kernel(h, p)) {
         return step_few(h, p, q_rot, k_cache, v_cache, o_part, lse_part, nullptr, st);
     } else if (use_tensor_kernel(p)) {
         const int T = p->cache_len + p->num_new;
@@ -1295,7 +1305,7 @@ evlnStatus_t evlnStep(evlnHandle_t h, const evlnStepParams* p, const void* q_new
     const long rows = (long)p->num_new * (p->num_q_heads / p->num_kv_heads);
     if (workspace_bytes < partial_bytes(resolve_splits(h, p), p->num_kv_heads, rows, p->head_dim))
         return EVLN_WORKSPACE_TOO_SMALL;
-    if (use_few_kernel(p) && p->num_new <= kFewFusedTokens &&
+    if (use_few_kernel(h, p) && p->num_new <= kFewFusedTokens &&
         !step_buffers_shared(p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, out, lse_out)) {
         s = check_rope_append(h, p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, k_cache, v_cache);
         if (s != EVLN_OK) return s;

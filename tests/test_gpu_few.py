@@ -36,6 +36,8 @@ def handle():
     (64, 8, 3068, 4, 0),          # 32 rows over a longer cache of eight kv heads: the one-CTA kernel
     (28, 4, 9000, 3, 0),          # more stages per block than the ring holds
     (7, 1, 20000, 1, 0),          # one kv head: the library splits
+    (6, 6, 25000, 17, 0),         # 17 rows over a long cache of six kv heads: the one-CTA kernel
+    (64, 8, 4292, 4, 1),          # 32 rows of eight kv heads in fewer splits than fill the SMs: clusters do
     (28, 4, 500, 1, 5),           # splits of one and two stages: clusters of one block
     (28, 4, 100, 1, 9),           # more splits than stages: empty splits
 ])
@@ -53,6 +55,28 @@ def test_step_of_few_rows_against_oracle(handle, hq, hkv, L, n, splits):
         bits.append((g["out"].view(torch.int16), g["lse"], g["q_rot"].reshape(-1).view(torch.int16), gs.k_cache.view(torch.int16)))
     for a, b in zip(*bits):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("hq,hkv,L,n", [
+    (64, 8, 4292, 4),             # 32 rows of eight kv heads: the one-CTA kernel
+    (28, 4, 24600, 4),            # 28 rows of four, from 24576 keys on
+    (28, 4, 24600, 3),            # ... 21 rows: the few-row kernel
+    (28, 4, 20000, 4),            # ... and below
+    (28, 4, 4292, 8),             # 56 rows
+    (28, 4, 4096, 196),           # CTA pairs
+])
+def test_reported_split_count_passed_on_gives_the_same_bits(handle, hq, hkv, L, n):
+    gen = torch.Generator(device="cuda:0").manual_seed(L + n)
+    q, k, v = (torch.randn((n, h, 128), generator=gen, device="cuda:0").to(torch.bfloat16) for h in (hq, hkv, hkv))
+    kc, vc = (torch.randn((hkv, L, 128), generator=gen, device="cuda:0").to(torch.bfloat16) for _ in range(2))
+    bits, splits = [], 0
+    for _ in range(2):
+        gs = GpuStep(handle, "bf16", hq, hkv, 128, L + n, 1e6, n, num_splits=splits, fused=True)
+        gs.k_cache[:, :L], gs.v_cache[:, :L] = kc, vc
+        g = gs.step(L, q, k, v)
+        splits = g["splits"]
+        bits.append((g["out"].view(torch.int16), g["lse"]))
+    assert all(torch.equal(a, b) for a, b in zip(*bits))
 
 
 @pytest.mark.parametrize("lens,new,chunk", [
