@@ -514,6 +514,7 @@ void longest_first(int batch, const int* lens, const int* offs, int* order)
 // (ascending), so an episode costs a few steps however many items it has.
 constexpr int kMaxPairs = 128;
 constexpr int kNextItemTiles = 5;        // from a pair's last product of an item to the first of its next one, in KV tiles
+constexpr double kSplitTiles = 0.3;      // what a split adds to the merge of its rows, in KV tiles
 double finish_time(int pairs, int G, int Hkv, int batch, const int* lens, const int* offs, const int* order, int chunk)
 {
     struct Run { double load; int count; } runs[kMaxPairs];
@@ -568,18 +569,25 @@ double finish_time(int pairs, int G, int Hkv, int batch, const int* lens, const 
 // of 16384 and 8000 tokens 104 and 91 (three and two ways); four of 4000 .. 16000 tokens 128 unsplit, 105 in up to four.
 int choose_chunk(int pairs, int G, int Hkv, int batch, const int* lens, const int* offs, const int* order, int nkv_max)
 {
-    long unsplit = 0;
-    for (int b = 0; b < batch; ++b) unsplit += (long)ceil_div((offs[b + 1] - offs[b]) * G, kUnitRows) * Hkv;
+    long unsplit = 0, tiles = 0;
+    for (int b = 0; b < batch; ++b) {
+        const int n = offs[b + 1] - offs[b], units = ceil_div(n * G, kUnitRows);
+        unsplit += (long)units * Hkv;
+        for (int u = 0; u < units; ++u) tiles += (long)unit_kv_tiles(lens[b], n, G, u, kUnitRows) * Hkv;
+    }
     if (unsplit >= 8L * pairs) return nkv_max;
-    const double rows = (double)offs[batch] * G * Hkv;
+    const double rows = (double)offs[batch] * G * Hkv, least = ((double)tiles + (double)kNextItemTiles * unsplit) / pairs;
     int best = nkv_max;
     double best_cost = 1e30;
-    for (int splits = 1; splits <= 8 && splits <= nkv_max; ++splits) {
+    for (int splits = 1, last = 0; splits <= kMaxSplits && splits <= nkv_max; ++splits) {
         const int chunk = ceil_div(nkv_max, splits);
+        if (chunk == last) continue;
+        last = chunk;
         // a KV tile takes a pair about 0.87 us with all of them at work; partials move at about 5.5 TB/s, each row
-        // written and read
-        const double moved = rows * (splits == 1 ? 0.5 : splits) * 1024.0 / 5.5e6 / 0.87;
-        const double cost = finish_time(pairs, G, Hkv, batch, lens, offs, order, chunk) + moved;
+        // written and read; and every part of a row makes its merge longer, whatever the rows
+        const double merge = rows * (splits == 1 ? 0.5 : splits) * 1024.0 / 5.5e6 / 0.87 + kSplitTiles * splits;
+        if (least + merge >= best_cost) break;       // (no pair is done before its share, and the merge only grows)
+        const double cost = finish_time(pairs, G, Hkv, batch, lens, offs, order, chunk) + merge;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = chunk; }
     }
     return best;

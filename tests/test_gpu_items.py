@@ -58,3 +58,22 @@ def test_paged_batch_of_few_rows_in_equal_shares(handle, hq, hkv, lens, new):
                                      x["new_offsets"], cfg.rope_theta, storage="bf16")
     check_output("bf16", out, lse, ref_out, ref_lse)
     _check_pools(x, cfg, k_pool, v_pool, okp, ovp)
+
+
+@pytest.mark.parametrize("hq,hkv,length,new,least", [
+    (7, 1, 20000, 64, 12),        # two row units of one kv head: in up to 8 parts 26.0 us, in as many as pay 18.7
+    (28, 4, 9000, 20, 9),
+    (28, 4, 700, 196, 1),
+])
+def test_paged_frame_of_one_long_episode(handle, hq, hkv, length, new, least):
+    cfg = dataclasses.replace(W.PAGED_B16, name="long", num_q_heads=hq, num_kv_heads=hkv, batch=1, seed=140 + new)
+    x = W.make_paged_inputs(cfg, [length], [new])
+    p = B.paged_params(hq, hkv, 128, 1, 64, x["num_pages"], len(x["page_table"][0]), cfg.rope_theta)
+    parts = B.evlnPagedWorkspaceSize(handle, p, [length], [0, new]) // (new * hq * 129 * 4)
+    assert parts >= least
+    out, lse, k_pool, v_pool = _gpu_paged(handle, cfg, x)
+    okp, ovp = f64(x["k_pool"]), f64(x["v_pool"])
+    ref_out, ref_lse = so.step_paged(f64(x["q_new"]), f64(x["k_new"]), f64(x["v_new"]), okp, ovp, x["page_table"], [length],
+                                     x["new_offsets"], cfg.rope_theta, storage="bf16")
+    check_output("bf16", out, lse, ref_out, ref_lse)
+    _check_pools(x, cfg, k_pool, v_pool, okp, ovp)
