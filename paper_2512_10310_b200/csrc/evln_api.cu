@@ -116,7 +116,8 @@ cudaError_t prepare_few()
 // Shared-memory limits of the kernels that take more than the default, on the current device.
 cudaError_t prepare_kernels()
 {
-    const std::pair<const void*, int> tc[5] = {{(const void*)attn_pair_kernel, kTcSmemBytes},
+    const std::pair<const void*, int> tc[6] = {{(const void*)attn_pair_kernel, kTcSmemBytes},
+                                               {(const void*)attn_paged_pair_kernel, kTcSmemBytes},
                                                {(const void*)attn_persistent_kernel<false, NoLens>, kPersistSmemBytes},
                                                {(const void*)attn_persistent_kernel<true, PagedLens>, kPersistSmemBytes},
                                                {(const void*)attn_solo_kernel, kSoloSmemBytes},
@@ -144,7 +145,7 @@ cudaError_t prepare_kernels()
 bool attention_register_pool_ok()
 {
     cudaFuncAttributes fa;
-    const void* kernels[5] = {(const void*)attn_pair_kernel, (const void*)attn_persistent_kernel<false, NoLens>, (const void*)attn_persistent_kernel<true, PagedLens>,
+    const void* kernels[6] = {(const void*)attn_pair_kernel, (const void*)attn_paged_pair_kernel, (const void*)attn_persistent_kernel<false, NoLens>, (const void*)attn_persistent_kernel<true, PagedLens>,
                               (const void*)attn_solo_kernel, (const void*)attn_packed_kernel};
     for (const void* k : kernels) {
         if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return false;
@@ -1473,6 +1474,10 @@ evlnStatus_t evlnPagedStepAttention(evlnHandle_t h, const evlnPagedParams* p, co
     if (smax == 1) {
         d.out = (__nv_bfloat16*)workspace;
         d.lse_out = a.lse_part;
+    }
+    if (items <= persistent_pairs(h, items)) {
+        const cudaError_t e = launch_pair_pdl(attn_paged_pair_kernel, dim3(2 * (unsigned)items), kTcSmemBytes, (cudaStream_t)stream, tm_q, tm_k, tm_v, a, bl, d);
+        return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
     }
     ItemTable table;
     int k = 0, place = -1, unit = 0, units = 0, slot = 0, splits = 0, tiles = 0;     // in the order decode_work numbers them

@@ -23,15 +23,17 @@ def handle():
     B.evlnDestroy(h)
 
 
-@pytest.mark.parametrize("batch", [
-    4,       # 64 work items: fewer than SM pairs
-    20,      # 320: dealt to the pairs by the item table
-    64,      # 1024: more than the table holds, dealt in turn
-    160,     # 2560: more than the pairs keep, two launches
+@pytest.mark.parametrize("batch,heads", [
+    (4, 16),       # 64 work items: fewer than SM pairs, a launch without persistent pairs
+    (37, 2),       # 74: as many as pairs
+    (38, 2),       # 76: more
+    (20, 16),      # 320: dealt to the pairs by the item table
+    (64, 16),      # 1024: more than the table holds, dealt in turn
+    (160, 16),     # 2560: more than the pairs keep, two launches
 ])
-def test_paged_batch_of_many_work_items(handle, batch):
+def test_paged_batch_of_many_work_items(handle, batch, heads):
     # one query head per kv head and 33 tokens: one unit per (episode, kv head) for the tile kernel
-    cfg = dataclasses.replace(W.PAGED_B16, name=f"many_{batch}", num_q_heads=16, num_kv_heads=16, batch=batch, seed=90 + batch)
+    cfg = dataclasses.replace(W.PAGED_B16, name=f"many_{batch}", num_q_heads=heads, num_kv_heads=heads, batch=batch, seed=90 + batch)
     lens = [(37 * b) % 301 for b in range(batch)]
     x = W.make_paged_inputs(cfg, lens, [33] * batch)
     out, lse, k_pool, v_pool = _gpu_paged(handle, cfg, x)
