@@ -16,7 +16,17 @@ from ctypes import (POINTER, Structure, byref, c_char_p, c_double, c_float, c_in
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
 LIB_PATH = os.path.join(_PKG, "lib", "libevln.so")
-NATIVE_PATH = os.path.join(_PKG, "lib", "_evln_native.so")
+
+
+def native_path() -> str:
+    """Where the CPython module of the hot calls lies.  It reads tensors through torch's C++ classes, so a binary is good
+    for the Python ABI and the torch version (which fixes the C++ ABI) that it was built against: both are in its name."""
+    import importlib.metadata
+    import sysconfig
+    return os.path.join(_PKG, "lib", f"_evln_native.{sysconfig.get_config_var('SOABI')}.torch{importlib.metadata.version('torch')}.so")
+
+
+NATIVE_PATH = native_path()
 _SOURCES = ["evln_api.cu", "attn_pair.cuh", "attn_few.cuh", "attn_simt.cuh", "combine.cuh", "rope_append.cuh",
             "common.cuh", "ptx_sm100.cuh", "gather_rope.cuh", "timeline_debug.cuh"]
 
@@ -108,7 +118,7 @@ def _build_cuda(src_dir, verbose):
 
 
 def _build_native(src):
-    """The CPython module of the hot calls (``lib/_evln_native.so``), against torch's C++ headers."""
+    """The CPython module of the hot calls (``NATIVE_PATH``), against torch's C++ headers."""
     import sysconfig
 
     import torch
@@ -351,7 +361,7 @@ def evlnStoreFetch(handle, params, h_k_store, h_v_store, src_slot, length, k_sto
 
 # ---- the calls a model makes per layer and step ----------------------------------------------
 
-# Built-ins of lib/_evln_native.so (csrc/py_native.cpp).  Through ctypes an evlnStep cost 16.5 us of
+# Built-ins of the module at NATIVE_PATH (csrc/py_native.cpp).  Through ctypes an evlnStep cost 16.5 us of
 # host time, twice what its three launches take, and more than the GPU needs for a step of a few tokens.
 kHotCalls = ("evlnRopeTable", "evlnRopeAppend", "evlnStepAttention", "evlnStepCombine", "evlnStep",
              "evlnPagedRopeAppend", "evlnPagedStepAttention", "evlnPagedStepCombine", "evlnPackedForward",

@@ -84,3 +84,22 @@ def test_null_handle_is_rejected(lib):
     v = ctypes.c_size_t(0)
     assert lib.evlnStepWorkspaceSize(None, ctypes.byref(p), ctypes.byref(v)) == B.EVLN_INVALID_VALUE
     assert lib.evlnDestroy(None) == B.EVLN_INVALID_VALUE
+
+
+def test_native_module_belongs_to_this_python_and_torch(lib, monkeypatch):
+    # a binary built against another torch is neither reused nor loaded: its name is another one
+    import importlib.metadata
+    import sysconfig
+
+    import torch
+    assert torch.__version__ in B.NATIVE_PATH and sysconfig.get_config_var("SOABI") in B.NATIVE_PATH
+    assert os.path.exists(B.NATIVE_PATH)
+    monkeypatch.setattr(importlib.metadata, "version", lambda name: "0.0.1")
+    other = B.native_path()
+    assert other != B.NATIVE_PATH and not os.path.exists(other)
+    built = []
+    monkeypatch.setattr(B, "NATIVE_PATH", other)
+    monkeypatch.setattr(B, "_build_native", built.append)
+    monkeypatch.setattr(B, "_build_cuda", lambda *a: None)
+    B.build_library()
+    assert len(built) == 1
