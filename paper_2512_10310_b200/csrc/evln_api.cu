@@ -626,25 +626,27 @@ void batch_schedule(int num_sms, int G, int Hkv, int batch, const int* lens, con
 // Stages of one kv head of an episode in the few-row kernel (none without new tokens).
 inline int few_stages(int L, int n) { return n > 0 ? ceil_div(L + n, kFewKeys) : 0; }
 
-// A batch whose episodes all bring few rows (action tokens): the few-row kernel, one block per work item.
-bool paged_few(const evlnPagedParams* p, const int* offs)
+// Most rows per kv head that an episode of the batch brings.
+long most_rows(const evlnPagedParams* p, const int* offs)
 {
-    const int G = p->num_q_heads / p->num_kv_heads;
-    for (int b = 0; b < p->batch; ++b)
-        if ((long)(offs[b + 1] - offs[b]) * G > kFewRows) return false;
-    return true;
+    int n = 0;
+    for (int b = 0; b < p->batch; ++b) n = std::max(n, offs[b + 1] - offs[b]);
+    return (long)n * (p->num_q_heads / p->num_kv_heads);
 }
 
 struct PagedPlan {
+    bool few;                // few-row kernel (a block per work item or per equal share)
     int chunk, share;        // KV tiles per work item, or (share > 0) 64-key stages per block
     int splits;              // most partials of a row
     long items;              // work items, or blocks
 };
 PagedPlan paged_schedule(evlnHandle_t h, const evlnPagedParams* p, const int* lens, const int* offs)
 {
-    PagedPlan plan = {1, 0, 1, 0};
+    PagedPlan plan = {false, 1, 0, 1, 0};
     const int Hkv = p->num_kv_heads;
-    if (paged_few(p, offs) && p->kv_chunk_tiles == 0) {
+    const long rows = most_rows(p, offs);
+    if (rows <= kFewRows && p->kv_chunk_tiles == 0) {
+        plan.few = true;
         // An equal share of all stages for every SM, but no row in more parts than a warp merges, nor in more
         // than the merge is worth: a stage takes about 0.41 us, another part of the longest row 0.2.
         long total = 0;
@@ -666,6 +668,11 @@ PagedPlan paged_schedule(evlnHandle_t h, const evlnPagedParams* p, const int* le
     longest_first(p->batch, lens, offs, order);
     batch_schedule(h->num_sms, p->num_q_heads / Hkv, Hkv, p->batch, lens, offs, order, false, p->kv_chunk_tiles, &plan.chunk, &plan.splits,
                    &plan.items);
+    // Few rows in work items of the caller's size: a block of the few-row kernel takes 0.8 us per 128-key tile of one
+    // row tile and 1.08 of two, a CTA pair 0.75.  So two row tiles run on pairs where the items are long and there is a
+    // pair for each (28/4 heads, 4 episodes of up to 9000 keys, 4 tokens each in items of 64 tiles 39.5 us against 47.0,
+    // of 8 tiles 18.6 against 15.9; 40 episodes of 4000 keys, items of 32 tiles 104 against 89).
+    plan.few = rows <= kFewRows && (rows <= 16 || plan.chunk <= 8 || plan.items > h->num_sms / 2);
     return plan;
 }
 
@@ -1400,15 +1407,14 @@ evlnStatus_t evlnPagedStepAttention(evlnHandle_t h, const evlnPagedParams* p, co
     if (workspace_bytes < partial_bytes(smax, p->num_kv_heads, rows, 128)) return EVLN_WORKSPACE_TOO_SMALL;
     if (items <= 0 || items * (plan.share > 0 ? plan.share : 1) > 0x3fffffffL) return EVLN_NOT_SUPPORTED;
 
-    if (paged_few(p, h_new_offsets)) {
+    if (plan.few) {
         CUtensorMap tm_k, tm_v;
         cuuint64_t dims[4] = {128, 64, (cuuint64_t)p->num_kv_heads, (cuuint64_t)p->num_pages};
         cuuint64_t strides[3] = {256, 64 * 256, (cuuint64_t)p->num_kv_heads * 64 * 256};
         cuuint32_t box[4] = {64, kFewKeys, 1, 1};
         if (!encode_map(h, &tm_k, k_pool, 4, dims, strides, box)) return EVLN_INVALID_VALUE;
         if (!encode_map(h, &tm_v, v_pool, 4, dims, strides, box)) return EVLN_INVALID_VALUE;
-        int most = 0;
-        for (int b = 0; b < p->batch; ++b) most = h_new_offsets[b + 1] - h_new_offsets[b] > most ? h_new_offsets[b + 1] - h_new_offsets[b] : most;
+        const int most = (int)most_rows(p, h_new_offsets);
         FewArgs a = {};
         a.o_part = (float*)workspace;
         a.lse_part = a.o_part + (size_t)smax * p->num_kv_heads * rows * 128;
@@ -1423,9 +1429,9 @@ evlnStatus_t evlnPagedStepAttention(evlnHandle_t h, const evlnPagedParams* p, co
         BatchLens bl;
         fill_lens(&bl, p, h_cache_lens, h_new_offsets, chunk, plan.share);
         if (plan.share == 0 && bl.item_off[p->batch] != (int)items) return EVLN_INVALID_VALUE;
-        const size_t smem = few_smem_bytes(kFewPagedStages, most * G, 1, false, 0) + kFewOutBytes;
+        const size_t smem = few_smem_bytes(kFewPagedStages, most, 1, false, 0) + kFewOutBytes;
         cudaStream_t st = (cudaStream_t)stream;
-        cudaError_t e = few_row_tiles(most * G) == 1
+        cudaError_t e = few_row_tiles(most) == 1
                             ? launch_pdl(attn_few_kernel<1, true, false, BatchLens>, dim3((int)items), dim3(kFewThreads), smem, st, tm_k, tm_v, a, bl)
                             : launch_pdl(attn_few_kernel<2, true, false, BatchLens>, dim3((int)items), dim3(kFewThreads), smem, st, tm_k, tm_v, a, bl);
         return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
@@ -1522,7 +1528,7 @@ evlnStatus_t evlnPagedStepCombine(evlnHandle_t h, const evlnPagedParams* p, cons
     a.out = out; a.lse_out = lse_out;
     a.Hkv = p->num_kv_heads; a.G = G; a.D = 128; a.rows = (int)rows; a.num_splits = smax;
     a.batch = p->batch; a.unit_rows = kUnitRows; a.chunk_tiles = chunk;
-    if (smax == 1 && !paged_few(p, h_new_offsets)) return launch_copy_out(h, a, (cudaStream_t)stream);
+    if (smax == 1 && !plan.few) return launch_copy_out(h, a, (cudaStream_t)stream);
     a.share = plan.share;
     a.div_share = make_fast_div((uint32_t)(plan.share > 0 ? plan.share : 1));
     BatchLens bl;

@@ -83,6 +83,9 @@ def test_reported_split_count_passed_on_gives_the_same_bits(handle, hq, hkv, L, 
     ([300, 64, 1], [1, 1, 1], 0),                 # shorter than a stage, one page, one key
     ([1000, 127, 128, 4000], [4, 2, 0, 3], 0),    # ragged, an episode without new tokens, two row tiles
     ([2500, 700], [1, 2], 4),                     # work items of the caller's size
+    ([2500, 700], [4, 1], 16),                    # ... long ones of two row tiles: CTA pairs
+    ([2500, 700], [4, 1], 24),                    # ... unsplit
+    ([2500, 700] * 10, [4, 1] * 10, 16),          # ... more of them than pairs: the few-row kernel
 ])
 def test_paged_batch_of_few_rows_against_oracle(handle, lens, new, chunk):
     cfg = dataclasses.replace(W.PAGED_B16, batch=len(lens), seed=60 + len(lens))
