@@ -1846,6 +1846,12 @@ extern "C" evlnStatus_t evlnGatherRope(evlnHandle_t h, const evlnGatherParams* p
     a.k_chunks = ceil_div(a.Hkv << a.vph_shift, 32);
     a.v_chunks = ceil_div(a.Hkv << (a.vph_shift + 1), 64);
     a.div_chunks = make_fast_div((uint32_t)(a.k_chunks + a.v_chunks));
+    if (gather_by_block(a.k_chunks, total, a.table != nullptr, p->dtype == EVLN_BF16, a.D)) {
+        if (p->dtype == EVLN_BF16) launch_pdl(gather_rope_block_kernel<__nv_bfloat16>, dim3((unsigned)total), dim3(kGatherBlockThreads), 0, st, a, segs);
+        else launch_pdl(gather_rope_block_kernel<float>, dim3((unsigned)total), dim3(kGatherBlockThreads), 0, st, a, segs);
+        const cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
+    }
     if (total * (a.k_chunks + a.v_chunks) > 0x7fffff00L) return EVLN_NOT_SUPPORTED;
     const dim3 grid((unsigned)((total * (a.k_chunks + a.v_chunks) + kGatherWarps - 1) / kGatherWarps)), block(32 * kGatherWarps);
     if (p->dtype == EVLN_BF16) launch_pdl(gather_rope_kernel<__nv_bfloat16>, grid, block, 0, st, a, segs);

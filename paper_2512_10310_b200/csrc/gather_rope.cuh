@@ -64,7 +64,8 @@ store_append_kernel(const GatherArgs a)
 
 // A warp per chunk of a destination token: 32 vector pairs of its keys, or 64 vectors of its values.  Warps
 // do not wait for each other, so a call of a few thousand tokens is one wave of short chains (a block
-// per token, all of it behind the angles: 6.5 us for 3392 tokens of 4 kv heads; this: 5.3).
+// per token, all of it behind the angles: 6.5 us for 3392 tokens of 4 kv heads; this: 5.3).  For tokens whose keys are
+// one chunk, and for few tokens: every further chunk of keys needs the token's angles again.
 constexpr int kGatherWarps = 8;
 
 template <typename T>
@@ -120,6 +121,59 @@ gather_rope_kernel(const GatherArgs a, const __grid_constant__ SegList segs)
         for (int i = 0; i < 2; ++i) {
             const int d = (it + 32 * i) & ((2 << a.vph_shift) - 1), g = (it + 32 * i) >> (a.vph_shift + 1);
             if (g < a.Hkv) *reinterpret_cast<uint4*>((T*)a.v_dst + ((long)g * a.dst_cap + pos) * D + d * V) = x[i];
+        }
+    }
+}
+
+// A block per destination token, which forms (or reads) the token's angles once for all its heads: more than one chunk of
+// keys, and enough tokens (of few, a warp per chunk spreads the work further).  3392 tokens of 8 kv heads: without a
+// table bf16 6.5 us, a warp per chunk 8.5, fp32 7.6 and 11.7; with one 5.8 and 6.0, 6.9 and 8.5.  32 heads of 250 fp32
+// tokens with a table 4.8 and 3.3, of 60 without one 4.9 and 3.3.  bf16 of head_dim 64 with a table (short rows, one
+// read of the angles per 64 channels) stays with the warps: 16 heads, 20000 tokens 39.8 and 33.4.
+constexpr int kGatherBlockThreads = 128;
+inline bool gather_by_block(int k_chunks, long tokens, bool table, bool bf16, int D)
+{
+    return k_chunks > 1 && tokens > (table ? 512 : 128) && !(table && bf16 && D == 64);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kGatherBlockThreads, 12)
+gather_rope_block_kernel(const GatherArgs a, const __grid_constant__ SegList segs)
+{
+    constexpr int V = VecTraits<T>::kVec;
+    __shared__ typename Rotation<T>::Angle s_angle[Rotation<T>::kAngles];
+    const int pos = (int)blockIdx.x;                       // working slot = new position id
+    const int D = a.D, half = D / 2;
+    int lo = 0, hi = a.num_segments;                       // largest s with dst_off[s] <= pos
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (segs.dst_off[mid] <= pos) lo = mid; else hi = mid;
+    }
+    const long src_slot = segs.src[lo] + (pos - segs.dst_off[lo]);
+    // (so far launch parameters only)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if ((int)threadIdx.x < half) {
+        const int j = threadIdx.x;
+        Rotation<T>::put(s_angle, j, a.table ? a.table[(long)(pos - a.table_first) * half + j] : rope_cos_sin(pos, j, D, a.log2_theta));
+    }
+    __syncthreads();
+
+    const int k_items = a.Hkv << a.vph_shift, v_items = a.Hkv << (a.vph_shift + 1);
+    for (int it = threadIdx.x; it < k_items + v_items; it += kGatherBlockThreads) {
+        if (it < k_items) {
+            const int k = it & ((1 << a.vph_shift) - 1), g = it >> a.vph_shift;
+            const T* src = (const T*)a.k_src + ((long)g * a.src_cap + src_slot) * D + k * V;
+            const uint4 lo_raw = *reinterpret_cast<const uint4*>(src), hi_raw = *reinterpret_cast<const uint4*>(src + half);
+            uint4 out_lo, out_hi;
+            Rotation<T>::turn(s_angle, k, lo_raw, hi_raw, out_lo, out_hi);
+            T* dst = (T*)a.k_dst + ((long)g * a.dst_cap + pos) * D + k * V;
+            *reinterpret_cast<uint4*>(dst) = out_lo;
+            *reinterpret_cast<uint4*>(dst + half) = out_hi;
+        } else {
+            const int e = it - k_items, d = e & ((2 << a.vph_shift) - 1), g = e >> (a.vph_shift + 1);
+            *reinterpret_cast<uint4*>((T*)a.v_dst + ((long)g * a.dst_cap + pos) * D + d * V) =
+                *reinterpret_cast<const uint4*>((const T*)a.v_src + ((long)g * a.src_cap + src_slot) * D + d * V);
         }
     }
 }

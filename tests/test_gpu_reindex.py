@@ -165,3 +165,42 @@ def test_offloaded_store_episode_matches_the_oracle(handle):
     assert np.array_equal(f64(h_k.permute(1, 0, 2)), k_raw) and np.array_equal(f64(h_v.permute(1, 0, 2)), v_raw)
     # frames admitted on the device need no fetch; later the uniform sampler moves a few per step
     assert max(moved) <= budget and np.mean(moved[budget + 2:]) <= 0.75 * budget
+
+
+@pytest.mark.parametrize("dtype,hkv,d,lengths", [
+    ("bf16", 8, 128, [128]),                  # two chunks of keys a token, few tokens: warps of their own
+    ("bf16", 8, 128, [100, 29]),              # ... one more: a block per token
+    ("bf16", 5, 128, [200, 0, 1, 150]),       # work items that end within a warp; with a table still by warps
+    ("bf16", 8, 128, [512, 1]),               # ... and from 513 tokens by blocks
+    ("bf16", 32, 64, [257]),
+    ("f32", 3, 128, [130]),
+    ("f32", 32, 128, [3, 140]),               # more work items than a block has threads, several times
+    ("f32", 9, 64, [300]),
+])
+def test_gather_of_tokens_with_many_heads(handle, dtype, hkv, d, lengths):
+    gen = torch.Generator().manual_seed(hkv + d)
+    tdt, dev, slots = {"bf16": torch.bfloat16, "f32": torch.float32}[dtype], "cuda:0", sum(lengths) + 50
+    k_raw, v_raw = (torch.randn((slots, hkv, d), generator=gen).to(tdt) for _ in range(2))
+    k_store, v_store = (t.to(dev).permute(1, 0, 2).contiguous() for t in (k_raw, v_raw))
+    segs, at = [], slots
+    for n in lengths:                         # taken from the back of the store
+        at -= n + 3
+        segs.append((at, n))
+    kw, vw = ro.gather_rope(f64(k_raw), f64(v_raw), segs, 1e4, storage=dtype)
+    total = sum(lengths)
+    table = torch.empty(B.evlnRopeTableBytes(d, total), dtype=torch.uint8, device=dev)
+    B.evlnRopeTable(handle, d, 1e4, 0, total, table)
+    bits = []
+    for tbl in (None, table):
+        k_work, v_work = (torch.full((hkv, total + 5, d), 7.0, dtype=tdt, device=dev) for _ in range(2))
+        p = B.gather_params(dtype, hkv, d, slots, total + 5, 1e4, tbl, 0, total if tbl is not None else 0)
+        assert B.evlnGatherRope(handle, p, [s for s, _ in segs], lengths, k_store, v_store, k_work, v_work) == total
+        got = k_work[:, :total].permute(1, 0, 2)
+        if dtype == "bf16":
+            assert bf16_ulp_distance(got, kw).max() <= 1
+        else:
+            assert np.abs(f64(got) - kw).max() <= 1e-6
+        assert np.array_equal(f64(v_work[:, :total].permute(1, 0, 2)), vw)
+        assert bool((k_work[:, total:] == 7.0).all()) and bool((v_work[:, total:] == 7.0).all())
+        bits.append(k_work)
+    assert torch.equal(*bits)
