@@ -169,8 +169,9 @@ evlnStatus_t evlnRopeTable(evlnHandle_t handle, int head_dim, double rope_theta,
 /* Step 1 (Sec. 3.2: contiguous position ids, RoPE, concatenation with the cache).
  * Rotates the new queries at positions L+i into q_rot (grouped by kv head), rotates the new
  * keys and stores them, with the values copied bit-exactly, into cache slots L .. L+n-1.
- * Angles, sines/cosines and the rotation products are formed in double precision and then
- * rounded to the storage dtype.  Slots outside L .. L+n-1 are not touched.
+ * Angles, sines and cosines are formed in double precision.  The rotation's products and sums carry
+ * at least 40 bits (f32: double; bf16: pairs of floats) and are rounded to float and then to the
+ * storage dtype.  Slots outside L .. L+n-1 are not touched.
  * Errors: EVLN_CACHE_FULL if L+n > cache_capacity; n = 0 returns EVLN_OK and launches nothing. */
 evlnStatus_t evlnRopeAppend(evlnHandle_t handle, const evlnStepParams* params,
                             const void* q_new, const void* k_new, const void* v_new,
@@ -179,12 +180,13 @@ evlnStatus_t evlnRopeAppend(evlnHandle_t handle, const evlnStepParams* params,
 
 /* Step 2 (Sec. 3.2: prefill of the current frame only, against the reused cache).
  * Causal attention of the n rotated queries over cache slots 0 .. L+n-1 (query i sees slots
- * 0 .. L+i), split over the keys; writes per-split normalised outputs and log-sum-exps into
- * `workspace`.  Must run after evlnRopeAppend of the same step on the same stream.
+ * 0 .. L+i), split over the keys; writes per-split normalised outputs [S, Hkv, n*G, D] and
+ * log-sum-exps [S, Hkv, n*G], all float, into `workspace` (S = evlnStepNumSplits, also when it is
+ * 1; a split that a row sees no key of has output 0 and log-sum-exp -inf).  Must run after evlnRopeAppend of the same step on the same stream.
  * bf16 with head_dim 128 runs on the tensor cores: CTA pairs over 256-row units of the packed
  * query rows, or, when all n * G rows of a kv head fit one 128-row tile (the few action tokens
- * decoded after a frame, Sec. 3.1), one CTA per (kv head, KV split) with the KV range spread
- * over all SMs.                                                                              */
+ * decoded after a frame, Sec. 3.1), one CTA per (kv head, KV split); at most 32 rows per kv head
+ * in clusters of blocks that merge a head's keys among themselves.                            */
 evlnStatus_t evlnStepAttention(evlnHandle_t handle, const evlnStepParams* params,
                                const void* q_rot, const void* k_cache, const void* v_cache,
                                void* workspace, size_t workspace_bytes, void* stream);
@@ -195,8 +197,13 @@ evlnStatus_t evlnStepCombine(evlnHandle_t handle, const evlnStepParams* params,
                              const void* workspace, void* out, float* lse_out, void* stream);
 
 /* The whole step in one call (Sec. 3.2): evlnRopeAppend, evlnStepAttention and evlnStepCombine
- * with the same arguments, enqueued on `stream`; same results bit for bit.  One launch instead of three for at most 32 query
- * rows per kv head, two when the keys are not split.
+ * with the same arguments, enqueued on `stream`; same results bit for bit.  Two launches instead of
+ * three where bf16 steps of head_dim 128 on CTA pairs are not split.  Steps of at most 32 query rows
+ * per kv head and 16 tokens: one launch, two when split (not where the one-CTA kernel serves them:
+ * more than 16 rows with 8 or more kv heads and 3072 or more keys, or more than 24 rows with 4 kv
+ * heads and 24576 or more keys).  q_rot may be q_new (n = 1, rotation in place) and `out` may lie
+ * over q_rot or the new tokens' tensors; such calls take the separate launches, unless `out` is just
+ * q_new.
  * All arguments are validated before the first launch; errors as for the three calls.          */
 evlnStatus_t evlnStep(evlnHandle_t handle, const evlnStepParams* params,
                       const void* q_new, const void* k_new, const void* v_new,
@@ -220,6 +227,8 @@ evlnStatus_t evlnPagedRopeAppend(evlnHandle_t handle, const evlnPagedParams* par
                                  const int* h_cache_lens, const int* h_new_offsets,
                                  const int* d_page_table, void* q_rot, void* k_pool, void* v_pool,
                                  void* stream);
+/* What the attention call leaves in `workspace` is for evlnPagedStepCombine of the same parameters
+ * only: its form depends on the kernel and the split counts that the library chose.           */
 evlnStatus_t evlnPagedStepAttention(evlnHandle_t handle, const evlnPagedParams* params,
                                     const void* q_rot, const void* k_pool, const void* v_pool,
                                     const int* h_cache_lens, const int* h_new_offsets,
