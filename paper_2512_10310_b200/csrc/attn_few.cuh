@@ -68,7 +68,7 @@ struct FewArgs {
     FastDiv div_share;
     float scale_log2;         // softmax scale * log2(e)
     FastDiv div_g;            // division by G
-    // contiguous only: the cache, for prefetches into L2 and for the fused append
+    // contiguous only: the cache, for the fused append
     __nv_bfloat16* k_cache;
     __nv_bfloat16* v_cache;
     int cache_cap;
@@ -145,7 +145,7 @@ attn_few_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant_
     const int q_off = stages * kFewStageBytes, bar_off = q_off + MT * 16 * 256, stat_off = bar_off + kFewBarBytes;
     const uint32_t bar_full = smem_base + bar_off, bar_empty = bar_full + 8 * kFewMaxStages;
     volatile int* s_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 16 * kFewMaxStages);
-    float* s_m = reinterpret_cast<float*>(smem_gen + stat_off);            // [kFewWarps][64] reference of each warp's rows
+    float* s_m = reinterpret_cast<float*>(smem_gen + stat_off);            // [kFewWarps][kFewRows] reference of each warp's rows
     float* s_l = s_m + kFewWarps * kFewRows;                               // ... and their sums
     float* s_in = s_l + kFewWarps * kFewRows;                              // [rows this block merges][cluster][kFewOStride]
     uint8_t* s_tail = smem_gen + stat_off + kFewStatBytes + (PAGED ? 0 : few_cluster_bytes(a.num_new * a.G, gridDim.x));

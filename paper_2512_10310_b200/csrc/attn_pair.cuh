@@ -1270,8 +1270,8 @@ attn_packed_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 }
 
 // One CTA per work item, for steps whose rows per kv head fit one 128-row tile (the few action
-// tokens that follow a frame, Sec. 3.1): the KV range is cut into as many splits as there are SMs,
-// and each CTA streams whole K/V tiles, so the step runs at the rate HBM delivers the cache.
+// tokens that follow a frame, Sec. 3.1): the KV range is cut into up to 32 splits (choose_splits_solo) and
+// each CTA streams whole K/V tiles, so that a long cache is read at the rate HBM delivers it.
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_solo_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const TcAttnArgs a)

@@ -23,7 +23,7 @@ struct CombineArgs {
     int rows;                // R = (total) new tokens * G
     int num_splits;          // contiguous: S for every row
     // batches: per-episode split counts are derived from the lengths
-    int batch, unit_rows, chunk_tiles;
+    int batch, chunk_tiles;
     int tail;                // batch of items sharing a cache prefix (own tokens tiled separately)
     FastDiv div_g;           // division by G, by the work-item size in KV tiles (chunk_tiles, at least 1):
     FastDiv div_chunk;       //   a row's warp decodes its place with multiplications (an integer division costs

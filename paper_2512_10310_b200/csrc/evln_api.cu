@@ -1527,7 +1527,7 @@ evlnStatus_t evlnPagedStepCombine(evlnHandle_t h, const evlnPagedParams* p, cons
     a.lse_part = a.o_part + (size_t)smax * p->num_kv_heads * rows * 128;
     a.out = out; a.lse_out = lse_out;
     a.Hkv = p->num_kv_heads; a.G = G; a.D = 128; a.rows = (int)rows; a.num_splits = smax;
-    a.batch = p->batch; a.unit_rows = kUnitRows; a.chunk_tiles = chunk;
+    a.batch = p->batch; a.chunk_tiles = chunk;
     if (smax == 1 && !plan.few) return launch_copy_out(h, a, (cudaStream_t)stream);
     a.share = plan.share;
     a.div_share = make_fast_div((uint32_t)(plan.share > 0 ? plan.share : 1));
@@ -1735,7 +1735,7 @@ extern "C" evlnStatus_t evlnPackedForward(evlnHandle_t h, const evlnPackedParams
     c.lse_part = c.o_part + (size_t)pl.smax * p->num_kv_heads * rows_a * 128;
     c.out = out; c.lse_out = lse_out;
     c.Hkv = p->num_kv_heads; c.G = G; c.D = 128; c.rows = (int)rows_a; c.num_splits = pl.smax;
-    c.batch = p->num_frames; c.unit_rows = kUnitRows; c.chunk_tiles = pl.chunk;
+    c.batch = p->num_frames; c.chunk_tiles = pl.chunk;
     c.tail = 1;
     c.map = make_packed_map(p->instr_len, p->frame_tokens, p->action_tokens, 1);
     return launch_combine<__nv_bfloat16>(h, c, 128, true, &bl, st);

@@ -56,20 +56,6 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok;
 }
 
-// one look, without the suspension try_wait may take
-__device__ __forceinline__ uint32_t mbar_test_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok;
-}
-
 // ---- TMA (tiled tensor loads into this CTA's shared memory) -----------------------------
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
                                             int x, int y, int z)
@@ -92,11 +78,6 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         "[%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
         "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
         : "memory");
-}
-// L2 prefetch of `bytes` (a multiple of 16) from a 16-byte boundary
-__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 // L2 prefetch of a tile (no shared-memory destination, no barrier)
 __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z)
@@ -256,11 +237,6 @@ __device__ __forceinline__ void cluster_arrive_relaxed()
 __device__ __forceinline__ void cluster_wait()
 {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// arrival that releases this thread's earlier writes (shared memory included) to the cluster
-__device__ __forceinline__ void cluster_arrive()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
 // asynchronous stores to shared memory of any CTA of the cluster; their bytes are counted on an mbarrier there
 __device__ __forceinline__ void st_async_f32x4(uint32_t cluster_addr, const float4& v, uint32_t cluster_bar)
