@@ -62,10 +62,10 @@ typedef enum {
 
 typedef enum { EVLN_BF16 = 0, EVLN_F32 = 1 } evlnDType_t;
 
-/* Attention kernel choice.  AUTO: tensor-core kernel (tcgen05 MMA, TMEM accumulators, TMA
- * tiles) for bf16 with head_dim 128; the fp32 SIMT kernel otherwise.  SIMT forces the
- * SIMT kernel (any dtype), which exists for the fp32 precision target and as an
- * independent on-device cross-check.                                                        */
+/* Attention kernel choice.  AUTO: tensor-core kernels for bf16 with head_dim 128 (tcgen05 MMA, TMEM
+ * accumulators, TMA tiles; mma.sync for few rows) and for fp32 (every float as three bf16 parts,
+ * fp32 sums: the accuracy of float FMAs); the SIMT kernel for bf16 with head_dim 64.  SIMT forces
+ * the SIMT kernel (float FMAs, any dtype), an independent on-device cross-check.                */
 typedef enum { EVLN_KERNEL_AUTO = 0, EVLN_KERNEL_SIMT = 1 } evlnKernel_t;
 
 typedef struct evlnContext* evlnHandle_t;

@@ -1,9 +1,5 @@
-// fp32 SIMT step attention (no tensor cores).
-//
-// The fp32 configuration asks for 1e-5 agreement with the fp64 oracle, which tf32 tensor-core
-// products cannot give, so this kernel evaluates the same split-KV causal attention with
-// float FMAs.  It is also the on-device cross-check of the tensor-core kernel for bf16 inputs, and
-// the path of bf16 with head_dim 64.
+// SIMT step attention in float FMAs (no tensor cores): bf16 with head_dim 64, and, when the caller asks for
+// it (EVLN_KERNEL_SIMT), any type as an on-device cross-check of the tensor-core kernels.
 //
 // Bound: the FMA pipes (4 D flop per visible pair; 128 FMA per SM and cycle).  A block of 256 threads
 // owns a tile of 16 * RPT packed query rows of one kv head and walks its split's keys 64 at a time:
@@ -41,6 +37,10 @@ struct SimtAttnArgs {
     int num_splits;
     int share;             // key tiles per block, 0: a block per (row block, kv head, split)
     float scale;
+    // attn_f32.cuh only:
+    float scale_lo;                 // rest of the scale
+    float scale2_hi, scale2_lo;     // scale * log2(e) rounded towards zero, and its rest (> 0)
+    int* status;                    // device status word
 };
 
 constexpr int kSimtThreads = 256;

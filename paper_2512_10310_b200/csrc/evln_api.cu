@@ -16,6 +16,7 @@
 
 #include "attn_simt.cuh"
 #include "attn_pair.cuh"
+#include "attn_f32.cuh"
 #include "attn_few.cuh"
 #include "combine.cuh"
 #include "gather_rope.cuh"
@@ -99,6 +100,15 @@ cudaError_t prepare_simt()
     return e;
 }
 
+template <int D>
+cudaError_t prepare_f32()
+{
+    cudaError_t e = cudaFuncSetAttribute(attn_f32_kernel<D, NoTable>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Plan<D>::kBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(attn_f32_kernel<D, SimtTiles>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Plan<D>::kBytes);
+    return e;
+}
+
 template <int MT>
 cudaError_t prepare_few()
 {
@@ -128,6 +138,8 @@ cudaError_t prepare_kernels()
     }
     cudaError_t e = prepare_few<1>();
     if (e == cudaSuccess) e = prepare_few<2>();
+    if (e == cudaSuccess) e = prepare_f32<128>();
+    if (e == cudaSuccess) e = prepare_f32<64>();
     if (e == cudaSuccess) e = prepare_simt<float, 128, 8>();
     if (e == cudaSuccess) e = prepare_simt<float, 128, 2>();
     if (e == cudaSuccess) e = prepare_simt<float, 64, 8>();
@@ -202,6 +214,12 @@ evlnStatus_t check_step_params(evlnHandle_t h, const evlnStepParams* p)
     if (!rope_table_covers(p->rope_table, p->rope_table_first_pos, p->rope_table_count, p->cache_len, p->num_new))
         return EVLN_INVALID_VALUE;
     return EVLN_OK;
+}
+
+// fp32 on the tensor cores (attn_f32.cuh), unless the caller asks for the kernel without them.
+inline bool use_f32_kernel(const evlnStepParams* p)
+{
+    return p->kernel == EVLN_KERNEL_AUTO && p->dtype == EVLN_F32;
 }
 
 inline bool use_tensor_kernel(const evlnStepParams* p)
@@ -377,6 +395,10 @@ size_t partial_bytes(int splits, int Hkv, long rows, int D)
 // has the SM to itself, 9.5 per tile when two share it.  So 128-row tiles are 1.4 times cheaper per row
 // where they fill the chip, 32-row tiles have twice the latency advantage where they would not.  A
 // split writes and re-reads a set of partials (about 5 TB/s out of L2).
+// fp32 has its 128-row tiles on the tensor cores (attn_f32.cuh): 2.25 us per 64-key tile (1.5 at head_dim 64) and, beside
+// what the others need, 3 us for its start, so that it takes over from 32-row blocks where those are walked for two or
+// three tiles, or are two to an SM.  (196 tokens of the 7B shape over 1024 cached 95.4 us in float FMAs, 29 so; one
+// key tile for 64 rows of head_dim 64 8.3 and 11.5.)
 struct SimtSchedule {
     int rows_per_thread, splits;
     int share;               // > 0: one block per SM, each that many key tiles of 128-row blocks (see attn_simt.cuh)
@@ -398,17 +420,22 @@ SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits, 
     const int tiles = ceil_div(p->cache_len + p->num_new, kSimtKeys);
     const double d = p->head_dim / 128.0;
     const double split_us = 0.3 + 2.0 * R * p->num_kv_heads * p->head_dim * 4 / 5e6;
+    // (Steps of more row blocks than the share table holds keep the split counts, and by that the workspaces, of the
+    // kernel without tensor cores.)
+    const bool tensor = use_f32_kernel(p) && ceil_div(R, 128) <= kSimtShareBlocks;
+    const double big_tile = tensor ? 0.75 / d + 1.5 : 13.3, big_start = tensor ? 7.1 + 2.8 * d : 7.0;
     SimtSchedule best = {8, splits > 0 ? splits : 1, 0};
     double best_cost = 1e30;
     const int smax = tiles < most_splits ? tiles : most_splits;
     for (int rpt = 8; rpt >= 2; rpt -= 6) {
         const long row_blocks = (long)ceil_div(R, 16 * rpt) * p->num_kv_heads;
+        if (use_f32_kernel(p) && !tensor && rpt != 8) break;
         for (int s = splits > 0 ? splits : 1; s <= (splits > 0 ? splits : smax); ++s) {
             const long blocks = row_blocks * s;
             const long at_once = rpt == 8 || blocks <= h->num_sms ? h->num_sms : 2 * h->num_sms;
-            const double tile_us = rpt == 8 ? 13.3 : at_once == h->num_sms ? 6.3 : 9.5;
+            const double tile_us = rpt == 8 ? big_tile : at_once == h->num_sms ? 6.3 : 9.5;
             const double waves = (double)((blocks + at_once - 1) / at_once);
-            const double cost = waves * (ceil_div(tiles, s) * tile_us * d + (rpt == 8 ? 7.0 : 5.0)) + split_us * s;
+            const double cost = waves * (ceil_div(tiles, s) * tile_us * d + (rpt == 8 ? big_start : 5.0)) + split_us * s;
             if (cost < best_cost - 1e-9) { best_cost = cost; best = {rpt, s, 0}; }
         }
     }
@@ -421,7 +448,7 @@ SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits, 
         int share = ceil_div(per_head * p->num_kv_heads, h->num_sms);
         if (share < ceil_div(most, kMaxSplits - 1)) share = ceil_div(most, kMaxSplits - 1);
         const int s = ceil_div(most - 1, share) + 1;
-        const double cost = share * 13.3 * d + 7.0 + 4.0 * ceil_div(share, t.off[1]) + split_us * (1.0 + (double)most / share);
+        const double cost = share * big_tile * d + big_start + (tensor ? 5.0 : 4.0) * ceil_div(share, t.off[1]) + split_us * (1.0 + (double)most / share);
         if (s <= most_splits && cost < best_cost - 1e-9) best = {8, s, share};
     }
     return best;
@@ -439,6 +466,38 @@ void launch_simt(const SimtSchedule& plan, const evlnStepParams* p, dim3 grid, c
         launch_pdl(attn_simt_kernel<T, D, 8, NoTable>, grid, dim3(kSimtThreads), simt_smem_bytes<D, 8>(), st, a, NoTable{});
     } else {
         launch_pdl(attn_simt_kernel<T, D, 2, NoTable>, grid, dim3(kSimtThreads), simt_smem_bytes<D, 2>(), st, a, NoTable{});
+    }
+}
+
+// The scale of the fp32 kernel in two floats each, with what its scores fall short of: the tensor core cuts the sums
+// behind every 16 channels off instead of rounding them (measured with normal numbers: 7.1e-8 of a score at 128 channels, half
+// of that at 64).
+void set_f32_scale(const evlnStepParams* p, SimtAttnArgs* a)
+{
+    const double scale = (p->softmax_scale > 0.f ? (double)p->softmax_scale : 1.0 / sqrt((double)p->head_dim)) * (1.0 + 5.5e-10 * p->head_dim);
+    const double scale2 = scale * 1.4426950408889634;
+    a->scale = (float)scale;
+    a->scale_lo = (float)(scale - (double)a->scale);
+    a->scale2_hi = (float)scale2;
+    if ((double)a->scale2_hi >= scale2) a->scale2_hi = nextafterf(a->scale2_hi, 0.f);
+    a->scale2_lo = (float)(scale2 - (double)a->scale2_hi);
+}
+
+template <int D>
+void launch_f32(const SimtSchedule& plan, const evlnStepParams* p, dim3 grid, cudaStream_t st, SimtAttnArgs a)
+{
+    if (plan.rows_per_thread == 2) {
+        launch_simt<float, D>(plan, p, grid, st, a);
+        return;
+    }
+    set_f32_scale(p, &a);
+    if (plan.share > 0) {
+        SimtTiles t;
+        fill_simt_tiles(p, &t);
+        const int blocks = ceil_div(t.off[kSimtShareBlocks] * p->num_kv_heads, plan.share);
+        launch_pdl(attn_f32_kernel<D, SimtTiles>, dim3(blocks), dim3(kF32Threads), F32Plan<D>::kBytes, st, a, t);
+    } else {
+        launch_pdl(attn_f32_kernel<D, NoTable>, grid, dim3(kF32Threads), F32Plan<D>::kBytes, st, a, NoTable{});
     }
 }
 
@@ -1255,10 +1314,14 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
         a.cache_len = p->cache_len; a.num_new = p->num_new; a.cache_cap = p->cache_capacity;
         a.num_splits = S; a.scale = scale;
         a.share = plan.share;
+        a.status = h->d_status;
         dim3 grid(ceil_div(R, 16 * plan.rows_per_thread), p->num_kv_heads, S);
         if (p->dtype == EVLN_BF16) {
             if (D == 128) launch_simt<__nv_bfloat16, 128>(plan, p, grid, st, a);
             else launch_simt<__nv_bfloat16, 64>(plan, p, grid, st, a);
+        } else if (use_f32_kernel(p)) {
+            if (D == 128) launch_f32<128>(plan, p, grid, st, a);
+            else launch_f32<64>(plan, p, grid, st, a);
         } else {
             if (D == 128) launch_simt<float, 128>(plan, p, grid, st, a);
             else launch_simt<float, 64>(plan, p, grid, st, a);

@@ -1,0 +1,85 @@
+"""The fp32 step attention on the tensor cores (three bf16 parts per float) at the edges of its tiles, and
+where its splitting of numbers ends."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2512_10310_b200 import binding as B
+from paper_2512_10310_b200 import workloads as W
+from tests.helpers import GpuStep, check_cache, check_output, f64, oracle_step
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def handle():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    h = B.evlnCreate(0)
+    yield h
+    B.evlnDestroy(h)
+
+
+def _inputs(hq, hkv, d, L, n):
+    cfg = W.StepConfig("f32", "f32", hq, hkv, d, L, n, 1e4, 1.0, 20 + L + n)
+    return cfg, W.make_step_inputs(cfg)
+
+
+def _step(handle, cfg, x, **options):
+    gs = GpuStep(handle, "f32", cfg.num_q_heads, cfg.num_kv_heads, cfg.head_dim, cfg.cache_len + cfg.num_new + 5, cfg.rope_theta,
+                 cfg.num_new, **options)
+    gs.load_cache(x["k_cache"], x["v_cache"])
+    return gs, gs.step(cfg.cache_len, x["q_new"], x["k_new"], x["v_new"])
+
+
+@pytest.mark.parametrize("hq,hkv,d,L,n,splits", [
+    (1, 1, 64, 0, 1, 0),           # one row, one key
+    (2, 1, 64, 256, 64, 0),        # 128 rows
+    (1, 1, 128, 62, 2, 1),         # keys end with their tile
+    (4, 2, 128, 63, 64, 0),        # ... and one key into the third
+    (7, 1, 128, 300, 18, 4),       # 126 rows
+    (43, 1, 64, 100, 3, 0),        # 129 rows: a row block of one row
+    (8, 1, 128, 449, 63, 8),       # 512 keys, a tile per split
+    (8, 1, 128, 450, 63, 8),       # ... and one key more
+    (2, 2, 64, 10, 3, 7),          # more splits than key tiles
+    (8, 4, 128, 0, 64, 0),         # no cache
+    (8, 4, 128, 200, 65, 0),       # 130 rows per head
+    (28, 4, 128, 1024, 196, 0),    # equal shares
+])
+def test_one_call_is_the_three_calls(handle, hq, hkv, d, L, n, splits):
+    cfg, x = _inputs(hq, hkv, d, L, n)
+    r = oracle_step("f32", x["k_cache"], x["v_cache"], x["q_new"], x["k_new"], x["v_new"], L, cfg.rope_theta)
+    three, a = _step(handle, cfg, x, num_splits=splits)
+    one, b = _step(handle, cfg, x, num_splits=splits, fused=True)
+    for gs, g in ((three, a), (one, b)):
+        check_cache(gs, r, L, n)
+        check_output("f32", g["out"], g["lse"], r["out"], r["lse"])
+    for key in ("out", "lse", "q_rot"):
+        assert torch.equal(a[key], b[key]), key
+    assert torch.equal(three.k_cache, one.k_cache) and torch.equal(three.v_cache, one.v_cache)
+
+
+@pytest.mark.parametrize("hq,hkv,d,L,n,scale", [
+    (2, 1, 64, 256, 64, 1e-36),    # the parts of such numbers are not exact: done again in floats
+    (4, 2, 128, 500, 70, 1e-36),
+    (4, 2, 128, 500, 70, 1e30),
+])
+@pytest.mark.parametrize("fused", [False, True])
+def test_values_of_any_size(handle, hq, hkv, d, L, n, scale, fused):
+    cfg, x = _inputs(hq, hkv, d, L, n)
+    x["v_cache"], x["v_new"] = x["v_cache"] * scale, x["v_new"] * scale
+    r = oracle_step("f32", x["k_cache"], x["v_cache"], x["q_new"], x["k_new"], x["v_new"], L, cfg.rope_theta)
+    _, g = _step(handle, cfg, x, fused=fused)
+    # (the output is linear in V: the fp32 gate, relative)
+    assert np.linalg.norm(f64(g["out"]) / scale - r["out"] / scale) <= 1e-5 * np.linalg.norm(r["out"] / scale)
+
+
+@pytest.mark.parametrize("hq,hkv,d,L,n", [(2, 1, 64, 256, 64), (4, 2, 128, 500, 70), (28, 4, 128, 1024, 196)])
+def test_scores_beyond_any_sum(handle, hq, hkv, d, L, n):
+    # one key so long that it either takes a row over or drops out of it, by the sign of one channel of the query
+    cfg, x = _inputs(hq, hkv, d, L, n)
+    x["k_cache"][L // 2] = 0.0
+    x["k_cache"][L // 2, :, 3] = -1.0e37
+    r = oracle_step("f32", x["k_cache"], x["v_cache"], x["q_new"], x["k_new"], x["v_new"], L, cfg.rope_theta)
+    _, g = _step(handle, cfg, x)
+    assert np.abs(f64(g["out"]) - r["out"]).max() <= 1e-5
