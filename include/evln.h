@@ -201,7 +201,8 @@ evlnStatus_t evlnStepCombine(evlnHandle_t handle, const evlnStepParams* params,
  * three where bf16 steps of head_dim 128 on CTA pairs are not split.  Steps of at most 32 query rows
  * per kv head and 16 tokens: one launch, two when split (not where the one-CTA kernel serves them:
  * more than 16 rows with 8 or more kv heads and 3072 or more keys, or more than 24 rows with 4 kv
- * heads and 24576 or more keys).  q_rot may be q_new (n = 1, rotation in place) and `out` may lie
+ * heads and 24576 or more keys).  fp32 steps of little work (a few hundred rows, a tile or two of keys
+ * per block): one launch.  q_rot may be q_new (n = 1, rotation in place) and `out` may lie
  * over q_rot or the new tokens' tensors; such calls take the separate launches, unless `out` is just
  * q_new.
  * All arguments are validated before the first launch; errors as for the three calls.          */

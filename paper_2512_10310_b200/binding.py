@@ -27,7 +27,7 @@ def native_path() -> str:
 
 
 NATIVE_PATH = native_path()
-_SOURCES = ["evln_api.cu", "attn_pair.cuh", "attn_few.cuh", "attn_simt.cuh", "attn_f32.cuh", "combine.cuh", "rope_append.cuh",
+_SOURCES = ["evln_api.cu", "attn_pair.cuh", "attn_few.cuh", "attn_simt.cuh", "attn_f32.cuh", "attn_f32_small.cuh", "combine.cuh", "rope_append.cuh",
             "common.cuh", "ptx_sm100.cuh", "gather_rope.cuh", "timeline_debug.cuh"]
 
 EVLN_OK, EVLN_INVALID_VALUE, EVLN_NOT_SUPPORTED, EVLN_CACHE_FULL = 0, 1, 2, 3

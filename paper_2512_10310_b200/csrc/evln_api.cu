@@ -17,6 +17,7 @@
 #include "attn_simt.cuh"
 #include "attn_pair.cuh"
 #include "attn_f32.cuh"
+#include "attn_f32_small.cuh"
 #include "attn_few.cuh"
 #include "combine.cuh"
 #include "gather_rope.cuh"
@@ -37,6 +38,7 @@ struct evlnContext {
     int* d_status;
     EncodeTiledFn encode;
     int max_clusters[5];     // clusters of 1, 2, 4, 8, 16 blocks of the few-row kernel that fit the device at once
+    int small_clusters[kSmallCluster];   // clusters of 1, 2, .. blocks of the small fp32 kernel
 };
 
 #ifdef EVLN_TIMELINE
@@ -106,6 +108,11 @@ cudaError_t prepare_f32()
     cudaError_t e = cudaFuncSetAttribute(attn_f32_kernel<D, NoTable>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Plan<D>::kBytes);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(attn_f32_kernel<D, SimtTiles>, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Plan<D>::kBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(attn_f32_small_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SmallPlan<D>::kBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(attn_f32_small_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SmallPlan<D>::kBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_f32_small_kernel<D, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
 
@@ -361,6 +368,33 @@ cudaError_t query_few_clusters(int* max_clusters)
     return cudaSuccess;
 }
 
+// The same for the small fp32 kernel, clusters of 1 .. kSmallCluster.
+cudaError_t query_small_clusters(int* max_clusters)
+{
+    for (int i = 0; i < kSmallCluster; ++i) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(i + 1);
+        cfg.blockDim = dim3(kSmallThreads);
+        cfg.dynamicSmemBytes = SmallPlan<128>::kBytes;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = i + 1;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, attn_f32_small_kernel<128, true>, &cfg);
+        if (e != cudaSuccess) {
+            if (i == 0) return e;
+            cudaGetLastError();            // this cluster size is not available
+            n = 0;
+        }
+        max_clusters[i] = n;
+    }
+    return cudaSuccess;
+}
+
 template <bool FUSED>
 cudaError_t launch_few(const FewPlan& f, int rows, cudaStream_t st, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const FewArgs& a)
 {
@@ -395,13 +429,16 @@ size_t partial_bytes(int splits, int Hkv, long rows, int D)
 // has the SM to itself, 9.5 per tile when two share it.  So 128-row tiles are 1.4 times cheaper per row
 // where they fill the chip, 32-row tiles have twice the latency advantage where they would not.  A
 // split writes and re-reads a set of partials (about 5 TB/s out of L2).
-// fp32 has its 128-row tiles on the tensor cores (attn_f32.cuh): 2.25 us per 64-key tile (1.5 at head_dim 64) and, beside
-// what the others need, 3 us for its start, so that it takes over from 32-row blocks where those are walked for two or
-// three tiles, or are two to an SM.  (196 tokens of the 7B shape over 1024 cached 95.4 us in float FMAs, 29 so; one
-// key tile for 64 rows of head_dim 64 8.3 and 11.5.)
+// fp32 runs on the tensor cores: 128-row tiles (attn_f32.cuh) take 2.25 us per 64-key tile (1.5 at head_dim 64) and 3 us more
+// for their start than the others; 32-row blocks (attn_f32_small.cuh) 3.7 us per tile (1.8), and evlnStep in one launch
+// where the blocks' rotations are not too many, which saves two launches of about 2 us each and the partials' round
+// trip.  So 128-row tiles begin where 32-row blocks would be walked for three tiles or more.  (One call, us: 64 tokens of 2
+// heads over 256 keys 9.6 with three launches of float FMAs, 7.9; 34 tokens of 28 heads over 518 keys 18.2 with float FMAs, 16.5 in
+// 128-row tiles, 17.1 in one launch; 243 tokens of 2 heads over 373 keys 18.5, 16.5 and, 32 rows in three launches, 14.1.)
 struct SimtSchedule {
     int rows_per_thread, splits;
     int share;               // > 0: one block per SM, each that many key tiles of 128-row blocks (see attn_simt.cuh)
+    bool one_launch;         // fp32 in 32-row blocks: evlnStep is one launch
 };
 // The row blocks' key tiles, at most kSimtShareBlocks blocks.
 void fill_simt_tiles(const evlnStepParams* p, SimtTiles* t)
@@ -412,6 +449,12 @@ void fill_simt_tiles(const evlnStepParams* p, SimtTiles* t)
         const int last = 128 * (rb + 1) < R ? 128 * (rb + 1) - 1 : R - 1;
         t->off[rb + 1] = t->off[rb] + (rb < blocks ? ceil_div(p->cache_len + last / G + 1, kSimtKeys) : 0);
     }
+}
+// Most tokens whose angles a block of the small fp32 kernel forms in a one-launch step: its rows' and its share of the new ones.
+inline int f32_angle_tokens(const evlnStepParams* p, int splits)
+{
+    const int G = p->num_q_heads / p->num_kv_heads, own = std::min((kSmallRows + G - 2) / G + 1, p->num_new);
+    return std::min(own + ceil_div(p->num_new, splits), p->num_new);
 }
 // (most_splits: bound on the splits of the library's own choice)
 SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits, int most_splits = kMaxSplits)
@@ -424,7 +467,7 @@ SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits, 
     // kernel without tensor cores.)
     const bool tensor = use_f32_kernel(p) && ceil_div(R, 128) <= kSimtShareBlocks;
     const double big_tile = tensor ? 0.75 / d + 1.5 : 13.3, big_start = tensor ? 7.1 + 2.8 * d : 7.0;
-    SimtSchedule best = {8, splits > 0 ? splits : 1, 0};
+    SimtSchedule best = {8, splits > 0 ? splits : 1, 0, false};
     double best_cost = 1e30;
     const int smax = tiles < most_splits ? tiles : most_splits;
     for (int rpt = 8; rpt >= 2; rpt -= 6) {
@@ -432,11 +475,27 @@ SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits, 
         if (use_f32_kernel(p) && !tensor && rpt != 8) break;
         for (int s = splits > 0 ? splits : 1; s <= (splits > 0 ? splits : smax); ++s) {
             const long blocks = row_blocks * s;
-            const long at_once = rpt == 8 || blocks <= h->num_sms ? h->num_sms : 2 * h->num_sms;
-            const double tile_us = rpt == 8 ? big_tile : at_once == h->num_sms ? 6.3 : 9.5;
-            const double waves = (double)((blocks + at_once - 1) / at_once);
-            const double cost = waves * (ceil_div(tiles, s) * tile_us * d + (rpt == 8 ? big_start : 5.0)) + split_us * s;
-            if (cost < best_cost - 1e-9) { best_cost = cost; best = {rpt, s, 0}; }
+            double cost;
+            bool one_launch = false;
+            if (tensor && rpt == 2) {
+                if (ceil_div(R, kSmallRows) > 65535) break;
+                const double block_us = ceil_div(tiles, s) * (3.8 * d - 0.1) + 1.0;
+                cost = (double)((blocks + h->num_sms - 1) / h->num_sms) * block_us + 6.0 + (split_us - 0.2) * s;
+                const int tokens = f32_angle_tokens(p, s), fit = tokens <= kSmallAngleTokens && s <= kSmallCluster ? h->small_clusters[s - 1] : 0;
+                if (fit > 0) {
+                    // what a thread rotates, in vectors, and the angles it forms for that (with a table or without: the split count, and
+                    // by that the result's bits, are the same)
+                    const double items = (std::min(R, kSmallRows) + 3.0 * ceil_div(p->num_new, s)) * d / 16.0, angles = tokens * d / 4.0;
+                    const double one = (double)((row_blocks + fit - 1) / fit) * (block_us + 0.4 * items + 0.4 * angles) + 3.0 + 0.05 * s;
+                    if (one < cost) { cost = one; one_launch = true; }
+                }
+            } else {
+                const long at_once = rpt == 8 || blocks <= h->num_sms ? h->num_sms : 2 * h->num_sms;
+                const double tile_us = rpt == 8 ? big_tile : at_once == h->num_sms ? 6.3 : 9.5;
+                const double waves = (double)((blocks + at_once - 1) / at_once);
+                cost = waves * (ceil_div(tiles, s) * tile_us * d + (rpt == 8 ? big_start : 5.0)) + split_us * s;
+            }
+            if (cost < best_cost - 1e-9) { best_cost = cost; best = {rpt, s, 0, one_launch}; }
         }
     }
     if (splits == 0 && ceil_div(R, 128) <= kSimtShareBlocks && (long)ceil_div(R, 128) * p->num_kv_heads * tiles > h->num_sms) {
@@ -449,7 +508,7 @@ SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits, 
         if (share < ceil_div(most, kMaxSplits - 1)) share = ceil_div(most, kMaxSplits - 1);
         const int s = ceil_div(most - 1, share) + 1;
         const double cost = share * big_tile * d + big_start + (tensor ? 5.0 : 4.0) * ceil_div(share, t.off[1]) + split_us * (1.0 + (double)most / share);
-        if (s <= most_splits && cost < best_cost - 1e-9) best = {8, s, share};
+        if (s <= most_splits && cost < best_cost - 1e-9) best = {8, s, share, false};
     }
     return best;
 }
@@ -472,9 +531,9 @@ void launch_simt(const SimtSchedule& plan, const evlnStepParams* p, dim3 grid, c
 // The scale of the fp32 kernel in two floats each, with what its scores fall short of: the tensor core cuts the sums
 // behind every 16 channels off instead of rounding them (measured with normal numbers: 7.1e-8 of a score at 128 channels, half
 // of that at 64).
-void set_f32_scale(const evlnStepParams* p, SimtAttnArgs* a)
+void set_f32_scale(const evlnStepParams* p, SimtAttnArgs* a, bool small)
 {
-    const double scale = (p->softmax_scale > 0.f ? (double)p->softmax_scale : 1.0 / sqrt((double)p->head_dim)) * (1.0 + 5.5e-10 * p->head_dim);
+    const double scale = (p->softmax_scale > 0.f ? (double)p->softmax_scale : 1.0 / sqrt((double)p->head_dim)) * (1.0 + (small ? 2.75e-10 : 5.5e-10) * p->head_dim);
     const double scale2 = scale * 1.4426950408889634;
     a->scale = (float)scale;
     a->scale_lo = (float)(scale - (double)a->scale);
@@ -486,12 +545,11 @@ void set_f32_scale(const evlnStepParams* p, SimtAttnArgs* a)
 template <int D>
 void launch_f32(const SimtSchedule& plan, const evlnStepParams* p, dim3 grid, cudaStream_t st, SimtAttnArgs a)
 {
+    set_f32_scale(p, &a, plan.rows_per_thread == 2);
     if (plan.rows_per_thread == 2) {
-        launch_simt<float, D>(plan, p, grid, st, a);
-        return;
-    }
-    set_f32_scale(p, &a);
-    if (plan.share > 0) {
+        launch_pdl(attn_f32_small_kernel<D, false>, dim3(grid.z, grid.x, grid.y), dim3(kSmallThreads), SmallPlan<D>::kBytes, st, a,
+                   make_fast_div((uint32_t)a.G), F32Fused{});
+    } else if (plan.share > 0) {
         SimtTiles t;
         fill_simt_tiles(p, &t);
         const int blocks = ceil_div(t.off[kSimtShareBlocks] * p->num_kv_heads, plan.share);
@@ -499,6 +557,28 @@ void launch_f32(const SimtSchedule& plan, const evlnStepParams* p, dim3 grid, cu
     } else {
         launch_pdl(attn_f32_kernel<D, NoTable>, grid, dim3(kF32Threads), F32Plan<D>::kBytes, st, a, NoTable{});
     }
+}
+
+// The whole step in one launch: a cluster per (row block, kv head), a block per split.
+template <int D>
+cudaError_t launch_f32_step(const evlnStepParams* p, int splits, cudaStream_t st, SimtAttnArgs a, const F32Fused& f)
+{
+    set_f32_scale(p, &a, true);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(splits, ceil_div(a.num_new * a.G, kSmallRows), a.Hkv);
+    cfg.blockDim = dim3(kSmallThreads);
+    cfg.dynamicSmemBytes = SmallPlan<D>::kBytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = splits;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, attn_f32_small_kernel<D, true>, a, make_fast_div((uint32_t)a.G), f);
 }
 
 int resolve_splits(evlnHandle_t h, const evlnStepParams* p)
@@ -1018,6 +1098,7 @@ evlnStatus_t evlnCreate(evlnHandle_t* handle, int device)
     if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int));
     if (e == cudaSuccess) e = prepare_kernels();
     if (e == cudaSuccess) e = query_few_clusters(h->max_clusters);
+    if (e == cudaSuccess) e = query_small_clusters(h->small_clusters);
     if (e == cudaSuccess && !attention_register_pool_ok()) {
         cudaFree(h->d_status);
         delete h;
@@ -1211,6 +1292,17 @@ static bool step_buffers_shared(const evlnStepParams* p, const void* q_new, cons
     return output_over_q_rot(p, q_rot, out, lse_out);
 }
 
+// New tokens given in the cache itself (rotated in place).  Where the blocks of several row blocks rotate the same keys, one
+// would read what another has written.
+static bool new_tokens_in_cache(const evlnStepParams* p, const void* k_new, const void* v_new, long k_stride, long v_stride, const void* k_cache,
+                                const void* v_cache)
+{
+    const size_t e = elem_bytes(p->dtype), kv_row = (size_t)p->num_kv_heads * p->head_dim, before_last = (size_t)(p->num_new - 1);
+    const size_t k_bytes = (before_last * k_stride + kv_row) * e, v_bytes = (before_last * v_stride + kv_row) * e, cache = kv_row * p->cache_capacity * e;
+    return overlap(k_new, k_bytes, k_cache, cache) || overlap(k_new, k_bytes, v_cache, cache) || overlap(v_new, v_bytes, k_cache, cache) ||
+           overlap(v_new, v_bytes, v_cache, cache);
+}
+
 // Attention of a step.  `direct` (may be null): the step's final output; when the keys are not split and
 // the pair kernel runs, it writes that itself and `done` says that there is nothing left to combine.
 struct DirectOut {
@@ -1394,6 +1486,28 @@ evlnStatus_t evlnStep(evlnHandle_t h, const evlnStepParams* p, const void* q_new
         s = step_few(h, p, q_rot, k_cache, v_cache, o_part, o_part + (size_t)S * p->num_kv_heads * rows * 128, &f, (cudaStream_t)stream);
         if (s != EVLN_OK || S == 1) return s;
         return evlnStepCombine(h, p, workspace, out, lse_out, stream);
+    }
+    if (use_f32_kernel(p) && p->num_kv_heads <= 65535) {
+        const SimtSchedule plan = simt_schedule(h, p, p->num_splits);
+        if (plan.one_launch && !new_tokens_in_cache(p, k_new, v_new, k_stride_tok, v_stride_tok, k_cache, v_cache) &&
+            !step_buffers_shared(p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, out, lse_out)) {
+            s = check_rope_append(h, p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, k_cache, v_cache);
+            if (s != EVLN_OK) return s;
+            SimtAttnArgs a = {};
+            a.q_rot = q_rot; a.k_cache = k_cache; a.v_cache = v_cache;
+            a.Hkv = p->num_kv_heads; a.G = p->num_q_heads / p->num_kv_heads;
+            a.cache_len = p->cache_len; a.num_new = p->num_new; a.cache_cap = p->cache_capacity;
+            a.num_splits = plan.splits;
+            F32Fused f = {};
+            f.q_new = (const float*)q_new; f.k_new = (const float*)k_new; f.v_new = (const float*)v_new;
+            f.q_stride = q_stride_tok; f.k_stride = k_stride_tok; f.v_stride = v_stride_tok;
+            f.out = (float*)out; f.lse_out = lse_out;
+            f.log2_theta = log2(p->rope_theta);
+            f.table = (const double2*)p->rope_table; f.table_first = p->rope_table_first_pos;
+            const cudaError_t e = p->head_dim == 128 ? launch_f32_step<128>(p, plan.splits, (cudaStream_t)stream, a, f)
+                                                     : launch_f32_step<64>(p, plan.splits, (cudaStream_t)stream, a, f);
+            return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
+        }
     }
     s = evlnRopeAppend(h, p, q_new, k_new, v_new, q_stride_tok, k_stride_tok, v_stride_tok, q_rot, k_cache, v_cache,
                        stream);
@@ -2008,6 +2122,7 @@ evlnStatus_t noalloc_setup(int device, NoAllocDevice** out)
         if (e != cudaSuccess || qres != cudaDriverEntryPointSuccess || !fn) return EVLN_CUDA_ERROR;
         e = prepare_kernels();
         if (e == cudaSuccess) e = query_few_clusters(d->ctx.max_clusters);
+        if (e == cudaSuccess) e = query_small_clusters(d->ctx.small_clusters);
         if (e != cudaSuccess) return EVLN_CUDA_ERROR;
         if (!attention_register_pool_ok()) return EVLN_NOT_SUPPORTED;
         d->ctx.device = device;

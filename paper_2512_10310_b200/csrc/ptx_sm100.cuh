@@ -240,9 +240,32 @@ __device__ __forceinline__ void cluster_arrive_relaxed()
 {
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }
+// ... with it: what this thread wrote (shared memory included) is visible to the cluster's threads after their wait
+__device__ __forceinline__ void cluster_arrive()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_wait()
 {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr)
+{
+    float x;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(cluster_addr) : "memory");
+    return x;
+}
+__device__ __forceinline__ float2 ld_cluster_f32x2(uint32_t cluster_addr)
+{
+    float2 x;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(x.x), "=f"(x.y) : "r"(cluster_addr) : "memory");
+    return x;
+}
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t cluster_addr)
+{
+    float4 x;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(cluster_addr) : "memory");
+    return x;
 }
 // asynchronous stores to shared memory of any CTA of the cluster; their bytes are counted on an mbarrier there
 __device__ __forceinline__ void st_async_f32x4(uint32_t cluster_addr, const float4& v, uint32_t cluster_bar)

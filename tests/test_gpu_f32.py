@@ -1,5 +1,5 @@
-"""The fp32 step attention on the tensor cores (three bf16 parts per float) at the edges of its tiles, and
-where its splitting of numbers ends."""
+"""The fp32 step attention on the tensor cores (three bf16 parts per float) at the edges of its tiles, where
+its splitting of numbers ends, and as one launch."""
 import numpy as np
 import pytest
 import torch
@@ -41,7 +41,12 @@ def _step(handle, cfg, x, **options):
     (43, 1, 64, 100, 3, 0),        # 129 rows: a row block of one row
     (8, 1, 128, 449, 63, 8),       # 512 keys, a tile per split
     (8, 1, 128, 450, 63, 8),       # ... and one key more
+    (8, 1, 64, 1000, 24, 16),      # as many splits as a cluster takes
+    (8, 1, 64, 1000, 24, 17),      # one more
     (2, 2, 64, 10, 3, 7),          # more splits than key tiles
+    (2, 2, 128, 30, 16, 1),        # 16 rows: one row tile
+    (3, 1, 128, 500, 11, 0),       # 33 rows: a block of one row
+    (1, 1, 128, 100, 81, 1),       # angles of more tokens than a block holds
     (8, 4, 128, 0, 64, 0),         # no cache
     (8, 4, 128, 200, 65, 0),       # 130 rows per head
     (28, 4, 128, 1024, 196, 0),    # equal shares
@@ -83,3 +88,18 @@ def test_scores_beyond_any_sum(handle, hq, hkv, d, L, n):
     r = oracle_step("f32", x["k_cache"], x["v_cache"], x["q_new"], x["k_new"], x["v_new"], L, cfg.rope_theta)
     _, g = _step(handle, cfg, x)
     assert np.abs(f64(g["out"]) - r["out"]).max() <= 1e-5
+
+
+def test_new_keys_rotated_in_place(handle):
+    # one kv head: its new tokens can be given in the cache slots they are stored to.  80 rows: more than one block's
+    hq, d, L, n = 4, 64, 100, 20
+    cfg, x = _inputs(hq, 1, d, L, n)
+    _, want = _step(handle, cfg, x, fused=True)
+    dev = "cuda:0"
+    p = B.step_params("f32", hq, 1, d, L, n, L + n, cfg.rope_theta)
+    kc, vc = (torch.cat([x[a], x[b]]).permute(1, 0, 2).contiguous().to(dev) for a, b in (("k_cache", "k_new"), ("v_cache", "v_new")))
+    q, out = x["q_new"].to(dev), torch.empty((n, hq, d), device=dev)
+    q_rot = torch.empty(B.evlnStepQRotSize(handle, p), dtype=torch.uint8, device=dev)
+    ws = torch.empty(B.evlnStepWorkspaceSize(handle, p), dtype=torch.uint8, device=dev)
+    B.evlnStep(handle, p, q, kc[0, L:].view(n, 1, d), vc[0, L:].view(n, 1, d), q_rot, kc, vc, ws, out, None)
+    assert torch.equal(out, want["out"])
