@@ -2,7 +2,7 @@
 //
 //   M = max_s lse_s,  w_s = e^{lse_s - M},  O = sum_s w_s O_s / sum_s w_s,  lse = M + log sum_s w_s
 //
-// One warp per packed query row: lane s holds lse_s (at most 32 splits), the maximum and the
+// One warp per packed query row (or per 32 channels of one: see the forms below): lane s holds lse_s (at most 32 splits), the maximum and the
 // weight sum are warp-shuffle reductions, then each lane merges D/32 contiguous channels with
 // vector loads.  The row is rounded once to the storage dtype and written to its place in the
 // token-major [n, Hq, D] output.  HBM/L2-bound: S*(D+1) floats in, D elements out per row.
@@ -33,13 +33,26 @@ struct CombineArgs {
     PackedMap map;           // where output token m goes (identity unless the call serves a packed sequence)
 };
 
-template <typename T, int D, bool PAGED, typename LensT>
-__global__ void __launch_bounds__(128)
+// Forms of the kernel, by the most parts of a row and by the rows; the sums keep the order of the parts in all of them, so
+// the bits are the same.
+//   few   at most kCombineFewParts: no loop behind the first loads, so that the kernel keeps 42 registers and a step of
+//         1400 blocks is one wave (196 tokens of the 7B shape: 64 registers and 1.2 waves before)
+//   many  a loop over the rest, eight parts at a time
+//   wide  few rows in many parts: a row's D / 32 warps take 32 channels each, a lane one float of each part, so that up to
+//         16 parts are on their way at once, on four times as many SMs
+constexpr int kCombineFew = 0, kCombineMany = 1, kCombineWide = 2;
+constexpr int kCombineFewParts = 4;
+
+template <typename T, int D, bool PAGED, typename LensT, int FORM>
+__global__ void __launch_bounds__(128, FORM == kCombineFew ? 12 : 1)
 combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
 {
-    constexpr int C = D / 32;
+    constexpr bool WIDE = FORM == kCombineWide;
+    constexpr int kWarps = WIDE ? D / 32 : 1;                   // warps per row
+    constexpr int C = WIDE ? 1 : D / 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t row = blockIdx.x * 4u + (uint32_t)warp;      // packed row within kv head (< 2^24, checked on the host)
+    const int col = WIDE ? (warp % kWarps) * 32 + lane : lane * C;      // the lane's first channel
+    const uint32_t row = (blockIdx.x * 4u + (uint32_t)warp) / kWarps;   // packed row within kv head (< 2^24, checked on the host)
     const int g = blockIdx.y;
     if (row >= (uint32_t)a.rows) return;
     const uint32_t row_tok = fast_div(row, a.div_g);            // its token among the call's new tokens ...
@@ -79,7 +92,7 @@ combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
     asm volatile("griddepcontrol.wait;" ::: "memory");          // programmatic dependent launch: inputs ready
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    constexpr int kPre = 4;
+    constexpr int kPre = WIDE ? 16 : kCombineFewParts;
     // (Letting every lane read all log-sum-exps of a row with few splits, so that the maximum and
     // the weights need no shuffles, was measured slower: 3.85 against 3.45 us at the 7B step.)
     float my_lse = (lane < S) ? a.lse_part[prow0 + lane * stride_s] : -INFINITY;
@@ -88,7 +101,7 @@ combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
 #pragma unroll
     for (int s = 0; s < kPre; ++s) {
         if (s < S) {
-            const float* op = a.o_part + (prow0 + s * stride_s) * D + lane * C;
+            const float* op = a.o_part + (prow0 + s * stride_s) * D + col;
             if (C == 4) {
                 float4 x = *reinterpret_cast<const float4*>(op);
                 pre[s][0] = x.x; pre[s][1] = x.y; pre[s][2] = x.z; pre[s][3] = x.w;
@@ -120,14 +133,14 @@ combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
     }
     // the remaining splits four at a time: their loads are in flight together, the sums keep the
     // order of the splits
-    constexpr int kBatch = 8;
-    for (int s0 = kPre; s0 < S; s0 += kBatch) {
+    constexpr int kBatch = WIDE ? 16 : 8;
+    for (int s0 = kPre; FORM != kCombineFew && s0 < S; s0 += kBatch) {
         float v[kBatch][C];
 #pragma unroll
         for (int k = 0; k < kBatch; ++k) {
             const int s = s0 + k;
             if (s < S) {
-                const float* op = a.o_part + (prow0 + s * stride_s) * D + lane * C;
+                const float* op = a.o_part + (prow0 + s * stride_s) * D + col;
                 if (C == 4) {
                     float4 x = *reinterpret_cast<const float4*>(op);
                     v[k][0] = x.x; v[k][1] = x.y; v[k][2] = x.z; v[k][3] = x.w;
@@ -154,10 +167,16 @@ combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
     const long tok = packed_row(a.map, (int)row_tok);
     const int h = g * a.G + row_head;
     const int Hq = a.Hkv * a.G;
-    T* dst = (T*)a.out + (tok * Hq + h) * D + lane * C;
+    T* dst = (T*)a.out + (tok * Hq + h) * D + col;
+    __align__(16) T y[C];
 #pragma unroll
-    for (int c = 0; c < C; ++c) from_float(acc[c] * inv, dst[c]);
-    if (a.lse_out && lane == 0) a.lse_out[tok * Hq + h] = (wsum > 0.f) ? M + logf(wsum) : -INFINITY;
+    for (int c = 0; c < C; ++c) from_float(acc[c] * inv, y[c]);
+    constexpr int kBytes = C * (int)sizeof(T);
+    if constexpr (kBytes == 16) *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(y);
+    else if constexpr (kBytes == 8) *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(y);
+    else if constexpr (kBytes == 4) *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(y);
+    else *dst = y[0];
+    if (a.lse_out && col == 0) a.lse_out[tok * Hq + h] = (wsum > 0.f) ? M + logf(wsum) : -INFINITY;
 }
 
 // The combine step of rows whose keys were not split: the one partial of a row is its output, rounded and put in its

@@ -849,6 +849,9 @@ void fill_lens(BatchLens* bl, const evlnPagedParams* p, const int* lens, const i
     }
 }
 
+// Up to 2048 rows a block per row (of 128 channels) fills the SMs no more than a few times over.  (8 tokens over 20656
+// keys, 224 rows in 28 parts: 18.0 us a step with a warp per row, 17.6 so; 16 paged episodes of one token 53.6 and 52.5.)
+constexpr long kCombineWideRows = 2048;
 template <typename T>
 evlnStatus_t launch_combine(evlnHandle_t h, const CombineArgs& args, int D, bool paged, const BatchLens* bl,
                             cudaStream_t st, const SimtTiles* shares = nullptr)
@@ -856,18 +859,25 @@ evlnStatus_t launch_combine(evlnHandle_t h, const CombineArgs& args, int D, bool
     CombineArgs a = args;
     a.div_g = make_fast_div((uint32_t)a.G);
     a.div_chunk = make_fast_div((uint32_t)(a.chunk_tiles > 0 ? a.chunk_tiles : 1));
-    dim3 grid(ceil_div(a.rows, 4), a.Hkv);
-    if (paged) {
-        if (D == 128) launch_pdl(combine_kernel<T, 128, true, BatchLens>, dim3(grid), dim3(128), 0, st, a, *bl);
-        else return EVLN_NOT_SUPPORTED;
-    } else if (shares) {
-        if (D == 128) launch_pdl(combine_kernel<T, 128, false, SimtTiles>, dim3(grid), dim3(128), 0, st, a, *shares);
-        else launch_pdl(combine_kernel<T, 64, false, SimtTiles>, dim3(grid), dim3(128), 0, st, a, *shares);
-    } else {
-        NoLens nl = {};
-        if (D == 128) launch_pdl(combine_kernel<T, 128, false, NoLens>, dim3(grid), dim3(128), 0, st, a, nl);
-        else launch_pdl(combine_kernel<T, 64, false, NoLens>, dim3(grid), dim3(128), 0, st, a, nl);
-    }
+    if (paged && D != 128) return EVLN_NOT_SUPPORTED;
+    const bool wide = a.num_splits > kCombineFewParts && (long)a.rows * a.Hkv <= kCombineWideRows;
+    const dim3 grid(ceil_div(a.rows, wide ? 128 / D : 4), a.Hkv);
+    auto launch = [&](auto form) {
+        constexpr int FORM = decltype(form)::value;
+        if (paged) {
+            launch_pdl(combine_kernel<T, 128, true, BatchLens, FORM>, grid, dim3(128), 0, st, a, *bl);
+        } else if (shares) {
+            if (D == 128) launch_pdl(combine_kernel<T, 128, false, SimtTiles, FORM>, grid, dim3(128), 0, st, a, *shares);
+            else launch_pdl(combine_kernel<T, 64, false, SimtTiles, FORM>, grid, dim3(128), 0, st, a, *shares);
+        } else {
+            NoLens nl = {};
+            if (D == 128) launch_pdl(combine_kernel<T, 128, false, NoLens, FORM>, grid, dim3(128), 0, st, a, nl);
+            else launch_pdl(combine_kernel<T, 64, false, NoLens, FORM>, grid, dim3(128), 0, st, a, nl);
+        }
+    };
+    if (a.num_splits <= kCombineFewParts) launch(std::integral_constant<int, kCombineFew>());
+    else if (wide) launch(std::integral_constant<int, kCombineWide>());
+    else launch(std::integral_constant<int, kCombineMany>());
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
 }
