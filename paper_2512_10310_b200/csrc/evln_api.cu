@@ -934,7 +934,9 @@ template <typename T, bool PAGED, typename LensT>
 void launch_rope_append(const RopeArgs& a, int tokens, cudaStream_t st, const LensT& lens)
 {
     const int items = rope_items(a), parts = tokens <= kRopeFewTokens ? ceil_div(items, kRopeThreadsMax) : 1;
-    launch_pdl(rope_append_kernel<T, PAGED, LensT>, dim3(tokens + (PAGED ? a.batch : 0), parts), rope_block(ceil_div(items, parts)), 0, st, a, lens);
+    const dim3 grid(tokens + (PAGED ? a.batch : 0), parts), block = rope_block(ceil_div(items, parts));
+    if (!PAGED && tokens <= kRopeFewTokens) launch_pdl(rope_append_kernel<T, PAGED, LensT, !PAGED>, grid, block, 0, st, a, lens);
+    else launch_pdl(rope_append_kernel<T, PAGED, LensT, false>, grid, block, 0, st, a, lens);
 }
 
 // CTA pairs of a persistent launch: one per two SMs, no more than there are items.
