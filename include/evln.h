@@ -185,8 +185,9 @@ evlnStatus_t evlnRopeAppend(evlnHandle_t handle, const evlnStepParams* params,
  * 1; a split that a row sees no key of has output 0 and log-sum-exp -inf).  Must run after evlnRopeAppend of the same step on the same stream.
  * bf16 with head_dim 128 runs on the tensor cores: CTA pairs over 256-row units of the packed
  * query rows, or, when all n * G rows of a kv head fit one 128-row tile (the few action tokens
- * decoded after a frame, Sec. 3.1), one CTA per (kv head, KV split); at most 32 rows per kv head
- * in clusters of blocks that merge a head's keys among themselves.                            */
+ * decoded after a frame, Sec. 3.1), one CTA per (kv head, KV split); short unsplit steps of few
+ * rows on one CTA per 128-row tile; at most 32 rows per kv head in clusters of blocks that merge a
+ * head's keys among themselves.                                                                */
 evlnStatus_t evlnStepAttention(evlnHandle_t handle, const evlnStepParams* params,
                                const void* q_rot, const void* k_cache, const void* v_cache,
                                void* workspace, size_t workspace_bytes, void* stream);
@@ -198,7 +199,7 @@ evlnStatus_t evlnStepCombine(evlnHandle_t handle, const evlnStepParams* params,
 
 /* The whole step in one call (Sec. 3.2): evlnRopeAppend, evlnStepAttention and evlnStepCombine
  * with the same arguments, enqueued on `stream`; same results bit for bit.  Two launches instead of
- * three where bf16 steps of head_dim 128 on CTA pairs are not split.  Steps of at most 32 query rows
+ * three where bf16 steps of head_dim 128 on CTA pairs or single CTAs are not split.  Steps of at most 32 query rows
  * per kv head and 16 tokens: one launch, two when split (not where the one-CTA kernel serves them:
  * more than 16 rows with 8 or more kv heads and 3072 or more keys, or more than 24 rows with 4 kv
  * heads and 24576 or more keys).  fp32 steps of little work (a few hundred rows, a tile or two of keys

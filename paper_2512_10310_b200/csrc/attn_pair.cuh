@@ -393,7 +393,7 @@ __device__ __forceinline__ void write_rows(const TcAttnArgs& a, const LensT& len
     const int first_row = w.unit * (CTAS * kTileM) + (int)rank * kTileM + (quarter << 5);   // episode-local
     const int r_local = first_row + lane;
     const int rows_here = rows_valid - first_row;                    // may be <= 0 or > 32
-    const bool direct = CTAS == 2 && d.out != nullptr && !(TAIL && !w.visual && d.act_split);
+    const bool direct = d.out != nullptr && !(TAIL && !w.visual && d.act_split);
     uint32_t regs[32];
     ptx::tmem_ld32(t_o, regs);
     ptx::tmem_ld_wait();
@@ -1274,9 +1274,9 @@ attn_packed_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 // each CTA streams whole K/V tiles, so that a long cache is read at the rate HBM delivers it.
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_solo_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                 const __grid_constant__ CUtensorMap tm_v, const TcAttnArgs a)
+                 const __grid_constant__ CUtensorMap tm_v, const TcAttnArgs a, const __grid_constant__ TcOutArgs d)
 {
-    attn_tc_body<false, false, false, NoLens, 1, NoTable>(tm_q, tm_k, tm_v, nullptr, nullptr, nullptr, a, NoLens{}, TcOutArgs{}, NoTable{});
+    attn_tc_body<false, false, false, NoLens, 1, NoTable>(tm_q, tm_k, tm_v, nullptr, nullptr, nullptr, a, NoLens{}, d, NoTable{});
 }
 
 }  // namespace evln

@@ -267,6 +267,16 @@ inline bool use_solo_kernel(const evlnStepParams* p)
     return use_tensor_kernel(p) && (long)p->num_new * (p->num_q_heads / p->num_kv_heads) <= kTileM;
 }
 
+// Short unsplit steps whose 128-row tiles leave SMs idle: a CTA per tile instead of a pair per two, which have not to meet
+// before they start nor at the end, and of which the first need fewer key tiles.  (28 layers, 7B shape: 256 tokens on an empty cache 271 us a
+// pass with pairs, 265 so; 400 359 and 357; 196 over 256 306 and 303.  For long walks the pairs' halved K/V traffic is worth more: 196
+// tokens over 4096 keys 15.8 us a layer and 16.8.)
+inline bool use_single_ctas(evlnHandle_t h, const evlnStepParams* p, int splits)
+{
+    const int G = p->num_q_heads / p->num_kv_heads, tiles = ceil_div(p->num_new * G, kTileM);
+    return splits == 1 && (long)tiles * p->num_kv_heads <= h->num_sms && ceil_div(p->cache_len + p->num_new, kTileN) <= 4;
+}
+
 // Split schedule of the one-CTA-per-item kernel, in microseconds: a CTA takes 0.9 per KV tile unless HBM (all
 // of K and V at most of its rate) takes longer, and a split adds partials of every row to write and merge.
 // (Measured over 500 .. 32000 cached keys, 4 and 8 kv heads, 35 .. 128 rows each: within 3 % of the best split
@@ -1348,6 +1358,7 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
         return step_few(h, p, q_rot, k_cache, v_cache, o_part, lse_part, nullptr, st);
     } else if (use_tensor_kernel(p)) {
         const int T = p->cache_len + p->num_new;
+        const bool alone = use_solo_kernel(p) || use_single_ctas(h, p, S);
         CUtensorMap tm_q, tm_k, tm_v;
         {
             cuuint64_t dims[3] = {128, (cuuint64_t)R, (cuuint64_t)p->num_kv_heads};
@@ -1364,22 +1375,28 @@ static evlnStatus_t step_attention(evlnHandle_t h, const evlnStepParams* p, cons
             // (a CTA on its own takes whole tiles: two 128-key boxes each)
             cuuint32_t box_k[3] = {64, 64, 1};
             cuuint32_t box_v[3] = {64, 128, 1};
-            if (!encode_map(h, &tm_k, k_cache, 3, dims, strides, use_solo_kernel(p) ? box_v : box_k)) return EVLN_INVALID_VALUE;
+            if (!encode_map(h, &tm_k, k_cache, 3, dims, strides, alone ? box_v : box_k)) return EVLN_INVALID_VALUE;
             if (!encode_map(h, &tm_v, v_cache, 3, dims, strides, box_v)) return EVLN_INVALID_VALUE;
         }
         TcAttnArgs a = {};
         a.o_part = o_part; a.lse_part = lse_part; a.page_table = nullptr; a.status = h->d_status;
         a.Hkv = p->num_kv_heads; a.G = G; a.rows = R;
         a.cache_len = p->cache_len; a.num_new = p->num_new; a.num_splits = S;
-        a.units_per_head = use_solo_kernel(p) ? 1 : ceil_div(R, kUnitRows);
+        a.units_per_head = ceil_div(R, alone ? kTileM : kUnitRows);
         a.scale_log2 = scale * 1.4426950408889634f;
         a.div_g = make_fast_div((uint32_t)G);
         a.div_s = make_fast_div((uint32_t)S);
         NoLens nl = {};
         // one work item per (unit, kv head, split): the kernels read it off the block index
         if (p->num_kv_heads > 65535) return EVLN_NOT_SUPPORTED;
-        if (use_solo_kernel(p)) {
-            launch_pdl(attn_solo_kernel, dim3(1, p->num_kv_heads, S), dim3(kTcThreads), kSoloSmemBytes, st, tm_q, tm_k, tm_v, a);
+        if (alone) {
+            TcOutArgs d = {};
+            if (S == 1 && direct) {
+                d.out = (__nv_bfloat16*)direct->out;
+                d.lse_out = direct->lse_out;
+                direct->done = true;
+            }
+            launch_pdl(attn_solo_kernel, dim3(a.units_per_head, p->num_kv_heads, S), dim3(kTcThreads), kSoloSmemBytes, st, tm_q, tm_k, tm_v, a, d);
         } else {
             TcOutArgs d = {};
             if (S == 1 && direct) {                // final rows, straight to the caller
