@@ -244,7 +244,9 @@ __device__ __forceinline__ void poly_ex2_pair(uint64_t x2, float& p0, float& p1)
 // of a sub-partition busy for as long as the tile's MMAs keep the tensor pipe busy, so a quarter of
 // them (one pair in eight scores) is computed on the FMA pipe, which has issue slots to spare;
 // a larger share costs more issue slots than it frees SFU cycles (measured: 25 % is 2-3 % faster
-// than none at every cache length, 50 % is slower).
+// than none at every cache length, 50 % is slower).  Not in persistent pairs over paged batches (POLY false), which run deepest
+// in the power cap: the cubic's instructions cost more energy than SFU time (16 episodes of a frame 432 us, 427 without; 4 of them 139 and 137).
+template <bool POLY>
 __device__ __forceinline__ void exp32(const uint32_t* s, uint32_t (&packed)[16], uint64_t scale2,
                                       uint64_t negm2, uint64_t& sum2a, uint64_t& sum2b)
 {
@@ -255,7 +257,7 @@ __device__ __forceinline__ void exp32(const uint32_t* s, uint32_t (&packed)[16],
         float x0, x1, p0, p1, p2, p3;
         ptx::unpack2(xa, x0, x1);
         p0 = ptx::ex2(x0); p1 = ptx::ex2(x1);
-        if (((e >> 2) & 1) == 0) {
+        if (POLY && ((e >> 2) & 1) == 0) {
             poly_ex2_pair(xb, p2, p3);
         } else {
             float x2, x3;
@@ -1125,7 +1127,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
             uint64_t sum2a = ptx::pack2(0.f, 0.f), sum2b = sum2a;
             {
                 uint32_t pk[16];
-                exp32(&s[0], pk, scale2, negm2, sum2a, sum2b);
+                exp32<!(PAGED && PERSIST)>(&s[0], pk, scale2, negm2, sum2a, sum2b);
                 while (ok && gj >= 2) {
                     const int r = wait_or_request(bar_pv_done + 8 * ((gj - 2) & 3), ((gj - 2) >> 2) & 1, kDevTimeoutSoftmaxO);
                     if (r == 0) break;
@@ -1158,7 +1160,7 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
                 const float neg_m2 = (m_ref == -INFINITY) ? 0.f : -m_ref;
                 const uint64_t negm2b = ptx::pack2(neg_m2, neg_m2);
                 uint32_t pk[16];
-                exp32(&s[32], pk, scale2, negm2b, sum2a, sum2b);
+                exp32<!(PAGED && PERSIST)>(&s[32], pk, scale2, negm2b, sum2a, sum2b);
                 ptx::tmem_st16(t_p + 16, pk);
             }
             {
