@@ -7,7 +7,7 @@
 // across key tiles: every tile's scores and every tile's products with V start from zero, and the tiles' results
 // are added in registers, rounded to nearest.
 //
-// Bound: the tensor pipe (6 x 4 D bf16 flop per visible pair).  A block of 16 + 1 warps owns 128 packed query rows of
+// Bound: the tensor pipe (6 x 4 D bf16 flop per visible pair), with all SMs at work the latency of K and V out of L2.  A block of 16 + 1 warps owns 128 packed query rows of
 // one kv head and walks its key tiles, 64 keys at a time:
 //   16 warps, four per TMEM lane quarter: a thread has a row, 16 of the tile's 64 score columns and a
 //            quarter of the channels.  Per tile they split the next K tile into its three parts (from
@@ -20,8 +20,8 @@
 //
 // SHARE: as in attn_simt.cuh, one block per SM with an equal share of all (row block, key tile) pairs.
 //
-// Measured: a tile 2.2 us at head_dim 128 (the products alone 1.9), 1.5 at 64; 196 tokens of the 7B shape over 1024 keys 96.7 us a step
-// in float FMAs, 33.5 so; 256 tokens over 2048 206 and 60; 252 tokens of 16 heads over 2031 123 and 37.
+// Measured: a tile 2.2 us at head_dim 128 (the products alone 1.9; about 3 with a block on every SM), 1.5 at 64; 196 tokens of the 7B shape over 1024 keys 96.7 us a step
+// in float FMAs, 33.0 so; 256 tokens over 2048 206 and 60; 252 tokens of 16 heads over 2031 123 and 37.
 #pragma once
 
 #include "attn_pair.cuh"
