@@ -73,7 +73,7 @@ store_append_kernel(const GatherArgs a)
 // per token, all of it behind the angles: 6.5 us for 3392 tokens of 4 kv heads; this: 5.3).  For tokens whose keys are
 // one chunk, and for few tokens: every further chunk of keys needs the token's angles again.
 // Bound by the warps in flight: six blocks an SM (40 registers, a few words spilled to L1) instead of the five that 48
-// registers leave, and 3392 kept tokens a layer are 736 -> 724 us for 28 re-indexed layers.
+// registers leave, and 3392 kept tokens a layer are 736 -> 724 us for 28 re-indexed layers (eight, at 32 registers: 780).
 constexpr int kGatherWarps = 8;
 
 template <typename T>
