@@ -33,8 +33,9 @@ struct CombineArgs {
     PackedMap map;           // where output token m goes (identity unless the call serves a packed sequence)
 };
 
-// Forms of the kernel, by the most parts of a row and by the rows; the sums keep the order of the parts in all of them, so
-// the bits are the same.
+// Forms of the kernel, by the most parts of a row and by the rows; the sums keep the order of the parts in all of them, and
+// all of them leave out the parts from kCombineFewParts on whose weight is 0 (an infinite value at a key of no weight is then
+// not multiplied by 0), so the bits are the same.
 //   few   at most kCombineFewParts: no loop behind the first loads, so that the kernel keeps 42 registers and a step of
 //         1400 blocks is one wave (196 tokens of the 7B shape: 64 registers and 1.2 waves before)
 //   many  a loop over the rest, eight parts at a time
@@ -128,10 +129,12 @@ combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
 #pragma unroll
     for (int s = 0; s < kPre; ++s) {
         const float ws = __shfl_sync(0xffffffffu, w, s);      // 0 for s >= S and for empty splits
+        if (s < kCombineFewParts || ws != 0.f) {              // (see the forms above)
 #pragma unroll
-        for (int c = 0; c < C; ++c) acc[c] = fmaf(ws, pre[s][c], acc[c]);
+            for (int c = 0; c < C; ++c) acc[c] = fmaf(ws, pre[s][c], acc[c]);
+        }
     }
-    // the remaining splits four at a time: their loads are in flight together, the sums keep the
+    // the remaining splits, kBatch at a time: their loads are in flight together, the sums keep the
     // order of the splits
     constexpr int kBatch = WIDE ? 16 : 8;
     for (int s0 = kPre; FORM != kCombineFew && s0 < S; s0 += kBatch) {

@@ -54,3 +54,34 @@ def test_merge_against_fp64(handle, dtype, hq, hkv, d, n, splits):
     eps = 2.0 ** -8 if dtype == "bf16" else 0.0
     assert bool(((out.double() - want).abs() <= eps * want.abs() + 40 * 2.0 ** -24 * 4.0).all())
     assert float((got_lse.double() - total).abs().max()) <= 16 * 2.0 ** -24 * float(total.abs().max().clamp(min=1.0))
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("hq,hkv,d,n,splits", [
+    (28, 4, 128, 73, 12),          # 2044 rows: a block per row
+    (28, 4, 128, 74, 12),          # 2072 rows: a warp per row
+    (14, 2, 64, 9, 17),
+])
+def test_parts_of_no_weight_are_left_out(handle, dtype, hq, hkv, d, n, splits):
+    # a part from the fifth on whose weight underflows to 0 holds infinite and undefined values: not in the sum, whatever the form
+    gen = torch.Generator(device=DEV).manual_seed(7 * splits + n)
+    p = B.step_params(dtype, hq, hkv, d, 32 * 64, n, 32 * 64 + n, 1e4, num_splits=splits)
+    rows = n * hq // hkv
+    o = torch.randn((splits, hkv, rows, d), generator=gen, device=DEV)
+    lse = 3.0 * torch.randn((splits, hkv, rows), generator=gen, device=DEV)
+    none = torch.rand((splits, hkv, rows), generator=gen, device=DEV) < 0.3
+    none[:4] = False
+    none[4] = True
+    lse[none] = -200.0
+    o[none] = 0.0
+    outs = []
+    for filler in (0.0, float("inf"), float("nan")):
+        part = o.clone()
+        part[none] = filler
+        ws = torch.cat([part.flatten(), lse.flatten()])
+        ws = torch.cat([ws, torch.zeros(max(0, (B.evlnStepWorkspaceSize(handle, p) - ws.numel() * 4 + 3) // 4), device=DEV)])
+        out = torch.empty((n, hq, d), dtype=torch.bfloat16 if dtype == "bf16" else torch.float32, device=DEV)
+        B.evlnStepCombine(handle, p, ws, out, None)
+        outs.append(out)
+    assert bool(torch.isfinite(outs[0]).all())
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])

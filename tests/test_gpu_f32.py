@@ -103,3 +103,27 @@ def test_new_keys_rotated_in_place(handle):
     ws = torch.empty(B.evlnStepWorkspaceSize(handle, p), dtype=torch.uint8, device=dev)
     B.evlnStep(handle, p, q, kc[0, L:].view(n, 1, d), vc[0, L:].view(n, 1, d), q_rot, kc, vc, ws, out, None)
     assert torch.equal(out, want["out"])
+
+
+@pytest.mark.parametrize("hq,hkv,d,L,n,splits,first,count", [
+    (8, 1, 64, 1000, 24, 12, 768, 64),         # split 9 of 12; evlnStep in one launch
+    (28, 4, 128, 1024, 196, 12, 960, 64),      # ... of 12, 128-row blocks
+])
+def test_infinite_values_of_keys_without_weight(handle, hq, hkv, d, L, n, splits, first, count):
+    # `count` keys whose scores are 150 below all others: what they hold is not in the result, in one call or in three
+    cfg, x = _inputs(hq, hkv, d, L, n)
+    slow = d // 2 - 1                          # the channel that turns least: half a radian over these positions
+    x["q_new"][:, :, slow] = 40.0
+    x["q_new"][:, :, slow + d // 2] = 0.0
+    keys = torch.cat([x["k_cache"], x["k_new"]])
+    keys[:, :, slow] = 0.0
+    keys[first:first + count, :, slow] = -80.0
+    values = torch.cat([x["v_cache"], x["v_new"]])
+    got = []
+    for filler in (0.0, float("inf")):
+        values[first:first + count] = filler
+        y = dict(x, k_cache=keys[:L], k_new=keys[L:], v_cache=values[:L], v_new=values[L:])
+        for fused in (False, True):
+            got.append(_step(handle, cfg, y, num_splits=splits, fused=fused)[1]["out"])
+    assert torch.equal(got[0], got[1]) and torch.equal(got[2], got[3])
+    assert bool(torch.isfinite(got[2]).all()) and torch.equal(got[0], got[2])
