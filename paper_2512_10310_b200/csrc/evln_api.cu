@@ -2059,9 +2059,11 @@ extern "C" evlnStatus_t evlnGatherRope(evlnHandle_t h, const evlnGatherParams* p
         return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
     }
     if (total * (a.k_chunks + a.v_chunks) > 0x7fffff00L) return EVLN_NOT_SUPPORTED;
-    const dim3 grid((unsigned)((total * (a.k_chunks + a.v_chunks) + kGatherWarps - 1) / kGatherWarps)), block(32 * kGatherWarps);
-    if (p->dtype == EVLN_BF16) launch_pdl(gather_rope_kernel<__nv_bfloat16>, grid, block, 0, st, a, segs);
-    else launch_pdl(gather_rope_kernel<float>, grid, block, 0, st, a, segs);
+    const long blocks = (total * (a.k_chunks + a.v_chunks) + kGatherWarps - 1) / kGatherWarps;
+    const dim3 grid((unsigned)blocks), block(32 * kGatherWarps);
+    const bool wave = gather_one_wave(a.Hkv << a.vph_shift, a.k_chunks, blocks, a.table != nullptr, h->num_sms);
+    if (p->dtype == EVLN_BF16) launch_pdl(wave ? gather_rope_kernel<__nv_bfloat16, true> : gather_rope_kernel<__nv_bfloat16, false>, grid, block, 0, st, a, segs);
+    else launch_pdl(wave ? gather_rope_kernel<float, true> : gather_rope_kernel<float, false>, grid, block, 0, st, a, segs);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? EVLN_OK : cuda_fail(h, e);
 }

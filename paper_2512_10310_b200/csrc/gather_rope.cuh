@@ -72,12 +72,23 @@ store_append_kernel(const GatherArgs a)
 // do not wait for each other, so a call of a few thousand tokens is one wave of short chains (a block
 // per token, all of it behind the angles: 6.5 us for 3392 tokens of 4 kv heads; this: 5.3).  For tokens whose keys are
 // one chunk, and for few tokens: every further chunk of keys needs the token's angles again.
-// Bound by the warps in flight: six blocks an SM (40 registers, a few words spilled to L1) instead of the five that 48
-// registers leave, and 3392 kept tokens a layer are 736 -> 724 us for 28 re-indexed layers (eight, at 32 registers: 780).
-constexpr int kGatherWarps = 8;
+// WAVE: all blocks run at once.  Then they are there while the previous kernel ends, and each warp requests its source rows into L2
+// meanwhile; bounded to 40 registers (a few words spilled to L1), so that six blocks fit an SM instead of the five that 48 registers
+// leave (28 re-indexed layers of 3392 kept tokens 774 us, 736 with the requests, 724 with six blocks; eight, at 32 registers: 780).
+// More tokens run in several rounds, whose blocks are not there ahead of time: requests and spills only cost (us a layer, 20000 tokens
+// of 4 kv heads without a table 20.5, 23.9 in the form for one wave; 5000 of 1 head 6.1 and 6.9).  Two rounds are a little faster so where
+// warps are full and the angles come from a table (1700 tokens of 32 kv heads of 64 channels 7.2 and 6.7, 5000 of 4 in fp32 5.5 and 5.2).
+constexpr int kGatherWarps = 8, kGatherWaveBlocks = 6;
+// Nor is that form used where the SMs have several blocks of little to request each (844 tokens of one kv head 2.16 us and 2.53; 250
+// 2.07 and 2.06, 3392 5.7 and 4.4), or a block's warps share a token's many chunks of keys (60 tokens of 32 kv heads 2.59 and 2.68).
+inline bool gather_one_wave(int k_items, int k_chunks, long blocks, bool table, int sms)
+{
+    if (blocks > (long)kGatherWaveBlocks * sms * (table && k_items >= 32 ? 2 : 1)) return false;
+    return k_chunks > 4 ? blocks > sms : blocks <= sms || k_items * blocks > 32L * sms;
+}
 
-template <typename T>
-__global__ void __launch_bounds__(32 * kGatherWarps, 6)
+template <typename T, bool WAVE>
+__global__ void __launch_bounds__(32 * kGatherWarps, WAVE ? kGatherWaveBlocks : 0)
 gather_rope_kernel(const GatherArgs a, const __grid_constant__ SegList segs)
 {
     constexpr int V = VecTraits<T>::kVec;
@@ -93,9 +104,7 @@ gather_rope_kernel(const GatherArgs a, const __grid_constant__ SegList segs)
         if (segs.dst_off[mid] <= pos) lo = mid; else hi = mid;
     }
     const long src_slot = segs.src[lo] + (pos - segs.dst_off[lo]);
-    // The warp's source rows on their way into L2 while the previous kernel ends (3392 kept tokens of a store of 64 frames:
-    // 774 us a re-indexed step of 28 layers, 758 so).
-    if (pos < a.num_tokens) {
+    if (WAVE && pos < a.num_tokens) {
         const bool is_k = chunk < a.k_chunks;
         const int row_lines = D * (int)sizeof(T) / 128, chunks = is_k ? a.k_chunks : a.v_chunks, lines = (a.Hkv * row_lines + chunks - 1) / chunks;
         const char* from = reinterpret_cast<const char*>((const T*)(is_k ? a.k_src : a.v_src) + src_slot * D);

@@ -176,6 +176,10 @@ def test_offloaded_store_episode_matches_the_oracle(handle):
     ("f32", 3, 128, [130]),
     ("f32", 32, 128, [3, 140]),               # more work items than a block has threads, several times
     ("f32", 9, 64, [300]),
+    ("bf16", 4, 128, [3550, 2]),              # as many blocks as 148 SMs run at once; without a table ...
+    ("bf16", 4, 128, [3550, 3]),              # ... and one more: in two rounds
+    ("f32", 2, 128, [7106]),                  # ... and with one
+    ("bf16", 1, 128, [2300, 71]),             # a quarter of the lanes
 ])
 def test_gather_of_tokens_with_many_heads(handle, dtype, hkv, d, lengths):
     gen = torch.Generator().manual_seed(hkv + d)
