@@ -36,16 +36,16 @@ struct CombineArgs {
 // Forms of the kernel, by the most parts of a row and by the rows; the sums keep the order of the parts in all of them, and
 // all of them leave out the parts from kCombineFewParts on whose weight is 0 (an infinite value at a key of no weight is then
 // not multiplied by 0), so the bits are the same.
-//   few   at most kCombineFewParts: no loop behind the first loads, so that the kernel keeps 42 registers and a step of
+//   few   at most kCombineFewParts: no loop behind the first loads, so that the kernel keeps 38 registers and a step of
 //         1400 blocks is one wave (196 tokens of the 7B shape: 64 registers and 1.2 waves before)
-//   many  a loop over the rest, eight parts at a time
+//   many  a loop over the rest, eight parts at a time; bounded to the 64 registers of eight blocks an SM
 //   wide  few rows in many parts: a row's D / 32 warps take 32 channels each, a lane one float of each part, so that up to
 //         16 parts are on their way at once, on four times as many SMs
 constexpr int kCombineFew = 0, kCombineMany = 1, kCombineWide = 2;
 constexpr int kCombineFewParts = 4;
 
 template <typename T, int D, bool PAGED, typename LensT, int FORM>
-__global__ void __launch_bounds__(128, FORM == kCombineFew ? 12 : 1)
+__global__ void __launch_bounds__(128, FORM == kCombineFew ? 12 : FORM == kCombineMany ? 8 : 1)
 combine_kernel(const CombineArgs a, const __grid_constant__ LensT lens)
 {
     constexpr bool WIDE = FORM == kCombineWide;

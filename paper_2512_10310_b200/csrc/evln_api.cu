@@ -859,9 +859,22 @@ void fill_lens(BatchLens* bl, const evlnPagedParams* p, const int* lens, const i
     }
 }
 
-// Up to 2048 rows a block per row (of 128 channels) fills the SMs no more than a few times over.  (8 tokens over 20656
-// keys, 224 rows in 28 parts: 18.0 us a step with a warp per row, 17.6 so; 16 paged episodes of one token 53.6 and 52.5.)
-constexpr long kCombineWideRows = 2048;
+// Few rows in many parts: a block per row (of 128 channels; five of them fit an SM) instead of a warp, where all those blocks run at once, or,
+// from nine parts on, in two rounds; elsewhere the warps are faster.  (us of a step of three calls, warps and blocks: 16 parts of 840 rows
+// 20.6 and 18.4, 27 of 280 15.8 and 15.3, 7 of 560 11.7 and 11.3, 9 of 1280 42.0 and 41.0, a paged one of 1372 19.2 and 18.4; but 5 of 1904 12.7
+// and 14.3, 7 of 1120 13.5 and 14.4, 7 of a paged 700 12.4 and 13.3, 9 of 1960 19.1 and 19.7.)  Steps in fp32, whose attention blocks leave more
+// room beside them, a little further: 7 of 632 12.1 and 11.2, 5 of 884 12.2 and 11.5, 13 of 1240 22.6 and 20.0.
+inline bool combine_wide(int parts, long blocks, bool f32, int sms)
+{
+    return parts > kCombineFewParts && blocks <= (parts > 8 ? 10L : f32 ? 7L : 4L) * sms;
+}
+// At most four parts: the form without a loop, where the other one's blocks (eight an SM) would not run at once, or are so few that its longer
+// start shows; not between, where more blocks beside the attention's last CTAs crowd the SMs that ended first.  (1372 blocks 21.1 us a step with
+// the loop and 20.8, 476 13.3 and 13.0, 256 13.6 and 13.2; but 640 12.3 and 12.8, 800 17.9 and 18.4, 1024 16.6 and 17.1.)
+inline bool combine_few(int parts, long blocks, int sms)
+{
+    return parts <= kCombineFewParts && (blocks <= 4L * sms || blocks > 8L * sms);
+}
 template <typename T>
 evlnStatus_t launch_combine(evlnHandle_t h, const CombineArgs& args, int D, bool paged, const BatchLens* bl,
                             cudaStream_t st, const SimtTiles* shares = nullptr)
@@ -870,7 +883,7 @@ evlnStatus_t launch_combine(evlnHandle_t h, const CombineArgs& args, int D, bool
     a.div_g = make_fast_div((uint32_t)a.G);
     a.div_chunk = make_fast_div((uint32_t)(a.chunk_tiles > 0 ? a.chunk_tiles : 1));
     if (paged && D != 128) return EVLN_NOT_SUPPORTED;
-    const bool wide = a.num_splits > kCombineFewParts && (long)a.rows * a.Hkv <= kCombineWideRows;
+    const bool wide = combine_wide(a.num_splits, (long)ceil_div(a.rows, 128 / D) * a.Hkv, sizeof(T) == 4, h->num_sms);
     const dim3 grid(ceil_div(a.rows, wide ? 128 / D : 4), a.Hkv);
     auto launch = [&](auto form) {
         constexpr int FORM = decltype(form)::value;
@@ -885,7 +898,7 @@ evlnStatus_t launch_combine(evlnHandle_t h, const CombineArgs& args, int D, bool
             else launch_pdl(combine_kernel<T, 64, false, NoLens, FORM>, grid, dim3(128), 0, st, a, nl);
         }
     };
-    if (a.num_splits <= kCombineFewParts) launch(std::integral_constant<int, kCombineFew>());
+    if (combine_few(a.num_splits, (long)grid.x * grid.y, h->num_sms)) launch(std::integral_constant<int, kCombineFew>());
     else if (wide) launch(std::integral_constant<int, kCombineWide>());
     else launch(std::integral_constant<int, kCombineMany>());
     cudaError_t e = cudaGetLastError();

@@ -21,8 +21,14 @@ def handle():
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("hq,hkv,d,n,splits", [
     (28, 4, 128, 73, 4),           # the most parts of the first form
-    (28, 4, 128, 73, 5),           # one more, 2044 rows: a block per row
-    (28, 4, 128, 74, 9),           # 2072 rows: not
+    (28, 4, 128, 73, 5),           # one more
+    (28, 4, 128, 74, 9),
+    (28, 4, 128, 86, 4),           # 4 parts of 602 blocks: the form with the loop
+    (28, 4, 128, 170, 3),          # ... of 1190 blocks: without it again
+    (28, 4, 128, 21, 5),           # 588 rows: a block per row; in fp32 up to 1000, from 9 parts on up to 1280 rows
+    (28, 4, 128, 22, 8),
+    (28, 4, 128, 45, 9),           # 1260 rows
+    (28, 4, 128, 46, 9),           # 1288 rows
     (28, 4, 128, 8, 16),           # all parts on their way at once
     (28, 4, 128, 8, 17),           # ... and one more
     (3, 1, 128, 1, 32),            # one token, the most parts
@@ -58,7 +64,7 @@ def test_merge_against_fp64(handle, dtype, hq, hkv, d, n, splits):
 
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("hq,hkv,d,n,splits", [
-    (28, 4, 128, 73, 12),          # 2044 rows: a block per row
+    (28, 4, 128, 45, 12),          # 1260 rows: a block per row
     (28, 4, 128, 74, 12),          # 2072 rows: a warp per row
     (14, 2, 64, 9, 17),
 ])
