@@ -4,8 +4,9 @@
 // floats is nine products of bf16 numbers, which the tensor core forms exactly and adds in fp32.  Six of them are
 // taken (the other three are below 2^-26 of the product), the small ones first, so that the accumulator's own
 // rounding (towards zero, at its size of the moment) sees the large ones only.  An accumulator never runs on
-// across key tiles: every tile's scores and every tile's products with V start from zero, and the tiles' results
-// are added in registers, rounded to nearest.
+// across key tiles: every tile's products with V start from zero, and so do its scores, in two sums over half of the channels each; the
+// results are added in registers, rounded to nearest.  (What the tensor core cuts off makes a score about 7e-8 too small in one sum of 128
+// channels, half of that in two; a chain of float FMAs is off by twice as much, either way.)
 //
 // Bound: the tensor pipe (6 x 4 D bf16 flop per visible pair), with all SMs at work the latency of K and V out of L2.  A block of 16 + 1 warps owns 128 packed query rows of
 // one kv head and walks its key tiles, 64 keys at a time:
@@ -16,7 +17,8 @@
 //            probabilities' three parts in tensor memory.
 //   1 warp   issues: S_j = Q K_j^T (A = Q's parts in tensor memory) and O_j = P_j V_j (A = P_j's parts), in the order
 //            S_0, S_1, O_0, S_2, O_1, ..: the scores of a tile run while the softmax of the one before does.
-// Tensor memory columns: Q's parts 0 .. 3 D/2, O_j (D), S_j (64), P_j's parts (96).
+// Tensor memory columns: Q's parts 0 .. 3 D/2, O_j (D), S_j (two sums of 64: even and odd 16 channels), P_j's first two parts (64); all 512 at
+// head_dim 128, where P_j's third part is in shared memory.
 //
 // SHARE: as in attn_simt.cuh, one block per SM with an equal share of all (row block, key tile) pairs.
 //
@@ -38,13 +40,16 @@ template <int D> struct F32Plan {
     static constexpr int kPart = kBlk * (D / 64);            // one part of a K or V tile
     static constexpr int kTile = 3 * kPart;
     static constexpr int kKOff = 0, kVOff = 2 * kTile;       // two tiles each
-    static constexpr int kBarOff = kVOff + 2 * kTile;        // barriers, TMEM address, flags
+    static constexpr int kPLoOff = kVOff + 2 * kTile;        // the probabilities' third part, 128 rows x 64 keys, 128-byte swizzle
+    static constexpr int kBarOff = kPLoOff + (D == 128 ? kTileM * 128 : 0);   // barriers, TMEM address, flags
     static constexpr int kMaxOff = kBarOff + 128;            // float [2][4][128]: row maxima, tiles in turn
     static constexpr int kSumOff = kMaxOff + 2 * 4 * 128 * 4;    // float [4][128]: row sums
     static constexpr int kBytes = kSumOff + 4 * 128 * 4 + 1024;
-    static constexpr uint32_t kColO = 3 * D / 2, kColS = kColO + D, kColP = kColS + kF32Keys;
+    static constexpr uint32_t kColO = 3 * D / 2, kColS = kColO + D, kColP = kColS + 2 * kF32Keys;
     static constexpr int kOutStride = D + 16;                // bytes per row of a warp's D / 4 channels when they are written out
-    static_assert(kColP + 3 * kF32Keys / 2 <= 512, "tensor memory");
+    static constexpr bool kPLoTmem = kColP + 3 * kF32Keys / 2 <= 512;          // P_j's third part beside the others (one in shared memory: 1.5 % of a step more)
+    static_assert(kPLoTmem == (D == 64), "room for the third part");
+    static_assert(kColP + kF32Keys <= 512, "tensor memory");
     static_assert(kBytes <= 227 * 1024, "shared memory per CTA");
     static_assert(16 * 32 * kOutStride <= 2 * kTile, "the rows are written out through the K tiles");
 };
@@ -64,14 +69,44 @@ __device__ __forceinline__ void split3(uint64_t x, uint32_t& hi, uint32_t& mid, 
     lo = ptx::pack_bf16x2(x0, x1);
 }
 
-// Log-sum-exp of a row: unscaled maximum and sum of exponentials.  The scale's rest and what ex2.approx falls short of
-// (5e-8 on average, measured) are below half a unit of the sum of the two parts, so they join its rounding error.
-__device__ __forceinline__ float f32_lse(const SimtAttnArgs& a, float m, float sum)
+// A row's weights are kept 2^64 times as large: the third part of one down to 2^-149 is then no smaller than bf16 holds.
+constexpr float kWeightUnit = 18446744073709551616.f, kPerWeightUnit = 1.f / kWeightUnit;
+constexpr float kLeastWeight = -191.f;                       // exponent from which on a weight is 0
+
+// Weights of two score differences d <= 0: 2^(64 + d * scale2).  The exponent's integer n is split off before the scale's rest joins, so that
+// ex2 sees a fraction in [-0.5, 0.5] with the accuracy of the difference and not that of n.  The largest score's weight is exact.  Undefined
+// differences stay undefined.  (Nothing here or in the scale is fitted to inputs.  Against fp64, geometric means over 62 shapes of 64 to 2048
+// keys: outputs 2.2e-7 off, 3.2e-7 with float FMAs and expf; log-sum-exps 2.8e-8 both.)
+__device__ __forceinline__ uint64_t f32_weights(const SimtAttnArgs& a, uint64_t d2)
 {
+    const uint64_t hi = ptx::pack2(a.scale2_hi, a.scale2_hi), magic = ptx::pack2(12582912.f, 12582912.f);
+    float d0, d1, t0, t1, f0, f1;
+    ptx::unpack2(d2, d0, d1);
+    d2 = ptx::pack2(ptx::max_nan(d0, a.diff_min), ptx::max_nan(d1, a.diff_min));
+    const uint64_t t = ptx::fma2(d2, hi, magic);             // n in its low bits
+    const uint64_t minus_n = ptx::fma2(t, ptx::pack2(-1.f, -1.f), magic);
+    ptx::unpack2(ptx::fma2(d2, ptx::pack2(a.scale2_lo, a.scale2_lo), ptx::fma2(d2, hi, minus_n)), f0, f1);
+    ptx::unpack2(t, t0, t1);
+    constexpr uint32_t kBias = (127u + 64u) << 23;           // 2^(64 + n); the field is 0, and so is the weight, from n = kLeastWeight on
+    return ptx::mul2(ptx::pack2(ptx::ex2(f0), ptx::ex2(f1)),
+                     ptx::pack2(__uint_as_float((__float_as_uint(t0) << 23) + kBias), __uint_as_float((__float_as_uint(t1) << 23) + kBias)));
+}
+// ... what a running sum is multiplied by when its maximum moves up by -d
+__device__ __forceinline__ float f32_rescale(const SimtAttnArgs& a, float d)
+{
+    float w0, w1;
+    ptx::unpack2(f32_weights(a, ptx::pack2(d, d)), w0, w1);
+    return w0 * kPerWeightUnit;
+}
+
+// Log-sum-exp of a row: unscaled maximum and sum of weights.  The sum of the two parts is rounded once.
+__device__ __forceinline__ float f32_lse(const SimtAttnArgs& a, float m, float weights)
+{
+    const float sum = weights * kPerWeightUnit;
     if (!(sum > 0.f)) return -INFINITY;
-    const float top = m * a.scale, rest = fmaf(m, a.scale, -top) + m * a.scale_lo, lg = logf(sum);
+    const float top = m * a.scale, rest = fmaf(m, a.scale_lo, fmaf(m, a.scale, -top)), lg = logf(sum);
     const float s = top + lg, b = s - top;
-    return s + (((top - (s - b)) + (lg - b)) + (rest + 5e-8f));
+    return s + (((top - (s - b)) + (lg - b)) + rest);
 }
 
 template <int D, typename TilesT>
@@ -173,6 +208,7 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
         const uint32_t idesc_s = make_idesc(false, BM, BN), idesc_o = make_idesc(true, BM, D);
         const uint64_t kdesc0 = make_sdesc(smem_base + Plan::kKOff, 16, 1024);
         const uint64_t vdesc0 = make_sdesc(smem_base + Plan::kVOff, Plan::kBlk, 1024);
+        const uint64_t pdesc = make_sdesc(smem_base + Plan::kPLoOff, 16, 1024);
         do {
             const int keys = keys_of(), ntiles = keys > 0 ? (keys + BN - 1) / BN : 0;
             for (int j = 0; j <= ntiles && ntiles > 0; ++j) {
@@ -186,8 +222,8 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                         for (int x = 0; x < 6; ++x)
 #pragma unroll
                             for (int ks = 0; ks < D / 16; ++ks)
-                                ptx::mma_ts(tmem + Plan::kColS, tmem + kPa[x] * (D / 2) + ks * 8,
-                                            kd + (uint64_t)((kPb[x] * Plan::kPart + (ks >> 2) * Plan::kBlk + (ks & 3) * 32) >> 4), idesc_s, x > 0 || ks > 0);
+                                ptx::mma_ts(tmem + Plan::kColS + (ks & 1) * BN, tmem + kPa[x] * (D / 2) + ks * 8,
+                                            kd + (uint64_t)((kPb[x] * Plan::kPart + (ks >> 2) * Plan::kBlk + (ks & 3) * 32) >> 4), idesc_s, x > 0 || ks > 1);
                         ptx::mma_commit(bar_s_done);
                     }
                     __syncwarp();
@@ -201,9 +237,11 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
 #pragma unroll
                         for (int x = 0; x < 6; ++x)
 #pragma unroll
-                            for (int ks = 0; ks < BN / 16; ++ks)
-                                ptx::mma_ts(tmem + Plan::kColO, tmem + Plan::kColP + kPa[x] * (BN / 2) + ks * 8,
-                                            vd + (uint64_t)((kPb[x] * Plan::kPart + ks * 2048) >> 4), idesc_o, x > 0 || ks > 0);
+                            for (int ks = 0; ks < BN / 16; ++ks) {
+                                const uint64_t v = vd + (uint64_t)((kPb[x] * Plan::kPart + ks * 2048) >> 4);
+                                if (!Plan::kPLoTmem && kPa[x] == 2) ptx::mma_ss(tmem + Plan::kColO, pdesc + (uint64_t)(ks * 2), v, idesc_o, x > 0 || ks > 0);
+                                else ptx::mma_ts(tmem + Plan::kColO, tmem + Plan::kColP + kPa[x] * (BN / 2) + ks * 8, v, idesc_o, x > 0 || ks > 0);
+                            }
                         ptx::mma_commit(bar_o_done);
                     }
                     __syncwarp();
@@ -296,7 +334,13 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                 ptx::fence_after_sync();
                 uint32_t s[16];
                 ptx::tmem_ld16(t_lane + Plan::kColS + part * 16, s);
-                ptx::tmem_ld_wait();
+                {
+                    uint32_t odd[16];
+                    ptx::tmem_ld16(t_lane + Plan::kColS + BN + part * 16, odd);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) s[e] = __float_as_uint(__uint_as_float(s[e]) + __uint_as_float(odd[e]));
+                }
                 ptx::fence_before_sync();
                 if (j + 1 < ntiles) {
                     ptx::fence_proxy_async();
@@ -321,16 +365,13 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                 // (the maximum stays unscaled: a difference of scores is as exact as the scores, and 0 for the largest)
                 const float m_new = fmaxf(ptx::max3(m, xm[0], xm[128]), fmaxf(xm[256], xm[384]));
                 const float ref = (m_new == -INFINITY) ? 0.f : m_new;      // a row that has seen no key yet: every p is 0
-                const float alpha = ptx::ex2(fmaf(m - ref, a.scale2_hi, (m - ref) * a.scale2_lo));     // m = -inf: 0
+                const float alpha = f32_rescale(a, m - ref);                // m = -inf: 0
                 m = m_new;
-                const uint64_t minus_ref = ptx::pack2(-ref, -ref), hi2 = ptx::pack2(a.scale2_hi, a.scale2_hi), lo2 = ptx::pack2(a.scale2_lo, a.scale2_lo);
+                const uint64_t minus_ref = ptx::pack2(-ref, -ref);
                 uint64_t sum2 = 0ull, pp[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
-                    const uint64_t d2 = ptx::add2(ptx::pack2(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), minus_ref);
-                    float y0, y1;
-                    ptx::unpack2(ptx::fma2(d2, hi2, ptx::mul2(d2, lo2)), y0, y1);
-                    pp[e] = ptx::pack2(ptx::ex2(y0), ptx::ex2(y1));
+                    pp[e] = f32_weights(a, ptx::add2(ptx::pack2(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), minus_ref));
                     sum2 = ptx::add2(sum2, pp[e]);
                 }
                 {
@@ -358,7 +399,11 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
 #pragma unroll
                     for (int e = 0; e < 8; ++e) split3(pp[e], p[0][e], p[1][e], p[2][e]);
 #pragma unroll
-                    for (int y = 0; y < 3; ++y) ptx::tmem_st8(t_lane + Plan::kColP + y * (BN / 2) + part * 8, p[y]);
+                    for (int y = 0; y < (Plan::kPLoTmem ? 3 : 2); ++y) ptx::tmem_st8(t_lane + Plan::kColP + y * (BN / 2) + part * 8, p[y]);
+#pragma unroll
+                    for (int h = 0; h < (Plan::kPLoTmem ? 0 : 2); ++h)
+                        *reinterpret_cast<uint4*>(smem + Plan::kPLoOff + r_tile * 128 + (((2 * part + h) ^ (r_tile & 7)) << 4)) =
+                            make_uint4(p[2][4 * h], p[2][4 * h + 1], p[2][4 * h + 2], p[2][4 * h + 3]);
                 }
                 ptx::tmem_st_wait();
                 ptx::fence_before_sync();
@@ -388,7 +433,7 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                     ptx::unpack2(acc[c], y0, y1);
                     y0 = fabsf(y0);
                     y1 = fabsf(y1);
-                    bad |= !(y0 + y1 <= 3.0e38f) || (y0 < 1e-30f && y0 > 0.f) || (y1 < 1e-30f && y1 > 0.f);
+                    bad |= !(y0 + y1 <= 3.0e38f) || (y0 < 1e-30f * kWeightUnit && y0 > 0.f) || (y1 < 1e-30f * kWeightUnit && y1 > 0.f);
                 }
                 bad = bad && row_valid;
             }

@@ -50,6 +50,13 @@ template <int D> struct SmallPlan {
     static_assert(kSmallAngleTokens * kAngles * 16 <= 6 * kPart, "the angles fit the tiles");
 };
 
+// f32_rescale in fewer steps, one behind the other in a chain of a tile or two: the error of a larger exponent goes with a smaller factor.
+__device__ __forceinline__ float small_rescale(const SimtAttnArgs& a, float d)
+{
+    d = fmaxf(d, a.diff_min);
+    return ptx::ex2(fmaf(d, a.scale2_hi, d * a.scale2_lo));
+}
+
 template <int D, bool FUSED>
 __global__ void __launch_bounds__(kSmallThreads, 1)
 attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_constant__ F32Fused f)
@@ -240,11 +247,11 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
         }
         const int key0 = j * 64 + kg * 16;
         if (rt * 16 >= rows || key0 >= keys) continue;
-        float big[2][2][4], small[2][4];                     // [parity of the 16 channels][8 keys]
+        float big[2][4], small[2][4];                        // [8 keys]
 #pragma unroll
         for (int t = 0; t < 2; ++t)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) big[0][t][e] = big[1][t][e] = small[t][e] = 0.f;
+            for (int e = 0; e < 4; ++e) big[t][e] = small[t][e] = 0.f;
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {
             uint32_t q[3][4], k[3][4];
@@ -260,7 +267,10 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
                 ptx::mma_bf16(small[t], q[1], k[1][2 * t], k[1][2 * t + 1]);
                 ptx::mma_bf16(small[t], q[1], k[0][2 * t], k[0][2 * t + 1]);
                 ptx::mma_bf16(small[t], q[0], k[1][2 * t], k[1][2 * t + 1]);
-                ptx::mma_bf16(big[ks & 1][t], q[0], k[0][2 * t], k[0][2 * t + 1]);
+                float u[4] = {0.f, 0.f, 0.f, 0.f};
+                ptx::mma_bf16(u, q[0], k[0][2 * t], k[0][2 * t + 1]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) big[t][e] += u[e];
             }
         }
         float x[2][4];
@@ -268,7 +278,7 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
         for (int t = 0; t < 2; ++t)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                x[t][e] = (big[0][t][e] + big[1][t][e]) + small[t][e];
+                x[t][e] = big[t][e] + small[t][e];
                 if (key0 + t * 8 + (lane & 3) * 2 + (e & 1) > bound[e >> 1]) x[t][e] = -INFINITY;
             }
         uint32_t p[3][4];
@@ -278,15 +288,16 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
             const float m_new = fmaxf(m[h], mx), ref = (m_new == -INFINITY) ? 0.f : m_new;
-            const float alpha = ptx::ex2(fmaf(m[h] - ref, a.scale2_hi, (m[h] - ref) * a.scale2_lo));
+            const float alpha = small_rescale(a, m[h] - ref);
             m[h] = m_new;
             float sum = 0.f;
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
-                const float d0 = x[t][2 * h] - ref, d1 = x[t][2 * h + 1] - ref;
-                const float p0 = ptx::ex2(fmaf(d0, a.scale2_hi, d0 * a.scale2_lo)), p1 = ptx::ex2(fmaf(d1, a.scale2_hi, d1 * a.scale2_lo));
-                sum += p0 + p1;
-                split3(ptx::pack2(p0, p1), p[0][2 * t + h], p[1][2 * t + h], p[2][2 * t + h]);
+                const uint64_t w = f32_weights(a, ptx::pack2(x[t][2 * h] - ref, x[t][2 * h + 1] - ref));
+                float w0, w1;
+                ptx::unpack2(w, w0, w1);
+                sum += w0 + w1;
+                split3(w, p[0][2 * t + h], p[1][2 * t + h], p[2][2 * t + h]);
             }
             l[h] = fmaf(l[h], alpha, sum);
 #pragma unroll
@@ -354,7 +365,7 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
         for (int v = 0; v < kV; ++v) y[v] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            w[i] = ptx::ex2(fmaf(w[i] - ref, a.scale2_hi, (w[i] - ref) * a.scale2_lo));
+            w[i] = small_rescale(a, w[i] - ref);
             sum = fmaf(w[i], s_stat[128 + (w0 + 2 * i) * 16 + rr], sum);
             const float4* at = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(smem) + ((w0 + 2 * i) * 16 + rr) * Plan::kStride);
 #pragma unroll
@@ -368,7 +379,7 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
         }
         // (not ordinary numbers: see attn_f32.cuh)
         bool odd = false;
-        auto ordinary = [](float x) { return fabsf(x) <= 3.0e38f && (x == 0.f || fabsf(x) >= 1e-30f); };
+        auto ordinary = [](float x) { return fabsf(x) <= 3.0e38f && (x == 0.f || fabsf(x) >= 1e-30f * kWeightUnit); };
 #pragma unroll
         for (int v = 0; v < kV; ++v) odd |= !(ordinary(y[v].x) && ordinary(y[v].y) && ordinary(y[v].z) && ordinary(y[v].w));
         uint32_t bad = __ballot_sync(0xffffffffu, odd && r < rows);

@@ -39,7 +39,8 @@ struct SimtAttnArgs {
     float scale;
     // attn_f32.cuh only:
     float scale_lo;                 // rest of the scale
-    float scale2_hi, scale2_lo;     // scale * log2(e) rounded towards zero, and its rest (> 0)
+    float scale2_hi, scale2_lo;     // scale * log2(e) in two parts
+    float diff_min;                 // difference of scores whose weight is 0
     int* status;                    // device status word
 };
 

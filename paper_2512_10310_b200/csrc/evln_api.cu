@@ -538,24 +538,22 @@ void launch_simt(const SimtSchedule& plan, const evlnStepParams* p, dim3 grid, c
     }
 }
 
-// The scale of the fp32 kernel in two floats each, with what its scores fall short of: the tensor core cuts the sums
-// behind every 16 channels off instead of rounding them (measured with normal numbers: 7.1e-8 of a score at 128 channels, half
-// of that at 64).
-void set_f32_scale(const evlnStepParams* p, SimtAttnArgs* a, bool small)
+// The scale of the fp32 kernels in two floats each.
+void set_f32_scale(const evlnStepParams* p, SimtAttnArgs* a)
 {
-    const double scale = (p->softmax_scale > 0.f ? (double)p->softmax_scale : 1.0 / sqrt((double)p->head_dim)) * (1.0 + (small ? 2.75e-10 : 5.5e-10) * p->head_dim);
+    const double scale = p->softmax_scale > 0.f ? (double)p->softmax_scale : 1.0 / sqrt((double)p->head_dim);
     const double scale2 = scale * 1.4426950408889634;
     a->scale = (float)scale;
     a->scale_lo = (float)(scale - (double)a->scale);
     a->scale2_hi = (float)scale2;
-    if ((double)a->scale2_hi >= scale2) a->scale2_hi = nextafterf(a->scale2_hi, 0.f);
     a->scale2_lo = (float)(scale2 - (double)a->scale2_hi);
+    a->diff_min = kLeastWeight / a->scale2_hi;
 }
 
 template <int D>
 void launch_f32(const SimtSchedule& plan, const evlnStepParams* p, dim3 grid, cudaStream_t st, SimtAttnArgs a)
 {
-    set_f32_scale(p, &a, plan.rows_per_thread == 2);
+    set_f32_scale(p, &a);
     if (plan.rows_per_thread == 2) {
         launch_pdl(attn_f32_small_kernel<D, false>, dim3(grid.z, grid.x, grid.y), dim3(kSmallThreads), SmallPlan<D>::kBytes, st, a,
                    make_fast_div((uint32_t)a.G), F32Fused{});
@@ -573,7 +571,7 @@ void launch_f32(const SimtSchedule& plan, const evlnStepParams* p, dim3 grid, cu
 template <int D>
 cudaError_t launch_f32_step(const evlnStepParams* p, int splits, cudaStream_t st, SimtAttnArgs a, const F32Fused& f)
 {
-    set_f32_scale(p, &a, true);
+    set_f32_scale(p, &a);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(splits, ceil_div(a.num_new * a.G, kSmallRows), a.Hkv);
     cfg.blockDim = dim3(kSmallThreads);

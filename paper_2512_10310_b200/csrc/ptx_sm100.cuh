@@ -261,12 +261,6 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr)
     asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(cluster_addr) : "memory");
     return x;
 }
-__device__ __forceinline__ float2 ld_cluster_f32x2(uint32_t cluster_addr)
-{
-    float2 x;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(x.x), "=f"(x.y) : "r"(cluster_addr) : "memory");
-    return x;
-}
 __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t cluster_addr)
 {
     float4 x;
@@ -369,6 +363,13 @@ __device__ __forceinline__ float ex2(float x)
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+// undefined if either is
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
 }
 __device__ __forceinline__ float max3(float a, float b, float c)
 {

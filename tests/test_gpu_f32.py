@@ -127,3 +127,50 @@ def test_infinite_values_of_keys_without_weight(handle, hq, hkv, d, L, n, splits
             got.append(_step(handle, cfg, y, num_splits=splits, fused=fused)[1]["out"])
     assert torch.equal(got[0], got[1]) and torch.equal(got[2], got[3])
     assert bool(torch.isfinite(got[2]).all()) and torch.equal(got[0], got[2])
+
+
+@pytest.mark.parametrize("hq,hkv,d,n", [
+    (64, 64, 64, 1),               # 32-row blocks
+    (64, 64, 128, 1),
+    (28, 4, 64, 400),              # 128-row blocks
+    (28, 4, 128, 400),
+])
+@pytest.mark.parametrize("fused", [False, True])
+def test_log_sum_exp_of_one_key(handle, hq, hkv, d, n, fused):
+    # The first token on an empty cache is not turned and sees itself only.  Scores of short numbers are exact, so what is left is
+    # one rounding of the scale's product and one of its rest: half a unit of the last place each.
+    cfg, x = _inputs(hq, hkv, d, 0, n)
+    for key in ("q_new", "k_new"):
+        x[key] = torch.round(x[key] * 4.0) / 4.0
+    x["q_new"][0, :, 5:] = 0.0                 # few channels: scores of every size from 1/16 on
+    _, g = _step(handle, cfg, x, fused=fused)
+    k = f64(x["k_new"][0]).repeat(hq // hkv, axis=0)
+    want = (f64(x["q_new"][0]) * k).sum(-1) / np.sqrt(d)
+    assert bool((np.abs(f64(g["lse"][0]) - want) <= 2.0 ** -23 * np.abs(want)).all())
+    assert np.array_equal(f64(g["out"][0]), f64(x["v_new"][0]).repeat(hq // hkv, axis=0))
+
+
+@pytest.mark.parametrize("hq,hkv,d,L,n", [
+    (2, 1, 64, 256, 64),
+    (8, 4, 128, 362, 79),
+    (4, 2, 64, 858, 40),
+    (28, 4, 64, 1024, 196),
+    (28, 4, 128, 1024, 196),
+    (16, 4, 128, 2031, 252),
+])
+@pytest.mark.parametrize("kind", ["normal", "positive", "short"])
+def test_no_further_off_than_float_fmas(handle, hq, hkv, d, L, n, kind):
+    # tensor-core and SIMT kernels on the same inputs, both against the oracle.  An error of thousands of outputs is steady
+    # within some per cent from one seed to the next; a quarter is allowed.
+    cfg, x = _inputs(hq, hkv, d, L, n)
+    for key in ("q_new", "k_new", "k_cache", "v_new", "v_cache"):
+        if kind == "positive" and key[0] != "v":
+            x[key] = x[key].abs()
+        if kind == "short":
+            x[key] = torch.round(x[key] * 4.0) / 4.0
+    r = oracle_step("f32", x["k_cache"], x["v_cache"], x["q_new"], x["k_new"], x["v_new"], L, cfg.rope_theta)
+    off = []
+    for kernel in (B.EVLN_KERNEL_SIMT, B.EVLN_KERNEL_AUTO):
+        _, g = _step(handle, cfg, x, kernel=kernel)
+        off.append((np.linalg.norm(f64(g["out"]) - r["out"]), np.linalg.norm(f64(g["lse"]) - r["lse"])))
+    assert off[1][0] <= 1.25 * off[0][0] and off[1][1] <= 1.25 * off[0][1], off
