@@ -69,6 +69,13 @@ __device__ __forceinline__ void split3(uint64_t x, uint32_t& hi, uint32_t& mid, 
     lo = ptx::pack_bf16x2(x0, x1);
 }
 
+// The parts are exact down to 2^-109 and no further off than 2^-134 below.  What that leaves out of a score is nothing (2^-30) unless the
+// number's partner is huge, so row blocks that meet a query or key of 2^90 (divided by a softmax scale above 1) are done in floats.
+__device__ __forceinline__ bool f32_huge(const SimtAttnArgs& a, uint32_t top)        // top: max_abs_bf16x2 of first parts
+{
+    return (top & 0x7fffu) >= a.huge || ((top >> 16) & 0x7fffu) >= a.huge;
+}
+
 // A row's weights are kept 2^64 times as large: the third part of one down to 2^-149 is then no smaller than bf16 holds.
 constexpr float kWeightUnit = 18446744073709551616.f, kPerWeightUnit = 1.f / kWeightUnit;
 constexpr float kLeastWeight = -191.f;                       // exponent from which on a weight is 0
@@ -91,12 +98,11 @@ __device__ __forceinline__ uint64_t f32_weights(const SimtAttnArgs& a, uint64_t 
     return ptx::mul2(ptx::pack2(ptx::ex2(f0), ptx::ex2(f1)),
                      ptx::pack2(__uint_as_float((__float_as_uint(t0) << 23) + kBias), __uint_as_float((__float_as_uint(t1) << 23) + kBias)));
 }
-// ... what a running sum is multiplied by when its maximum moves up by -d
+// ... what a running sum is multiplied by when its maximum moves up by -d (in fewer steps: the error of a larger exponent goes with a smaller factor)
 __device__ __forceinline__ float f32_rescale(const SimtAttnArgs& a, float d)
 {
-    float w0, w1;
-    ptx::unpack2(f32_weights(a, ptx::pack2(d, d)), w0, w1);
-    return w0 * kPerWeightUnit;
+    d = fmaxf(d, a.diff_min);
+    return ptx::ex2(fmaf(d, a.scale2_hi, d * a.scale2_lo));
 }
 
 // Log-sum-exp of a row: unscaled maximum and sum of weights.  The sum of the two parts is rounded once.
@@ -271,17 +277,20 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                 if (t_row + i * kRowStep < rows) x[i] = *reinterpret_cast<const ulonglong2*>(from + tid * 4 + i * (kF32Compute * 4));
             }
         };
-        auto store_tile = [&](const ulonglong2 (&x)[kVecs], uint8_t* to) {
+        int turn = 0;
+        auto store_tile = [&](const ulonglong2 (&x)[kVecs], uint8_t* to, bool is_k) {
+            uint32_t top = 0;
 #pragma unroll
             for (int i = 0; i < kVecs; ++i) {
                 uint2 p[3];
                 split3(x[i].x, p[0].x, p[1].x, p[2].x);
                 split3(x[i].y, p[0].y, p[1].y, p[2].y);
+                if (is_k) top = ptx::max_abs_bf16x2(ptx::max_abs_bf16x2(top, p[0].x), p[0].y);
 #pragma unroll
                 for (int y = 0; y < 3; ++y) *reinterpret_cast<uint2*>(to + t_place + i * (kRowStep * 128) + y * Plan::kPart) = p[y];
             }
+            if (is_k && f32_huge(a, top)) atomicOr(&s_bad[turn & 1], 1);
         };
-        int turn = 0;
         do {
             const int row0 = rb * BM, t_lo = j_lo * BN, keys = keys_of(), ntiles = keys > 0 ? (keys + BN - 1) / BN : 0;
             const int row = row0 + r_tile;
@@ -306,6 +315,7 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                     q[c] = make_ulonglong2(0ull, 0ull);
                     if (row_valid) q[c] = reinterpret_cast<const ulonglong2*>(qrow)[c];
                 }
+                uint32_t top = 0;
                 __syncwarp();
 #pragma unroll
                 for (int h = 0; h < kCh / 16; ++h) {
@@ -314,11 +324,13 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                     for (int c = 0; c < 4; ++c) {
                         split3(q[4 * h + c].x, p[0][2 * c], p[1][2 * c], p[2][2 * c]);
                         split3(q[4 * h + c].y, p[0][2 * c + 1], p[1][2 * c + 1], p[2][2 * c + 1]);
+                        top = ptx::max_abs_bf16x2(ptx::max_abs_bf16x2(top, p[0][2 * c]), p[0][2 * c + 1]);
                     }
 #pragma unroll
                     for (int y = 0; y < 3; ++y) ptx::tmem_st8(t_lane + y * (D / 2) + part * (kCh / 2) + h * 8, p[y]);
                 }
-                store_tile(x, smem + Plan::kKOff + (base & 1) * Plan::kTile);
+                if (f32_huge(a, top)) atomicOr(&s_bad[turn & 1], 1);
+                store_tile(x, smem + Plan::kKOff + (base & 1) * Plan::kTile, true);
                 ptx::tmem_st_wait();
                 ptx::fence_before_sync();
                 ptx::fence_proxy_async();
@@ -328,7 +340,7 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
             for (int j = 0; j < ntiles; ++j) {
                 const int gj = base + j;
                 // (tile j - 1 of the scores is done, and with it that K buffer)
-                if (j + 1 < ntiles) store_tile(x, smem + Plan::kKOff + ((gj + 1) & 1) * Plan::kTile);
+                if (j + 1 < ntiles) store_tile(x, smem + Plan::kKOff + ((gj + 1) & 1) * Plan::kTile, true);
                 load_tile(x, vb + (long)j * BN * D, keys - j * BN);
                 warp_wait(bar_s_done, gj & 1, kDevTimeoutSoftmaxS, a.status, s_abort, lane);
                 ptx::fence_after_sync();
@@ -339,7 +351,12 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                     ptx::tmem_ld16(t_lane + Plan::kColS + BN + part * 16, odd);
                     ptx::tmem_ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) s[e] = __float_as_uint(__uint_as_float(s[e]) + __uint_as_float(odd[e]));
+                    for (int e = 0; e < 16; e += 2) {
+                        float lo, hi;
+                        ptx::unpack2(ptx::add2(ptx::pack2(__uint_as_float(s[e]), __uint_as_float(s[e + 1])), ptx::pack2(__uint_as_float(odd[e]), __uint_as_float(odd[e + 1]))), lo, hi);
+                        s[e] = __float_as_uint(lo);
+                        s[e + 1] = __float_as_uint(hi);
+                    }
                 }
                 ptx::fence_before_sync();
                 if (j + 1 < ntiles) {
@@ -379,7 +396,7 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                     ptx::unpack2(sum2, s0, s1);
                     l = l * alpha + (s0 + s1);
                 }
-                store_tile(x, smem + Plan::kVOff + (gj & 1) * Plan::kTile);        // (the product of tile j - 2 is done)
+                store_tile(x, smem + Plan::kVOff + (gj & 1) * Plan::kTile, false);        // (the product of tile j - 2 is done)
                 if (j + 2 < ntiles) load_tile(x, kb + (long)(j + 2) * BN * D, keys - (j + 2) * BN);
                 if (j > 0) {
                     warp_wait(bar_o_done, (gj - 1) & 1, kDevTimeoutSoftmaxO, a.status, s_abort, lane);
@@ -438,7 +455,7 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                 bad = bad && row_valid;
             }
             s_sum[part * 128 + r_tile] = l;
-            if (bad) s_bad[turn & 1] = 1;
+            if (bad) atomicOr(&s_bad[turn & 1], 1);
             all_compute();
             if (tid == 0) s_bad[(turn & 1) ^ 1] = 0;
             if (*(volatile int*)&s_bad[turn & 1] == 0) {

@@ -43,19 +43,13 @@ template <int D> struct SmallPlan {
     static constexpr int kStride = D + 4;                                  // floats per row of an output
     static constexpr int kStatOff = kQOff + 3 * kQPart;                    // float [2][8][16]: the warps' maxima and sums
     static constexpr int kLseOff = kStatOff + 2 * 8 * 16 * 4;              // float [32]
-    static constexpr int kBytes = kLseOff + kSmallRows * 4 + 1024;
+    static constexpr int kHugeOff = kLseOff + kSmallRows * 4;              // int
+    static constexpr int kBytes = kHugeOff + 16 + 1024;
     static constexpr int kAngles = D / 2 + D / 16;                         // places of a token's angles
     static_assert(8 * 16 * kStride * 4 <= 6 * kPart, "the warps' outputs fit the tiles");
     static_assert(kSmallRows * kStride * 4 <= 3 * kQPart, "the rows to merge fit the queries");
     static_assert(kSmallAngleTokens * kAngles * 16 <= 6 * kPart, "the angles fit the tiles");
 };
-
-// f32_rescale in fewer steps, one behind the other in a chain of a tile or two: the error of a larger exponent goes with a smaller factor.
-__device__ __forceinline__ float small_rescale(const SimtAttnArgs& a, float d)
-{
-    d = fmaxf(d, a.diff_min);
-    return ptx::ex2(fmaf(d, a.scale2_hi, d * a.scale2_lo));
-}
 
 template <int D, bool FUSED>
 __global__ void __launch_bounds__(kSmallThreads, 1)
@@ -99,12 +93,16 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
             if (r >= lo && r < hi) x[i] = *reinterpret_cast<const ulonglong2*>(from + tid * 4 + i * (NT * 4));
         }
     };
-    auto store_tile = [&](const ulonglong2 (&x)[kVecs], uint8_t* to) {
+    int* s_huge = reinterpret_cast<int*>(smem + Plan::kHugeOff);
+    if (tid == 0) *s_huge = 0;
+    uint32_t top = 0;                                        // largest query and key parts
+    auto store_tile = [&](const ulonglong2 (&x)[kVecs], uint8_t* to, bool is_k) {
 #pragma unroll
         for (int i = 0; i < kVecs; ++i) {
             uint2 p[3];
             split3(x[i].x, p[0].x, p[1].x, p[2].x);
             split3(x[i].y, p[0].y, p[1].y, p[2].y);
+            if (is_k) top = ptx::max_abs_bf16x2(ptx::max_abs_bf16x2(top, p[0].x), p[0].y);
 #pragma unroll
             for (int y = 0; y < 3; ++y) *reinterpret_cast<uint2*>(to + t_place + i * (kRowStep * 128) + y * Plan::kPart) = p[y];
         }
@@ -114,6 +112,7 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
         uint2 p[3];
         split3(x.x, p[0].x, p[1].x, p[2].x);
         split3(x.y, p[0].y, p[1].y, p[2].y);
+        top = ptx::max_abs_bf16x2(ptx::max_abs_bf16x2(top, p[0].x), p[0].y);
         uint8_t* at = smem + Plan::kQOff + (c >> 4) * Plan::kQBlk + r * 128 + ((((c & 15) >> 1) ^ (r & 7)) << 4) + (c & 1) * 8;
 #pragma unroll
         for (int y = 0; y < 3; ++y) *reinterpret_cast<uint2*>(at + y * Plan::kQPart) = p[y];
@@ -236,8 +235,8 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
 
     for (int j = 0; j < ntiles; ++j) {
         __syncthreads();                                     // everyone is done with tile j - 1 (and the angles)
-        store_tile(kx, smem + Plan::kKOff);
-        store_tile(vx, smem + Plan::kVOff);
+        store_tile(kx, smem + Plan::kKOff, true);
+        store_tile(vx, smem + Plan::kVOff, false);
         __syncthreads();
         if (j + 1 < ntiles) {
             zero_tile(kx);
@@ -288,7 +287,7 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
             const float m_new = fmaxf(m[h], mx), ref = (m_new == -INFINITY) ? 0.f : m_new;
-            const float alpha = small_rescale(a, m[h] - ref);
+            const float alpha = f32_rescale(a, m[h] - ref);
             m[h] = m_new;
             float sum = 0.f;
 #pragma unroll
@@ -328,6 +327,7 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
 
     // ---- the four warps of a row into shared memory, where the tiles were ----
     __syncthreads();
+    if (f32_huge(a, top)) *s_huge = 1;
     {
         float* s_o = reinterpret_cast<float*>(smem) + warp * 16 * Plan::kStride;
 #pragma unroll
@@ -365,7 +365,7 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
         for (int v = 0; v < kV; ++v) y[v] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            w[i] = small_rescale(a, w[i] - ref);
+            w[i] = f32_rescale(a, w[i] - ref);
             sum = fmaf(w[i], s_stat[128 + (w0 + 2 * i) * 16 + rr], sum);
             const float4* at = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(smem) + ((w0 + 2 * i) * 16 + rr) * Plan::kStride);
 #pragma unroll
@@ -378,7 +378,7 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
             }
         }
         // (not ordinary numbers: see attn_f32.cuh)
-        bool odd = false;
+        bool odd = *s_huge != 0;
         auto ordinary = [](float x) { return fabsf(x) <= 3.0e38f && (x == 0.f || fabsf(x) >= 1e-30f * kWeightUnit); };
 #pragma unroll
         for (int v = 0; v < kV; ++v) odd |= !(ordinary(y[v].x) && ordinary(y[v].y) && ordinary(y[v].z) && ordinary(y[v].w));

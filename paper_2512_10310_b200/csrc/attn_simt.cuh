@@ -41,6 +41,7 @@ struct SimtAttnArgs {
     float scale_lo;                 // rest of the scale
     float scale2_hi, scale2_lo;     // scale * log2(e) in two parts
     float diff_min;                 // difference of scores whose weight is 0
+    uint32_t huge;                  // magnitude (a bf16 number's bits) from which on a query or key is not split
     int* status;                    // device status word
 };
 

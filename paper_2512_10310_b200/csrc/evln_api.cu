@@ -223,10 +223,12 @@ evlnStatus_t check_step_params(evlnHandle_t h, const evlnStepParams* p)
     return EVLN_OK;
 }
 
-// fp32 on the tensor cores (attn_f32.cuh), unless the caller asks for the kernel without them.
+// fp32 on the tensor cores (attn_f32.cuh), unless the caller asks for the kernel without them, or for a softmax scale with which scores of
+// ordinary size come from queries and keys whose products leave the range of floats (2^-60 to 2^60 keep them far from it).
 inline bool use_f32_kernel(const evlnStepParams* p)
 {
-    return p->kernel == EVLN_KERNEL_AUTO && p->dtype == EVLN_F32;
+    const bool ordinary = p->softmax_scale == 0.f || (p->softmax_scale >= 0x1p-60f && p->softmax_scale <= 0x1p60f);
+    return p->kernel == EVLN_KERNEL_AUTO && p->dtype == EVLN_F32 && ordinary;
 }
 
 inline bool use_tensor_kernel(const evlnStepParams* p)
@@ -548,6 +550,10 @@ void set_f32_scale(const evlnStepParams* p, SimtAttnArgs* a)
     a->scale2_hi = (float)scale2;
     a->scale2_lo = (float)(scale2 - (double)a->scale2_hi);
     a->diff_min = kLeastWeight / a->scale2_hi;
+    const float huge = 0x1p90f / std::max(a->scale, 1.f);
+    uint32_t bits;
+    memcpy(&bits, &huge, sizeof(bits));
+    a->huge = bits >> 16;
 }
 
 template <int D>

@@ -80,6 +80,24 @@ def test_values_of_any_size(handle, hq, hkv, d, L, n, scale, fused):
 
 
 @pytest.mark.parametrize("hq,hkv,d,L,n", [(2, 1, 64, 256, 64), (4, 2, 128, 500, 70), (28, 4, 128, 1024, 196)])
+@pytest.mark.parametrize("q_size,k_size,softmax_scale", [
+    (1e-36, 1e36, 0.0),            # the queries' third parts are below bf16's least number, and the keys are as large
+    (1e36, 1e-36, 0.0),
+    (1e-30, 1e30, 0.0),            # all parts exact
+    (2.0 ** -56, 2.0 ** -56, 2.0 ** 110),      # products of parts below the least float
+    (1e-2, 1e-2, 1e3),
+])
+@pytest.mark.parametrize("fused", [False, True])
+def test_queries_and_keys_of_any_size(handle, hq, hkv, d, L, n, q_size, k_size, softmax_scale, fused):
+    cfg, x = _inputs(hq, hkv, d, L, n)
+    x["q_new"] = x["q_new"] * q_size
+    x["k_cache"], x["k_new"] = x["k_cache"] * k_size, x["k_new"] * k_size
+    r = oracle_step("f32", x["k_cache"], x["v_cache"], x["q_new"], x["k_new"], x["v_new"], L, cfg.rope_theta, scale=softmax_scale)
+    _, g = _step(handle, cfg, x, fused=fused, scale=softmax_scale)
+    check_output("f32", g["out"], g["lse"], r["out"], r["lse"])
+
+
+@pytest.mark.parametrize("hq,hkv,d,L,n", [(2, 1, 64, 256, 64), (4, 2, 128, 500, 70), (28, 4, 128, 1024, 196)])
 def test_scores_beyond_any_sum(handle, hq, hkv, d, L, n):
     # one key so long that it either takes a row over or drops out of it, by the sign of one channel of the query
     cfg, x = _inputs(hq, hkv, d, L, n)
