@@ -78,6 +78,15 @@ __device__ __forceinline__ bool f32_huge(const SimtAttnArgs& a, uint32_t top)   
 
 // A row's weights are kept 2^64 times as large: the third part of one down to 2^-149 is then no smaller than bf16 holds.
 constexpr float kWeightUnit = 18446744073709551616.f, kPerWeightUnit = 1.f / kWeightUnit;
+// A value's parts are 2^-134 off at most, and with weights of 2^64 each a row's sum over 2^24 keys 2^-46: bits of sums below 2^-18 may be
+// lost, if the row's values are of the kind whose third part is not exact.
+constexpr float kSmallSum = 3.814697265625e-6f;
+__device__ __forceinline__ bool f32_small(float sum) { return sum != 0.f && fabsf(sum) < kSmallSum; }
+__device__ __forceinline__ bool f32_inexact(const float4& v)                         // any of them not 0 and below 2^-109
+{
+    auto tiny = [](float x) { return __float_as_uint(x) * 2u - 1u < 2u * 0x09000000u - 1u; };
+    return tiny(v.x) || tiny(v.y) || tiny(v.z) || tiny(v.w);
+}
 constexpr float kLeastWeight = -191.f;                       // exponent from which on a weight is 0
 
 // Weights of two score differences d <= 0: 2^(64 + d * scale2).  The exponent's integer n is split off before the scale's rest joins, so that
@@ -134,7 +143,8 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
     const uint32_t bar_o_done = bar_s_done + 8;              // O_j there
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + Plan::kBarOff + 32);
     volatile int* s_abort = reinterpret_cast<volatile int*>(smem + Plan::kBarOff + 36);
-    int* s_bad = reinterpret_cast<int*>(smem + Plan::kBarOff + 40);      // [2], row blocks in turn
+    int* s_bad = reinterpret_cast<int*>(smem + Plan::kBarOff + 40);      // [2], row blocks in turn: 1 done again, 2 small sums
+    int* s_inexact = s_bad + 2;                                          // [2]
     float* s_max = reinterpret_cast<float*>(smem + Plan::kMaxOff);
     float* s_sum = reinterpret_cast<float*>(smem + Plan::kSumOff);
 
@@ -192,7 +202,7 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
         ptx::mbar_init(bar_o_done, 1);
         ptx::fence_barrier_init();
         *s_abort = 0;
-        s_bad[0] = s_bad[1] = 0;
+        s_bad[0] = s_bad[1] = s_inexact[0] = s_inexact[1] = 0;
     }
     if (warp == kF32Compute / 32) {
         ptx::tmem_alloc(ptx::smem_u32(s_tmem), 512);
@@ -427,7 +437,7 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                 ptx::fence_proxy_async();
                 arrive(bar_p_ready);
             }
-            bool bad = false;
+            bool bad = false, small = false;
             if (ntiles > 0) {
                 warp_wait(bar_o_done, (base + ntiles - 1) & 1, kDevTimeoutSoftmaxO, a.status, s_abort, lane);
                 ptx::fence_after_sync();
@@ -441,24 +451,32 @@ attn_f32_kernel(const SimtAttnArgs a, const __grid_constant__ TilesT tiles)
                         acc[(h + c) / 2] = ptx::add2(acc[(h + c) / 2], ptx::pack2(__uint_as_float(o[c]), __uint_as_float(o[c + 1])));
                 }
                 ptx::fence_before_sync();
-                // Infinities and undefined numbers do not split, numbers near the smallest normal ones lose their
-                // last part, and a masked key's probability of 0 times an infinite value is undefined: a row block
-                // whose results are not all ordinary is done again row by row, in floats, each row over the keys it sees.
+                // Infinities and undefined numbers do not split, and a masked key's probability of 0 times an infinite value is
+                // undefined: a row block whose results are not all finite is done again row by row, in floats, each row over the keys
+                // it sees; so are small sums of values whose parts are not exact.
 #pragma unroll
                 for (int c = 0; c < kCh / 2; ++c) {
                     float y0, y1;
                     ptx::unpack2(acc[c], y0, y1);
-                    y0 = fabsf(y0);
-                    y1 = fabsf(y1);
-                    bad |= !(y0 + y1 <= 3.0e38f) || (y0 < 1e-30f * kWeightUnit && y0 > 0.f) || (y1 < 1e-30f * kWeightUnit && y1 > 0.f);
+                    bad |= !(fabsf(y0) + fabsf(y1) <= 3.0e38f);
+                    small |= f32_small(y0) || f32_small(y1);
                 }
                 bad = bad && row_valid;
+                small = small && row_valid;
             }
             s_sum[part * 128 + r_tile] = l;
-            if (bad) atomicOr(&s_bad[turn & 1], 1);
+            if (bad || small) atomicOr(&s_bad[turn & 1], (bad ? 1 : 0) + (small ? 2 : 0));
             all_compute();
-            if (tid == 0) s_bad[(turn & 1) ^ 1] = 0;
-            if (*(volatile int*)&s_bad[turn & 1] == 0) {
+            if (tid == 0) s_bad[(turn & 1) ^ 1] = s_inexact[(turn & 1) ^ 1] = 0;
+            int again = *(volatile int*)&s_bad[turn & 1];
+            if (again == 2) {                                // (a look at the values costs a fraction of doing the block again)
+                bool inexact = false;
+                for (int i = tid; i < keys * (D / 4); i += kF32Compute) inexact |= f32_inexact(reinterpret_cast<const float4*>(vb)[i]);
+                if (inexact) s_inexact[turn & 1] = 1;
+                all_compute();
+                again = *(volatile int*)&s_inexact[turn & 1];
+            }
+            if (again == 0) {
                 const float sum = (s_sum[r_tile] + s_sum[128 + r_tile]) + (s_sum[256 + r_tile] + s_sum[384 + r_tile]);
                 const float inv = (sum > 0.f) ? 1.f / sum : 0.f;
                 const long prow0 = ((long)split * a.Hkv + g) * R + row0 + quarter * 32;

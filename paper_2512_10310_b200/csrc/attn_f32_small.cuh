@@ -377,12 +377,20 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
                 y[v].w = fmaf(w[i], x.w, y[v].w);
             }
         }
-        // (not ordinary numbers: see attn_f32.cuh)
-        bool odd = *s_huge != 0;
-        auto ordinary = [](float x) { return fabsf(x) <= 3.0e38f && (x == 0.f || fabsf(x) >= 1e-30f * kWeightUnit); };
+        // (done again in floats: see attn_f32.cuh)
+        bool odd = *s_huge != 0, low = false;
 #pragma unroll
-        for (int v = 0; v < kV; ++v) odd |= !(ordinary(y[v].x) && ordinary(y[v].y) && ordinary(y[v].z) && ordinary(y[v].w));
+        for (int v = 0; v < kV; ++v) {
+            odd |= !(fabsf(y[v].x) + fabsf(y[v].y) + fabsf(y[v].z) + fabsf(y[v].w) <= 3.0e38f);
+            low |= f32_small(y[v].x) || f32_small(y[v].y) || f32_small(y[v].z) || f32_small(y[v].w);
+        }
         uint32_t bad = __ballot_sync(0xffffffffu, odd && r < rows);
+        const uint32_t lows = __ballot_sync(0xffffffffu, low && r < rows);
+        if (lows & ~bad) {
+            bool inexact = false;
+            for (int i = lane; i < keys * (D / 4); i += 32) inexact |= f32_inexact(reinterpret_cast<const float4*>(vb)[i]);
+            if (__any_sync(0xffffffffu, inexact)) bad |= lows;
+        }
         const long prow0 = ((long)split * a.Hkv + g) * R + row0;
         if (r < rows) {
             const float inv = (sum > 0.f) ? 1.f / sum : 0.f;

@@ -66,6 +66,7 @@ def test_one_call_is_the_three_calls(handle, hq, hkv, d, L, n, splits):
 
 @pytest.mark.parametrize("hq,hkv,d,L,n,scale", [
     (2, 1, 64, 256, 64, 1e-36),    # the parts of such numbers are not exact: done again in floats
+    (28, 4, 128, 1024, 196, 1e-37),
     (4, 2, 128, 500, 70, 1e-36),
     (4, 2, 128, 500, 70, 1e30),
 ])
@@ -192,3 +193,35 @@ def test_no_further_off_than_float_fmas(handle, hq, hkv, d, L, n, kind):
         _, g = _step(handle, cfg, x, kernel=kernel)
         off.append((np.linalg.norm(f64(g["out"]) - r["out"]), np.linalg.norm(f64(g["lse"]) - r["lse"])))
     assert off[1][0] <= 1.25 * off[0][0] and off[1][1] <= 1.25 * off[0][1], off
+
+
+@pytest.mark.parametrize("hq,hkv,d,L,n,first", [
+    (2, 1, 64, 256, 64, 130),      # 32-row blocks
+    (28, 4, 128, 1024, 196, 500),  # equal shares of 128-row blocks
+    (28, 4, 64, 0, 400, 0),        # 128-row blocks, the first key seen by all
+])
+def test_small_sums_of_ordinary_values(handle, hq, hkv, d, L, n, first):
+    # A channel whose only value is at a key of weight 1e-34: as accurate as any, and the other channels are the bits
+    # that they are with something else in it, so nothing was done again in floats for its sake.
+    cfg, x = _inputs(hq, hkv, d, L, n)
+    slow = d // 2 - 1                          # the channel that turns least
+    x["q_new"][:, :, slow] = 40.0
+    x["q_new"][:, :, slow + d // 2] = 0.0
+    keys, values = torch.cat([x["k_cache"], x["k_new"]]), torch.cat([x["v_cache"], x["v_new"]])
+    keys[:, :, slow] = 0.0
+    keys[first] = 0.0
+    keys[first, :, slow] = -75.0 * d ** 0.5 / 40.0
+    outs = []
+    for other in (1.0, 0.0):
+        values[:, :, 5] = other
+        values[first, :, 5] = 1.0
+        y = dict(x, k_cache=keys[:L], k_new=keys[L:], v_cache=values[:L], v_new=values[L:])
+        outs.append(_step(handle, cfg, y)[1]["out"])
+    r = oracle_step("f32", y["k_cache"], y["v_cache"], y["q_new"], y["k_new"], y["v_new"], L, cfg.rope_theta)
+    rows = slice(1 if L == 0 else 0, None)     # (the first token of an empty cache sees that key only)
+    want, got = r["out"][rows, :, 5], f64(outs[1])[rows, :, 5]
+    assert np.abs(want).max() < 1e-30
+    # the weight's exponent is 75 to 80: a score of that size is some units of 2^-24 of itself off
+    assert bool((np.abs(got - want) <= 4e-5 * np.abs(want)).all())
+    keep = [c for c in range(d) if c != 5]
+    assert torch.equal(outs[0][rows][:, :, keep], outs[1][rows][:, :, keep])
