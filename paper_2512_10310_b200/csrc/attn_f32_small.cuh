@@ -202,6 +202,7 @@ attn_f32_small_kernel(const SimtAttnArgs a, const FastDiv div_g, const __grid_co
         }
         for (int it = q_items * 2 + tid; it < kSmallRows * (D / 4); it += NT) store_q(it / (D / 4), it % (D / 4), make_ulonglong2(0ull, 0ull));
         // the new keys and values are in the cache when all blocks of the cluster are here
+        __syncwarp();
         ptx::cluster_arrive();
         ptx::cluster_wait();
         load_rows(kx, kb, max(0, cached), keys);
