@@ -240,7 +240,7 @@ def test_strided_views_of_a_fused_qkv_buffer(handle, n):
 
 
 def test_one_call_step_fp32(handle):
-    # the one-call form on the fp32 configuration (SIMT attention kernel)
+    # the one-call form on the fp32 configuration (one launch, a cluster per row block)
     cfg = W.TINY_F32
     x = W.make_step_inputs(cfg)
     L, n = cfg.cache_len, cfg.num_new
