@@ -107,11 +107,13 @@ __device__ __forceinline__ uint64_t f32_weights(const SimtAttnArgs& a, uint64_t 
     return ptx::mul2(ptx::pack2(ptx::ex2(f0), ptx::ex2(f1)),
                      ptx::pack2(__uint_as_float((__float_as_uint(t0) << 23) + kBias), __uint_as_float((__float_as_uint(t1) << 23) + kBias)));
 }
-// ... what a running sum is multiplied by when its maximum moves up by -d (in fewer steps: the error of a larger exponent goes with a smaller factor)
+// ... what a running sum is multiplied by when its maximum moves up by -d, in fewer steps: the error of a larger exponent goes with a
+// smaller factor.  Factors below the least normal number are kept (ex2 alone would make them 0).
 __device__ __forceinline__ float f32_rescale(const SimtAttnArgs& a, float d)
 {
     d = fmaxf(d, a.diff_min);
-    return ptx::ex2(fmaf(d, a.scale2_hi, d * a.scale2_lo));
+    const float x = fmaf(d, a.scale2_hi, d * a.scale2_lo);
+    return x < -64.f ? ptx::ex2(x + 64.f) * kPerWeightUnit : ptx::ex2(x);
 }
 
 // Log-sum-exp of a row: unscaled maximum and sum of weights.  The sum of the two parts is rounded once.

@@ -196,12 +196,16 @@ def test_no_further_off_than_float_fmas(handle, hq, hkv, d, L, n, kind):
 
 
 @pytest.mark.parametrize("hq,hkv,d,L,n,first", [
-    (2, 1, 64, 256, 64, 130),      # 32-row blocks
-    (28, 4, 128, 1024, 196, 500),  # equal shares of 128-row blocks
-    (28, 4, 64, 0, 400, 0),        # 128-row blocks, the first key seen by all
+    (2, 1, 64, 256, 64, 128),      # 32-row blocks
+    (28, 4, 128, 1024, 196, 512),  # equal shares of 128-row blocks
+    (28, 4, 64, 0, 400, 0),        # 128-row blocks, the first keys seen by all
 ])
-def test_small_sums_of_ordinary_values(handle, hq, hkv, d, L, n, first):
-    # A channel whose only value is at a key of weight 1e-34: as accurate as any, and the other channels are the bits
+@pytest.mark.parametrize("count,depth,value", [
+    (1, 75.0, 1.0),
+    (64, 88.0, 1000.0),            # a key tile whose weights are below the least normal number
+])
+def test_small_sums_of_ordinary_values(handle, hq, hkv, d, L, n, first, count, depth, value):
+    # A channel whose only values are at keys of weights below 1e-33: as accurate as any, and the other channels are the bits
     # that they are with something else in it, so nothing was done again in floats for its sake.
     cfg, x = _inputs(hq, hkv, d, L, n)
     slow = d // 2 - 1                          # the channel that turns least
@@ -209,19 +213,19 @@ def test_small_sums_of_ordinary_values(handle, hq, hkv, d, L, n, first):
     x["q_new"][:, :, slow + d // 2] = 0.0
     keys, values = torch.cat([x["k_cache"], x["k_new"]]), torch.cat([x["v_cache"], x["v_new"]])
     keys[:, :, slow] = 0.0
-    keys[first] = 0.0
-    keys[first, :, slow] = -75.0 * d ** 0.5 / 40.0
+    keys[first:first + count] = 0.0
+    keys[first:first + count, :, slow] = -depth * d ** 0.5 / 40.0
     outs = []
     for other in (1.0, 0.0):
         values[:, :, 5] = other
-        values[first, :, 5] = 1.0
+        values[first:first + count, :, 5] = value
         y = dict(x, k_cache=keys[:L], k_new=keys[L:], v_cache=values[:L], v_new=values[L:])
         outs.append(_step(handle, cfg, y)[1]["out"])
     r = oracle_step("f32", y["k_cache"], y["v_cache"], y["q_new"], y["k_new"], y["v_new"], L, cfg.rope_theta)
-    rows = slice(1 if L == 0 else 0, None)     # (the first token of an empty cache sees that key only)
+    rows = slice(count if L == 0 else 0, None)     # (the first tokens of an empty cache see those keys only)
     want, got = r["out"][rows, :, 5], f64(outs[1])[rows, :, 5]
     assert np.abs(want).max() < 1e-30
-    # the weight's exponent is 75 to 80: a score of that size is some units of 2^-24 of itself off
+    # the weight's exponent is 75 to 95: a score of that size is some units of 2^-24 of itself off
     assert bool((np.abs(got - want) <= 4e-5 * np.abs(want)).all())
     keep = [c for c in range(d) if c != 5]
     assert torch.equal(outs[0][rows][:, :, keep], outs[1][rows][:, :, keep])
