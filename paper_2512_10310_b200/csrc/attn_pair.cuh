@@ -960,11 +960,15 @@ __device__ __forceinline__ void attn_tc_body(const CUtensorMap& tm_q, const CUte
         int nrare = 0;                // meetings on bar_rare so far
         auto move_reference = [&](int released, bool mine, float want) -> bool {
             s_cand[part * 128 + r_tile] = mine ? want : m_ref;
-            if (lane == 0) s_rel[quarter * kParts + part] = released;
+            // (A persistent pair's first product of an item is not issued before all warps have read the rows of the item
+            // before, each after its first tile.  A warp that has not done so yet would wait for itself below: as long as there is
+            // one, nothing of this item is consumed, so that is what it reports.)
+            const int report = PERSIST && turn > 0 && released < first + 2 ? first : released;
+            if (lane == 0) s_rel[quarter * kParts + part] = report;
             __syncwarp();
             if (lane == 0) s_req[quarter] = 1;
             if (!meet(bar_rare, nrare++)) return false;
-            int r_min = released;
+            int r_min = report;
             float m_new = m_ref;
 #pragma unroll
             for (int c = 0; c < kParts; ++c) {

@@ -8,7 +8,7 @@ import torch
 from oracle import step_oracle as so
 from paper_2512_10310_b200 import binding as B
 from paper_2512_10310_b200 import workloads as W
-from tests.helpers import check_output, f64
+from tests.helpers import GpuStep, check_output, f64, oracle_step
 from tests.test_gpu_paged import _check_pools, _gpu_paged
 
 pytestmark = pytest.mark.gpu
@@ -76,6 +76,46 @@ def test_paged_frame_of_one_long_episode(handle, hq, hkv, length, new, least):
     out, lse, k_pool, v_pool = _gpu_paged(handle, cfg, x)
     okp, ovp = f64(x["k_pool"]), f64(x["v_pool"])
     ref_out, ref_lse = so.step_paged(f64(x["q_new"]), f64(x["k_new"]), f64(x["v_new"]), okp, ovp, x["page_table"], [length],
+                                     x["new_offsets"], cfg.rope_theta, storage="bf16")
+    check_output("bf16", out, lse, ref_out, ref_lse)
+    _check_pools(x, cfg, k_pool, v_pool, okp, ovp)
+
+
+RISING = [(130, 17.0), (200, 34.0), (300, 51.0), (420, 68.0)]      # (token, its key): second tile, both halves, third, fourth
+
+
+def _rising_scores(q, k, starts, lengths):
+    # each of these keys is 60 above the one before for all queries, so a row's reference moves at each of them
+    q[:, :, 63], q[:, :, 127] = 40.0, 0.0       # the channel that turns least
+    k[:, :, 63] = 0.0
+    for start, n in zip(starts, lengths):
+        for tok, value in RISING:
+            if tok < n:
+                k[start + tok, :, 63] = value
+
+
+def test_references_move_in_later_items_of_a_pair(handle):
+    # 232 work items on contiguous caches: a pair's second and third start while rows of the one before are still to be read
+    # (0.3: a bf16 operand's rounding grows with the logits that it makes, 1.04 % of a row's rms at 1.0, and values up to 4 are rounded by
+    # more than the absolute gate; neither is what is tested)
+    cfg = dataclasses.replace(W.STEP_7B, name="rising", num_q_heads=64, num_kv_heads=8, cache_len=0, num_new=900, input_scale=0.3, seed=61)
+    x = W.make_step_inputs(cfg)
+    _rising_scores(x["q_new"], x["k_new"], [0], [900])
+    r = oracle_step("bf16", x["k_cache"], x["v_cache"], x["q_new"], x["k_new"], x["v_new"], 0, cfg.rope_theta)
+    for fused in (False, True):
+        gs = GpuStep(handle, "bf16", 64, 8, 128, 900, cfg.rope_theta, 900, fused=fused)
+        g = gs.step(0, x["q_new"], x["k_new"], x["v_new"])
+        check_output("bf16", g["out"], g["lse"], r["out"], r["lse"])
+
+
+def test_references_move_in_later_items_of_a_paged_batch(handle):
+    new = [450, 300, 470, 140, 431, 260]
+    cfg = dataclasses.replace(W.PAGED_B16, name="rising", num_q_heads=64, num_kv_heads=8, batch=len(new), seed=62)
+    x = W.make_paged_inputs(cfg, [0] * len(new), new)
+    _rising_scores(x["q_new"], x["k_new"], x["new_offsets"], new)
+    out, lse, k_pool, v_pool = _gpu_paged(handle, cfg, x)
+    okp, ovp = f64(x["k_pool"]), f64(x["v_pool"])
+    ref_out, ref_lse = so.step_paged(f64(x["q_new"]), f64(x["k_new"]), f64(x["v_new"]), okp, ovp, x["page_table"], [0] * len(new),
                                      x["new_offsets"], cfg.rope_theta, storage="bf16")
     check_output("bf16", out, lse, ref_out, ref_lse)
     _check_pools(x, cfg, k_pool, v_pool, okp, ovp)
