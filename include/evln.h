@@ -65,7 +65,12 @@ typedef enum { EVLN_BF16 = 0, EVLN_F32 = 1 } evlnDType_t;
 /* Attention kernel choice.  AUTO: tensor-core kernels for bf16 with head_dim 128 (tcgen05 MMA, TMEM
  * accumulators, TMA tiles; mma.sync for few rows) and for fp32 (every float as three bf16 parts,
  * fp32 sums: the accuracy of float FMAs); the SIMT kernel for bf16 with head_dim 64.  SIMT forces
- * the SIMT kernel (float FMAs, any dtype), an independent on-device cross-check.                */
+ * the SIMT kernel (float FMAs, any dtype), an independent on-device cross-check.
+ * fp32 in AUTO: numbers of any size give what floats give, except that a value below 2^-134 counts as
+ * 0.  What does not split into bf16 parts is done in floats, a 128- or 32-row block of queries (or a row) at a
+ * time and slower: queries or keys of 2^90 and more (divided by a softmax scale above 1), results that
+ * are not finite or reach 2^64, and tiny results of values below 2^-109.  Softmax scales outside
+ * 2^-60 .. 2^60 take the SIMT kernel.                                                            */
 typedef enum { EVLN_KERNEL_AUTO = 0, EVLN_KERNEL_SIMT = 1 } evlnKernel_t;
 
 typedef struct evlnContext* evlnHandle_t;
@@ -329,7 +334,7 @@ evlnStatus_t evlnPackedForward(evlnHandle_t handle, const evlnPackedParams* para
  * clears it for the current device.
  * Limits and errors: parameters whose split workspace (evlnStepWorkspaceSize) exceeds
  * EVLN_NOALLOC_SCRATCH_BYTES are rejected with EVLN_WORKSPACE_TOO_SMALL and nothing is
- * launched, except that the SIMT kernel with num_splits = 0 takes as many splits as fit
+ * launched, except that fp32 and SIMT steps with num_splits = 0 take as many splits as fit
  * (rejected only if one does not); other errors as for evlnStepAttention / evlnStepCombine.
  * Sharing: every call on a device uses the same scratch array, which keeps the previous
  * call's contents (each call overwrites every partial it later reads, so nothing needs

@@ -1,12 +1,12 @@
 // fp32 step attention on the 5th-generation tensor cores.
 //
-// A float is exactly the sum of three bf16 numbers (8 + 8 + 8 bits and the signs of the rests), so a product of
+// A float is exactly the sum of three bf16 numbers (8 + 8 + 8 bits and the signs of the rests; down to 2^-109), so a product of
 // floats is nine products of bf16 numbers, which the tensor core forms exactly and adds in fp32.  Six of them are
 // taken (the other three are below 2^-26 of the product), the small ones first, so that the accumulator's own
 // rounding (towards zero, at its size of the moment) sees the large ones only.  An accumulator never runs on
 // across key tiles: every tile's products with V start from zero, and so do its scores, in two sums over half of the channels each; the
-// results are added in registers, rounded to nearest.  (What the tensor core cuts off makes a score about 7e-8 too small in one sum of 128
-// channels, half of that in two; a chain of float FMAs is off by twice as much, either way.)
+// results are added in registers, rounded to nearest.  (A score of 128 normal channels against fp64: in one sum 1.3e-7 off, of which
+// 1.0e-7 is what the tensor core cuts off, always towards zero; in two sums 8.6e-8 and 6e-8; a chain of float FMAs 1.5e-7, either way.)
 //
 // Bound: the tensor pipe (6 x 4 D bf16 flop per visible pair), with all SMs at work the latency of K and V out of L2.  A block of 16 + 1 warps owns 128 packed query rows of
 // one kv head and walks its key tiles, 64 keys at a time:
@@ -14,7 +14,7 @@
 //            quarter of the channels.  Per tile they split the next K tile into its three parts (from
 //            registers into swizzled shared memory), take the scores, exchange the row maximum (four threads a
 //            row), split the V tile, add the previous tile's product to the accumulator in registers, and leave the
-//            probabilities' three parts in tensor memory.
+//            probabilities' three parts in tensor memory (at head_dim 128 the third in shared memory).
 //   1 warp   issues: S_j = Q K_j^T (A = Q's parts in tensor memory) and O_j = P_j V_j (A = P_j's parts), in the order
 //            S_0, S_1, O_0, S_2, O_1, ..: the scores of a tile run while the softmax of the one before does.
 // Tensor memory columns: Q's parts 0 .. 3 D/2, O_j (D), S_j (two sums of 64: even and odd 16 channels), P_j's first two parts (64); all 512 at
@@ -22,8 +22,8 @@
 //
 // SHARE: as in attn_simt.cuh, one block per SM with an equal share of all (row block, key tile) pairs.
 //
-// Measured: a tile 2.2 us at head_dim 128 (the products alone 1.9; about 3 with a block on every SM), 1.5 at 64; 196 tokens of the 7B shape over 1024 keys 96.7 us a step
-// in float FMAs, 33.0 so; 256 tokens over 2048 206 and 60; 252 tokens of 16 heads over 2031 123 and 37.
+// Measured: a tile 2.2 us at head_dim 128 (the products alone 1.9; about 3 with a block on every SM), 1.5 at 64; 196 tokens of the 7B shape over 1024 keys 95.3 us a step
+// in float FMAs, 33.2 so (32.0 with the scores in one sum); 256 tokens over 2048 206 and 62; 252 tokens of 16 heads over 2031 123 and 37.9.
 #pragma once
 
 #include "attn_pair.cuh"

@@ -5,8 +5,8 @@
 // A block: 32 packed query rows of one kv head (two 16-row tiles) and a split of its keys, 64 at a time.  All warps split
 // the K and V tiles into their parts (registers to swizzled shared memory, the next tile's loads in flight); then warp
 // (w % 2, w / 2) has 16 rows and 16 of the tile's keys to itself: scores, probabilities and a running maximum, sum and
-// output of its own.  Every product starts from zero and is added in registers, the small parts on their
-// own, so that the tensor core's cut-off sums stay as short as in attn_f32.cuh.  The four warps of a row are merged in shared memory.
+// output of its own.  The large parts' product of every 16 channels and every tile's product with V start from zero and are
+// added in registers, the small parts of a score are a sum of their own, so that the tensor core cuts off even less than in attn_f32.cuh.  The four warps of a row are merged in shared memory.
 //
 // FUSED: evlnStep as one launch.  The splits of a row block are a cluster.  Its blocks rotate the row block's queries (each
 // all of them, into q_rot and its own shared memory) and the new keys (a share each, into the cache with the values; blocks of

@@ -463,7 +463,7 @@ __device__ __forceinline__ void write_rows(const TcAttnArgs& a, const LensT& len
 
 // --- the kernel ---------------------------------------------------------------------------
 // CTAS = 2: launched with a cluster of 2 CTAs along x: query tile = cluster rank.
-// CTAS = 1: no cluster; one query tile (all the rows of a kv head fit in it).
+// CTAS = 1: no cluster; a query tile per CTA (all rows of a kv head, or a unit of 128 of a short unsplit step).
 
 // TAIL: a packed sequence (Sec. 3.3) in one launch.  Its visual run is an ordinary causal prefill on the
 // cache (tm_q, tm_k, tm_v).  Its action chunks are a batch of items that share the first L_b tokens of
@@ -1275,7 +1275,8 @@ attn_packed_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     attn_tc_body<false, true, true, BatchLens, 2, ItemTable>(tm_q, tm_k, tm_v, &tm_qt, &tm_kt, &tm_vt, a, lens, d, table);
 }
 
-// One CTA per work item, for steps whose rows per kv head fit one 128-row tile (the few action
+// One CTA per work item, for short unsplit steps (a CTA per 128-row tile, final rows to the caller where the call
+// allows) and for steps whose rows per kv head fit one tile (the few action
 // tokens that follow a frame, Sec. 3.1): the KV range is cut into up to 32 splits (choose_splits_solo) and
 // each CTA streams whole K/V tiles, so that a long cache is read at the rate HBM delivers it.
 __global__ void __launch_bounds__(kTcThreads, 1)

@@ -435,8 +435,8 @@ size_t partial_bytes(int splits, int Hkv, long rows, int D)
     return round_up((size_t)splits * Hkv * rows * (D + 1) * sizeof(float), 256);
 }
 
-// Row tile and split count of the SIMT kernel (splits > 0: given), by a model of measured times at
-// head_dim 128 (head_dim 64: about half).  A block of 128 rows runs alone on its SM, 13.3 us per 64-key
+// Row tile and split count of the SIMT and fp32 kernels (splits > 0: given), by a model of measured times at
+// head_dim 128 (head_dim 64: about half).  SIMT: a block of 128 rows runs alone on its SM, 13.3 us per 64-key
 // tile and 7 us for its start and write-out; a block of 32 rows takes 6.3 us per tile and 5 us when it
 // has the SM to itself, 9.5 per tile when two share it.  So 128-row tiles are 1.4 times cheaper per row
 // where they fill the chip, 32-row tiles have twice the latency advantage where they would not.  A
@@ -490,7 +490,6 @@ SimtSchedule simt_schedule(evlnHandle_t h, const evlnStepParams* p, int splits, 
             double cost;
             bool one_launch = false;
             if (tensor && rpt == 2) {
-                if (ceil_div(R, kSmallRows) > 65535) break;
                 const double block_us = ceil_div(tiles, s) * (3.8 * d - 0.1) + 1.0;
                 cost = (double)((blocks + h->num_sms - 1) / h->num_sms) * block_us + 6.0 + (split_us - 0.2) * s;
                 const int tokens = f32_angle_tokens(p, s), fit = tokens <= kSmallAngleTokens && s <= kSmallCluster ? h->small_clusters[s - 1] : 0;
@@ -1343,7 +1342,7 @@ static bool new_tokens_in_cache(const evlnStepParams* p, const void* k_new, cons
 }
 
 // Attention of a step.  `direct` (may be null): the step's final output; when the keys are not split and
-// the pair kernel runs, it writes that itself and `done` says that there is nothing left to combine.
+// the pair or the one-CTA kernel runs, it writes that itself and `done` says that there is nothing left to combine.
 struct DirectOut {
     void* out;
     float* lse_out;
@@ -2212,7 +2211,7 @@ extern "C" evlnStatus_t evlnStepAttentionNoAlloc(const evlnStepParams* p, const 
     if (p->num_new == 0) return EVLN_OK;
     evlnStepParams fitting = *p;
     if (need > (size_t)EVLN_NOALLOC_SCRATCH_BYTES) {
-        // The fp32 kernel splits to fill the chip, up to 2.3 times faster than what fits here for large steps, so it is
+        // The fp32 and SIMT kernels split to fill the chip, up to 2.3 times faster than what fits here for large steps, so it is
         // this call that makes do with fewer splits.  (The schedules of the other kernels take about as few as they can.)
         const size_t one = partial_bytes(1, p->num_kv_heads, (long)p->num_new * (p->num_q_heads / p->num_kv_heads), p->head_dim);
         const int fit = (int)(EVLN_NOALLOC_SCRATCH_BYTES / one);

@@ -95,7 +95,7 @@ def test_no_alloc_rejects_oversized_problems():
     (32, 16, 128, 100, 2000),     # 33.0 MB in one split: just inside
 ])
 def test_no_alloc_takes_the_splits_that_fit(hq, hkv, d, L, n):
-    # steps of the SIMT kernel whose own split count needs more than the built-in scratch
+    # fp32 steps whose own split count needs more than the built-in scratch
     if not torch.cuda.is_available():
         pytest.skip("needs a CUDA device")
     dev = "cuda:0"
